@@ -93,10 +93,10 @@ const char *rs_last_error(const rs_ctx *ctx);
  * are the ones the library's tuner chose on a GB300 (the tuner, its
  * coordinate descent and its result check are in the Python package).
  *   link_blocks_per_sm  big-node link search: resident warps per SM the
- *                       kernel is compiled for, in units of eight (4, 5 or 6:
- *                       32, 40 or 48 warps);
- *   nn_blocks_per_sm    big-node nearest-neighbour search, the same (5, 6
- *                       or 7);
+ *                       kernel is compiled for (4, 5 or 6: 24, 32 or 40
+ *                       warps);
+ *   nn_blocks_per_sm    big-node nearest-neighbour search, the same in units
+ *                       of eight (5, 6 or 7: 40, 48 or 56 warps);
  *   kd_levels           big-node levels whose members are put in k-d order
  *                       (0-3; deeper levels keep their parent's order);
  *   bracket_min         big nodes above this many members search with the

@@ -41,6 +41,8 @@
 #include <cmath>
 #include <cstring>
 
+#include <cuda_fp16.h>
+
 #include "rs_refine.cuh"
 
 namespace {
@@ -1003,76 +1005,9 @@ __device__ __forceinline__ Box6 box_empty()
     return b;
 }
 
-__device__ __forceinline__ void box_add(Box6 &b, float4 p, float4 v)
-{
-    b.plo.x = fminf(b.plo.x, p.x); b.plo.y = fminf(b.plo.y, p.y); b.plo.z = fminf(b.plo.z, p.z);
-    b.phi.x = fmaxf(b.phi.x, p.x); b.phi.y = fmaxf(b.phi.y, p.y); b.phi.z = fmaxf(b.phi.z, p.z);
-    b.vlo.x = fminf(b.vlo.x, v.x); b.vlo.y = fminf(b.vlo.y, v.y); b.vlo.z = fminf(b.vlo.z, v.z);
-    b.vhi.x = fmaxf(b.vhi.x, v.x); b.vhi.y = fmaxf(b.vhi.y, v.y); b.vhi.z = fmaxf(b.vhi.z, v.z);
-}
-
-__device__ __forceinline__ void box_merge(Box6 &b, const Box6 &c)
-{
-    b.plo.x = fminf(b.plo.x, c.plo.x); b.plo.y = fminf(b.plo.y, c.plo.y); b.plo.z = fminf(b.plo.z, c.plo.z);
-    b.phi.x = fmaxf(b.phi.x, c.phi.x); b.phi.y = fmaxf(b.phi.y, c.phi.y); b.phi.z = fmaxf(b.phi.z, c.phi.z);
-    b.vlo.x = fminf(b.vlo.x, c.vlo.x); b.vlo.y = fminf(b.vlo.y, c.vlo.y); b.vlo.z = fminf(b.vlo.z, c.vlo.z);
-    b.vhi.x = fmaxf(b.vhi.x, c.vhi.x); b.vhi.y = fmaxf(b.vhi.y, c.vhi.y); b.vhi.z = fmaxf(b.vhi.z, c.vhi.z);
-}
-
 // warp min/max votes on order-preserving integer images
 __device__ __forceinline__ float wmin_f(float x) { return ord_f(__reduce_min_sync(0xffffffffu, ord_i(x))); }
 __device__ __forceinline__ float wmax_f(float x) { return ord_f(__reduce_max_sync(0xffffffffu, ord_i(x))); }
-
-// Leaf boxes and the packed member copy, one warp per leaf over the whole
-// level (tiles of 256 members, eight leaves each).
-__global__ void __launch_bounds__(TQ) k_bvh_leaves(LevelBufs L, NodeArrays nd, const int64_t *box_base, BoxStore B,
-                                                   MemberStore MS, const float4 *wpos, const float4 *wvel)
-{
-    const int k = L.tile_rank[blockIdx.x], q0 = L.tile_q0[blockIdx.x] + 32 * warp_id();
-    const int node = L.list[k], first = nd.first[node], n = nd.count[node];
-    if (q0 >= n) return;
-    const int m = q0 + lane_id();
-    const bool ok = m < n;
-    float4 p = make_float4(0, 0, 0, 0), v = p;
-    if (ok) {
-        p = wpos[first + m];
-        v = wvel[first + m];
-        MS.a[first + m] = make_float4(p.x, p.y, p.z, v.x);
-        MS.b[first + m] = make_float2(v.y, v.z);
-    }
-    Box6 b;
-    b.plo = make_float4(wmin_f(ok ? p.x : INFINITY), wmin_f(ok ? p.y : INFINITY), wmin_f(ok ? p.z : INFINITY), 0.f);
-    b.phi = make_float4(wmax_f(ok ? p.x : -INFINITY), wmax_f(ok ? p.y : -INFINITY), wmax_f(ok ? p.z : -INFINITY), 0.f);
-    b.vlo = make_float4(wmin_f(ok ? v.x : INFINITY), wmin_f(ok ? v.y : INFINITY), wmin_f(ok ? v.z : INFINITY), 0.f);
-    b.vhi = make_float4(wmax_f(ok ? v.x : -INFINITY), wmax_f(ok ? v.y : -INFINITY), wmax_f(ok ? v.z : -INFINITY), 0.f);
-    if (lane_id() == 0) box_put(box_shift(B, box_base[k]), q0 / BVH_LEAF, b);
-}
-
-// one block per node: the levels above the leaves
-__global__ void __launch_bounds__(256) k_bvh_build(LevelBufs L, NodeArrays nd, const int64_t *box_base, BoxStore B)
-{
-    const int k = blockIdx.x;
-    if (k >= L.K) return;
-    const int node = L.list[k], n = nd.count[node];
-    const int nl = (int)ceil_div(n, BVH_LEAF);
-    const BoxStore bx = box_shift(B, box_base[k]);
-    const int H = bvh_levels(nl);
-    int64_t off_prev = 0, off = nl;
-    int cprev = nl;
-    for (int h = 1; h < H; h++) {
-        const int cnt = (cprev + 31) >> BVH_LOG;
-        for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-            Box6 b = box_get(bx, off_prev + 32 * i);
-            const int e = min(cprev, 32 * i + 32);
-            for (int c = 32 * i + 1; c < e; c++) box_merge(b, box_get(bx, off_prev + c));
-            box_put(bx, off + i, b);
-        }
-        __syncthreads();
-        off_prev = off;
-        off += cnt;
-        cprev = cnt;
-    }
-}
 
 __device__ __forceinline__ float point_box_d2(float4 p, float4 v, const Box6 &b, const Metric6 &m)
 {
@@ -1169,70 +1104,159 @@ __device__ __forceinline__ float point_box_far2(float4 p, float4 v, const Box6 &
     return (fx * fx + fy * fy + fz * fz) * m.ax + (fu * fu + fv * fv + fw * fw) * m.av;
 }
 
-// One block per node, once the linking length is known.  The boxes are
-// rebuilt over the members that can have a friend (nearest-neighbour value
-// within reach; the link search skips the others as candidates and as
-// queries), which drops the phase-space outliers that stretch them.  A box
-// whose members all can have a friend and whose diameter is within the
-// clique margin is flagged, and the members of every maximal flagged box (a
-// flagged box whose parent is not flagged) are joined.
-__global__ void __launch_bounds__(256) k_bvh_linkbox(LevelBufs L, NodeArrays nd, const int64_t *box_base, BoxStore B,
-                                                     const float4 *wpos, const float4 *wvel, const float *dnn,
-                                                     int *parent, rs_dev_status *st)
+// ---- building the boxes ----
+// Two forms.  Before the searches (LINK false): boxes over all members, and
+// the packed member copy.  Once the linking length is known (LINK true): the
+// boxes are rebuilt over the members that can have a friend (nearest-
+// neighbour value within reach; the others are neither queries nor
+// candidates, and their packed x becomes infinite, which no box is within
+// reach of), which drops the phase-space outliers that stretch them.  A box
+// whose members all can have a friend and whose diameter is within the clique
+// margin is flagged, and its members are joined: a leaf's when its members'
+// union-find entries are first written, an upper box's by joining the first
+// members of its children (a flagged box's children are flagged, their
+// diameters being no larger).
+__device__ __forceinline__ float link_part(double l2)
+{
+    return fmaxf((float)(l2 * (1.0 + RS_BAND)), (float)(l2 * (1.0 + 3e-6)));
+}
+
+// the union of one box per lane, in every lane
+__device__ __forceinline__ Box6 warp_box(const Box6 &c)
+{
+    Box6 b;
+    b.plo = make_float4(wmin_f(c.plo.x), wmin_f(c.plo.y), wmin_f(c.plo.z), 0.f);
+    b.phi = make_float4(wmax_f(c.phi.x), wmax_f(c.phi.y), wmax_f(c.phi.z), 0.f);
+    b.vlo = make_float4(wmin_f(c.vlo.x), wmin_f(c.vlo.y), wmin_f(c.vlo.z), 0.f);
+    b.vhi = make_float4(wmax_f(c.vhi.x), wmax_f(c.vhi.y), wmax_f(c.vhi.z), 0.f);
+    return b;
+}
+
+// Leaf boxes (one warp a leaf) and the boxes of 32 leaves above them.  A
+// block takes the 1024 members of one such box: the tiles' grid, of which the
+// blocks of every fourth tile work.  Against one thread a leaf in one block a
+// node (the link form before: 3.5 ms of a 16.8M-particle path, its largest
+// node alone on one SM), the loads coalesce and a large node spreads over the
+// device.
+template <bool LINK>
+__global__ void __launch_bounds__(TQ) k_bvh_leaves(LevelBufs L, NodeArrays nd, const int64_t *box_base, BoxStore B,
+                                                   MemberStore MS, const float4 *wpos, const float4 *wvel,
+                                                   const float *dnn, int *parent, int *csize, int *cmin,
+                                                   rs_dev_status *st)
+{
+    __shared__ float bs[32][12];
+    __shared__ unsigned char cs[32];
+    const int qb = L.tile_q0[blockIdx.x];
+    if (qb & 1023) return;
+    const int k = L.tile_rank[blockIdx.x];
+    const int node = L.list[k], first = nd.first[node], n = nd.count[node];
+    const int lane = lane_id();
+    const BoxStore bx = box_shift(B, box_base[k]);
+    Metric6 met;
+    met.ax = L.met[k].ax;
+    met.av = L.met[k].av;
+    const float part = LINK ? link_part(L.l2[k]) : 0.f;
+    const float clim = LINK ? (float)(L.l2[k] * RS_CLIQUE_MARGIN) : 0.f;
+    for (int j = warp_id(); j < 32; j += TQ / 32) {
+        const int q0 = qb + 32 * j, m = q0 + lane;
+        if (q0 >= n) break;
+        const bool ok = m < n;
+        bool act = ok;
+        float4 p = make_float4(0, 0, 0, 0), v = p;
+        if (ok) {
+            if (LINK) {
+                mem_get(mem_shift(MS, first), m, p, v);
+                act = dnn[first + m] <= part;
+                if (!act) MS.a[first + m].x = INFINITY;
+            } else {
+                p = wpos[first + m];
+                v = wvel[first + m];
+                MS.a[first + m] = make_float4(p.x, p.y, p.z, v.x);
+                MS.b[first + m] = make_float2(v.y, v.z);
+            }
+        }
+        Box6 b = box_empty();
+        if (act) {
+            b.plo = b.phi = p;
+            b.vlo = b.vhi = v;
+        }
+        b = warp_box(b);
+        bool clique = false;
+        if (LINK) {
+            clique = __ballot_sync(0xffffffffu, act) == __ballot_sync(0xffffffffu, ok) && box_diam2(b, met) <= clim;
+            if (ok) {
+                parent[first + m] = clique ? first + q0 : first + m;
+                csize[first + m] = 0;
+                cmin[first + m] = 0x7fffffff;
+            }
+        }
+        if (lane == 0) {
+            box_put(bx, q0 / BVH_LEAF, b);
+            if (LINK) bx.cl[q0 / BVH_LEAF] = cs[j] = clique ? 1 : 0;
+            float *o = bs[j];
+            o[0] = b.plo.x; o[1] = b.plo.y; o[2] = b.plo.z; o[3] = b.vlo.x; o[4] = b.vlo.y; o[5] = b.vlo.z;
+            o[6] = b.phi.x; o[7] = b.phi.y; o[8] = b.phi.z; o[9] = b.vhi.x; o[10] = b.vhi.y; o[11] = b.vhi.z;
+        }
+    }
+    __syncthreads();
+    const int nl = (int)ceil_div(n, BVH_LEAF), i0 = qb / BVH_LEAF;
+    if (warp_id() != 0 || nl < 2) return;
+    const bool have = i0 + lane < nl;
+    Box6 b = box_empty();
+    if (have) {
+        const float *o = bs[lane];
+        b.plo = make_float4(o[0], o[1], o[2], 0.f);
+        b.vlo = make_float4(o[3], o[4], o[5], 0.f);
+        b.phi = make_float4(o[6], o[7], o[8], 0.f);
+        b.vhi = make_float4(o[9], o[10], o[11], 0.f);
+    }
+    b = warp_box(b);
+    const bool clique = LINK && !__any_sync(0xffffffffu, have && !cs[lane]) && box_diam2(b, met) <= clim;
+    if (lane == 0) {
+        box_put(bx, nl + (qb >> 10), b);
+        if (LINK) bx.cl[nl + (qb >> 10)] = clique ? 1 : 0;
+    }
+    if (clique && have && lane > 0) uf_union(parent, first + qb, first + qb + 32 * lane, st);
+}
+
+// the levels above, one block a node, one warp a box
+template <bool LINK>
+__global__ void __launch_bounds__(256) k_bvh_build(LevelBufs L, NodeArrays nd, const int64_t *box_base, BoxStore B,
+                                                   int *parent, rs_dev_status *st)
 {
     const int k = blockIdx.x;
     if (k >= L.K) return;
-    const int node = L.list[k], first = nd.first[node], n = nd.count[node];
-    const Metric6 met = L.met[k];
-    const LinkLim lm = link_lim(L.l2[k]);
-    const float lim = (float)(L.l2[k] * RS_CLIQUE_MARGIN);
-    __shared__ int lv_s[2 * BVH_MAXH];
-    if (threadIdx.x == 0) bvh_fill(lv_s, (int)ceil_div(n, BVH_LEAF));
-    __syncthreads();
-    BvhView V;
-    bvh_set(V, B, box_base[k], n, lv_s);
-    // leaves; the flag holds "every member can have a friend" until the end
-    for (int i = threadIdx.x; i < V.nl; i += blockDim.x) {
-        Box6 b = box_empty();
-        bool all = true;
-        const int e = min(n, (i + 1) * BVH_LEAF);
-        for (int m = i * BVH_LEAF; m < e; m++) {
-            if (dnn[first + m] <= lm.part)
-                box_add(b, wpos[first + m], wvel[first + m]);
-            else
-                all = false;
-        }
-        box_put(V.S, i, b);
-        V.S.cl[i] = all ? 1 : 0;
-    }
-    __syncthreads();
-    for (int h = 1; h < V.H; h++) {
-        const int cprev = V.cnt[h - 1];
-        for (int i = threadIdx.x; i < V.cnt[h]; i += blockDim.x) {
-            Box6 b = box_get(V.S, V.off[h - 1] + 32 * i);
-            bool all = V.S.cl[V.off[h - 1] + 32 * i] != 0;
-            const int e = min(cprev, 32 * i + 32);
-            for (int c = 32 * i + 1; c < e; c++) {
-                box_merge(b, box_get(V.S, V.off[h - 1] + c));
-                all = all && V.S.cl[V.off[h - 1] + c] != 0;
+    const int node = L.list[k], n = nd.count[node], first = nd.first[node];
+    const int nl = (int)ceil_div(n, BVH_LEAF);
+    const BoxStore bx = box_shift(B, box_base[k]);
+    const int H = bvh_levels(nl), lane = lane_id();
+    Metric6 met;
+    met.ax = L.met[k].ax;
+    met.av = L.met[k].av;
+    const float clim = LINK ? (float)(L.l2[k] * RS_CLIQUE_MARGIN) : 0.f;
+    int cprev = (nl + 31) >> BVH_LOG;
+    int64_t off_prev = nl, off = nl + cprev;
+    for (int h = 2; h < H; h++) {
+        const int cnt = (cprev + 31) >> BVH_LOG;
+        for (int i = warp_id(); i < cnt; i += 8) {
+            const int c = 32 * i + lane;
+            const bool have = c < cprev;
+            Box6 b = box_empty();
+            if (have) b = box_get(bx, off_prev + c);
+            b = warp_box(b);
+            const bool clique = LINK && !__any_sync(0xffffffffu, have && !bx.cl[off_prev + c]) &&
+                                box_diam2(b, met) <= clim;
+            if (lane == 0) {
+                box_put(bx, off + i, b);
+                if (LINK) bx.cl[off + i] = clique ? 1 : 0;
             }
-            box_put(V.S, V.off[h] + i, b);
-            V.S.cl[V.off[h] + i] = all ? 1 : 0;
+            if (clique && have && lane > 0)
+                uf_union(parent, first + (int)bvh_m0(h, i), first + (int)bvh_m0(h - 1, c), st);
         }
         __syncthreads();
-    }
-    const int total = V.off[V.H - 1] + 1;
-    for (int b = threadIdx.x; b < total; b += blockDim.x)
-        if (V.S.cl[b] && !(box_diam2(box_get(V.S, b), met) <= lim)) V.S.cl[b] = 0;
-    __syncthreads();
-    for (int b = threadIdx.x; b < total; b += blockDim.x) {
-        if (!V.S.cl[b]) continue;
-        int h = 0;
-        while (h + 1 < V.H && V.off[h + 1] <= b) h++;
-        const int i = b - V.off[h];
-        if (h + 1 < V.H && V.S.cl[V.off[h + 1] + (i >> BVH_LOG)]) continue;  // not maximal
-        const int m0 = (int)bvh_m0(h, i), m1 = (int)min((int64_t)n, bvh_m0(h, i + 1));
-        for (int m = m0 + 1; m < m1; m++) uf_union(parent, first + m0, first + m, st);
+        off_prev = off;
+        off += cnt;
+        cprev = cnt;
     }
 }
 
@@ -1516,115 +1540,100 @@ __device__ __forceinline__ int join_friend(int *parent, int a, int b, int rq, rs
     return uf_union_root(parent, a, b, st);
 }
 
-// Child c = 32 i + lane of stack entry `ent` for a friends-of-friends search
-// of member q: true when the child can hold a friend after q (its member
-// range extends past q + 1 and its box is within reach).  A clique box wholly
-// within reach is joined with one union and not searched.
-__device__ __forceinline__ bool link_child(const BvhView &V, int ent, int lane, int q, int own, float4 pq, float4 vq,
-                                           const Metric6 &met, const LinkLim &lm, int *parent, int first, int rq,
-                                           rs_dev_status *st)
+// ---- friends-of-friends at l: one warp per leaf, pairs found by the matrix units ----
+// A warp takes the 32 members of a leaf together.  It walks the hierarchy
+// once for all of them, box against box, for the leaves within reach of its
+// own leaf's box; keeps, of each such leaf's 32 members, those within reach of
+// the box (a tenth to a seventh of them on the catalogues of synth.py); and
+// tests the kept ones, 32 at a time, against its 32 members.  That test is a
+// contraction: with coordinates u = (x - c) w relative to the leaf box's
+// centre c, in units of the linking radius, d^2 - T = -2 u_q.u_c + |u_c|^2 +
+// (|u_q|^2 - T) is one m16n8k8 half-precision product for 16 x 8 pairs (six
+// coordinates and |u_c|^2 in two halves against ones, the query's term in the
+// accumulator), and its sign alone is used: a pair it calls far is farther
+// than the linking radius, because T leaves room for every rounding:
+//   the rounded points u^ (half, relative 2^-11) differ from u by at most
+//   delta = 1.02 2^-11 (|u_q| + |u_c|) + 3.1e-4 (the float32 steps before,
+//   and subnormal halves even if they counted as zero), so friends have
+//   |u^_q - u^_c| <= 1 + delta; the norms are taken of the rounded points, so
+//   the product is |u^_q - u^_c|^2 up to float32 accumulation and the second
+//   half's rounding, below 2^-18 (|u_q| + |u_c|)^2 + 1e-4.
+// T stays below 1.02 for the usual boxes (2.7 linking lengths in radius), so
+// the few pairs it lets through (about 20 of 1024) are nearly all friends;
+// they are queued and evaluated 32 at a time in full, as float32 differences
+// of the members' own coordinates with the float64 recheck in the band.  A
+// leaf whose box is too large for half precision (or whose l is 0) queues
+// every kept pair instead.
+//
+// Bound by instruction issue and the latency of the dependent walk.  Walking
+// once a leaf instead of once a query cut the link of the 134M-particle path
+// (7 levels) from 240 to 68 ms, of 9.6M members in independent groups from 46
+// to 13.8 ms, of a 2M path from 4.3 to 0.85 ms.  32 resident warps (64
+// registers) against 40 (48, spilling: 74 ms) and 48 (81 ms).
+constexpr int LK_STACK = 256;   // link stack entries per warp
+constexpr int LK_LEAVES = 128;  // pending leaves per warp
+constexpr int LK_RING = 128;    // kept candidates per warp (a ring; 32 are consumed at a time)
+constexpr float LK_RMAX = 100.f;  // largest box radius, in linking lengths, for the half-precision test
+
+__device__ __forceinline__ void mma_m16n8k8_f16(float (&d)[4], unsigned a0, unsigned a1, unsigned b0, float c0,
+                                                float c1, float c2, float c3)
 {
-    if (ent < 0) return false;
-    const int ch = (ent >> 24) - 1, c = 32 * (ent & 0xffffff) + lane;
-    if (!(c < V.cnt[ch] && !(ch == 0 && c == own) && bvh_m0(ch, c + 1) > (int64_t)q + 1)) return false;
-    const int64_t bi = V.off[ch] + c;
-    const Box6 bx = box_get(V.S, bi);
-    // the clique flag is loaded with the box, not after the reach test, so
-    // its latency overlaps the box loads instead of following them
-    const unsigned char clique = V.S.cl[bi];
-    if (!(point_box_d2(pq, vq, bx, met) <= lm.lim)) return false;
-    if (clique && point_box_far2(pq, vq, bx, met) <= lm.cl_lim) {
-        join_friend(parent, first + q, first + (int)bvh_m0(ch, c), rq, st);
-        return false;
-    }
-    return true;
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%7,%8,%9,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(b0), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
 }
 
-constexpr int LK_STACK = 256;  // link stack entries per warp
-constexpr int LK_LEAVES = 128; // pending leaves per warp
-constexpr int LK_BATCH = 2;    // leaves scanned together
-
-// Friends-of-friends pairs of member q with the members after it (outside
-// its own leaf) by a whole warp; returns this lane's tie count.  The search
-// pops two boxes at a time and collects the leaves within reach in a list,
-// which it scans LK_BATCH leaves at a time (one member per lane and leaf), so
-// several independent loads are in flight per warp.
-__device__ __forceinline__ int w32_link(const BvhView &V, const MemberStore &M, const float *D, int n,
-                                        int q, float4 pq, float4 vq, const Metric6 &met, const Metric6 *met64,
-                                        const double *l2p, const LinkLim &lm, int own,
-                                        int *parent, int first, int *si, int *lf, int &rq, rs_dev_status *st,
-                                        int node)
+// box-to-box lower bound on the squared distance (each gap is one rounded
+// float32 difference of members' coordinates, as in point_box_d2)
+__device__ __forceinline__ float box_box_d2(const Box6 &a, const Box6 &b, const Metric6 &m)
 {
-    const int lane = lane_id();
-    int tie = 0;
-    if (V.H < 2) return 0;
-    if (lane == 0) si[0] = (V.H - 1) << 24;
-    int sp = 1, nl = 0;
-    __syncwarp();
-    const unsigned below = (1u << lane) - 1u;
-    for (int it = 0; (sp > 0 || nl > 0) && it < (1 << 24); it++) {
-        if (sp > 0 && nl <= LK_LEAVES - 64) {
-            const int ea = si[sp - 1];
-            const int eb = sp >= 2 ? si[sp - 2] : -1;
-            __syncwarp();
-            sp -= eb >= 0 ? 2 : 1;
-            const bool na = link_child(V, ea, lane, q, own, pq, vq, met, lm, parent, first, rq, st);
-            const bool nb = link_child(V, eb, lane, q, own, pq, vq, met, lm, parent, first, rq, st);
-            const unsigned ma = __ballot_sync(FULLW, na), mb = __ballot_sync(FULLW, nb);
-            if (sp + __popc(ma) + __popc(mb) > LK_STACK) {
-                if (lane == 0) dev_fail(st, DEV_OVERFLOW, 55, node);
-                return tie;
-            }
-            const int ents[2] = {ea, eb};
-            const unsigned ms[2] = {ma, mb};
-            const bool nd2[2] = {na, nb};
-            for (int u = 0; u < 2; u++) {
-                if (!ms[u]) continue;
-                const int ch = (ents[u] >> 24) - 1, c = 32 * (ents[u] & 0xffffff) + lane;
-                const int slot = __popc(ms[u] & below);
-                if (ch == 0) {
-                    if (nd2[u]) lf[nl + slot] = c;
-                    nl += __popc(ms[u]);
-                } else {
-                    if (nd2[u]) si[sp + slot] = (ch << 24) | c;
-                    sp += __popc(ms[u]);
-                }
-            }
-            __syncwarp();
-            continue;
-        }
-        // scan the collected leaves
-        while (nl > 0) {
-            const int kk = min(nl, LK_BATCH);
-            nl -= kk;
-            int mm[LK_BATCH];
-#pragma unroll
-            for (int u = 0; u < LK_BATCH; u++) mm[u] = u < kk ? lf[nl + u] * BVH_LEAF + lane : -1;
-            __syncwarp();
-            float dd[LK_BATCH];
-            float4 pp[LK_BATCH], vv[LK_BATCH];
-#pragma unroll
-            for (int u = 0; u < LK_BATCH; u++) {
-                dd[u] = INFINITY;
-                if (mm[u] > q && mm[u] < n) {
-                    dd[u] = D[mm[u]];
-                    mem_get(M, mm[u], pp[u], vv[u]);
-                }
-            }
-            int nr = 0x7fffffff;
-#pragma unroll
-            for (int u = 0; u < LK_BATCH; u++) {
-                if (dd[u] <= lm.part) {
-                    const int r = pair_test(lm, met, met64, l2p, pq, vq, pp[u], vv[u]);
-                    tie += r >> 1;
-                    if (r & 1) nr = min(nr, join_friend(parent, first + q, first + mm[u], rq, st));
-                }
-            }
-            rq = min(rq, (int)__reduce_min_sync(FULLW, (unsigned)nr));
-        }
-    }
-    return tie;
+    const float gx = fmaxf(0.f, fmaxf(b.plo.x - a.phi.x, a.plo.x - b.phi.x)),
+                gy = fmaxf(0.f, fmaxf(b.plo.y - a.phi.y, a.plo.y - b.phi.y)),
+                gz = fmaxf(0.f, fmaxf(b.plo.z - a.phi.z, a.plo.z - b.phi.z));
+    const float gu = fmaxf(0.f, fmaxf(b.vlo.x - a.vhi.x, a.vlo.x - b.vhi.x)),
+                gv = fmaxf(0.f, fmaxf(b.vlo.y - a.vhi.y, a.vlo.y - b.vhi.y)),
+                gw = fmaxf(0.f, fmaxf(b.vlo.z - a.vhi.z, a.vlo.z - b.vhi.z));
+    return (gx * gx + gy * gy + gz * gz) * m.ax + (gu * gu + gv * gv + gw * gw) * m.av;
 }
+
+// the six coordinates of a member relative to the box centre, in units of
+// the linking radius, rounded to half; returns the squared norm of the
+// rounded point
+struct HalfPoint {
+    __half h[6];
+};
+__device__ __forceinline__ float half_point(float4 p, float4 v, float4 pc, float4 vc, float wx, float wv, HalfPoint &o)
+{
+    const float u[6] = {(p.x - pc.x) * wx, (p.y - pc.y) * wx, (p.z - pc.z) * wx,
+                        (v.x - vc.x) * wv, (v.y - vc.y) * wv, (v.z - vc.z) * wv};
+    float s = 0.f;
+#pragma unroll
+    for (int d = 0; d < 6; d++) {
+        o.h[d] = __float2half_rn(u[d]);
+        const float r = __half2float(o.h[d]);
+        s = fmaf(r, r, s);
+    }
+    return s;
+}
+
+__device__ __forceinline__ unsigned pack2(__half a, __half b)
+{
+    return (unsigned)__half_as_ushort(a) | ((unsigned)__half_as_ushort(b) << 16);
+}
+
+struct LinkWarp {
+    uint4 cand[32];         // 32 candidates (or, at first, the queries) as eight halves
+    float4 qa[32];          // the queries: px, py, pz, vx
+    float2 qb[32];          //              vy, vz
+    float4 box[4];          // the leaf's box (plo, phi, vlo, vhi)
+    float4 pc, vc;          // its centre; .w: the metric's weights over the linking radius
+    int ring[LK_RING];      // kept candidates (member of the node)
+    int pairs[64];          // (query lane << 26) | member, to be evaluated
+    int stack[LK_STACK];
+    int leaf[LK_LEAVES];
+    int rq[32];             // per query: a member of its set
+    int lv[2 * BVH_MAXH];
+};
 
 // friends-of-friends at l, one warp per leaf of 32 consecutive members, pairs
 // with the candidate after the query in the node's member order; only
@@ -1633,16 +1642,15 @@ __device__ __forceinline__ int w32_link(const BvhView &V, const MemberStore &M, 
 // a small block frees its slot as soon as its own few warps end instead of
 // waiting for the slowest of eight.
 constexpr int LK_WARPS = 2;
-template <int MINB>
-__global__ void __launch_bounds__(LK_WARPS * 32, MINB * (TQ / 32) / LK_WARPS)
-    k_bvh_link(LevelBufs L, NodeArrays nd, const int64_t *box_base, BoxStore B, MemberStore MS, const float *dnn,
-               int *parent, rs_dev_status *st)
+template <int WARPS>
+__global__ void __launch_bounds__(LK_WARPS * 32, WARPS / LK_WARPS)
+    k_bvh_link(LevelBufs L, NodeArrays nd, const int64_t *box_base, BoxStore B, MemberStore MS, int *parent,
+               rs_dev_status *st)
 {
     static_assert((TQ / 32) % LK_WARPS == 0, "a tile's warps fill whole blocks");
-    __shared__ int si_s[LK_WARPS][LK_STACK];
-    __shared__ int lf_s[LK_WARPS][LK_LEAVES];
-    __shared__ int lv_s[LK_WARPS][2 * BVH_MAXH];
+    __shared__ LinkWarp sh[LK_WARPS];
     const int w = warp_id(), lane = lane_id();
+    LinkWarp &S = sh[w];
     // the grid holds exactly the tiles' warps: block b takes warps
     // (b % bpt) * LK_WARPS + w of tile b / bpt
     constexpr int bpt = (TQ / 32) / LK_WARPS;
@@ -1650,43 +1658,262 @@ __global__ void __launch_bounds__(LK_WARPS * 32, MINB * (TQ / 32) / LK_WARPS)
     const int k = L.tile_rank[tile], q0 = L.tile_q0[tile] + 32 * jw;
     const int node = L.list[k], first = nd.first[node], n = nd.count[node];
     if (q0 >= n) return;
+    const MemberStore M = mem_shift(MS, first);
+    const int mo = q0 + lane;
+    float4 po = make_float4(INFINITY, 0, 0, 0), vo = make_float4(0, 0, 0, 0);
+    if (mo < n) mem_get(M, mo, po, vo);
+    // (a member without a neighbour within reach has an infinite packed x)
+    const bool act = po.x < INFINITY;
+    const unsigned actm = __ballot_sync(FULLW, act);
+    if (!actm) return;
     Metric6 met;  // float32 factors only; the float64 ones are read where needed
     met.ax = L.met[k].ax;
     met.av = L.met[k].av;
     const Metric6 *met64 = L.met + k;
     const double *l2p = L.l2 + k;
     const LinkLim lm = link_lim(L.l2[k]);
-    const MemberStore M = mem_shift(MS, first);
-    const float *D = dnn + first;
-    const int mo = q0 + lane;
-    const bool have = mo < n;
-    const bool act = have && D[mo] <= lm.part;
-    unsigned rem = __ballot_sync(FULLW, act);
-    if (!rem) return;
-    float4 po = make_float4(0, 0, 0, 0), vo = po;
-    if (have) mem_get(M, mo, po, vo);
     BvhView V;
-    bvh_view(V, B, box_base[k], n, lv_s[w]);
+    bvh_view(V, B, box_base[k], n, S.lv);
     const int own = q0 / BVH_LEAF;
-    int tie = 0;
-    while (rem) {
-        const int j = __ffs(rem) - 1;
-        rem &= rem - 1;
-        const int q = q0 + j;
-        const float4 pq = shfl4(po, j), vq = shfl4(vo, j);
-        // a member of the query's set (its parent), refined as unions report roots
-        int rq = __ldcg(&parent[first + q]);
-        // pairs inside the own leaf, lane > j
-        int nr = 0x7fffffff;
-        if (lane > j && act) {
-            const int r = pair_test(lm, met, met64, l2p, pq, vq, po, vo);
-            tie += r >> 1;
-            if (r & 1) nr = join_friend(parent, first + q, first + mo, rq, st);
-        }
-        rq = min(rq, (int)__reduce_min_sync(FULLW, (unsigned)nr));
-        tie += w32_link(V, M, D, n, q, pq, vq, met, met64, l2p, lm, own, parent, first, si_s[w], lf_s[w], rq, st,
-                        node);
+    S.qa[lane] = make_float4(po.x, po.y, po.z, vo.x);
+    S.qb[lane] = make_float2(vo.y, vo.z);
+    S.rq[lane] = act ? __ldcg(&parent[first + mo]) : 0;
+
+    // ---- half-precision frame: centre, weights, the queries' fragments ----
+    bool brute;
+    unsigned a[4];
+    float cr[4];
+    {
+    const Box6 bx = box_get(V.S, own);
+    const float4 pc = make_float4(0.5f * bx.plo.x + 0.5f * bx.phi.x, 0.5f * bx.plo.y + 0.5f * bx.phi.y,
+                                  0.5f * bx.plo.z + 0.5f * bx.phi.z, 0.f);
+    const float4 vc = make_float4(0.5f * bx.vlo.x + 0.5f * bx.vhi.x, 0.5f * bx.vlo.y + 0.5f * bx.vhi.y,
+                                  0.5f * bx.vlo.z + 0.5f * bx.vhi.z, 0.f);
+    const float wx = sqrtf(met.ax / lm.part), wv = sqrtf(met.av / lm.part);
+    const float rb = sqrtf(point_box_far2(pc, vc, bx, met) / lm.part);
+    brute = !(rb <= LK_RMAX && lm.part < 1e30f);
+    if (lane == 0) {
+        S.box[0] = bx.plo;
+        S.box[1] = bx.phi;
+        S.box[2] = bx.vlo;
+        S.box[3] = bx.vhi;
+        S.pc = make_float4(pc.x, pc.y, pc.z, wx);
+        S.vc = make_float4(vc.x, vc.y, vc.z, wv);
     }
+    const float rsum = 2.f * rb + 1.01f;
+    const float dl = 1.02f * 4.8828125e-4f * rsum + 3.1e-4f;
+    const float T = (1.f + dl) * (1.f + dl) * 1.00002f + 3.814697265625e-6f * rsum * rsum + 1.e-4f;
+        HalfPoint h;
+        float s = half_point(act && !brute ? po : pc, act && !brute ? vo : vc, pc, vc, wx, wv, h);
+        const __half2 m2 = __float2half2_rn(-2.f);
+        __half2 c0 = __hmul2(__halves2half2(h.h[0], h.h[1]), m2), c1 = __hmul2(__halves2half2(h.h[2], h.h[3]), m2),
+                c2 = __hmul2(__halves2half2(h.h[4], h.h[5]), m2);
+        uint4 row;
+        row.x = pack2(__low2half(c0), __high2half(c0));
+        row.y = pack2(__low2half(c1), __high2half(c1));
+        row.z = pack2(__low2half(c2), __high2half(c2));
+        row.w = 0x3c003c00u;  // (1, 1)
+        S.cand[lane] = row;
+        s = act ? s - T : 60000.f;
+        __syncwarp();
+        const unsigned *cw = (const unsigned *)S.cand;
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            a[i] = cw[4 * (8 * i + (lane >> 2)) + (lane & 3)];
+            cr[i] = __shfl_sync(FULLW, s, 8 * i + (lane >> 2));
+        }
+        __syncwarp();
+    }
+
+    int tie = 0, np = 0;               // queued pairs
+    int head = 0, nc = 0;              // ring of kept candidates
+    const unsigned below = (1u << lane) - 1u;
+    // evaluates up to 32 queued pairs, one a lane
+    auto flush = [&](int cnt) {
+        np -= cnt;
+        const int code = lane < cnt ? S.pairs[np + lane] : 0;
+        const int r = code >> 26, m = code & 0x3ffffff;
+        if (lane < cnt && m > q0 + r) {
+            float4 pm, vm;
+            mem_get(M, m, pm, vm);
+            const float4 x = S.qa[r];
+            const float2 y = S.qb[r];
+            const float4 pq = make_float4(x.x, x.y, x.z, 0.f), vq = make_float4(x.w, y.x, y.y, 0.f);
+            const int f = pair_test(lm, met, met64, l2p, pq, vq, pm, vm);
+            tie += f >> 1;
+            if (f & 1) {
+                const int root = join_friend(parent, first + q0 + r, first + m, ((volatile int *)S.rq)[r], st);
+                if (root != 0x7fffffff) atomicMin(&S.rq[r], root);
+            }
+        }
+        __syncwarp();
+    };
+    // tests the oldest cnt (at most 32) kept candidates against the queries
+    auto test = [&](int cnt) {
+        const int m = S.ring[(head + lane) & (LK_RING - 1)];
+        unsigned mask = 0;
+        if (!brute) {
+            uint4 c = make_uint4(0u, 0u, 0u, 0x00007b00u);  // padding: |u|^2 = 57344, never near
+            if (lane < cnt) {
+                float4 pm, vm;
+                mem_get(M, m, pm, vm);
+                HalfPoint h;
+                const float4 pc = S.pc, vc = S.vc;
+                const float s = half_point(pm, vm, pc, vc, pc.w, vc.w, h);
+                const __half hi = __float2half_rn(s), lo = __float2half_rn(s - __half2float(hi));
+                c = make_uint4(pack2(h.h[0], h.h[1]), pack2(h.h[2], h.h[3]), pack2(h.h[4], h.h[5]), pack2(hi, lo));
+            }
+            S.cand[lane] = c;
+            __syncwarp();
+            const unsigned *cw = (const unsigned *)S.cand;
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const unsigned b = cw[4 * (8 * j + (lane >> 2)) + (lane & 3)];
+                float d0[4], d1[4];
+                mma_m16n8k8_f16(d0, a[0], a[1], b, cr[0], cr[0], cr[1], cr[1]);
+                mma_m16n8k8_f16(d1, a[2], a[3], b, cr[2], cr[2], cr[3], cr[3]);
+                // the sign bits, oldest at the top: bit 31 - (8 j + i)
+#pragma unroll
+                for (int i = 0; i < 4; i++) mask = __funnelshift_l(__float_as_uint(d0[i]), mask, 1);
+#pragma unroll
+                for (int i = 0; i < 4; i++) mask = __funnelshift_l(__float_as_uint(d1[i]), mask, 1);
+            }
+            __syncwarp();
+        } else {
+            for (int e = 0; e < 32; e++) {
+                const int row = 16 * ((e >> 2) & 1) + 8 * ((e >> 1) & 1) + (lane >> 2);
+                const int col = 8 * (e >> 3) + 2 * (lane & 3) + (e & 1);
+                if (((actm >> row) & 1u) && col < cnt) mask |= 0x80000000u >> e;
+            }
+        }
+        for (;;) {
+            const unsigned bm = __ballot_sync(FULLW, mask != 0);
+            if (!bm) break;
+            const int e = mask ? __clz(mask) : 0;
+            const int row = 16 * ((e >> 2) & 1) + 8 * ((e >> 1) & 1) + (lane >> 2);
+            const int col = 8 * (e >> 3) + 2 * (lane & 3) + (e & 1);
+            if (mask) {
+                mask &= ~(0x80000000u >> e);
+                S.pairs[np + __popc(bm & below)] = (row << 26) | S.ring[(head + col) & (LK_RING - 1)];
+            }
+            np += __popc(bm);
+            __syncwarp();
+            if (np >= 32) flush(32);
+        }
+        head = (head + cnt) & (LK_RING - 1);
+        nc -= cnt;
+    };
+    // whether the child box of this lane of stack entry `ent` has to be
+    // searched: it reaches the leaf's own members or later ones, and its box
+    // is within reach.  A clique box wholly within l of a query joins it with
+    // one union; it is searched only for queries it holds near and far
+    // members of.
+    auto own_box = [&]() {
+        Box6 b;
+        b.plo = S.box[0];
+        b.phi = S.box[1];
+        b.vlo = S.box[2];
+        b.vhi = S.box[3];
+        return b;
+    };
+    auto child = [&](int ent) -> bool {
+        bool want = false, clique = false;
+        Box6 cb = box_empty();
+        int c = 0, ch = 0;
+        if (ent >= 0) {
+            ch = (ent >> 24) - 1;
+            c = 32 * (ent & 0xffffff) + lane;
+            if (c < V.cnt[ch] && bvh_m0(ch, c + 1) > (int64_t)q0) {
+                const int64_t bi = V.off[ch] + c;
+                cb = box_get(V.S, bi);
+                clique = V.S.cl[bi] != 0;
+                want = box_box_d2(own_box(), cb, met) <= lm.lim;
+            }
+        }
+        unsigned cm = __ballot_sync(FULLW, want && clique && !(ch == 0 && c == own));
+        while (cm) {
+            const int s = __ffs(cm) - 1;
+            cm &= cm - 1;
+            Box6 b;
+            b.plo = shfl4(cb.plo, s);
+            b.phi = shfl4(cb.phi, s);
+            b.vlo = shfl4(cb.vlo, s);
+            b.vhi = shfl4(cb.vhi, s);
+            const int m0 = (int)bvh_m0(ch, __shfl_sync(FULLW, c, s));
+            const float4 x = S.qa[lane];
+            const float2 y = S.qb[lane];
+            const float4 po = make_float4(x.x, x.y, x.z, 0.f), vo = make_float4(x.w, y.x, y.y, 0.f);
+            const bool near = ((actm >> lane) & 1u) && point_box_d2(po, vo, b, met) <= lm.lim;
+            const bool all = near && point_box_far2(po, vo, b, met) <= lm.cl_lim;
+            if (all) {
+                const int root = join_friend(parent, first + mo, first + m0, S.rq[lane], st);
+                if (root != 0x7fffffff) S.rq[lane] = min(S.rq[lane], root);
+            }
+            const bool open = __any_sync(FULLW, near && !all);
+            if (lane == s) want = open;
+        }
+        return want;
+    };
+
+    if (lane == 0) S.stack[0] = (V.H - 1) << 24;
+    int sp = V.H >= 2 ? 1 : 0, nl = 0;
+    if (V.H < 2) {
+        if (lane == 0) S.leaf[0] = own;
+        nl = 1;
+    }
+    __syncwarp();
+    for (int it = 0; (sp > 0 || nl > 0 || nc > 0) && it < (1 << 24); it++) {
+        if (sp > 0 && nl <= LK_LEAVES - 64) {
+            const int ea = S.stack[sp - 1];
+            const int eb = sp >= 2 ? S.stack[sp - 2] : -1;
+            __syncwarp();
+            sp -= eb >= 0 ? 2 : 1;
+#pragma unroll 1
+            for (int u = 0; u < 2; u++) {
+                const int ent = u == 0 ? ea : eb;
+                if (ent < 0) break;
+                const bool want = child(ent);
+                const unsigned m = __ballot_sync(FULLW, want);
+                const int ch = (ent >> 24) - 1, c = 32 * (ent & 0xffffff) + lane;
+                const int slot = __popc(m & below);
+                if (ch == 0) {
+                    if (want) S.leaf[nl + slot] = c;
+                    nl += __popc(m);
+                } else {
+                    if (sp + __popc(m) > LK_STACK) {
+                        if (lane == 0) dev_fail(st, DEV_OVERFLOW, 55, node);
+                        return;
+                    }
+                    if (want) S.stack[sp + slot] = (ch << 24) | c;
+                    sp += __popc(m);
+                }
+            }
+            __syncwarp();
+            continue;
+        }
+        // the members of the collected leaves within reach of the own box,
+        // two leaves at a time (their loads overlap)
+        if (nl > 0) {
+            const int m0 = S.leaf[nl - 1] * BVH_LEAF + lane;
+            const int m1 = nl >= 2 ? S.leaf[nl - 2] * BVH_LEAF + lane : n;
+            nl = max(0, nl - 2);
+            float4 p0 = make_float4(INFINITY, 0, 0, 0), u0 = make_float4(0, 0, 0, 0), p1 = p0, u1 = u0;
+            if (m0 < n) mem_get(M, m0, p0, u0);
+            if (m1 < n) mem_get(M, m1, p1, u1);
+            const Box6 bx = own_box();
+            const bool k0 = point_box_d2(p0, u0, bx, met) <= lm.lim;
+            const bool k1 = point_box_d2(p1, u1, bx, met) <= lm.lim;
+            const unsigned b0 = __ballot_sync(FULLW, k0), b1 = __ballot_sync(FULLW, k1);
+            if (k0) S.ring[(head + nc + __popc(b0 & below)) & (LK_RING - 1)] = m0;
+            nc += __popc(b0);
+            if (k1) S.ring[(head + nc + __popc(b1 & below)) & (LK_RING - 1)] = m1;
+            nc += __popc(b1);
+            __syncwarp();
+        }
+        const bool last = sp == 0 && nl == 0;
+        while (nc >= 32 || (last && nc > 0)) test(min(nc, 32));
+    }
+    if (np > 0) flush(np);
     tie = warp_sum(tie);
     if (lane == 0 && tie) atomicAdd(&L.tie[k], tie);
 }
@@ -2453,17 +2680,6 @@ __global__ void k_lvl_l2(LevelBufs L, NodeArrays nd, double f, int sub_n, rs_dev
     }
 }
 
-__global__ void k_lvl_iota(LevelBufs L, NodeArrays nd, int *parent, int *csize, int *cmin)
-{
-    const int k = L.tile_rank[blockIdx.x], q0 = L.tile_q0[blockIdx.x];
-    const int node = L.list[k], first = nd.first[node], n = nd.count[node];
-    const int q = q0 + threadIdx.x;
-    if (q >= n) return;
-    parent[first + q] = first + q;
-    csize[first + q] = 0;
-    cmin[first + q] = 0x7fffffff;
-}
-
 __global__ void k_lvl_comp(LevelBufs L, NodeArrays nd, const int *widx, int *parent, int *csize, int *cmin,
                            rs_dev_status *st)
 {
@@ -2874,9 +3090,11 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
             ms.a = carve<float4>(sp2, M);
             ms.b = carve<float2>(sp2, M);
         }
-        RS_LAUNCH(ctx, "rf_bvh_leaves", k_bvh_leaves, T, TQ, 0, L, nd, (const int64_t *)bo, boxes, ms,
-                  (const float4 *)wpos, (const float4 *)wvel);
-        RS_LAUNCH(ctx, "rf_bvh_build", k_bvh_build, K, 256, 0, L, nd, (const int64_t *)bo, boxes);
+        RS_LAUNCH(ctx, "rf_bvh_leaves", k_bvh_leaves<false>, T, TQ, 0, L, nd, (const int64_t *)bo, boxes, ms,
+                  (const float4 *)wpos, (const float4 *)wvel, (const float *)nullptr, (int *)nullptr, (int *)nullptr,
+                  (int *)nullptr, ctx->d_status);
+        RS_LAUNCH(ctx, "rf_bvh_build", k_bvh_build<false>, K, 256, 0, L, nd, (const int64_t *)bo, boxes,
+                  (int *)nullptr, ctx->d_status);
         // ---- random member subsets of the nodes above sub_n (Sec. 3.2) ----
         int2 *sub_q = nullptr;
         int *sub_len = ctr + 13;
@@ -2975,25 +3193,27 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
         RS_LAUNCH(ctx, "rf_lvl_band_exact", k_lvl_band_exact, ceil_div(nbv, W_WARPS), W_WARPS * 32, 0, L, nd,
                   (const int64_t *)bo, boxes, ms, (const float *)dnn, ctx->d_status);
         RS_LAUNCH(ctx, "rf_lvl_l2", k_lvl_l2, K, 128, 0, L, nd, f, (int)sub_n, ctx->d_status);
-        RS_LAUNCH(ctx, "rf_lvl_iota", k_lvl_iota, T, TQ, 0, L, nd, uf, csize, cmin);
-        RS_LAUNCH(ctx, "rf_bvh_linkbox", k_bvh_linkbox, K, 256, 0, L, nd, (const int64_t *)bo, boxes,
-                  (const float4 *)wpos, (const float4 *)wvel, (const float *)dnn, uf, ctx->d_status);
+        RS_LAUNCH(ctx, "rf_link_leaves", k_bvh_leaves<true>, T, TQ, 0, L, nd, (const int64_t *)bo, boxes, ms,
+                  (const float4 *)wpos, (const float4 *)wvel, (const float *)dnn, uf, csize, cmin, ctx->d_status);
+        RS_LAUNCH(ctx, "rf_link_build", k_bvh_build<true>, K, 256, 0, L, nd, (const int64_t *)bo, boxes, uf,
+                  ctx->d_status);
         {
-            // one warp per leaf job, LK_WARPS to a block; compiled for 8 x
-            // rs_tuning::link_blocks_per_sm resident warps per SM
+            // one warp per leaf job, LK_WARPS to a block; compiled for 24, 32
+            // or 40 resident warps per SM (rs_tuning::link_blocks_per_sm = 4,
+            // 5 or 6)
             const int64_t njobs = T * (TQ / 32), lg = ceil_div(njobs, LK_WARPS);
             switch (ctx->tune.link_blocks_per_sm) {
             case 4:
-                RS_LAUNCH(ctx, "rf_lvl_link", k_bvh_link<4>, lg, LK_WARPS * 32, 0, L, nd, (const int64_t *)bo, boxes,
-                          ms, (const float *)dnn, uf, ctx->d_status);
+                RS_LAUNCH(ctx, "rf_lvl_link", k_bvh_link<24>, lg, LK_WARPS * 32, 0, L, nd, (const int64_t *)bo, boxes,
+                          ms, uf, ctx->d_status);
                 break;
             case 6:
-                RS_LAUNCH(ctx, "rf_lvl_link", k_bvh_link<6>, lg, LK_WARPS * 32, 0, L, nd, (const int64_t *)bo, boxes,
-                          ms, (const float *)dnn, uf, ctx->d_status);
+                RS_LAUNCH(ctx, "rf_lvl_link", k_bvh_link<40>, lg, LK_WARPS * 32, 0, L, nd, (const int64_t *)bo, boxes,
+                          ms, uf, ctx->d_status);
                 break;
             default:
-                RS_LAUNCH(ctx, "rf_lvl_link", k_bvh_link<5>, lg, LK_WARPS * 32, 0, L, nd, (const int64_t *)bo, boxes,
-                          ms, (const float *)dnn, uf, ctx->d_status);
+                RS_LAUNCH(ctx, "rf_lvl_link", k_bvh_link<32>, lg, LK_WARPS * 32, 0, L, nd, (const int64_t *)bo, boxes,
+                          ms, uf, ctx->d_status);
             }
         }
         RS_LAUNCH(ctx, "rf_lvl_comp", k_lvl_comp, T, TQ, 0, L, nd, (const int *)widx, uf, csize, cmin,
