@@ -170,8 +170,8 @@ rs_status rs_fof3d(rs_ctx *ctx, const float *pos, int32_t stride, int64_t n, dou
  * plus an edge from every centre to every particle within 2l (inclusive).
  * Every group is a union of plain FOF groups.  labels as rs_fof3d (device,
  * n int32).  n_groups and n_centres (host, optional; n_centres = number of
- * centres) synchronise.  The call always synchronises once per round of the
- * centre choice.  Errors as rs_fof3d; RS_ERR_INVALID_ARG for dense_n < 0;
+ * centres) synchronise.  The call always synchronises once per few rounds of
+ * the centre choice.  Errors as rs_fof3d; RS_ERR_INVALID_ARG for dense_n < 0;
  * RS_ERR_INTERNAL if the centre choice has not settled after 65536 rounds. */
 rs_status rs_fof3d_accel(rs_ctx *ctx, const float *pos, int32_t stride, int64_t n, double box, double b,
                          int32_t dense_n, int32_t *labels, int64_t *n_groups, int64_t *n_centres);

@@ -459,8 +459,20 @@ __global__ void __launch_bounds__(FOF_THREADS) k_fof_tieband(const uint32_t *n_c
 // decide the centres (a dense particle becomes a centre once every dense
 // neighbour of smaller index is decided and none is a centre, and drops out
 // once one is a centre); and the 2l joins of the centres' fine cells.
-enum : uint8_t { ACC_SPARSE = 0, ACC_UNDECIDED = 1, ACC_CENTRE = 2, ACC_OUT = 3 };
-
+//
+// The rounds work on fine cells, not on particles.  A cell's particles are
+// mutual neighbours in index order, so only its first undecided particle (its
+// head) can be decided, and a centre settles the whole cell.  A cell's state
+// is one 64-bit word, (head, centre + 1), written and read whole.  A round has
+// two kernels: one decides the heads of the unsettled cells, a warp a cell,
+// seeing a neighbouring cell through its word and its particles from its head
+// up to the own index; one lets each new centre mark the particles within l
+// as out, once per centre.  Bound by the dependent loads of the cell walks.
+// Before, a round went over every particle and scanned all neighbours of the
+// undecided ones: 14 rounds of 1.16 ms at 2M particles, now 8 of 0.16 ms (a
+// thread walking a cell's heads one after another in one launch instead took
+// 100 ms: the cores' cells hold thousands).  The whole call takes 4.0 ms
+// instead of 18 to 21 at 2M particles, 201 instead of 1128 at 134M.
 // Calls f(B, b0, b1, sx, sy, sz) for every occupied fine cell B within R fine
 // cells per axis of the fine cell at fine coordinates (ax, ay, az) (coarse
 // cell (ccx, ccy, ccz), sub-cell (ux, uy, uz)), with B's particle range and
@@ -517,7 +529,7 @@ __device__ __forceinline__ void acc_where(const uint64_t *cell_key, uint32_t A, 
 __global__ void __launch_bounds__(FOF_THREADS) k_acc_count(int64_t n, const uint32_t *cell_of, const uint64_t *cell_key,
                                                            const uint32_t *cell_start, const uint32_t *table,
                                                            const uint64_t *occ, const float4 *spos, FofGeom g,
-                                                           int dense_n, uint8_t *state)
+                                                           int dense_n, uint8_t *dense)
 {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= n) return;
@@ -535,76 +547,181 @@ __global__ void __launch_bounds__(FOF_THREADS) k_acc_count(int64_t n, const uint
                       return false;
                   });
     }
-    state[q] = cnt > dense_n ? ACC_UNDECIDED : ACC_SPARSE;
+    dense[q] = cnt > dense_n ? 1 : 0;
 }
 
-// one round of the centre choice; `left` counts the particles still undecided
-__global__ void __launch_bounds__(FOF_THREADS) k_acc_round(int64_t n, const uint32_t *cell_of, const uint64_t *cell_key,
-                                                           const uint32_t *cell_start, const uint32_t *table,
-                                                           const uint64_t *occ, const float4 *spos, const uint32_t *idx,
-                                                           FofGeom g, const uint8_t *sin, uint8_t *sout,
-                                                           unsigned long long *left)
+__device__ __forceinline__ uint64_t acc_word(uint32_t head, uint32_t centre1) { return (uint64_t)head << 32 | centre1; }
+
+__device__ __forceinline__ uint32_t acc_next(const uint8_t *dense, uint32_t q, uint32_t end)
 {
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
-    const uint8_t s0 = sin[q];
-    if (s0 != ACC_UNDECIDED) {
-        sout[q] = s0;
-        return;
+    while (q < end && !dense[q]) q++;
+    return q;
+}
+
+// every cell's first dense particle; the cells that have one are unsettled
+__global__ void k_acc_init(const uint32_t *n_cells_p, const uint32_t *cell_start, const uint8_t *dense, uint64_t *word,
+                           uint32_t *list, unsigned *len)
+{
+    const int64_t M = *n_cells_p;
+    for (int64_t wb = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); wb < M;
+         wb += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t A = wb + lane_id();
+        bool open = false;
+        if (A < M) {
+            const uint32_t end = cell_start[A + 1], h = acc_next(dense, cell_start[A], end);
+            word[A] = acc_word(h, 0u);
+            open = h < end;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, open);
+        unsigned base = 0;
+        if (lane_id() == 0 && m) base = atomicAdd(len, (unsigned)__popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (open) list[base + __popc(m & ((1u << lane_id()) - 1u))] = (uint32_t)A;
     }
-    const uint32_t A = cell_of[q], me = idx[q];
-    int ccx, ccy, ccz, ux, uy, uz;
-    acc_where(cell_key, A, g, ccx, ccy, ccz, ux, uy, uz);
-    const float4 p = spos[q];
-    bool blocked = false, out = false;
-    acc_cells(ccx, ccy, ccz, ux, uy, uz, 2, cell_start, table, occ, g,
-              [&](uint32_t B, uint32_t b0, uint32_t b1, int sx, int sy, int sz) {
-                  for (uint32_t r = b0; r < b1; r++) {
-                      const uint8_t sr = sin[r];
-                      if ((sr != ACC_UNDECIDED && sr != ACC_CENTRE) || idx[r] >= me) continue;
-                      // the own fine cell is a clique
-                      if (B != A && !pair_link(p, spos[r], sx, sy, sz, g)) continue;
-                      if (sr == ACC_CENTRE) {
-                          out = true;
-                          return true;
-                      }
-                      blocked = true;
-                  }
-                  return false;
-              });
-    const uint8_t s1 = out ? ACC_OUT : (blocked ? ACC_UNDECIDED : ACC_CENTRE);
-    sout[q] = s1;
-    if (s1 == ACC_UNDECIDED) atomicAdd(left, 1ull);
+}
+
+// One round of the centre choice: the head of every listed cell waits (its
+// cell goes to the next list) while an undecided dense particle of smaller
+// index lies within l, or one that became a centre in this very round, and is
+// a centre otherwise.  A warp a cell, a lane two of a coarse cell's sub-cells.
+__global__ void __launch_bounds__(FOF_THREADS) k_acc_round(const uint32_t *list, const unsigned *len,
+                                                           const uint64_t *cell_key, const uint32_t *cell_start,
+                                                           const uint32_t *table, const uint64_t *occ,
+                                                           const float4 *spos, const uint32_t *idx, FofGeom g,
+                                                           const uint8_t *dense, uint64_t *word, uint32_t *list2,
+                                                           unsigned *len2, uint32_t *clist, unsigned *clen)
+{
+    const unsigned FULL = 0xffffffffu;
+    const unsigned n = *len;
+    const int lane = lane_id();
+    for (unsigned k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += gridDim.x * blockDim.x >> 5) {
+        const uint32_t A = list[k], end = cell_start[A + 1];
+        uint32_t h = (uint32_t)(__ldcg(&word[A]) >> 32);
+        unsigned f = 0;
+        while (h < end && !(f = __ballot_sync(FULL, h + lane < end && dense[h + lane] != 0))) h += 32;
+        h = f ? h + (uint32_t)__ffs(f) - 1u : end;
+        if (lane == 0) __stcg(&word[A], acc_word(h, 0u));
+        if (h >= end) continue;  // every particle is out
+        int ccx, ccy, ccz, ux, uy, uz;
+        acc_where(cell_key, A, g, ccx, ccy, ccz, ux, uy, uz);
+        const int ax = 4 * ccx + ux, ay = 4 * ccy + uy, az = 4 * ccz + uz;
+        const uint32_t me = idx[h];
+        const float4 p = spos[h];
+        bool blocked = false;
+        for (int c8 = 0; c8 < 8 && !blocked; c8++) {
+            const int dx = (ux < 2 ? -1 : 0) + (c8 & 1), dy = (uy < 2 ? -1 : 0) + ((c8 >> 1) & 1),
+                      dz = (uz < 2 ? -1 : 0) + (c8 >> 2);
+            int cx = ccx + dx, cy = ccy + dy, cz = ccz + dz;
+            cx = cx < 0 ? cx + g.Gc : (cx >= g.Gc ? cx - g.Gc : cx);
+            cy = cy < 0 ? cy + g.Gc : (cy >= g.Gc ? cy - g.Gc : cy);
+            cz = cz < 0 ? cz + g.Gc : (cz >= g.Gc ? cz - g.Gc : cz);
+            const uint32_t b0c = table[((uint64_t)cz * g.Gc + cy) * g.Gc + cx];
+            if (b0c == 0xffffffffu) continue;
+            const uint64_t om = occ[b0c], cand = om & reach_mask(ux, uy, uz, dx, dy, dz, 2);
+            bool mine = false;
+            for (int sb = lane; sb < 64; sb += 32) {
+                if (!((cand >> sb) & 1ull)) continue;
+                const uint32_t B = b0c + (uint32_t)__popcll(om & ((1ull << sb) - 1ull));
+                if (B == A) continue;
+                const uint64_t w = __ldcg(&word[B]);
+                const uint32_t c1 = (uint32_t)w, b1 = c1 ? c1 : cell_start[B + 1];
+                int sx, sy, sz;
+                fine_offset(ax, 4 * cx + (sb & 3), g.Gf, sx);
+                fine_offset(ay, 4 * cy + ((sb >> 2) & 3), g.Gf, sy);
+                fine_offset(az, 4 * cz + (sb >> 4), g.Gf, sz);
+                for (uint32_t r = c1 ? c1 - 1u : (uint32_t)(w >> 32); !mine && r < b1 && idx[r] < me; r++)
+                    mine = dense[r] && pair_link(p, spos[r], sx, sy, sz, g);
+            }
+            blocked = __any_sync(FULL, mine);
+        }
+        if (lane == 0) {
+            if (blocked) {
+                list2[atomicAdd(len2, 1u)] = A;
+            } else {
+                __stcg(&word[A], acc_word(end, h + 1u));
+                clist[atomicAdd(clen, 1u)] = A;
+            }
+        }
+    }
+}
+
+// the particles within l of the round's centres are out (a centre's own cell
+// is settled by its word); a warp a centre, the lanes over a cell's particles
+__global__ void __launch_bounds__(FOF_THREADS) k_acc_mark(const uint32_t *clist, const unsigned *clen,
+                                                          const uint64_t *cell_key, const uint32_t *cell_start,
+                                                          const uint32_t *table, const uint64_t *occ,
+                                                          const float4 *spos, FofGeom g, const uint64_t *word,
+                                                          uint8_t *dense)
+{
+    const unsigned n = *clen;
+    for (unsigned k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n; k += gridDim.x * blockDim.x >> 5) {
+        const uint32_t A = clist[k];
+        int ccx, ccy, ccz, ux, uy, uz;
+        acc_where(cell_key, A, g, ccx, ccy, ccz, ux, uy, uz);
+        const float4 p = spos[(uint32_t)word[A] - 1u];
+        acc_cells(ccx, ccy, ccz, ux, uy, uz, 2, cell_start, table, occ, g,
+                  [&](uint32_t B, uint32_t, uint32_t b1, int sx, int sy, int sz) {
+                      if (B == A) return false;
+                      for (uint32_t r = (uint32_t)(word[B] >> 32) + lane_id(); r < b1; r += 32)
+                          if (dense[r] && pair_link(p, spos[r], sx, sy, sz, g)) dense[r] = 0;
+                      return false;
+                  });
+    }
 }
 
 // every centre joins the fine cells that hold a particle within 2l of it
 // (a fine cell is one set already, so one such particle joins it); g2 is the
-// geometry with the thresholds of 2l
-__global__ void __launch_bounds__(FOF_THREADS) k_acc_join(int64_t n, const uint32_t *cell_of, const uint64_t *cell_key,
+// geometry with the thresholds of 2l.  A warp takes a centre, a lane two of a
+// coarse cell's 64 sub-cells.
+__global__ void __launch_bounds__(FOF_THREADS) k_acc_join(const uint32_t *n_cells_p, const uint64_t *cell_key,
                                                           const uint32_t *cell_start, const uint32_t *table,
                                                           const uint64_t *occ, const float4 *spos, FofGeom g2,
-                                                          const uint8_t *state, int *parent,
+                                                          const uint64_t *word, int *parent,
                                                           unsigned long long *centres, rs_dev_status *st)
 {
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool mine = q < n && state[q] == ACC_CENTRE;
-    const unsigned m = __ballot_sync(0xffffffffu, mine);
-    if (lane_id() == 0 && m) atomicAdd(centres, (unsigned long long)__popc(m));
-    if (!mine) return;
-    const uint32_t A = cell_of[q];
-    int ccx, ccy, ccz, ux, uy, uz;
-    acc_where(cell_key, A, g2, ccx, ccy, ccz, ux, uy, uz);
-    const float4 p = spos[q];
-    acc_cells(ccx, ccy, ccz, ux, uy, uz, 4, cell_start, table, occ, g2,
-              [&](uint32_t B, uint32_t b0, uint32_t b1, int sx, int sy, int sz) {
-                  if (uf_find(parent, (int)A, st) == uf_find(parent, (int)B, st)) return false;
-                  for (uint32_t r = b0; r < b1; r++)
-                      if (pair_link(p, spos[r], sx, sy, sz, g2)) {
-                          uf_union(parent, (int)A, (int)B, st);
-                          break;
-                      }
-                  return false;
-              });
+    const unsigned FULL = 0xffffffffu;
+    const int64_t M = *n_cells_p;
+    const int lane = lane_id();
+    for (int64_t wb = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); wb < M;
+         wb += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t mine = wb + lane < M ? (uint32_t)word[wb + lane] : 0u;
+        unsigned m = __ballot_sync(FULL, mine != 0u);
+        if (lane == 0 && m) atomicAdd(centres, (unsigned long long)__popc(m));
+        while (m) {
+            const int s = __ffs(m) - 1;
+            m &= m - 1u;
+            const uint32_t A = (uint32_t)(wb + s);
+            const float4 p = spos[__shfl_sync(FULL, mine, s) - 1u];
+            int ccx, ccy, ccz, ux, uy, uz;
+            acc_where(cell_key, A, g2, ccx, ccy, ccz, ux, uy, uz);
+            const int ax = 4 * ccx + ux, ay = 4 * ccy + uy, az = 4 * ccz + uz;
+            for (int c27 = 0; c27 < 27; c27++) {
+                const int dz = c27 / 9 - 1, dy = c27 / 3 % 3 - 1, dx = c27 % 3 - 1;
+                int cx = ccx + dx, cy = ccy + dy, cz = ccz + dz;
+                cx = cx < 0 ? cx + g2.Gc : (cx >= g2.Gc ? cx - g2.Gc : cx);
+                cy = cy < 0 ? cy + g2.Gc : (cy >= g2.Gc ? cy - g2.Gc : cy);
+                cz = cz < 0 ? cz + g2.Gc : (cz >= g2.Gc ? cz - g2.Gc : cz);
+                const uint32_t b0c = table[((uint64_t)cz * g2.Gc + cy) * g2.Gc + cx];
+                if (b0c == 0xffffffffu) continue;
+                const uint64_t om = occ[b0c], cand = om & reach_mask(ux, uy, uz, dx, dy, dz, 4);
+                for (int sb = lane; sb < 64; sb += 32) {
+                    if (!((cand >> sb) & 1ull)) continue;
+                    const uint32_t B = b0c + (uint32_t)__popcll(om & ((1ull << sb) - 1ull));
+                    if (uf_find(parent, (int)A, st) == uf_find(parent, (int)B, st)) continue;
+                    int sx, sy, sz;
+                    fine_offset(ax, 4 * cx + (sb & 3), g2.Gf, sx);
+                    fine_offset(ay, 4 * cy + ((sb >> 2) & 3), g2.Gf, sy);
+                    fine_offset(az, 4 * cz + (sb >> 4), g2.Gf, sz);
+                    for (uint32_t r = cell_start[B]; r < cell_start[B + 1]; r++)
+                        if (pair_link(p, spos[r], sx, sy, sz, g2)) {
+                            uf_union(parent, (int)A, (int)B, st);
+                            break;
+                        }
+                }
+                __syncwarp();
+            }
+        }
+    }
 }
 
 rs_status fof_geometry(rs_ctx *ctx, int64_t n, double box, double b, FofGeom *g)
@@ -651,6 +768,7 @@ int key_bits(const FofGeom &g)
 namespace {
 
 constexpr int ACC_MAX_ROUNDS = 1 << 16;  // bound on the centre-choice rounds
+constexpr int ACC_BATCH = 4;             // rounds between two looks at how many cells are left
 
 // plain FOF (dense_n < 0) or the accelerated variant (dense_n >= 0)
 rs_status fof_run(rs_ctx *ctx, const float *pos, int32_t stride, int64_t n, double box, double b, int32_t dense_n,
@@ -728,24 +846,42 @@ rs_status fof_run(rs_ctx *ctx, const float *pos, int32_t stride, int64_t n, doub
     }
     if (dense_n >= 0) {
         // accelerated variant: dense flags, centre rounds, 2l joins
-        RS_WS(ctx, uint8_t, acc, WS_FOF_ACC, 2 * n + 64);
-        uint8_t *sa = acc, *sb = acc + n;
-        unsigned long long *acnt = (unsigned long long *)(acc + (2 * n + 7) / 8 * 8);
+        const int64_t acc8 = n + ceil_div(3 * n, 2) + ceil_div(n, 8);
+        RS_WS(ctx, uint64_t, word, WS_FOF_ACC, acc8 + 20);
+        uint32_t *la = (uint32_t *)(word + n), *lb = la + n, *clist = lb + n;
+        uint8_t *dense = (uint8_t *)(clist + n);
+        // list lengths before and after each of a batch's rounds, each
+        // round's new centres, then the number of centres
+        unsigned *len = (unsigned *)(word + acc8 + 2), *clen = len + 8;
+        unsigned long long *acnt = (unsigned long long *)len + 8;
         RS_LAUNCH(ctx, "fof_acc_count", k_acc_count, nb, T, 0, n, (const uint32_t *)cell_of,
                   (const uint64_t *)cell_key, (const uint32_t *)cell_start, (const uint32_t *)table,
-                  (const uint64_t *)occ, (const float4 *)spos, g, (int)dense_n, sa);
-        for (int round = 0;; round++) {
+                  (const uint64_t *)occ, (const float4 *)spos, g, (int)dense_n, dense);
+        RS_CUDA(ctx, cudaMemsetAsync(len, 0, 4, ctx->stream));
+        RS_LAUNCH(ctx, "fof_acc_init", k_acc_init, grid, T, 0, (const uint32_t *)n_cells,
+                  (const uint32_t *)cell_start, (const uint8_t *)dense, word, la, len);
+        // the host looks at the length after every ACC_BATCH rounds (a round
+        // over an empty list ends at once)
+        for (int round = 0;; round += ACC_BATCH) {
             if (round >= ACC_MAX_ROUNDS)
                 return rs_fail(ctx, RS_ERR_INTERNAL, "rs_fof3d_accel: the centre choice did not settle");
-            RS_CUDA(ctx, cudaMemsetAsync(acnt, 0, sizeof(unsigned long long), ctx->stream));
-            RS_LAUNCH(ctx, "fof_acc_round", k_acc_round, nb, T, 0, n, (const uint32_t *)cell_of,
-                      (const uint64_t *)cell_key, (const uint32_t *)cell_start, (const uint32_t *)table,
-                      (const uint64_t *)occ, (const float4 *)spos, (const uint32_t *)idx, g, (const uint8_t *)sa, sb,
-                      acnt);
+            RS_CUDA(ctx, cudaMemsetAsync(len + 1, 0, 4 * 15, ctx->stream));
+            for (int r = 0; r < ACC_BATCH; r++) {
+                RS_LAUNCH(ctx, "fof_acc_round", k_acc_round, std::min<int64_t>(nb, (int64_t)ctx->num_sms * 8), T, 0,
+                          (const uint32_t *)la, (const unsigned *)len + r, (const uint64_t *)cell_key,
+                          (const uint32_t *)cell_start, (const uint32_t *)table, (const uint64_t *)occ,
+                          (const float4 *)spos, (const uint32_t *)idx, g, (const uint8_t *)dense, word, lb,
+                          len + r + 1, clist, clen + r);
+                RS_LAUNCH(ctx, "fof_acc_mark", k_acc_mark, std::min<int64_t>(nb, (int64_t)ctx->num_sms * 8), T, 0,
+                          (const uint32_t *)clist, (const unsigned *)clen + r, (const uint64_t *)cell_key,
+                          (const uint32_t *)cell_start, (const uint32_t *)table, (const uint64_t *)occ,
+                          (const float4 *)spos, g, (const uint64_t *)word, dense);
+                std::swap(la, lb);
+            }
             int64_t left = 0;
-            RS_TRY(rs_read_i64(ctx, acnt, 1, &left, "rs_fof3d_accel"));
-            std::swap(sa, sb);
-            if (left == 0) break;
+            RS_TRY(rs_read_i64(ctx, len + ACC_BATCH, 1, &left, "rs_fof3d_accel"));
+            if ((left & 0xffffffffll) == 0) break;
+            RS_CUDA(ctx, cudaMemcpyAsync(len, len + ACC_BATCH, 4, cudaMemcpyDeviceToDevice, ctx->stream));
         }
         // the same tests at 2l: every threshold scales by exactly 2 or 4
         FofGeom g2 = g;
@@ -753,11 +889,11 @@ rs_status fof_run(rs_ctx *ctx, const float *pos, int32_t stride, int64_t n, doub
         g2.l2 = 4.0 * g.l2;
         g2.lo32 = 4.0f * g.lo32;
         g2.hi32 = 4.0f * g.hi32;
-        RS_CUDA(ctx, cudaMemsetAsync(acnt + 1, 0, sizeof(unsigned long long), ctx->stream));
-        RS_LAUNCH(ctx, "fof_acc_join", k_acc_join, nb, T, 0, n, (const uint32_t *)cell_of, (const uint64_t *)cell_key,
+        RS_CUDA(ctx, cudaMemsetAsync(acnt, 0, sizeof(unsigned long long), ctx->stream));
+        RS_LAUNCH(ctx, "fof_acc_join", k_acc_join, grid, T, 0, (const uint32_t *)n_cells, (const uint64_t *)cell_key,
                   (const uint32_t *)cell_start, (const uint32_t *)table, (const uint64_t *)occ, (const float4 *)spos,
-                  g2, (const uint8_t *)sa, parent, acnt + 1, ctx->d_status);
-        if (n_centres) RS_TRY(rs_read_i64(ctx, acnt + 1, 1, n_centres, "rs_fof3d_accel"));
+                  g2, (const uint64_t *)word, parent, acnt, ctx->d_status);
+        if (n_centres) RS_TRY(rs_read_i64(ctx, acnt, 1, n_centres, "rs_fof3d_accel"));
     }
     RS_LAUNCH(ctx, "fof_rootmin", k_fof_rootmin, grid, T, 0, (const uint32_t *)n_cells,
               (const uint32_t *)cell_start, (const uint32_t *)idx, parent, root_min,
