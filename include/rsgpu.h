@@ -102,13 +102,16 @@ const char *rs_last_error(const rs_ctx *ctx);
  *   bracket_min         big nodes above this many members search with the
  *                       sampled bracket of the linking length (>= 1024);
  *   mid_max             subtrees of at most this many members run in the
- *                       128-thread tier (33-256); larger ones up to 1024 run
- *                       in the 256-thread tier;
- *   tiny_max            subtrees of at most this many members run one per
- *                       warp (10-32);
+ *                       128-thread tier, and below 128 in the one-warp tier
+ *                       (33-256); larger ones up to 1024 run in the
+ *                       256-thread tier;
+ *   tiny_max            subtrees of at most this many members run in a
+ *                       warp's registers (10-32);
  *   small_ctas_per_sm, mid_ctas_per_sm, tiny_ctas_per_sm
- *                       persistent CTAs per SM of the three subtree tiers
- *                       (1-2, 1-8, 1-16);
+ *                       persistent CTAs per SM of the subtree tiers: one more
+ *                       than the first in the 256-thread tier (1-2), the
+ *                       second in the 128-thread tier and three times as many
+ *                       one-warp ones (1-8), the third in the last (1-16);
  *   fof_link_ctas_per_sm  CTAs per SM of the grid-stride 3D link (1-64). */
 typedef struct {
     int32_t link_blocks_per_sm;

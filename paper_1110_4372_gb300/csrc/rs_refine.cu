@@ -19,10 +19,11 @@
 //    exact k-th select, union-find, children, recursion with an explicit
 //    stack), as a persistent work queue; a second instance with 128 threads
 //    and MID_N-member shared arrays takes the subtrees of at most MID_N
-//    members, which the first forwards to it;
+//    members, and a third with one warp those of at most WARP_N, each
+//    forwarded by the one before;
 //  * tiny nodes (<= TINY_N = 32 members): one warp holds the node in
 //    registers, a member per lane, and builds its whole subtree with warp
-//    shuffles and votes, eight subtrees per CTA at a time; the middle
+//    shuffles and votes, eight subtrees per CTA at a time; the one-warp
 //    instance forwards them here.
 //
 // Exactness: means and dispersions come from exact fixed-point integer sums;
@@ -49,10 +50,11 @@ namespace {
 
 constexpr int SMALL_N = 1024;       // largest node handled by one CTA
 constexpr int SMALL_THREADS = 256;
-constexpr int STACK_CAP = 256;
 constexpr int MID_N = 256;          // largest node of the middle CTA size
 constexpr int MID_THREADS = 128;
-constexpr int TINY_N = 32;          // largest node handled by one warp
+constexpr int WARP_N = 128;         // largest node of the one-warp CTAs
+constexpr int WARP_CTAS = 24;       // of which this many fit an SM (16 and 20 are 15% slower)
+constexpr int TINY_N = 32;          // largest node handled in one warp's registers
 constexpr int TINY_WARPS = 8;       // warps per block of the tiny-node kernel
 constexpr int TINY_STACK = 32;      // pending nodes per warp
 constexpr int TQ = 256;             // big-node tile (members per CTA)
@@ -80,10 +82,18 @@ __device__ __forceinline__ int ord_i(float f)
 
 __device__ __forceinline__ float ord_f(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
 
-__global__ void k_fill_s32(int32_t *p, int64_t n, int32_t v)
+// start values of the unwrap decision, and the size table of the subtree kernels
+__global__ void k_refine_init(int64_t G, int *gred, int *gmin, int nmax, double f, SizeTab *tab)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = v;
+    if (i < 12 * G) gred[i] = 0x7f800000;
+    if (i < G) gmin[i] = 0x7fffffff;
+    if (i <= nmax) {
+        long long kk = (long long)ceil(f * (double)i);
+        kk = kk < 1 ? 1 : (kk > i ? i : kk);
+        tab[i].inv_n = 1.0 / (double)i;
+        tab[i].kk = kk;
+    }
 }
 
 // group of member slot m (off[g] <= base + m < off[g + 1])
@@ -219,74 +229,186 @@ __global__ void k_make_roots(int64_t G, const int64_t *off, const int *gmin, con
     else small_list[atomicAdd(small_len, 1)] = id;
 }
 
+// pruning slack of the box bounds, and the margin of clique boxes (both explained
+// at the boxes, below)
+#define RS_PRUNE_SLACK 1.000003814697265625f  // 1 + 2^-18
+#define RS_CLIQUE_MARGIN 0.99999237060546875  // 1 - 2^-17
+
+// linking limits of one node: float32 band edges around l^2 (decided in
+// float64 inside them), the reporting band for ties, and the pruning radius
+struct LinkLim {
+    float lo, hi, tlo, thi, part, lim, cl_lim;
+    double l2, l;
+};
+
+__device__ __forceinline__ LinkLim link_lim(double l2)
+{
+    LinkLim r;
+    r.l2 = l2;
+    r.l = sqrt(l2);
+    r.lo = (float)(l2 * (1.0 - RS_BAND));
+    r.hi = (float)(l2 * (1.0 + RS_BAND));
+    r.tlo = (float)(l2 * (1.0 - 3e-6));
+    r.thi = (float)(l2 * (1.0 + 3e-6));
+    r.part = fmaxf(r.hi, r.thi);
+    r.lim = r.part * RS_PRUNE_SLACK;
+    r.cl_lim = (float)(l2 * RS_CLIQUE_MARGIN);
+    return r;
+}
+
+// the float32 edge of the linking and the tie bands: no pair beyond it matters
+__device__ __forceinline__ float link_part(double l2)
+{
+    return fmaxf((float)(l2 * (1.0 + RS_BAND)), (float)(l2 * (1.0 + 3e-6)));
+}
+
+// ---------------------------------------------------------------------------
+// half-precision points for the matrix units
+// ---------------------------------------------------------------------------
+// Pairs are screened by m16n8k8 half-precision products.  With points u of
+// six coordinates rounded to half, the product of (-2 u_q, 1, 1) and (u_c,
+// hi, lo) -- hi + lo the squared norm of the rounded u_c in two halves -- plus
+// |u_q|^2 in the float32 accumulator is |u^_q - u^_c|^2 for 16 x 8 pairs.  The
+// rounded points differ from the exact ones by at most
+//   delta = 1.02 2^-11 (|u_q| + |u_c|) + 3.1e-4
+// in all (half's relative 2^-11, the float32 steps before, and subnormal
+// halves even if they counted as zero), so the product's square root is
+// within delta of the pair's distance, up to float32 accumulation and lo's
+// rounding, below 2^-18 (|u_q| + |u_c|)^2 + 1e-4 on the square.  Screens use
+// these bounds one-sidedly: what they drop cannot matter, and what they pass
+// is evaluated in full.
+__device__ __forceinline__ void mma_m16n8k8_f16(float (&d)[4], unsigned a0, unsigned a1, unsigned b0, float c0,
+                                                float c1, float c2, float c3)
+{
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%7,%8,%9,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(b0), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
+}
+
+// the eight halves of a point: six coordinates u = (x - c) w, and the squared
+// norm s of the rounded coordinates in two halves
+__device__ __forceinline__ uint4 half_point(float4 p, float4 v, float4 pc, float4 vc, float wx, float wv, float &s)
+{
+    const __half2 h0 = __floats2half2_rn((p.x - pc.x) * wx, (p.y - pc.y) * wx),
+                  h1 = __floats2half2_rn((p.z - pc.z) * wx, (v.x - vc.x) * wv),
+                  h2 = __floats2half2_rn((v.y - vc.y) * wv, (v.z - vc.z) * wv);
+    const float2 f0 = __half22float2(h0), f1 = __half22float2(h1), f2 = __half22float2(h2);
+    s = f0.x * f0.x + f0.y * f0.y + f1.x * f1.x + f1.y * f1.y + f2.x * f2.x + f2.y * f2.y;
+    const __half hi = __float2half_rn(s);
+    const __half2 n = __halves2half2(hi, __float2half_rn(s - __half2float(hi)));
+    return make_uint4(*(const unsigned *)&h0, *(const unsigned *)&h1, *(const unsigned *)&h2, *(const unsigned *)&n);
+}
+
+constexpr unsigned HALF_ONES = 0x3c003c00u;  // (1, 1)
+constexpr unsigned HALF_FAR = 0x00007b00u;   // a squared norm of 57344: near nothing (with zero coordinates)
+
+// word t of a query's operand from word t of its point
+__device__ __forceinline__ unsigned half_query(unsigned word, int t)
+{
+    const __half2 h = __hmul2(*(const __half2 *)&word, __float2half2_rn(-2.f));
+    return t < 3 ? *(const unsigned *)&h : HALF_ONES;
+}
+
+__device__ __forceinline__ float half_norm(unsigned word3)
+{
+    const float2 f = __half22float2(*(const __half2 *)&word3);
+    return f.x + f.y;
+}
+
+// bound on the product's value over pairs at most d apart, a point of norm nq
+// against points within d of it
+__device__ __forceinline__ float half_bound(float d, float nq)
+{
+    const float rs = 2.f * nq + d;
+    const float e = d + 1.02f * 4.8828125e-4f * rs + 3.1e-4f;
+    return e * e * 1.00002f + 3.814697265625e-6f * rs * rs + 1.e-4f;
+}
+
+// bound on the distance of a point of norm nq from the one whose product with
+// it (without a threshold) is m
+__device__ __forceinline__ float half_reach(float m, float nq)
+{
+    const float s = sqrtf(fmaxf(m, 0.f)), rs = 2.f * nq + s;
+    const float d = sqrtf(s * s + 4.2e-6f * rs * rs + 2.e-4f);
+    return d + 1.05f * 4.8828125e-4f * (2.f * nq + d) + 3.5e-4f;
+}
+
 // ---------------------------------------------------------------------------
 // small nodes: whole subtree in one CTA
 // ---------------------------------------------------------------------------
 template <int NMAX, int NT>
 struct SmallShared {
-    float px[NMAX], py[NMAX], pz[NMAX], vx[NMAX], vy[NMAX], vz[NMAX];
+    float4 a[NMAX];   // px, py, pz, vx
+    float2 b[NMAX];   // vy, vz
+    uint4 half[NMAX]; // the node's points (from 0); later, counts of the child partition
     int idx[NMAX];
     float dnn[NMAX];
-    int par[NMAX];
-    int csize[NMAX];
-    int cmin[NMAX];
-    unsigned long long key[NMAX];
-    float tp[6][NMAX];
-    int tidx[NMAX];
+    int par[NMAX];    // union-find; before it, the band's members
+    int csize[2 * NMAX];  // component sizes, then child numbers; before, the band's values (doubles)
+    int pairs[NT / 32][64];
+    int2 child[NMAX / 2];  // (smallest particle index, first position) of the children
+    // pending nodes: pairwise disjoint and larger than the next tier's limit
+    // (at least 10, rs_tuning::tiny_max's least)
+    static constexpr int STACK_CAP = NMAX / 10 + 2;
     int4 stack[STACK_CAP];
-    int sp;
-    int job;
     MomAcc wacc[NT / 32];
     Metric6 met;
     double l2;
-    float lo32, hi32, tlo32, thi32;
-    int nband, below, tie, nchild;
-    int pick;
+    float4 pc, vc;  // the half frame's centre; .w: weights
+    float t32;
+    int sp, job, umax, nband, below, tie, nchild, next[2];
 };
 
 template <class SS>
 __device__ __forceinline__ float4 sp4(const SS &S, int i)
 {
-    return make_float4(S.px[i], S.py[i], S.pz[i], 0.f);
+    const float4 x = S.a[i];
+    return make_float4(x.x, x.y, x.z, 0.f);
 }
 template <class SS>
 __device__ __forceinline__ float4 sv4(const SS &S, int i)
 {
-    return make_float4(S.vx[i], S.vy[i], S.vz[i], 0.f);
-}
-
-// in-place ascending bitonic sort of S.key[0 .. P), P a power of two
-__device__ void bitonic_u64(unsigned long long *key, int P)
-{
-    for (int k = 2; k <= P; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int t = threadIdx.x; t < P / 2; t += blockDim.x) {
-                int i = 2 * j * (t / j) + (t % j);
-                int l = i + j;
-                bool up = (i & k) == 0;
-                unsigned long long a = key[i], b = key[l];
-                if ((a > b) == up) {
-                    key[i] = b;
-                    key[l] = a;
-                }
-            }
-            __syncthreads();
-        }
-    }
+    const float2 y = S.b[i];
+    return make_float4(S.a[i].w, y.x, y.y, 0.f);
 }
 
 // One CTA of NT threads per subtree of at most NMAX members; nodes of at most
 // `fwd_limit` members (roots or children) go to the next queue, whose kernel
 // runs after this one (members are written back in their final order).
+//
+// A node's n^2 pair loops run on the matrix units, 16 members (a warp's rows)
+// against 8 a product.  Nearest neighbours take two passes: the smallest
+// product of each row, then the pairs whose product could be the row's
+// nearest given it; those are evaluated in float32.  The friends-of-friends
+// pass screens the pairs after each member at the linking length.  Passed
+// pairs are queued by the warp and evaluated 32 at a time, so results are
+// those of the full loops.  The k-th value is found by bisection on its bits
+// in one warp, and the children are placed by a stable count instead of a
+// sort, so a node costs about 20 block barriers instead of 130.
+//
+// Issue-bound in the largest instance, by instruction fetch in the one-warp
+// one (its warps run at different places of the code, hence one copy of the
+// pair loops for both rounds and little unrolling: 2.05 -> 1.52 ms), and
+// earlier by the float64 unit, which executes about 2 lanes a clock: what can
+// be is taken from tables, done in float32 with the same rounding, or left to
+// k_tree_stats.  5.0M members in 29,000 groups of 20-600: nodes above 256
+// members 6.9 -> 2.0 ms, 33-256 3.9 -> 2.5 ms (as one 128-thread tier 4.1), up
+// to 32 1.08 -> 0.67 ms.
 template <int NMAX, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
     k_small_subtree(const int *queue, const int *queue_len, int *queue_head, float4 *wpos, float4 *wvel, int *widx,
-                    int fwd_limit, int *fwd_q, int *fwd_len, NodeArrays nd, double box, double f, int min_n,
-                    rs_dev_status *st)
+                    int fwd_limit, int *fwd_q, int *fwd_len, NodeArrays nd, const SizeTab *size_tab, double box,
+                    int min_n, rs_dev_status *st)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SmallShared<NMAX, NT> &S = *reinterpret_cast<SmallShared<NMAX, NT> *>(smem_raw);
-    const int tid = threadIdx.x;
+    constexpr int NW = NT / 32, PER = NMAX / NT;
+    static_assert(NW * 32 * PER == NMAX, "");
+    const unsigned FULL = 0xffffffffu;
+    const int tid = threadIdx.x, lane = lane_id(), w = warp_id();
+    const unsigned below_me = (1u << lane) - 1u;
+    const int g = lane >> 2, t4 = lane & 3;  // the product's row and column group of this lane
+    int *cmin = S.csize + NMAX;
     for (;;) {
         if (tid == 0) S.job = atomicAdd(queue_head, 1);
         __syncthreads();
@@ -302,12 +424,8 @@ __global__ void __launch_bounds__(NT, MINB)
         }
         for (int i = tid; i < n0; i += NT) {
             float4 p = wpos[base + i], v = wvel[base + i];
-            S.px[i] = p.x;
-            S.py[i] = p.y;
-            S.pz[i] = p.z;
-            S.vx[i] = v.x;
-            S.vy[i] = v.y;
-            S.vz[i] = v.z;
+            S.a[i] = make_float4(p.x, p.y, p.z, v.x);
+            S.b[i] = make_float2(v.y, v.z);
             S.idx[i] = widx[base + i];
         }
         if (tid == 0) {
@@ -317,242 +435,408 @@ __global__ void __launch_bounds__(NT, MINB)
         __syncthreads();
         for (int guard = 0; guard < 1 << 20; guard++) {
             if (S.sp == 0) break;
-            __syncthreads();
-            int4 top;
-            top = S.stack[S.sp - 1];
-            __syncthreads();
-            if (tid == 0) S.sp--;
+            const int4 top = S.stack[S.sp - 1];
             const int lf = top.x, cnt = top.y, node = top.z, lev = top.w;
             // ---- moments (exact) ----
             {
-                MomRef ref = mom_ref(sp4(S, lf), sv4(S, lf));
+                const MomRef ref = mom_ref(sp4(S, lf), sv4(S, lf));
                 MomAcc a;
                 mom_zero(a);
                 for (int i = lf + tid; i < lf + cnt; i += NT) mom_add(a, sp4(S, i), sv4(S, i), ref);
                 mom_warp_reduce(a);
-                if (lane_id() == 0) S.wacc[warp_id()] = a;
+                if (lane == 0) S.wacc[w] = a;
                 __syncthreads();
-                if (tid == 0) {
-                    MomAcc t = S.wacc[0];
-                    for (int w = 1; w < NT / 32; w++) mom_merge(t, S.wacc[w]);
-                    MomOut o = mom_finalize(t, sp4(S, lf), sv4(S, lf), cnt, box);
-                    for (int d = 0; d < 3; d++) {
-                        nd.xbar[3 * node + d] = o.xbar[d];
-                        nd.vbar[3 * node + d] = o.vbar[d];
+                if (w == 0) {
+                    const float4 pr = sp4(S, lf), vr = sv4(S, lf);
+                    const MomOutWarp o = mom_finalize_warp(S.wacc, NW, pr, vr, size_tab[cnt].inv_n, box);
+                    if (lane < 3) {
+                        nd.xbar[3 * node + lane] = o.xbar;
+                        nd.vbar[3 * node + lane] = o.vbar;
                     }
-                    nd.sigx[node] = o.sigx;
-                    nd.sigv[node] = o.sigv;
-                    S.met = metric_of(o.sigx, o.sigv);
-                    S.nband = 0;
-                    S.below = 0;
-                    S.tie = 0;
-                    S.nchild = 0;
+                    const Metric6 m = metric_of_warp(o.sigx, o.sigv);
+                    if (lane == 0) {
+                        nd.sigx[node] = o.sigx;
+                        nd.sigv[node] = o.sigv;
+                        S.met = m;
+                        const float fx = (float)o.sigx, fv = (float)o.sigv;
+                        // half frame: units of a quarter dispersion about the mean, so
+                        // |u| <= 4 sqrt(2 n) = 181 and subnormal halves stay far below
+                        // the distances
+                        S.pc = make_float4(o.cx[0], o.cx[1], o.cx[2], fx > 0.f ? 4.f / fx : 0.f);
+                        S.vc = make_float4(o.cx[3], o.cx[4], o.cx[5], fv > 0.f ? 4.f / fv : 0.f);
+                        S.umax = 0;
+                        S.nband = 0;
+                        S.below = 0;
+                        S.tie = 0;
+                        S.nchild = 0;
+                        S.next[0] = S.next[1] = 0;
+                        S.sp--;
+                    }
                 }
                 __syncthreads();
             }
             const Metric6 met = S.met;
-            // ---- nearest neighbours (float32) ----
-            for (int q = lf + tid; q < lf + cnt; q += NT) {
-                const float4 pq = sp4(S, q), vq = sv4(S, q);
-                float best = INFINITY;
-                for (int c = lf; c < lf + cnt; c++) {
-                    if (c == q) continue;
-                    float d2 = d2_32(pq, vq, sp4(S, c), sv4(S, c), met);
-                    best = fminf(best, d2);
-                }
-                S.dnn[q] = best;
-            }
-            __syncthreads();
-            // ---- k-th smallest, float32 ----
-            int P = 1;
-            while (P < cnt) P <<= 1;
-            for (int i = tid; i < P; i += NT)
-                S.key[i] = i < cnt ? (unsigned long long)__float_as_uint(S.dnn[lf + i]) : ~0ull;
-            __syncthreads();
-            bitonic_u64(S.key, P);
-            long long kk = (long long)ceil(f * (double)cnt);
-            if (kk < 1) kk = 1;
-            if (kk > cnt) kk = cnt;
-            const float t32 = __uint_as_float((unsigned)S.key[kk - 1]);
-            const float blo = (float)((double)t32 * (1.0 - 2.0 * RS_BAND));
-            const float bhi = (float)((double)t32 * (1.0 + 2.0 * RS_BAND));
-            __syncthreads();
-            // ---- band members: exact float64 nearest-neighbour distances ----
-            // (one warp per band member, lanes over the candidates)
-            double *bval = reinterpret_cast<double *>(S.key);
-            int *blist = S.tidx;
-            for (int q = lf + tid; q < lf + cnt; q += NT) {
-                const float dq = S.dnn[q];
-                if (dq < blo)
-                    atomicAdd(&S.below, 1);
-                else if (dq <= bhi)
-                    blist[atomicAdd(&S.nband, 1)] = q;
-            }
-            __syncthreads();
-            for (int b = warp_id(); b < S.nband; b += NT / 32) {
-                const int q = blist[b];
-                const float4 pq = sp4(S, q), vq = sv4(S, q);
-                const float lim = S.dnn[q] * (float)(1.0 + 2.0 * RS_BAND);
-                double best = INFINITY;
-                for (int c = lf + lane_id(); c < lf + cnt; c += 32) {
-                    if (c == q) continue;
-                    const float4 pc = sp4(S, c), vc = sv4(S, c);
-                    if (d2_32(pq, vq, pc, vc, met) <= lim) best = fmin(best, d2_64(pq, vq, pc, vc, met));
-                }
-                for (int o = 16; o > 0; o >>= 1) best = fmin(best, __shfl_xor_sync(0xffffffffu, best, o));
-                if (lane_id() == 0) bval[b] = best;
-            }
-            __syncthreads();
-            // rank the band: the exact k-th value is the (k - 1 - below)-th
+            const int nblk = (cnt + 7) >> 3, ntile = (cnt + 15) >> 4;
             {
-                const int nb = S.nband, want = (int)(kk - 1) - S.below;
-                if (want < 0 || want >= nb) {
-                    if (tid == 0) dev_fail(st, DEV_INTERNAL, 40, node);
-                }
-                for (int b = tid; b < nb; b += NT) {
-                    int r = 0;
-                    const double vb = bval[b];
-                    for (int c = 0; c < nb; c++) r += (bval[c] < vb || (bval[c] == vb && c < b)) ? 1 : 0;
-                    if (r == want) S.l2 = vb;
-                }
-                __syncthreads();
-            }
-            const double l2 = S.l2;
-            if (tid == 0) {
-                S.lo32 = (float)(l2 * (1.0 - RS_BAND));
-                S.hi32 = (float)(l2 * (1.0 + RS_BAND));
-                S.tlo32 = (float)(l2 * (1.0 - 3e-6));
-                S.thi32 = (float)(l2 * (1.0 + 3e-6));
-                nd.lnk[node] = sqrt(l2 / met.scale);
-            }
-            for (int i = lf + tid; i < lf + cnt; i += NT) S.par[i] = i;
-            __syncthreads();
-            // ---- friends-of-friends at l (inclusive) ----
-            {
-                const float lo = S.lo32, hi = S.hi32, tlo = S.tlo32, thi = S.thi32;
-                const float part = fmaxf(hi, thi);
-                const double l = sqrt(l2);
-                int tie = 0;
-                // warp-uniform candidate loop from the warp's first query: the
-                // candidate test and its loads are the same for every lane
-                for (int qb = lf + 32 * warp_id(); qb < lf + cnt; qb += NT) {
-                    const int q = qb + lane_id();
-                    const bool act = q < lf + cnt && S.dnn[q] <= part;
-                    if (!__any_sync(0xffffffffu, act)) continue;
-                    const float4 pq = act ? sp4(S, q) : make_float4(0, 0, 0, 0);
-                    const float4 vq = act ? sv4(S, q) : make_float4(0, 0, 0, 0);
-                    for (int c = qb + 1; c < lf + cnt; c++) {
-                        if (S.dnn[c] > part) continue;
-                        const float4 pc = sp4(S, c), vc = sv4(S, c);
-                        if (!act || c <= q) continue;
-                        const float d2 = d2_32(pq, vq, pc, vc, met);
-                        if (d2 > part) continue;
-                        // below both bands: a friend, and not a tie-band pair
-                        bool link = d2 < fminf(lo, tlo);
-                        if (!link) {
-                            const double e = d2_64(pq, vq, pc, vc, met);
-                            link = e <= l2;
-                            if (l2 > 0 && e != l2 && fabs(sqrt(e) - l) <= 1e-6 * l) tie++;
+                float um = 0.f;
+                const float4 pc = S.pc, vc = S.vc;
+                for (int i = tid; i < 8 * nblk; i += NT) {
+                    uint4 h = make_uint4(0u, 0u, 0u, HALF_FAR);
+                    if (i < cnt) {
+                        float s;
+                        h = half_point(sp4(S, lf + i), sv4(S, lf + i), pc, vc, pc.w, vc.w, s);
+                        if (!(s < 5e4f)) {  // outside half's range: every pair will be evaluated
+                            s = INFINITY;
+                            h = make_uint4(0u, 0u, 0u, 0u);
                         }
-                        if (link) uf_union_s(S.par, q, c, st);
+                        um = fmaxf(um, s);
+                        S.dnn[lf + i] = INFINITY;
+                    }
+                    S.half[i] = h;
+                }
+                um = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(um)));
+                if (lane == 0) atomicMax(&S.umax, __float_as_int(um));
+            }
+            __syncthreads();
+            const bool in_range = __int_as_float(S.umax) < 5e4f;
+            const unsigned *hw = reinterpret_cast<const unsigned *>(S.half);
+            int *queue_w = S.pairs[w];
+            double l2 = 0.0;
+            float lo = 0.f, part = 0.f, lu = 0.f;
+            bool screen = in_range;
+            int tie = 0;
+            // Two rounds over the tiles: nearest neighbours, then (after the
+            // linking length) friends.  One copy of the code for both: the
+            // one-warp CTAs run at different places of it, and what they wait
+            // for most is the instruction cache.
+#pragma unroll 1
+            for (int round = 0; round < 2; round++) {
+                if (round == 1) {
+                    __syncthreads();
+                    // ---- k-th smallest, float32: bisection on the bits, in one warp ----
+                    const int kk = (int)size_tab[cnt].kk;
+                    if (w == 0) {
+                        unsigned v[NMAX / 32];
+                        unsigned x0 = 0xffffffffu, x1 = 0u;
+#pragma unroll
+                        for (int r = 0; r < NMAX / 32; r++) {
+                            const int i = 32 * r + lane;
+                            v[r] = i < cnt ? __float_as_uint(S.dnn[lf + i]) : 0xffffffffu;
+                            x0 = min(x0, v[r]);
+                            if (i < cnt) x1 = max(x1, v[r]);
+                        }
+                        x0 = __reduce_min_sync(FULL, x0);
+                        x1 = __reduce_max_sync(FULL, x1);
+                        while (x0 < x1) {  // the smallest x with kk values at most x
+                            const unsigned mid = x0 + ((x1 - x0) >> 1);
+                            int c = 0;
+#pragma unroll
+                            for (int r = 0; r < NMAX / 32; r++) c += v[r] <= mid ? 1 : 0;
+                            if (__reduce_add_sync(FULL, (unsigned)c) >= (unsigned)kk) x1 = mid;
+                            else x0 = mid + 1u;
+                        }
+                        if (lane == 0) S.t32 = __uint_as_float(x0);
+                    }
+                    __syncthreads();
+                    const float t32 = S.t32;
+                    // t32 (1 -+ 2 RS_BAND), rounded once: 2 RS_BAND = 2^-19
+                    const float blo = fmaf(t32, (float)(-2.0 * RS_BAND), t32),
+                                bhi = fmaf(t32, (float)(2.0 * RS_BAND), t32);
+                    // ---- band members: exact float64 nearest-neighbour distances ----
+                    // (the whole block over the candidates of one band member after another)
+                    unsigned long long *bval = reinterpret_cast<unsigned long long *>(S.csize);
+                    int *blist = S.par;
+                    for (int i = tid; i < 32 * ((cnt + 31) / 32); i += NT) {
+                        const float dq = i < cnt ? S.dnn[lf + i] : INFINITY;
+                        const unsigned bm = __ballot_sync(FULL, dq < blo);
+                        if (lane == 0 && bm) atomicAdd(&S.below, __popc(bm));
+                        if (i < cnt && dq >= blo && dq <= bhi) {
+                            const int b = atomicAdd(&S.nband, 1);
+                            blist[b] = lf + i;
+                            bval[b] = 0x7ff0000000000000ull;  // +infinity
+                        }
+                    }
+                    __syncthreads();
+                    const int nb = S.nband;
+                    for (int b = 0; b < nb; b++) {
+                        const int q = blist[b];
+                        const float4 pq = sp4(S, q), vq = sv4(S, q);
+                        const float lim = S.dnn[q] * (float)(1.0 + 2.0 * RS_BAND);
+#pragma unroll 1
+                        for (int c = lf + tid; c < lf + cnt; c += NT) {
+                            if (c == q) continue;
+                            const float4 pc = sp4(S, c), vc = sv4(S, c);
+                            if (d2_32(pq, vq, pc, vc, met) <= lim)
+                                atomicMin(&bval[b],
+                                          (unsigned long long)__double_as_longlong(d2_64(pq, vq, pc, vc, met)));
+                        }
+                    }
+                    __syncthreads();
+                    // rank the band: the exact k-th value is the (k - 1 - below)-th
+                    const int want = kk - 1 - S.below;
+                    if ((want < 0 || want >= nb) && tid == 0) dev_fail(st, DEV_INTERNAL, 40, node);
+                    for (int b = tid; b < nb; b += NT) {
+                        int r = 0;
+                        const unsigned long long vb = bval[b];
+                        for (int c = 0; c < nb; c++) r += (bval[c] < vb || (bval[c] == vb && c < b)) ? 1 : 0;
+                        if (r == want) {
+                            S.l2 = __longlong_as_double((long long)vb);
+                            nd.lnk[node] = S.l2;  // k_tree_stats makes it a length
+                        }
+                    }
+                    __syncthreads();
+                    l2 = S.l2;
+                    for (int i = lf + tid; i < lf + cnt; i += NT) {
+                        S.par[i] = i;
+                        S.csize[i] = 0;
+                        cmin[i] = 0x7fffffff;
+                    }
+                    __syncthreads();
+                    lo = fminf((float)(l2 * (1.0 - RS_BAND)), (float)(l2 * (1.0 - 3e-6)));
+                    part = link_part(l2);
+                    // the linking length in the half frame's units (a metric
+                    // whose scale float32 cannot hold screens nothing)
+                    const float sc = (float)met.scale;
+                    lu = 4.f * sqrtf(part / sc) * 1.000001f;
+                    screen = in_range && lu < 1e4f && sc > 1e-30f && part > 1e-30f;
+                }
+                int np = 0;
+                auto flush = [&](int k) {
+                    np -= k;
+                    const int code = lane < k ? queue_w[np + lane] : 0, q = lf + (code >> 10), c = lf + (code & 1023);
+                    if (q != c) {
+                        const float4 pq = sp4(S, q), vq = sv4(S, q), pc = sp4(S, c), vc = sv4(S, c);
+                        const float d2 = d2_32(pq, vq, pc, vc, met);
+                        if (round == 0) {
+                            atomicMin(reinterpret_cast<int *>(&S.dnn[q]), __float_as_int(d2));
+                        } else if (d2 <= part) {
+                            // below both bands: a friend, and not a tie-band pair
+                            bool link = d2 < lo;
+                            if (!link) {
+                                const double e = d2_64(pq, vq, pc, vc, met), l = sqrt(l2);
+                                link = e <= l2;
+                                if (l2 > 0 && e != l2 && fabs(sqrt(e) - l) <= 1e-6 * l) tie++;
+                            }
+                            if (link) uf_union_s(S.par, q, c, st);
+                        }
+                    }
+                    __syncwarp();
+                };
+                for (;;) {
+                    int tl = 0;
+                    if (lane == 0) tl = atomicAdd(&S.next[round], 1);
+                    tl = __shfl_sync(FULL, tl, 0);
+                    if (tl >= ntile) break;
+                    const int r0 = 16 * tl + g, r1 = r0 + 8;  // this lane's two rows
+                    const int q0 = min(r0, cnt - 1), q1 = min(r1, cnt - 1);
+                    const unsigned a0 = half_query(hw[4 * q0 + t4], t4), a1 = half_query(hw[4 * q1 + t4], t4);
+                    const float s0 = half_norm(hw[4 * q0 + 3]), s1 = half_norm(hw[4 * q1 + 3]);
+                    bool k0 = r0 < cnt, k1 = r1 < cnt;
+                    float d0 = lu, d1 = lu;
+                    if (round == 0) {
+                        // the smallest product of each row: the nearest is at
+                        // most sqrt(m) + delta away, so its own product is at
+                        // most the bound for that distance
+                        float m0 = INFINITY, m1 = INFINITY;
+#pragma unroll 2
+                        for (int j = 0; j < nblk; j++) {
+                            float d[4];
+                            mma_m16n8k8_f16(d, a0, a1, hw[4 * (8 * j + g) + t4], s0, s0, s1, s1);
+                            if ((j >> 1) == tl) {  // not itself
+                                const int c = 8 * j + 2 * t4;
+                                if (c == r0) d[0] = INFINITY;
+                                if (c + 1 == r0) d[1] = INFINITY;
+                                if (c == r1) d[2] = INFINITY;
+                                if (c + 1 == r1) d[3] = INFINITY;
+                            }
+                            m0 = fminf(m0, fminf(d[0], d[1]));
+                            m1 = fminf(m1, fminf(d[2], d[3]));
+                        }
+#pragma unroll
+                        for (int o = 1; o < 4; o <<= 1) {
+                            m0 = fminf(m0, __shfl_xor_sync(FULL, m0, o));
+                            m1 = fminf(m1, __shfl_xor_sync(FULL, m1, o));
+                        }
+                        d0 = half_reach(m0, sqrtf(s0));
+                        d1 = half_reach(m1, sqrtf(s1));
+                    } else {
+                        k0 = k0 && S.dnn[lf + q0] <= part;
+                        k1 = k1 && S.dnn[lf + q1] <= part;
+                        if (!__any_sync(FULL, k0 || k1)) continue;
+                    }
+                    const float c0 = !k0 ? 60000.f : (screen ? s0 - half_bound(d0, sqrtf(s0)) : -INFINITY);
+                    const float c1 = !k1 ? 60000.f : (screen ? s1 - half_bound(d1, sqrtf(s1)) : -INFINITY);
+                    for (int jb = round == 0 ? 0 : 2 * tl; jb < nblk; jb += 8) {
+                        // the signs of eight blocks' products, oldest at the top
+                        unsigned mask = 0;
+                        const int je = min(8, nblk - jb);
+#pragma unroll 2
+                        for (int j = 0; j < je; j++) {
+                            float d[4];
+                            mma_m16n8k8_f16(d, a0, a1, hw[4 * (8 * (jb + j) + g) + t4], c0, c0, c1, c1);
+#pragma unroll
+                            for (int i = 0; i < 4; i++) mask = __funnelshift_l(__float_as_uint(d[i]), mask, 1);
+                        }
+                        mask <<= 32 - 4 * je;
+                        while (__any_sync(FULL, mask != 0)) {
+                            bool push = false;
+                            int q = 0, c = 0;
+                            if (mask) {
+                                const int e = __clz(mask);
+                                mask &= ~(0x80000000u >> e);
+                                q = (e & 2) ? r1 : r0;
+                                c = 8 * (jb + (e >> 2)) + 2 * t4 + (e & 1);
+                                push = c < cnt && (round == 0 ? c != q : c > q);
+                            }
+                            const unsigned bm = __ballot_sync(FULL, push);
+                            if (push) queue_w[np + __popc(bm & below_me)] = (q << 10) | c;
+                            np += __popc(bm);
+                            __syncwarp();
+                            // evaluate when full, and what is left at the end
+                            if (np >= 32) flush(32);
+                        }
                     }
                 }
-                tie = warp_sum(tie);
-                if (lane_id() == 0 && tie) atomicAdd(&S.tie, tie);
+                if (np > 0) flush(np);
+            }
+            tie = warp_sum(tie);
+            if (lane == 0 && tie) atomicAdd(&S.tie, tie);
+            __syncthreads();
+            // ---- components (lanes of one component add once) ----
+            // each warp takes a run of the members, PER a lane
+            const int run = 32 * ((cnt + 32 * NW - 1) / (32 * NW)), i0 = w * run;
+#pragma unroll
+            for (int r = 0; r < PER; r++) {
+                const int i = i0 + 32 * r + lane;
+                const bool ok = 32 * r < run && i < cnt;
+                const int root = ok ? uf_find_s(S.par, lf + i) : -1;
+                const unsigned peers = __match_any_sync(FULL, root);
+                const int mi = (int)__reduce_min_sync(peers, ok ? (unsigned)S.idx[lf + i] : 0x7fffffffu);
+                if (ok && (peers & below_me) == 0) {
+                    atomicAdd(&S.csize[root], __popc(peers));
+                    atomicMin(&cmin[root], mi);
+                }
             }
             __syncthreads();
-            // ---- components ----
+            // ---- children, numbered as found; the others are the rest ----
             for (int i = lf + tid; i < lf + cnt; i += NT) {
-                S.csize[i] = 0;
-                S.cmin[i] = 0x7fffffff;
-            }
-            __syncthreads();
-            for (int i = lf + tid; i < lf + cnt; i += NT) {
-                int r = uf_find_s(S.par, i);
-                S.par[i] = r;
-                atomicAdd(&S.csize[r], 1);
-                atomicMin(&S.cmin[r], S.idx[i]);
-            }
-            __syncthreads();
-            // ---- children first (by smallest particle index), then the rest ----
-            for (int i = tid; i < P; i += NT) {
-                unsigned long long k = ~0ull;
-                if (i < cnt) {
-                    int r = S.par[lf + i];
-                    int sz = S.csize[r];
-                    unsigned hiw = (sz >= min_n && sz < cnt) ? (unsigned)S.cmin[r] : 0xffffffffu;
-                    k = ((unsigned long long)hiw << 32) | (unsigned)i;
-                }
-                S.key[i] = k;
-            }
-            __syncthreads();
-            bitonic_u64(S.key, P);
-            for (int p = tid; p < cnt; p += NT) {
-                int o = lf + (int)(S.key[p] & 0xffffffffu);
-                S.tp[0][p] = S.px[o];
-                S.tp[1][p] = S.py[o];
-                S.tp[2][p] = S.pz[o];
-                S.tp[3][p] = S.vx[o];
-                S.tp[4][p] = S.vy[o];
-                S.tp[5][p] = S.vz[o];
-                S.tidx[p] = S.idx[o];
-            }
-            __syncthreads();
-            for (int p = tid; p < cnt; p += NT) {
-                S.px[lf + p] = S.tp[0][p];
-                S.py[lf + p] = S.tp[1][p];
-                S.pz[lf + p] = S.tp[2][p];
-                S.vx[lf + p] = S.tp[3][p];
-                S.vy[lf + p] = S.tp[4][p];
-                S.vz[lf + p] = S.tp[5][p];
-                S.idx[lf + p] = S.tidx[p];
-            }
-            __syncthreads();
-            for (int p = tid; p < cnt; p += NT) {
-                const unsigned hiw = (unsigned)(S.key[p] >> 32);
-                if (hiw == 0xffffffffu) continue;
-                if (p > 0 && (unsigned)(S.key[p - 1] >> 32) == hiw) continue;
-                int e = p + 1;
-                while (e < cnt && (unsigned)(S.key[e] >> 32) == hiw) e++;
-                int id = atomicAdd(nd.counter, 1);
-                if (id >= nd.cap) {
-                    dev_fail(st, DEV_OVERFLOW, 41, id);
-                    continue;
-                }
-                nd.parent[id] = node;
-                nd.level[id] = lev + 1;
-                nd.first[id] = base + lf + p;
-                nd.count[id] = e - p;
-                nd.minidx[id] = (int)hiw;
-                nd.nchild[id] = 0;
-                nd.tie[id] = 0;
-                nd.root[id] = nd.root[node];
-                nd.shift[id] = nd.shift[node];
-                atomicAdd(&S.nchild, 1);
-                if (e - p <= fwd_limit) {  // its subtree goes to the next, smaller kernel
-                    fwd_q[atomicAdd(fwd_len, 1)] = id;
-                    continue;
-                }
-                int s = atomicAdd(&S.sp, 1);
-                if (s >= STACK_CAP) {
-                    dev_fail(st, DEV_OVERFLOW, 42, s);
-                    atomicSub(&S.sp, 1);
+                if (S.par[i] != i) continue;
+                const int sz = S.csize[i];
+                if (sz >= min_n && sz < cnt) {
+                    const int c = atomicAdd(&S.nchild, 1);
+                    S.child[c] = make_int2(cmin[i], sz);
+                    cmin[i] = c;
                 } else {
-                    S.stack[s] = make_int4(lf + p, e - p, id, lev + 1);
+                    cmin[i] = -1;
                 }
             }
             __syncthreads();
+            const int nc = S.nchild;
+            if (nc > 0) {
+                // their places (by smallest particle index, the rest after
+                // them) and their nodes
+                unsigned short *wc = reinterpret_cast<unsigned short *>(S.half);  // [NW][nc + 1]
+                for (int i = tid; i < NW * (nc + 1); i += NT) wc[i] = 0;
+                int *place = reinterpret_cast<int *>(wc + NW * (nc + 1) + ((NW * (nc + 1)) & 1));
+                for (int c = tid; c <= nc; c += NT) {
+                    const int2 me = c < nc ? S.child[c] : make_int2(0x7fffffff, 0);
+                    int at = 0;
+                    for (int o = 0; o < nc; o++) {
+                        const int2 ch = S.child[o];
+                        at += ch.x < me.x ? ch.y : 0;
+                    }
+                    place[c] = at;
+                    if (c == nc) continue;
+                    const int id = atomicAdd(nd.counter, 1);
+                    if (id >= nd.cap) {
+                        dev_fail(st, DEV_OVERFLOW, 41, id);
+                        continue;
+                    }
+                    nd.parent[id] = node;
+                    nd.level[id] = lev + 1;
+                    nd.first[id] = base + lf + at;
+                    nd.count[id] = me.y;
+                    nd.minidx[id] = me.x;
+                    nd.nchild[id] = 0;
+                    nd.tie[id] = 0;
+                    nd.root[id] = nd.root[node];
+                    nd.shift[id] = nd.shift[node];
+                    if (me.y <= fwd_limit) {  // its subtree goes to the next, smaller kernel
+                        fwd_q[atomicAdd(fwd_len, 1)] = id;
+                        continue;
+                    }
+                    const int s = atomicAdd(&S.sp, 1);
+                    if (s >= SmallShared<NMAX, NT>::STACK_CAP) {
+                        dev_fail(st, DEV_OVERFLOW, 42, s);
+                        atomicSub(&S.sp, 1);
+                    } else {
+                        S.stack[s] = make_int4(lf + at, me.y, id, lev + 1);
+                    }
+                }
+                __syncthreads();
+                // stable places: the members of one child before this one, in
+                // its warp's run and in the runs of the warps before
+                int grp[PER], rank[PER];
+#pragma unroll
+                for (int r = 0; r < PER; r++) {
+                    const int i = i0 + 32 * r + lane;
+                    const bool ok = 32 * r < run && i < cnt;
+                    int c = ok ? cmin[uf_find_s(S.par, lf + i)] : -2;
+                    if (c == -1) c = nc;
+                    const unsigned peers = __match_any_sync(FULL, c);
+                    const unsigned before = ok ? wc[w * (nc + 1) + c] : 0u;
+                    __syncwarp();
+                    if (ok && (peers & below_me) == 0) wc[w * (nc + 1) + c] = (unsigned short)(before + __popc(peers));
+                    __syncwarp();
+                    grp[r] = c;
+                    rank[r] = (int)before + __popc(peers & below_me);
+                }
+                __syncthreads();
+                for (int c = tid; c <= nc; c += NT) {
+                    unsigned tot = 0;
+                    for (int u = 0; u < NW; u++) {
+                        const unsigned x = wc[u * (nc + 1) + c];
+                        wc[u * (nc + 1) + c] = (unsigned short)tot;
+                        tot += x;
+                    }
+                }
+                float4 ra[PER];
+                float2 rb[PER];
+                int ri[PER];
+#pragma unroll
+                for (int r = 0; r < PER; r++) {
+                    const int i = i0 + 32 * r + lane;
+                    if (32 * r < run && i < cnt) {
+                        ra[r] = S.a[lf + i];
+                        rb[r] = S.b[lf + i];
+                        ri[r] = S.idx[lf + i];
+                    }
+                }
+                __syncthreads();
+#pragma unroll
+                for (int r = 0; r < PER; r++) {
+                    const int i = i0 + 32 * r + lane;
+                    if (32 * r < run && i < cnt) {
+                        const int to = lf + place[grp[r]] + wc[w * (nc + 1) + grp[r]] + rank[r];
+                        S.a[to] = ra[r];
+                        S.b[to] = rb[r];
+                        S.idx[to] = ri[r];
+                    }
+                }
+            }
             if (tid == 0) {
-                nd.nchild[node] = S.nchild;
+                nd.nchild[node] = nc;
                 nd.tie[node] = S.tie;
             }
             __syncthreads();
         }
         // members in their final order (the tiny-node kernel reads its nodes here)
         for (int i = tid; i < n0; i += NT) {
+            const float4 x = S.a[i];
+            const float2 y = S.b[i];
             widx[base + i] = S.idx[i];
-            wpos[base + i] = make_float4(S.px[i], S.py[i], S.pz[i], 0.f);
-            wvel[base + i] = make_float4(S.vx[i], S.vy[i], S.vz[i], 0.f);
+            wpos[base + i] = make_float4(x.x, x.y, x.z, 0.f);
+            wvel[base + i] = make_float4(x.w, y.x, y.y, 0.f);
         }
         __syncthreads();
     }
@@ -590,8 +874,9 @@ __device__ __forceinline__ unsigned long long warp_sort_u64(unsigned long long k
 // then children first by smallest particle index and the rest after them.
 __global__ void __launch_bounds__(TINY_WARPS * 32)
     k_tiny_subtree(const int *queue, const int *queue_len, int *queue_head, const float4 *wpos, const float4 *wvel,
-                   int *widx, NodeArrays nd, double box, double f, int min_n, rs_dev_status *st)
+                   int *widx, NodeArrays nd, const SizeTab *size_tab, double box, int min_n, rs_dev_status *st)
 {
+    __shared__ MomAcc acc_s[TINY_WARPS];
     __shared__ int par_s[TINY_WARPS][32];
     __shared__ int csz_s[TINY_WARPS][32];
     __shared__ int cmin_s[TINY_WARPS][32];
@@ -633,28 +918,19 @@ __global__ void __launch_bounds__(TINY_WARPS * 32)
             mom_zero(a);
             if (mine) mom_add(a, p, v, mom_ref(pr, vr));
             mom_warp_reduce(a);
-            Metric6 met;
-            {
-                double ax64 = 0, av64 = 0, scale = 0;
-                if (lane == 0) {
-                    const MomOut o = mom_finalize(a, pr, vr, cnt, box);
-                    for (int d = 0; d < 3; d++) {
-                        nd.xbar[3 * node + d] = o.xbar[d];
-                        nd.vbar[3 * node + d] = o.vbar[d];
-                    }
-                    nd.sigx[node] = o.sigx;
-                    nd.sigv[node] = o.sigv;
-                    const Metric6 m = metric_of(o.sigx, o.sigv);
-                    ax64 = m.ax64;
-                    av64 = m.av64;
-                    scale = m.scale;
-                }
-                met.ax64 = __shfl_sync(FULL, ax64, 0);
-                met.av64 = __shfl_sync(FULL, av64, 0);
-                met.scale = __shfl_sync(FULL, scale, 0);
-                met.ax = (float)met.ax64;
-                met.av = (float)met.av64;
+            if (lane == 0) acc_s[w] = a;
+            __syncwarp();
+            const MomOutWarp o = mom_finalize_warp(&acc_s[w], 1, pr, vr, size_tab[cnt].inv_n, box);
+            __syncwarp();
+            if (lane < 3) {
+                nd.xbar[3 * node + lane] = o.xbar;
+                nd.vbar[3 * node + lane] = o.vbar;
             }
+            if (lane == 0) {
+                nd.sigx[node] = o.sigx;
+                nd.sigv[node] = o.sigv;
+            }
+            const Metric6 met = metric_of_warp(o.sigx, o.sigv);
             // ---- nearest neighbours (float32) ----
             float dnn = INFINITY;
             for (int c = off; c < off + cnt; c++) {
@@ -662,9 +938,7 @@ __global__ void __launch_bounds__(TINY_WARPS * 32)
                 if (mine && c != lane) dnn = fminf(dnn, d2_32(p, v, pc, vc, met));
             }
             // ---- k-th smallest, float32: the member of rank k - 1 by (value, lane) ----
-            long long kk = (long long)ceil(f * (double)cnt);
-            if (kk < 1) kk = 1;
-            if (kk > cnt) kk = cnt;
+            const int kk = (int)size_tab[cnt].kk;
             int rank = 0;
             for (int c = off; c < off + cnt; c++) {
                 const float dc = __shfl_sync(FULL, dnn, c);
@@ -672,8 +946,7 @@ __global__ void __launch_bounds__(TINY_WARPS * 32)
             }
             const unsigned pick = __ballot_sync(FULL, mine && rank == kk - 1);
             const float t32 = __shfl_sync(FULL, dnn, pick ? __ffs(pick) - 1 : off);
-            const float blo = (float)((double)t32 * (1.0 - 2.0 * RS_BAND));
-            const float bhi = (float)((double)t32 * (1.0 + 2.0 * RS_BAND));
+            const float blo = fmaf(t32, (float)(-2.0 * RS_BAND), t32), bhi = fmaf(t32, (float)(2.0 * RS_BAND), t32);
             // ---- band members: exact float64 nearest-neighbour distances ----
             const bool inband = mine && dnn >= blo && dnn <= bhi;
             const int below = __popc(__ballot_sync(FULL, mine && dnn < blo));
@@ -688,20 +961,22 @@ __global__ void __launch_bounds__(TINY_WARPS * 32)
             // the exact k-th value is the (k - 1 - below)-th smallest band value
             const int want = (int)(kk - 1) - below;
             const unsigned bmask = __ballot_sync(FULL, inband);
+            // (non-negative doubles order as their bits; the float64 unit is
+            // what this kernel waits for most)
+            const long long eb = __double_as_longlong(ex);
             int brank = 0;
-            for (int c = off; c < off + cnt; c++) {
-                const double ec = __shfl_sync(FULL, ex, c);
-                if (inband && ((bmask >> c) & 1u) && (ec < ex || (ec == ex && c < lane))) brank++;
+            for (unsigned m = bmask; m; m &= m - 1u) {
+                const int c = __ffs(m) - 1;
+                const long long ec = __shfl_sync(FULL, eb, c);
+                if (inband && (ec < eb || (ec == eb && c < lane))) brank++;
             }
             const unsigned bp = __ballot_sync(FULL, inband && brank == want);
             if (!bp && lane == 0) dev_fail(st, DEV_INTERNAL, 45, node);
             const double l2 = bp ? __shfl_sync(FULL, ex, __ffs(bp) - 1) : 0.0;
-            if (lane == 0) nd.lnk[node] = sqrt(l2 / met.scale);
+            if (lane == 0) nd.lnk[node] = l2;  // k_tree_stats makes it a length
             // ---- friends-of-friends at l (inclusive) ----
-            const float lo = (float)(l2 * (1.0 - RS_BAND)), hi = (float)(l2 * (1.0 + RS_BAND));
-            const float tlo = (float)(l2 * (1.0 - 3e-6)), thi = (float)(l2 * (1.0 + 3e-6));
-            const float part = fmaxf(hi, thi);
-            const double l = sqrt(l2);
+            const float lo = fminf((float)(l2 * (1.0 - RS_BAND)), (float)(l2 * (1.0 - 3e-6)));
+            const float part = link_part(l2);
             par[lane] = lane;
             __syncwarp();
             int tie = 0;
@@ -713,9 +988,9 @@ __global__ void __launch_bounds__(TINY_WARPS * 32)
                 const float d2 = d2_32(p, v, pc, vc, met);
                 if (d2 > part) continue;
                 // below both bands: a friend, and not a tie-band pair
-                bool link = d2 < fminf(lo, tlo);
+                bool link = d2 < lo;
                 if (!link) {
-                    const double e = d2_64(p, v, pc, vc, met);
+                    const double e = d2_64(p, v, pc, vc, met), l = sqrt(l2);
                     link = e <= l2;
                     if (l2 > 0 && e != l2 && fabs(sqrt(e) - l) <= 1e-6 * l) tie++;
                 }
@@ -888,7 +1163,6 @@ __global__ void k_lvl_finalize(LevelBufs L, NodeArrays nd, double box)
 // skipped only when that bound exceeds the current radius by 2^-18 relative,
 // which can never skip a member whose float32 distance would change the
 // result.
-#define RS_PRUNE_SLACK 1.000003814697265625f  // 1 + 2^-18
 
 struct Box6 {
     float4 plo, phi, vlo, vhi;
@@ -1064,29 +1338,6 @@ __device__ __forceinline__ void bvh_view(BvhView &V, const BoxStore &B, int64_t 
 // that reaches the whole box within the same margin joins it with a single
 // union.  These pairs lie strictly inside the linking length, never in the
 // tie band.  The flag is kept in the box store's flag byte.
-#define RS_CLIQUE_MARGIN 0.99999237060546875  // 1 - 2^-17
-
-// linking limits of one node: float32 band edges around l^2 (decided in
-// float64 inside them), the reporting band for ties, and the pruning radius
-struct LinkLim {
-    float lo, hi, tlo, thi, part, lim, cl_lim;
-    double l2, l;
-};
-
-__device__ __forceinline__ LinkLim link_lim(double l2)
-{
-    LinkLim r;
-    r.l2 = l2;
-    r.l = sqrt(l2);
-    r.lo = (float)(l2 * (1.0 - RS_BAND));
-    r.hi = (float)(l2 * (1.0 + RS_BAND));
-    r.tlo = (float)(l2 * (1.0 - 3e-6));
-    r.thi = (float)(l2 * (1.0 + 3e-6));
-    r.part = fmaxf(r.hi, r.thi);
-    r.lim = r.part * RS_PRUNE_SLACK;
-    r.cl_lim = (float)(l2 * RS_CLIQUE_MARGIN);
-    return r;
-}
 
 __device__ __forceinline__ float box_diam2(const Box6 &b, const Metric6 &m)
 {
@@ -1116,11 +1367,6 @@ __device__ __forceinline__ float point_box_far2(float4 p, float4 v, const Box6 &
 // union-find entries are first written, an upper box's by joining the first
 // members of its children (a flagged box's children are flagged, their
 // diameters being no larger).
-__device__ __forceinline__ float link_part(double l2)
-{
-    return fmaxf((float)(l2 * (1.0 + RS_BAND)), (float)(l2 * (1.0 + 3e-6)));
-}
-
 // the union of one box per lane, in every lane
 __device__ __forceinline__ Box6 warp_box(const Box6 &c)
 {
@@ -1545,19 +1791,10 @@ __device__ __forceinline__ int join_friend(int *parent, int a, int b, int rq, rs
 // once for all of them, box against box, for the leaves within reach of its
 // own leaf's box; keeps, of each such leaf's 32 members, those within reach of
 // the box (a tenth to a seventh of them on the catalogues of synth.py); and
-// tests the kept ones, 32 at a time, against its 32 members.  That test is a
-// contraction: with coordinates u = (x - c) w relative to the leaf box's
-// centre c, in units of the linking radius, d^2 - T = -2 u_q.u_c + |u_c|^2 +
-// (|u_q|^2 - T) is one m16n8k8 half-precision product for 16 x 8 pairs (six
-// coordinates and |u_c|^2 in two halves against ones, the query's term in the
-// accumulator), and its sign alone is used: a pair it calls far is farther
-// than the linking radius, because T leaves room for every rounding:
-//   the rounded points u^ (half, relative 2^-11) differ from u by at most
-//   delta = 1.02 2^-11 (|u_q| + |u_c|) + 3.1e-4 (the float32 steps before,
-//   and subnormal halves even if they counted as zero), so friends have
-//   |u^_q - u^_c| <= 1 + delta; the norms are taken of the rounded points, so
-//   the product is |u^_q - u^_c|^2 up to float32 accumulation and the second
-//   half's rounding, below 2^-18 (|u_q| + |u_c|)^2 + 1e-4.
+// screens the kept ones, 32 at a time, against its 32 members on the matrix
+// units, in units of the linking radius about the leaf box's centre: a pair
+// whose product minus T, the bound for pairs within the linking radius (see
+// the half-precision points), is positive is no friend.
 // T stays below 1.02 for the usual boxes (2.7 linking lengths in radius), so
 // the few pairs it lets through (about 20 of 1024) are nearly all friends;
 // they are queued and evaluated 32 at a time in full, as float32 differences
@@ -1575,14 +1812,6 @@ constexpr int LK_LEAVES = 128;  // pending leaves per warp
 constexpr int LK_RING = 128;    // kept candidates per warp (a ring; 32 are consumed at a time)
 constexpr float LK_RMAX = 100.f;  // largest box radius, in linking lengths, for the half-precision test
 
-__device__ __forceinline__ void mma_m16n8k8_f16(float (&d)[4], unsigned a0, unsigned a1, unsigned b0, float c0,
-                                                float c1, float c2, float c3)
-{
-    asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%7,%8,%9,%10};"
-        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-        : "r"(a0), "r"(a1), "r"(b0), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
-}
-
 // box-to-box lower bound on the squared distance (each gap is one rounded
 // float32 difference of members' coordinates, as in point_box_d2)
 __device__ __forceinline__ float box_box_d2(const Box6 &a, const Box6 &b, const Metric6 &m)
@@ -1594,31 +1823,6 @@ __device__ __forceinline__ float box_box_d2(const Box6 &a, const Box6 &b, const 
                 gv = fmaxf(0.f, fmaxf(b.vlo.y - a.vhi.y, a.vlo.y - b.vhi.y)),
                 gw = fmaxf(0.f, fmaxf(b.vlo.z - a.vhi.z, a.vlo.z - b.vhi.z));
     return (gx * gx + gy * gy + gz * gz) * m.ax + (gu * gu + gv * gv + gw * gw) * m.av;
-}
-
-// the six coordinates of a member relative to the box centre, in units of
-// the linking radius, rounded to half; returns the squared norm of the
-// rounded point
-struct HalfPoint {
-    __half h[6];
-};
-__device__ __forceinline__ float half_point(float4 p, float4 v, float4 pc, float4 vc, float wx, float wv, HalfPoint &o)
-{
-    const float u[6] = {(p.x - pc.x) * wx, (p.y - pc.y) * wx, (p.z - pc.z) * wx,
-                        (v.x - vc.x) * wv, (v.y - vc.y) * wv, (v.z - vc.z) * wv};
-    float s = 0.f;
-#pragma unroll
-    for (int d = 0; d < 6; d++) {
-        o.h[d] = __float2half_rn(u[d]);
-        const float r = __half2float(o.h[d]);
-        s = fmaf(r, r, s);
-    }
-    return s;
-}
-
-__device__ __forceinline__ unsigned pack2(__half a, __half b)
-{
-    return (unsigned)__half_as_ushort(a) | ((unsigned)__half_as_ushort(b) << 16);
 }
 
 struct LinkWarp {
@@ -1703,16 +1907,13 @@ __global__ void __launch_bounds__(LK_WARPS * 32, WARPS / LK_WARPS)
     const float rsum = 2.f * rb + 1.01f;
     const float dl = 1.02f * 4.8828125e-4f * rsum + 3.1e-4f;
     const float T = (1.f + dl) * (1.f + dl) * 1.00002f + 3.814697265625e-6f * rsum * rsum + 1.e-4f;
-        HalfPoint h;
-        float s = half_point(act && !brute ? po : pc, act && !brute ? vo : vc, pc, vc, wx, wv, h);
-        const __half2 m2 = __float2half2_rn(-2.f);
-        __half2 c0 = __hmul2(__halves2half2(h.h[0], h.h[1]), m2), c1 = __hmul2(__halves2half2(h.h[2], h.h[3]), m2),
-                c2 = __hmul2(__halves2half2(h.h[4], h.h[5]), m2);
-        uint4 row;
-        row.x = pack2(__low2half(c0), __high2half(c0));
-        row.y = pack2(__low2half(c1), __high2half(c1));
-        row.z = pack2(__low2half(c2), __high2half(c2));
-        row.w = 0x3c003c00u;  // (1, 1)
+        float s;
+        const bool in = act && !brute;
+        uint4 row = half_point(in ? po : pc, in ? vo : vc, pc, vc, wx, wv, s);
+        row.x = half_query(row.x, 0);
+        row.y = half_query(row.y, 1);
+        row.z = half_query(row.z, 2);
+        row.w = HALF_ONES;
         S.cand[lane] = row;
         s = act ? s - T : 60000.f;
         __syncwarp();
@@ -1753,15 +1954,13 @@ __global__ void __launch_bounds__(LK_WARPS * 32, WARPS / LK_WARPS)
         const int m = S.ring[(head + lane) & (LK_RING - 1)];
         unsigned mask = 0;
         if (!brute) {
-            uint4 c = make_uint4(0u, 0u, 0u, 0x00007b00u);  // padding: |u|^2 = 57344, never near
+            uint4 c = make_uint4(0u, 0u, 0u, HALF_FAR);
             if (lane < cnt) {
                 float4 pm, vm;
                 mem_get(M, m, pm, vm);
-                HalfPoint h;
                 const float4 pc = S.pc, vc = S.vc;
-                const float s = half_point(pm, vm, pc, vc, pc.w, vc.w, h);
-                const __half hi = __float2half_rn(s), lo = __float2half_rn(s - __half2float(hi));
-                c = make_uint4(pack2(h.h[0], h.h[1]), pack2(h.h[2], h.h[3]), pack2(h.h[4], h.h[5]), pack2(hi, lo));
+                float s;
+                c = half_point(pm, vm, pc, vc, pc.w, vc.w, s);
             }
             S.cand[lane] = c;
             __syncwarp();
@@ -2676,7 +2875,7 @@ __global__ void k_lvl_l2(LevelBufs L, NodeArrays nd, double f, int sub_n, rs_dev
     found = __syncthreads_or(found);
     if (threadIdx.x == 0) {
         if (!found) dev_fail(st, DEV_INTERNAL, 50, node);
-        nd.lnk[node] = sqrt(L.l2[k] / L.met[k].scale);
+        nd.lnk[node] = L.l2[k];  // k_tree_stats makes it a length
     }
 }
 
@@ -2791,6 +2990,10 @@ __global__ void k_tree_stats(NodeArrays nd, int n_nodes, unsigned long long *out
         tie += (unsigned long long)nd.tie[i];
         sum += (unsigned long long)nd.count[i];
         maxl = max(maxl, nd.level[i]);
+        // the node's linking length in units of Eq. 1, from the square in its
+        // scaled metric (here, 32 nodes a float64 instruction, and not in the
+        // node's own block)
+        nd.lnk[i] = sqrt(nd.lnk[i] / metric_of(nd.sigx[i], nd.sigv[i]).scale);
     }
     seeds = warp_sum(seeds);
     tie = warp_sum(tie);
@@ -2920,18 +3123,18 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
     int *shift_bits = gmisc, *gmin = gmisc + G, *slot_group = gmisc + 2 * G, *gred = gmisc + 2 * G + M;
     // node queues: big lists (ping-pong) and the small queue; counters
     // counters first (16 ints = 64 bytes, so everything after stays 8-byte aligned)
-    RS_WS(ctx, int, q, WS_RF_NODEQ, 5 * cap + 16);
+    RS_WS(ctx, int, q, WS_RF_NODEQ, 6 * cap + 16);
     int *ctr = q, *big_a = q + 16, *big_b = q + 16 + cap, *small_q = q + 16 + 2 * cap, *tiny_q = q + 16 + 3 * cap,
-        *mid_q = q + 16 + 4 * cap;
+        *mid_q = q + 16 + 4 * cap, *warp_q = q + 16 + 5 * cap;
     // ctr: [0] big_a len, [1] big_b len, [2] small len, [3] small head, [4] band len,
     // [6..7] bracket fallback flag, [8] tiny len, [9] tiny head, [10] k-d ranges,
-    // [11] middle len, [12] middle head, [13] subset query list length
+    // [11] middle len, [12] middle head, [13] subset query list length,
+    // [14] warp-tier len, [15] warp-tier head
     RS_CUDA(ctx, cudaMemsetAsync(ctr, 0, sizeof(int) * 16, ctx->stream));
 
-    const int gb = (int)std::min<int64_t>(G, (int64_t)ctx->num_sms * 8);
-    RS_LAUNCH(ctx, "rf_unwrap_init", k_fill_s32, ceil_div(12 * G, 256), 256, 0, (int32_t *)gred, 12 * G,
-              (int32_t)0x7f800000);
-    RS_LAUNCH(ctx, "rf_unwrap_init", k_fill_s32, ceil_div(G, 256), 256, 0, (int32_t *)gmin, G, (int32_t)0x7fffffff);
+    RS_WS(ctx, SizeTab, size_tab, WS_RF_SIZES, SMALL_N + 1);
+    RS_LAUNCH(ctx, "rf_init", k_refine_init, ceil_div(std::max<int64_t>(12 * G, SMALL_N + 1), 256), 256, 0, G, gred,
+              gmin, SMALL_N, f, size_tab);
     RS_LAUNCH(ctx, "rf_group_unwrap", k_unwrap_tiles, ceil_div(M, 256), 256, 0, G, goff, perm, n, M, pos, stride,
               boxf, slot_group, gred, gmin, ctx->d_status);
     RS_LAUNCH(ctx, "rf_unwrap_bits", k_unwrap_bits, ceil_div(G, 256), 256, 0, G, (const int *)gred, boxf, shift_bits,
@@ -3244,26 +3447,32 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
     }
 
     // ---- small nodes: whole subtrees ----
-    // three size classes, each forwarding its smaller subtrees to the next
+    // four size classes, each forwarding its smaller subtrees to the next
     {
-        auto kbig = k_small_subtree<SMALL_N, SMALL_THREADS, 2>;
+        auto kbig = k_small_subtree<SMALL_N, SMALL_THREADS, 3>;
         auto kmid = k_small_subtree<MID_N, MID_THREADS, 8>;
+        auto kwarp = k_small_subtree<WARP_N, 32, WARP_CTAS>;
         const size_t sbig = sizeof(SmallShared<SMALL_N, SMALL_THREADS>);
         const size_t smid = sizeof(SmallShared<MID_N, MID_THREADS>);
+        const size_t swarp = sizeof(SmallShared<WARP_N, 32>);
         RS_CUDA(ctx, cudaFuncSetAttribute(kbig, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sbig));
         RS_CUDA(ctx, cudaFuncSetAttribute(kmid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smid));
         const rs_tuning &tu = ctx->tune;
-        RS_LAUNCH(ctx, "rf_small_subtree", kbig, (int64_t)ctx->num_sms * tu.small_ctas_per_sm, SMALL_THREADS, sbig,
-                  (const int *)small_q, (const int *)(ctr + 2), ctr + 3, wpos, wvel, widx,
-                  std::min(tu.mid_max, MID_N), mid_q, ctr + 11, nd, box, f, (int)min_n, ctx->d_status);
+        const int mid_max = std::min(tu.mid_max, MID_N), tiny_max = std::min(tu.tiny_max, TINY_N);
+        RS_LAUNCH(ctx, "rf_small_subtree", kbig, (int64_t)ctx->num_sms * (tu.small_ctas_per_sm + 1), SMALL_THREADS, sbig,
+                  (const int *)small_q, (const int *)(ctr + 2), ctr + 3, wpos, wvel, widx, mid_max, mid_q, ctr + 11,
+                  nd, (const SizeTab *)size_tab, box, (int)min_n, ctx->d_status);
         RS_LAUNCH(ctx, "rf_mid_subtree", kmid, (int64_t)ctx->num_sms * tu.mid_ctas_per_sm, MID_THREADS, smid,
                   (const int *)mid_q, (const int *)(ctr + 11), ctr + 12, wpos, wvel, widx,
-                  std::min(tu.tiny_max, TINY_N), tiny_q, ctr + 8, nd, box, f, (int)min_n, ctx->d_status);
+                  std::min(mid_max, WARP_N), warp_q, ctr + 14, nd, (const SizeTab *)size_tab, box, (int)min_n,
+                  ctx->d_status);
+        RS_LAUNCH(ctx, "rf_warp_subtree", kwarp, (int64_t)ctx->num_sms * WARP_CTAS * tu.mid_ctas_per_sm / 8, 32, swarp,
+                  (const int *)warp_q, (const int *)(ctr + 14), ctr + 15, wpos, wvel, widx, tiny_max, tiny_q, ctr + 8,
+                  nd, (const SizeTab *)size_tab, box, (int)min_n, ctx->d_status);
+        RS_LAUNCH(ctx, "rf_tiny_subtree", k_tiny_subtree, (int64_t)ctx->num_sms * tu.tiny_ctas_per_sm,
+                  TINY_WARPS * 32, 0, (const int *)tiny_q, (const int *)(ctr + 8), ctr + 9, (const float4 *)wpos,
+                  (const float4 *)wvel, widx, nd, (const SizeTab *)size_tab, box, (int)min_n, ctx->d_status);
     }
-    RS_LAUNCH(ctx, "rf_tiny_subtree", k_tiny_subtree, (int64_t)ctx->num_sms * ctx->tune.tiny_ctas_per_sm,
-              TINY_WARPS * 32, 0,
-              (const int *)tiny_q, (const int *)(ctr + 8), ctr + 9, (const float4 *)wpos, (const float4 *)wvel, widx,
-              nd, box, f, (int)min_n, ctx->d_status);
 
     // ---- summary ----
     RS_WS(ctx, unsigned long long, so, WS_RF_MISC3, 4);

@@ -151,22 +151,40 @@ __device__ __forceinline__ void mom_merge(MomAcc &a, const MomAcc &b)
     add128(a.qv_lo, a.qv_hi, b.qv_lo, b.qv_hi);
 }
 
+// Warp sum of 128-bit values modulo 2^128, in every lane: five pieces of 27
+// bits, each summed by one redux (32 (2^27 - 1) < 2^32).  Replaces five
+// rounds of shuffled 128-bit adds (a fifth of the instructions).
+// Not inlined: the subtree kernels' code has to stay small.
+static __device__ __noinline__ ulonglong2 warp_sum128(unsigned long long lo, unsigned long long hi)
+{
+    const unsigned m = (1u << 27) - 1u;
+    const unsigned r0 = __reduce_add_sync(0xffffffffu, (unsigned)lo & m),
+                   r1 = __reduce_add_sync(0xffffffffu, (unsigned)(lo >> 27) & m),
+                   r2 = __reduce_add_sync(0xffffffffu, (unsigned)((lo >> 54) | (hi << 10)) & m),
+                   r3 = __reduce_add_sync(0xffffffffu, (unsigned)(hi >> 17) & m),
+                   r4 = __reduce_add_sync(0xffffffffu, (unsigned)(hi >> 44));
+    lo = r0;
+    hi = ((unsigned long long)r3 << 17) + ((unsigned long long)r4 << 44);
+    add128(lo, hi, (unsigned long long)r1 << 27, 0ull);
+    add128(lo, hi, (unsigned long long)r2 << 54, (unsigned long long)(r2 >> 10));
+    return make_ulonglong2(lo, hi);
+}
+
 __device__ __forceinline__ void mom_warp_reduce(MomAcc &a)
 {
+    ulonglong2 r;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        MomAcc b;
-#pragma unroll
-        for (int i = 0; i < 6; i++) {
-            b.s_lo[i] = __shfl_xor_sync(0xffffffffu, a.s_lo[i], o);
-            b.s_hi[i] = __shfl_xor_sync(0xffffffffu, a.s_hi[i], o);
-        }
-        b.qx_lo = __shfl_xor_sync(0xffffffffu, a.qx_lo, o);
-        b.qx_hi = __shfl_xor_sync(0xffffffffu, a.qx_hi, o);
-        b.qv_lo = __shfl_xor_sync(0xffffffffu, a.qv_lo, o);
-        b.qv_hi = __shfl_xor_sync(0xffffffffu, a.qv_hi, o);
-        mom_merge(a, b);
+    for (int i = 0; i < 6; i++) {
+        r = warp_sum128(a.s_lo[i], a.s_hi[i]);
+        a.s_lo[i] = r.x;
+        a.s_hi[i] = r.y;
     }
+    r = warp_sum128(a.qx_lo, a.qx_hi);
+    a.qx_lo = r.x;
+    a.qx_hi = r.y;
+    r = warp_sum128(a.qv_lo, a.qv_hi);
+    a.qv_lo = r.x;
+    a.qv_hi = r.y;
 }
 
 __device__ __forceinline__ void atomic_add128(unsigned long long *lo, unsigned long long *hi, unsigned long long alo,
@@ -251,6 +269,79 @@ __device__ __forceinline__ MomOut mom_finalize(const MomAcc &a, float4 pref, flo
     o.sigv = vv > 0 ? sqrt(vv) : 0.0;
     return o;
 }
+
+// mom_finalize by a whole warp over np partial sums, a quantity a lane (the
+// float64 chain is what it costs: serially 100 operations, here the depth of
+// one division and one square root).  Lane d < 3 gets the mean's components d;
+// sigx, sigv and the unwrapped mean cx (float32) are in every lane.
+struct MomOutWarp {
+    double xbar, vbar, sigx, sigv;
+    float cx[6];
+};
+
+__device__ __forceinline__ MomOutWarp mom_finalize_warp(const MomAcc *part, int np, float4 pref, float4 vref,
+                                                        double inv_n, double box)
+{
+    const unsigned FULL = 0xffffffffu;
+    const int lane = lane_id(), j = lane & 7;
+    unsigned long long lo = 0, hi = 0;
+    for (int i = 0; i < np; i++) {
+        const unsigned long long *v = reinterpret_cast<const unsigned long long *>(part + i);
+        add128(lo, hi, v[j < 6 ? j : 2 * j], v[j < 6 ? j + 6 : 2 * j + 1]);
+    }
+    static_assert(sizeof(MomAcc) == 16 * 8, "s_lo, s_hi, then (lo, hi) of qx and of qv");
+    // s128_to_double of the sums and u128_to_double of the squares at once
+    const bool neg = j < 6 && (long long)hi < 0;
+    if (neg) {
+        lo = ~lo + 1ull;
+        hi = ~hi + (lo == 0 ? 1ull : 0ull);
+    }
+    const double a = u128_to_double(lo, hi) * (j < 6 ? RS_FX_INV : RS_FX_INV * RS_FX_INV), s = neg ? -a : a;
+    const float ref = j < 3 ? (j == 0 ? pref.x : (j == 1 ? pref.y : pref.z))
+                            : (j == 3 ? vref.x : (j == 4 ? vref.y : vref.z));
+    const double at = (double)ref + s * inv_n;
+    MomOutWarp o;
+    o.xbar = j < 3 ? wrap_box(at, box) : 0.0;
+    o.vbar = __shfl_sync(FULL, at, (lane + 3) & 31);
+#pragma unroll
+    for (int i = 0; i < 6; i++) o.cx[i] = __shfl_sync(FULL, (float)at, i);
+    // even lanes the positions' dispersion, odd lanes the velocities'
+    const int v3 = 3 * (lane & 1);
+    const double sa = __shfl_sync(FULL, s, v3), sb = __shfl_sync(FULL, s, v3 + 1), sc = __shfl_sync(FULL, s, v3 + 2),
+                 q = __shfl_sync(FULL, s, 6 + (lane & 1));
+    double s2 = 0;
+    s2 += sa * sa;
+    s2 += sb * sb;
+    s2 += sc * sc;
+    const double var = (q - s2 * inv_n) * inv_n;
+    const double sig = var > 0 ? sqrt(var) : 0.0;
+    o.sigx = __shfl_sync(FULL, sig, 0);
+    o.sigv = __shfl_sync(FULL, sig, 1);
+    return o;
+}
+
+// metric_of by a warp: the two reciprocals in one division
+__device__ __forceinline__ Metric6 metric_of_warp(double sigx, double sigv)
+{
+    const double s = (lane_id() & 1) ? sigv : sigx;
+    const double r = s > 0 ? 1.0 / (s * s) : 0.0;
+    const double ax = __shfl_sync(0xffffffffu, r, 0), av = __shfl_sync(0xffffffffu, r, 1);
+    const double mx = ax > av ? ax : av;
+    Metric6 m;
+    m.scale = mx > 0 ? 1.0 / mx : 1.0;
+    m.ax64 = ax * m.scale;
+    m.av64 = av * m.scale;
+    m.ax = (float)m.ax64;
+    m.av = (float)m.av64;
+    return m;
+}
+
+// Per member count: its float64 reciprocal and k = ceil(f n) clamped to
+// [1, n], for the kernels whose nodes each would spend a division on them.
+struct SizeTab {
+    double inv_n;
+    long long kk;
+};
 
 // Metric of Eq. 1 with a common scale that keeps both factors <= 1.
 __device__ __forceinline__ Metric6 metric_of(double sigx, double sigv)

@@ -1,8 +1,9 @@
-"""The big-node searches work leaf against leaf (32 members a leaf): node
-sizes at the edges of leaves and of the boxes above them, and inputs that
-leave the half-precision pair filter (leaf boxes far larger than the linking
-length, a zero linking length) or that the clique boxes serve (dense cores,
-copies).  Trees and tie counts must equal the float64 oracle's exactly."""
+"""The refinement screens pairs by half-precision products: big nodes leaf
+against leaf (32 members a leaf), small ones by tiles of 16 x 8 pairs in one
+block.  Node sizes at the edges of leaves, tiles and tiers, and inputs that
+leave the screen's range (boxes far larger than the linking length, a zero
+linking length) or that the clique boxes serve (dense cores, copies).  Trees
+and tie counts must equal the float64 oracle's exactly."""
 import numpy as np
 import pytest
 
@@ -46,17 +47,39 @@ def _members(kind, n, rng):
     ("blob", 33_000, 0.7), ("pairs", 1500, 0.7), ("pairs", 5001, 0.9), ("copies", 1500, 0.7), ("copies", 6000, 0.5),
     ("core", 3000, 0.7), ("core", 6001, 0.9), ("still", 1100, 0.7), ("still", 5000, 0.7)])
 def test_leaf_searches_match_oracle(kind, n, f):
-    from paper_1110_4372_gb300 import rsgpu
     rng = np.random.default_rng([n, len(kind)])
     box = 20.0
     p, v = _members(kind, n, rng)
     # one corner of the box, so that the group wraps
     cat = synth.Catalogue(pos=synth.wrap(p, box), vel=v.astype(np.float32), box=box, truth=np.zeros(n, np.int32),
                           comp_parent=np.zeros(0, np.int32), comp_n=np.zeros(0))
-    b = 0.4 * n ** (1 / 3) / box
+    o = _check(cat, f)
+    assert np.diff(o["offsets"]).max() > 1024
+
+
+@pytest.mark.parametrize("kind", ["blob", "pairs", "copies", "core", "still"])
+@pytest.mark.parametrize("f", [0.5, 0.7])
+def test_subtree_tiers_match_oracle(kind, f):
+    rng = np.random.default_rng([7, len(kind)])
+    sizes = [10, 11, 31, 32, 33, 34, 47, 48, 49, 63, 65, 127, 128, 129, 255, 256, 257, 258, 272, 273, 500, 511, 513,
+             777, 1008, 1009, 1023, 1024]
+    box = 40.0
+    parts = [_members(kind, k, rng) for k in sizes]
+    at = np.stack(np.meshgrid(*[np.arange(4) * 10.0] * 3), -1).reshape(-1, 3)[:len(sizes)]
+    p = np.vstack([q[0] + c for q, c in zip(parts, at)])
+    v = np.vstack([q[1] for q in parts])
+    mix = rng.permutation(len(p))
+    cat = synth.Catalogue(pos=synth.wrap(p[mix], box), vel=v[mix].astype(np.float32), box=box,
+                          truth=np.zeros(len(p), np.int32), comp_parent=np.zeros(0, np.int32), comp_n=np.zeros(0))
+    o = _check(cat, f)
+    assert o["tree"].n_nodes >= 20
+
+
+def _check(cat, f):
+    from paper_1110_4372_gb300 import rsgpu
+    b = 0.4 * cat.n ** (1 / 3) / cat.box
     g = run_gpu_path(rsgpu.Context(), rsgpu, cat, f=f, b=b, assign=False)
     o = run_oracle_path(cat, f=f, b=b, assign=False)
-    assert np.diff(o["offsets"]).max() > 1024
     # what the searches decide (the moments of a core of 1e-4 Mpc/h reach the
     # fixed-point sums' resolution, 2^-32)
     gd, od = gpu_tree_dict(g["tree"]), oracle_tree_dict(o["tree"])
@@ -65,3 +88,4 @@ def test_leaf_searches_match_oracle(kind, n, f):
         for q in ("members", "parent_key", "nchild", "tie"):
             assert a[q] == od[k][q], (k, q)
         assert abs(a["lnk"] - od[k]["lnk"]) <= 1e-6 * od[k]["lnk"], k
+    return o
