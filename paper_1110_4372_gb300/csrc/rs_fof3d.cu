@@ -26,6 +26,7 @@
 namespace {
 
 constexpr int FOF_THREADS = 256;
+constexpr int64_t FOF_ONE_PASS = 8192;  // particles linked in one pass (see k_fof_link)
 constexpr double BAND_REL = 9.5367431640625e-07;  // 2^-20, relative on d^2
 
 struct FofGeom {
@@ -54,10 +55,12 @@ __device__ __forceinline__ int fine_coord(float x, float inv, int Gf)
     return f;
 }
 
+// keys of the particles; the coarse table starts empty
 __global__ void k_fof_keys(const float *pos, int stride, int64_t n, FofGeom g, uint64_t *keys, uint32_t *vals,
-                           rs_dev_status *st)
+                           uint32_t *table, int64_t ncoarse, rs_dev_status *st)
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (int64_t c = i; c < ncoarse; c += (int64_t)gridDim.x * blockDim.x) table[c] = 0xffffffffu;
     if (i >= n) return;
     float x, y, z;
     load_pos(pos, stride, i, x, y, z);
@@ -70,34 +73,64 @@ __global__ void k_fof_keys(const float *pos, int stride, int64_t n, FofGeom g, u
     vals[i] = (uint32_t)i;
 }
 
-// sorted positions as float4 and cell-start flags
-__global__ void k_fof_gather(const float *pos, int stride, int64_t n, const uint64_t *keys, const uint32_t *idx,
-                             float4 *spos, uint32_t *flag)
-{
-    int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
-    float x, y, z;
-    load_pos(pos, stride, idx[q], x, y, z);
-    spos[q] = make_float4(x, y, z, 0.f);
-    flag[q] = (q == 0 || keys[q] != keys[q - 1]) ? 1u : 0u;
-}
+// One pass over the sorted keys: sorted positions as float4, the fine cells
+// numbered (runs of equal keys, by a scan with look-back: a warp takes rows of
+// 32 keys and counts run starts by votes), and every per-cell array started
+// where its cell is.  One launch instead of a gather, a copy, a scan of three
+// launches, the numbering and three fills over n.
+constexpr int CELL_ROWS = 8;  // rows of 32 particles per warp
+constexpr int64_t CELL_TILE = (int64_t)CELL_ROWS * FOF_THREADS;
 
-// after an exclusive scan of flag: cell_of[q] = scan[q] + flag[q] - 1
-__global__ void k_fof_cells(int64_t n, const uint64_t *keys, const uint32_t *scan, const uint32_t *flag,
-                            uint32_t *cell_of, uint32_t *cell_start, uint64_t *cell_key, uint32_t *table,
-                            const uint32_t *n_cells)
+__global__ void __launch_bounds__(FOF_THREADS) k_fof_cells(const float *pos, int stride, int64_t n, const uint64_t *keys,
+                                                           const uint32_t *idx, float4 *spos, uint32_t *cell_of,
+                                                           uint32_t *cell_start, uint64_t *cell_key, uint32_t *table,
+                                                           uint64_t *occ, int *parent, int *root_min,
+                                                           uint32_t *n_cells, RsLookback lb, rs_dev_status *st)
 {
-    int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
-    uint32_t c = scan[q] + flag[q] - 1u;
-    cell_of[q] = c;
-    if (flag[q]) {
-        cell_start[c] = (uint32_t)q;
-        cell_key[c] = keys[q];
-        uint64_t coarse = keys[q] >> 6;
-        if (q == 0 || (keys[q - 1] >> 6) != coarse) table[coarse] = c;
+    const unsigned FULL = 0xffffffffu;
+    const int64_t tile = rs_next_tile(lb);
+    const int lane = lane_id();
+    const int64_t base = tile * CELL_TILE + (int64_t)warp_id() * 32 * CELL_ROWS;
+    uint64_t key[CELL_ROWS];
+    unsigned starts[CELL_ROWS], coarse[CELL_ROWS];
+    int count = 0;
+#pragma unroll
+    for (int j = 0; j < CELL_ROWS; j++) {
+        const int64_t q = base + 32 * j + lane;
+        key[j] = q < n ? keys[q] : 0;
+        uint64_t prev = __shfl_up_sync(FULL, key[j], 1);
+        if (lane == 0 && q > 0 && q < n) prev = keys[q - 1];
+        starts[j] = __ballot_sync(FULL, q < n && (q == 0 || key[j] != prev));
+        coarse[j] = __ballot_sync(FULL, q < n && (q == 0 || (key[j] >> 6) != (prev >> 6)));
+        count += __popc(starts[j]);
     }
-    if (q == n - 1) cell_start[*n_cells] = (uint32_t)n;
+    uint32_t tot;
+    uint32_t c0 = rs_block_scan<FOF_THREADS>(lane == 0 ? (uint32_t)count : 0u, tot);
+    c0 = __shfl_sync(FULL, c0, 0) + (uint32_t)rs_lookback(lb, tile, tot, st);
+    const unsigned upto = (2u << lane) - 1u;
+#pragma unroll
+    for (int j = 0; j < CELL_ROWS; j++) {
+        const int64_t q = base + 32 * j + lane;
+        const uint32_t c = c0 + (uint32_t)__popc(starts[j] & upto) - 1u;
+        c0 += (uint32_t)__popc(starts[j]);
+        if (q >= n || c >= n) continue;  // (a look-back that ran out of time leaves wrong numbers)
+        float x, y, z;
+        load_pos(pos, stride, idx[q], x, y, z);
+        spos[q] = make_float4(x, y, z, 0.f);
+        cell_of[q] = c;
+        if ((starts[j] >> lane) & 1u) {
+            cell_start[c] = (uint32_t)q;
+            cell_key[c] = key[j];
+            occ[c] = 0;
+            parent[c] = (int)c;
+            root_min[c] = 0x7fffffff;
+            if ((coarse[j] >> lane) & 1u) table[key[j] >> 6] = c;
+        }
+        if (q == n - 1) {
+            *n_cells = c + 1u;
+            cell_start[c + 1u] = (uint32_t)n;
+        }
+    }
 }
 
 // occupancy mask of each coarse cell, kept at its first fine cell
@@ -108,19 +141,6 @@ __global__ void k_fof_occ(const uint32_t *n_cells_p, const uint64_t *cell_key, c
         const uint64_t k = cell_key[c];
         atomicOr((unsigned long long *)&occ[table[k >> 6]], 1ull << (k & 63));
     }
-}
-
-__global__ void k_fill_u32(uint32_t *p, int64_t n, uint32_t v)
-{
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (; i < n; i += stride) p[i] = v;
-}
-
-__global__ void k_iota_i32(int *p, int64_t n)
-{
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = (int)i;
 }
 
 // sub-cells (4 per axis, bit (z << 4) | (y << 2) | x) of the coarse cell at
@@ -215,6 +235,13 @@ __device__ __forceinline__ int nth_bit64(uint64_t m, int j)
 // rest.  Coarse cells numbered below A's hold only fine cells of smaller
 // index and are not visited.
 //
+// Pass 2 takes all cells at once, for boxes so small that the passes' chains
+// of dependent loads cost more than their pairs (32,768 particles: 166 us in
+// one pass, 76 in two, so up to 8192 only).  Where the rows of 32 cells do not
+// fill the device a warp takes only 8 / split of the eight coarse cells, so
+// that more warps share the chain, and the root kernels between the passes are
+// left out (32,768 particles: 117 -> 76 us).
+//
 // A warp takes 32 consecutive fine cells, a lane each.  For each of the
 // eight coarse cells around them every lane forms its mask of candidate fine
 // cells; the warp then numbers all lanes' candidates (a prefix sum of the
@@ -223,13 +250,17 @@ __device__ __forceinline__ int nth_bit64(uint64_t m, int j)
 __global__ void __launch_bounds__(FOF_THREADS, 6) k_fof_link(const uint32_t *n_cells_p, const uint64_t *cell_key,
                                                             const uint32_t *cell_start, const uint32_t *table,
                                                             const uint64_t *occ, const float4 *spos, int *parent,
-                                                            const int *uroot, FofGeom g, int pass, rs_dev_status *st)
+                                                            const int *uroot, FofGeom g, int pass, int split,
+                                                            rs_dev_status *st)
 {
     const unsigned FULL = 0xffffffffu;
     const int64_t M = *n_cells_p;
     const int lane = lane_id();
-    const int64_t wfirst = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31));
-    for (int64_t wb = wfirst; wb < M; wb += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t warps = (int64_t)gridDim.x * blockDim.x >> 5;
+    for (int64_t u = warp0; u < (M + 31) / 32 * split; u += warps) {
+        const int64_t wb = u / split * 32;
+        const int s0 = (int)(u % split) * (8 / split), s1 = s0 + 8 / split;
         const int64_t A = wb + lane;
         const bool va = A < M;
         uint64_t ca = 0;
@@ -251,7 +282,7 @@ __global__ void __launch_bounds__(FOF_THREADS, 6) k_fof_link(const uint32_t *n_c
         // a root of A's set (sets only grow, so a coarse cell whose common
         // root equals it is in A's set for the rest of the pass)
         const int ra = (va && uroot) ? uf_find(parent, (int)A, st) : -1;
-        for (int s8 = 0; s8 < 8; s8++) {
+        for (int s8 = s0; s8 < s1; s8++) {
             const int dz = loz + (s8 >> 2), dy = loy + ((s8 >> 1) & 1), dx = lox + (s8 & 1);
             int cz = ccz + dz, cy = ccy + dy, cx = ccx + dx;
             cz = cz < 0 ? cz + g.Gc : (cz >= g.Gc ? cz - g.Gc : cz);
@@ -265,7 +296,7 @@ __global__ void __launch_bounds__(FOF_THREADS, 6) k_fof_link(const uint32_t *n_c
                     b0c = table[cc];
                     if (b0c != 0xffffffffu && !(ra >= 0 && uroot[b0c] == ra)) {
                         om = occ[b0c];
-                        const uint64_t near = reach_mask(ux, uy, uz, dx, dy, dz, 1);
+                        const uint64_t near = pass < 2 ? reach_mask(ux, uy, uz, dx, dy, dz, 1) : 0ull;
                         cand = om & (pass == 0 ? near : reach_mask(ux, uy, uz, dx, dy, dz, 2) & ~near);
                         if (cc == ca) cand &= ~((2ull << sa) - 1ull);  // sub-cells after A's
                     }
@@ -796,53 +827,49 @@ rs_status fof_run(rs_ctx *ctx, const float *pos, int32_t stride, int64_t n, doub
     RS_WS(ctx, uint64_t, k1, WS_SORT_K1, n);
     RS_WS(ctx, uint32_t, v0, WS_SORT_V0, n);
     RS_WS(ctx, uint32_t, v1, WS_SORT_V1, n);
-    RS_LAUNCH(ctx, "fof_keys", k_fof_keys, nb, T, 0, pos, stride, n, g, k0, v0, ctx->d_status);
+    RS_WS(ctx, uint32_t, table, WS_FOF_TABLE, ncoarse);
+    RS_LAUNCH(ctx, "fof_keys", k_fof_keys, nb, T, 0, pos, stride, n, g, k0, v0, table, ncoarse, ctx->d_status);
     bool alt = false;
     RS_TRY(rs_radix_sort_u64(ctx, k0, k1, v0, v1, n, key_bits(g), &alt, "sort_fof"));
     uint64_t *keys = alt ? k1 : k0;
     uint32_t *idx = alt ? v1 : v0;
 
     RS_WS(ctx, float4, spos, WS_FOF_POS4, n);
-    RS_WS(ctx, uint32_t, flag, WS_FOF_MISC, 2 * n + 8);
-    uint32_t *scan = flag + n;
-    uint32_t *n_cells = flag + 2 * n;  // device scalar
-    RS_LAUNCH(ctx, "fof_gather", k_fof_gather, nb, T, 0, pos, stride, n, (const uint64_t *)keys,
-              (const uint32_t *)idx, spos, flag);
-    RS_CUDA(ctx, cudaMemcpyAsync(scan, flag, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, ctx->stream));
-    RS_TRY(rs_scan_u32(ctx, scan, n, n_cells));
-
+    RS_WS(ctx, uint32_t, misc, WS_FOF_MISC, n + 8);
+    uint32_t *n_cells = misc;                                     // device scalar
+    unsigned long long *cnt = (unsigned long long *)(misc + 2);  // groups, tie-band pairs
+    int *uroot = (int *)(misc + 8);  // common root of each coarse cell between the link passes
     RS_WS(ctx, uint32_t, cell_of, WS_FOF_CELLOF, n);
     RS_WS(ctx, uint32_t, cell_start, WS_FOF_CELLSTART, n + 1);
     RS_WS(ctx, uint64_t, cell_key, WS_FOF_CELLKEY, n);
-    RS_WS(ctx, uint32_t, table, WS_FOF_TABLE, ncoarse);
-    int fill_blocks = (int)std::min<int64_t>(ceil_div(ncoarse, T), (int64_t)ctx->num_sms * 16);
-    RS_LAUNCH(ctx, "fof_table_clear", k_fill_u32, fill_blocks, T, 0, table, ncoarse, 0xffffffffu);
-    RS_LAUNCH(ctx, "fof_cells", k_fof_cells, nb, T, 0, n, (const uint64_t *)keys, (const uint32_t *)scan,
-              (const uint32_t *)flag, cell_of, cell_start, cell_key, table, (const uint32_t *)n_cells);
     RS_WS(ctx, uint64_t, occ, WS_FOF_OCC, n);
-    RS_CUDA(ctx, cudaMemsetAsync(occ, 0, sizeof(uint64_t) * n, ctx->stream));
+    RS_WS(ctx, int, parent, WS_FOF_PARENT, n);
+    RS_WS(ctx, int, root_min, WS_FOF_ROOTMIN, n);
+    const int64_t ctiles = ceil_div(n, CELL_TILE);
+    RsLookback lb;
+    RS_TRY(rs_lookback_init(ctx, ctiles, &lb));
+    RS_LAUNCH(ctx, "fof_cells", k_fof_cells, ctiles, T, 0, pos, stride, n, (const uint64_t *)keys,
+              (const uint32_t *)idx, spos, cell_of, cell_start, cell_key, table, occ, parent, root_min, n_cells, lb,
+              ctx->d_status);
     const int64_t grid = std::min<int64_t>(nb, (int64_t)ctx->num_sms * ctx->tune.fof_link_ctas_per_sm);
     RS_LAUNCH(ctx, "fof_occ", k_fof_occ, grid, T, 0, (const uint32_t *)n_cells, (const uint64_t *)cell_key,
               (const uint32_t *)table, occ);
-
-    RS_WS(ctx, int, parent, WS_FOF_PARENT, n);
-    RS_WS(ctx, int, root_min, WS_FOF_ROOTMIN, n);
-    RS_LAUNCH(ctx, "fof_iota", k_iota_i32, nb, T, 0, parent, n);
-    RS_LAUNCH(ctx, "fof_fill", k_fill_u32, std::min<int64_t>(nb, (int64_t)ctx->num_sms * 16), T, 0,
-              (uint32_t *)root_min, n, 0x7fffffffu);
-    // (flag's first n words are free once the cells are numbered: they hold
-    // the common root of each coarse cell between the passes)
-    int *uroot = (int *)flag;
-    for (int pass = 0; pass < 2; pass++) {
-        if (pass == 1) {
+    const int64_t rows = ceil_div(n, 32), warps = (int64_t)ctx->num_sms * 48;
+    const bool small = n <= FOF_ONE_PASS;
+    int split = 1;
+    while (split < 8 && rows * split * 2 <= 2 * warps) split *= 2;
+    const int64_t lgrid = split > 1 ? ceil_div(rows * split, T / 32) : grid;
+    const bool roots = split == 1;  // the root kernels pay where most warps run more than one row
+    for (int pass = small ? 2 : 0; pass < (small ? 3 : 2); pass++) {
+        if (pass == 1 && roots) {
             RS_LAUNCH(ctx, "fof_uroot_first", k_fof_uroot_first, grid, T, 0, (const uint32_t *)n_cells,
                       (const uint64_t *)cell_key, (const uint32_t *)table, parent, uroot, ctx->d_status);
             RS_LAUNCH(ctx, "fof_uroot_check", k_fof_uroot_check, grid, T, 0, (const uint32_t *)n_cells,
                       (const uint64_t *)cell_key, (const uint32_t *)table, parent, uroot, ctx->d_status);
         }
-        RS_LAUNCH(ctx, "fof_link", k_fof_link, grid, T, 0, (const uint32_t *)n_cells, (const uint64_t *)cell_key,
+        RS_LAUNCH(ctx, "fof_link", k_fof_link, lgrid, T, 0, (const uint32_t *)n_cells, (const uint64_t *)cell_key,
                   (const uint32_t *)cell_start, (const uint32_t *)table, (const uint64_t *)occ, (const float4 *)spos,
-                  parent, pass == 1 ? (const int *)uroot : nullptr, g, pass, ctx->d_status);
+                  parent, pass == 1 && roots ? (const int *)uroot : nullptr, g, pass, split, ctx->d_status);
     }
     if (dense_n >= 0) {
         // accelerated variant: dense flags, centre rounds, 2l joins
@@ -901,7 +928,6 @@ rs_status fof_run(rs_ctx *ctx, const float *pos, int32_t stride, int64_t n, doub
     RS_LAUNCH(ctx, "fof_labels", k_fof_labels, nb, T, 0, n, (const uint32_t *)idx, (const uint32_t *)cell_of,
               parent, (const int *)root_min, labels, ctx->d_status);
     if (n_groups || n_tieband) {
-        unsigned long long *cnt = (unsigned long long *)(flag + 2 * n + 2);
         RS_CUDA(ctx, cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), ctx->stream));
         if (n_groups)
             RS_LAUNCH(ctx, "fof_count_roots", k_fof_count_roots, grid, T, 0, (const uint32_t *)n_cells,
@@ -938,60 +964,108 @@ extern "C" rs_status rs_fof3d_accel(rs_ctx *ctx, const float *pos, int32_t strid
 // ---------------------------------------------------------------------------
 namespace {
 
-// Members per label.  The lanes of a warp that share a label add together
-// (one atomic per distinct label in the warp): neighbours in the input often
-// belong to one group, whose counter would otherwise take one atomic per
-// member.
-__global__ void k_gs_count(int64_t n, const int32_t *labels, uint32_t *count, rs_dev_status *st)
+// Members per label besides the label's own particle (which alone makes most
+// of a catalogue's groups and needs no count).  A block counts GS_TILE
+// particles in a shared hash table before it adds to memory: the members of a
+// large group, spread over the catalogue, would otherwise queue on its one
+// counter (33M particles: 2.02 -> 0.24 ms).
+constexpr int GS_THREADS = 256;
+constexpr int GS_TILE = 16384;
+constexpr int GS_SLOTS = 4096;
+constexpr int GS_PROBES = 8;
+
+__global__ void __launch_bounds__(GS_THREADS) k_gs_count(int64_t n, const int32_t *labels, uint32_t *count,
+                                                         rs_dev_status *st)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int32_t l = -1;
-    if (i < n) {
-        l = labels[i];
+    __shared__ int32_t slot[GS_SLOTS];
+    __shared__ uint32_t num[GS_SLOTS];
+    for (int s = threadIdx.x; s < GS_SLOTS; s += GS_THREADS) {
+        slot[s] = -1;
+        num[s] = 0;
+    }
+    __syncthreads();
+    const int64_t i0 = (int64_t)blockIdx.x * GS_TILE;
+    for (int64_t i = i0 + threadIdx.x; i < min(n, i0 + GS_TILE); i += GS_THREADS) {
+        const int32_t l = labels[i];
         if (l < 0 || l > i) {
             dev_fail(st, DEV_BADARG, 20, i);
-            l = -1;
+            continue;
         }
+        if (l == i) continue;
+        unsigned h = ((unsigned)l * 2654435761u) >> 20;  // Knuth's multiplicative hash, 12 bits
+        bool done = false;
+        for (int p = 0; p < GS_PROBES && !done; p++, h = (h + 1) & (GS_SLOTS - 1)) {
+            int32_t have = ((volatile int32_t *)slot)[h];
+            if (have == -1) have = atomicCAS(&slot[h], -1, l);
+            if (have == -1 || have == l) {
+                atomicAdd(&num[h], 1u);
+                done = true;
+            }
+        }
+        if (!done) atomicAdd(&count[l], 1u);
     }
-    const unsigned peers = __match_any_sync(0xffffffffu, l);
-    if (l >= 0 && lane_id() == __ffs(peers) - 1) atomicAdd(&count[l], (uint32_t)__popc(peers));
+    __syncthreads();
+    for (int s = threadIdx.x; s < GS_SLOTS; s += GS_THREADS)
+        if (num[s]) atomicAdd(&count[slot[s]], num[s]);
 }
 
-// root flags: groups of >= min_n members, keyed by their label (= root index)
-__global__ void k_gs_rootflag(int64_t n, const int32_t *labels, const uint32_t *count, int32_t min_n,
-                              uint32_t *rflag)
+// One pass with look-back: the members of groups of >= min_n members, in
+// index order, and the groups (numbered by their label, the root's index)
+// with their sizes.  The scanned sum packs groups << 31 | members.
+constexpr int GS_ROWS = 8;
+constexpr int64_t GS_SCAN_TILE = (int64_t)GS_ROWS * GS_THREADS;
+
+__global__ void __launch_bounds__(GS_THREADS) k_gs_select(int64_t n, const int32_t *labels, const uint32_t *count,
+                                                          int32_t min_n, uint32_t *members, uint32_t *group,
+                                                          int64_t *sizes, int64_t cap, uint32_t *tot, RsLookback lb,
+                                                          rs_dev_status *st)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    rflag[i] = (labels[i] == (int32_t)i && count[i] >= (uint32_t)min_n) ? 1u : 0u;  // label i is in range
+    const unsigned FULL = 0xffffffffu;
+    const int64_t tile = rs_next_tile(lb);
+    const int lane = lane_id();
+    const int64_t base = tile * GS_SCAN_TILE + (int64_t)warp_id() * 32 * GS_ROWS;
+    unsigned mem[GS_ROWS], root[GS_ROWS];
+    uint32_t size[GS_ROWS];
+    unsigned long long sum = 0;
+#pragma unroll
+    for (int j = 0; j < GS_ROWS; j++) {
+        const int64_t i = base + 32 * j + lane;
+        const int32_t l = i < n ? labels[i] : -1;
+        size[j] = l >= 0 && l <= i ? count[l] + 1u : 0u;
+        const bool in = size[j] >= (uint32_t)min_n && size[j] > 0u;
+        mem[j] = __ballot_sync(FULL, in);
+        root[j] = __ballot_sync(FULL, in && l == i);
+        sum += (unsigned long long)__popc(root[j]) << 31 | (unsigned)__popc(mem[j]);
+    }
+    unsigned long long all;
+    unsigned long long at = rs_block_scan<GS_THREADS>(lane == 0 ? sum : 0ull, all);
+    at = __shfl_sync(FULL, at, 0) + rs_lookback(lb, tile, all, st);
+    uint32_t m0 = (uint32_t)(at & 0x7fffffffull), g0 = (uint32_t)(at >> 31);
+    const unsigned below = (1u << lane) - 1u;
+#pragma unroll
+    for (int j = 0; j < GS_ROWS; j++) {
+        const int64_t i = base + 32 * j + lane;
+        const uint32_t m = m0 + (uint32_t)__popc(mem[j] & below), g = g0 + (uint32_t)__popc(root[j] & below);
+        if (((mem[j] >> lane) & 1u) && m < n) members[m] = (uint32_t)i;
+        if ((root[j] >> lane) & 1u) {
+            group[i] = g;
+            if (g < cap) sizes[g] = size[j];
+        }
+        m0 += (uint32_t)__popc(mem[j]);
+        g0 += (uint32_t)__popc(root[j]);
+    }
+    if ((tile + 1) * GS_SCAN_TILE >= n && threadIdx.x == GS_THREADS - 1) {
+        tot[0] = g0;
+        tot[1] = m0;
+    }
 }
 
-// member flags
-__global__ void k_gs_memflag(int64_t n, const int32_t *labels, const uint32_t *count, int32_t min_n,
-                             uint32_t *mflag)
+// the members' group numbers
+__global__ void k_gs_keys(int64_t m, const uint32_t *members, const int32_t *labels, const uint32_t *group,
+                          uint32_t *keys)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int32_t l = labels[i];
-    mflag[i] = (l >= 0 && l <= i && count[l] >= (uint32_t)min_n) ? 1u : 0u;
-}
-
-__global__ void k_gs_compact(int64_t n, const int32_t *labels, const uint32_t *mflag, const uint32_t *mscan,
-                             const uint32_t *rscan, uint32_t *keys, uint32_t *vals)
-{
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || !mflag[i]) return;
-    uint32_t p = mscan[i];
-    keys[p] = rscan[labels[i]];
-    vals[p] = (uint32_t)i;
-}
-
-__global__ void k_gs_sizes(int64_t n, const uint32_t *rflag, const uint32_t *rscan, const uint32_t *count,
-                           int64_t *offsets)
-{
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || !rflag[i]) return;
-    offsets[rscan[i]] = count[i];
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < m) keys[p] = group[labels[members[p]]];
 }
 
 }  // namespace
@@ -1012,19 +1086,16 @@ extern "C" rs_status rs_group_sort(rs_ctx *ctx, const int32_t *labels, int64_t n
     }
     RsStageGuard running(&ctx->in_gs);
     RsRange range("rs_group_sort");
-    const int64_t T = 256, nb = ceil_div(n, T);
     RS_WS(ctx, uint32_t, count, WS_GS_COUNT, n);
-    RS_WS(ctx, uint32_t, fl, WS_GS_FLAG, 4 * n + 8);
-    uint32_t *rflag = fl, *rscan = fl + n, *mflag = fl + 2 * n, *mscan = fl + 3 * n;
-    uint32_t *tot = fl + 4 * n;  // [0] groups, [1] members
+    RS_WS(ctx, uint32_t, fl, WS_GS_FLAG, n + 8);
+    uint32_t *tot = fl, *group = fl + 8;  // tot: groups, members
     RS_CUDA(ctx, cudaMemsetAsync(count, 0, sizeof(uint32_t) * n, ctx->stream));
-    RS_LAUNCH(ctx, "gs_count", k_gs_count, nb, T, 0, n, labels, count, ctx->d_status);
-    RS_LAUNCH(ctx, "gs_rootflag", k_gs_rootflag, nb, T, 0, n, labels, (const uint32_t *)count, min_n, rflag);
-    RS_LAUNCH(ctx, "gs_memflag", k_gs_memflag, nb, T, 0, n, labels, (const uint32_t *)count, min_n, mflag);
-    RS_CUDA(ctx, cudaMemcpyAsync(rscan, rflag, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, ctx->stream));
-    RS_CUDA(ctx, cudaMemcpyAsync(mscan, mflag, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, ctx->stream));
-    RS_TRY(rs_scan_u32(ctx, rscan, n, tot));
-    RS_TRY(rs_scan_u32(ctx, mscan, n, tot + 1));
+    RS_LAUNCH(ctx, "gs_count", k_gs_count, ceil_div(n, GS_TILE), GS_THREADS, 0, n, labels, count, ctx->d_status);
+    const int64_t tiles = ceil_div(n, GS_SCAN_TILE);
+    RsLookback lb;
+    RS_TRY(rs_lookback_init(ctx, tiles, &lb));
+    RS_LAUNCH(ctx, "gs_select", k_gs_select, tiles, GS_THREADS, 0, n, labels, (const uint32_t *)count, min_n,
+              (uint32_t *)perm, group, offsets, offsets_cap, tot, lb, ctx->d_status);
     uint32_t h2[2];
     RS_CUDA(ctx, cudaMemcpyAsync(ctx->h_scratch, tot, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
     RS_TRY(rs_sync_check(ctx, "rs_group_sort"));
@@ -1037,17 +1108,15 @@ extern "C" rs_status rs_group_sort(rs_ctx *ctx, const int32_t *labels, int64_t n
     uint32_t *k0 = (uint32_t *)kbuf, *k1 = (uint32_t *)kbuf + Mm;
     RS_WS(ctx, uint32_t, vtmp, WS_SORT_V1, Mm);
     uint32_t *v0 = (uint32_t *)perm;
-    RS_LAUNCH(ctx, "gs_compact", k_gs_compact, nb, T, 0, n, labels, (const uint32_t *)mflag,
-              (const uint32_t *)mscan, (const uint32_t *)rscan, k0, v0);
+    RS_LAUNCH(ctx, "gs_keys", k_gs_keys, ceil_div(Mm, 256), 256, 0, Mm, (const uint32_t *)v0, labels,
+              (const uint32_t *)group, k0);
     int bits = 0;
     while (bits < 32 && ((uint64_t)(G > 0 ? G - 1 : 0) >> bits) != 0) bits++;
     bool alt = false;
     RS_TRY(rs_radix_sort_u32(ctx, k0, k1, v0, vtmp, Mm, bits, &alt, "sort_gs"));
     if (alt)
         RS_CUDA(ctx, cudaMemcpyAsync(perm, vtmp, sizeof(uint32_t) * Mm, cudaMemcpyDeviceToDevice, ctx->stream));
-    RS_CUDA(ctx, cudaMemsetAsync(offsets, 0, sizeof(int64_t) * (G + 1), ctx->stream));
-    RS_LAUNCH(ctx, "gs_sizes", k_gs_sizes, nb, T, 0, n, (const uint32_t *)rflag, (const uint32_t *)rscan,
-              (const uint32_t *)count, offsets);
+    RS_CUDA(ctx, cudaMemsetAsync(offsets + G, 0, sizeof(int64_t), ctx->stream));
     RS_TRY(rs_scan_i64(ctx, offsets, G + 1, nullptr));
     return rs_sync_check(ctx, "rs_group_sort");
 }

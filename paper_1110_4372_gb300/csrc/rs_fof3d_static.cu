@@ -37,7 +37,9 @@ constexpr int64_t r256(int64_t b) { return (b + 255) / 256 * 256; }
 constexpr int64_t SZ_STATUS = r256(sizeof(rs_dev_status));
 constexpr int64_t SZ_K = r256(8 * STATIC_MAX_N);                       // sort keys (x2)
 constexpr int64_t SZ_V = r256(4 * STATIC_MAX_N);                       // sort values (x2)
-constexpr int64_t SZ_HIST = r256(4 * 256 * ((STATIC_MAX_N + STATIC_SORT_TILE - 1) / STATIC_SORT_TILE));
+constexpr int64_t STATIC_SORT_PASSES = 4;  // keys of at most 2^20 cells x 64 sub-cells, and the one past them
+constexpr int64_t SZ_HIST =
+    r256(4 * STATIC_SORT_PASSES * (320 + 256 * ((STATIC_MAX_N + STATIC_SORT_TILE - 1) / STATIC_SORT_TILE)));
 constexpr int64_t SZ_SCAN = r256(STATIC_SCAN_BYTES);
 constexpr int64_t SZ_POS4 = r256(16 * STATIC_MAX_N);
 constexpr int64_t SZ_MISC = r256(4 * (2 * STATIC_MAX_N + 8));

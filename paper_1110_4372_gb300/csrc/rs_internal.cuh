@@ -179,8 +179,9 @@ __host__ __device__ static inline int64_t ceil_div(int64_t a, int64_t b) { retur
 // In-place exclusive prefix sum; *total (device, optional) receives the sum.
 rs_status rs_scan_u32(rs_ctx *ctx, uint32_t *data, int64_t n, uint32_t *total);
 rs_status rs_scan_i64(rs_ctx *ctx, int64_t *data, int64_t n, int64_t *total);
-// keys per radix-sort tile; the histogram workspace holds 256 counts per tile
-constexpr int64_t RS_SORT_TILE = 2048;
+// keys per radix-sort tile; the sort workspace holds, per pass of 8 key bits,
+// 320 words and 256 words per tile
+constexpr int64_t RS_SORT_TILE = 4096;
 // Stable LSD radix sort of (key, value) pairs on key bits [0, nbits).  The
 // caller provides both ping-pong buffers; *out_in_alt says whether the
 // sorted data ended in (k1, v1).
@@ -231,6 +232,91 @@ __device__ __forceinline__ T warp_max(T v)
 __device__ __forceinline__ double f64_mul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double f64_add(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ double f64_sub(double a, double b) { return __dsub_rn(a, b); }
+
+// ---- one-pass scans over tiles ----
+// A scan kernel takes its tile from a counter (so every earlier tile is
+// running or done), publishes the tile's sum, adds up its predecessors' sums
+// back to the first whose prefix is known, and publishes its own prefix.  A
+// state word is 0 until then, a sum with bit 62 set, or an inclusive prefix
+// with bit 63 set.  The wait for a predecessor is bounded.
+struct RsLookback {
+    unsigned *next;
+    unsigned long long *state;
+};
+// cleared counter and states for a scan of this many tiles (rs_scan_sort.cu)
+rs_status rs_lookback_init(rs_ctx *ctx, int64_t tiles, RsLookback *lb);
+
+// the block's tile
+__device__ __forceinline__ int64_t rs_next_tile(const RsLookback &lb)
+{
+    __shared__ unsigned tile;
+    if (threadIdx.x == 0) tile = atomicAdd(lb.next, 1u);
+    __syncthreads();
+    return tile;
+}
+
+// exclusive prefix of v over the block's THREADS threads; tot: the sum
+template <int THREADS, typename T>
+__device__ __forceinline__ T rs_block_scan(T v, T &tot)
+{
+    constexpr int WARPS = THREADS / 32;
+    static_assert(WARPS <= 32, "");
+    __shared__ T wsum[WARPS];
+    const int lane = lane_id(), w = warp_id();
+    T x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const T y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[w] = x;
+    __syncthreads();
+    T s = lane < WARPS ? wsum[lane] : T(0);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const T y = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += y;
+    }
+    tot = __shfl_sync(0xffffffffu, s, WARPS - 1);
+    const T before = __shfl_sync(0xffffffffu, s, w > 0 ? w - 1 : 0);
+    __syncthreads();
+    return (w > 0 ? before : T(0)) + x - v;
+}
+
+// the sum over all earlier tiles, in every thread (sum below 2^62)
+__device__ __forceinline__ unsigned long long rs_lookback(const RsLookback &lb, int64_t tile, unsigned long long sum,
+                                                          rs_dev_status *st)
+{
+    constexpr unsigned long long SUM = 1ull << 62, PREFIX = 1ull << 63;
+    __shared__ unsigned long long before_s;
+    if (warp_id() == 0) {
+        volatile unsigned long long *s = lb.state;
+        const int lane = lane_id();
+        unsigned long long before = 0;
+        if (lane == 0) s[tile] = tile == 0 ? PREFIX | sum : SUM | sum;
+        for (int64_t t = tile - 1; t >= 0; t -= 32) {
+            // the 32 tiles up to t, the nearest in lane 0
+            unsigned long long x = t >= lane ? s[t - lane] : PREFIX;
+            for (int it = 0; it < RS_SPIN_LIMIT && __any_sync(0xffffffffu, x == 0); it++)
+                if (x == 0) x = s[t - lane];
+            const unsigned zero = __ballot_sync(0xffffffffu, x == 0);
+            if (zero) {
+                if (lane == 0) dev_fail(st, DEV_TIMEOUT, 92, tile);
+                break;
+            }
+            const unsigned pre = __ballot_sync(0xffffffffu, (x >> 63) != 0);
+            const int stop = pre ? __ffs(pre) - 1 : 31;
+            before += warp_sum(lane <= stop ? x & (SUM - 1) : 0ull);
+            if (pre) break;
+        }
+        if (lane == 0) {
+            if (tile > 0) s[tile] = PREFIX | (before + sum);
+            before_s = before;
+        }
+    }
+    __syncthreads();
+    return before_s;
+}
 
 // Fine cells per side of the 3D FOF grid for (n, box, b): the side s is the
 // largest with sqrt(3) s (1 + 2 err) < l, err being the float32 error of a

@@ -2737,23 +2737,34 @@ __global__ void __launch_bounds__(TQ) k_lvl_hist(LevelBufs L, NodeArrays nd, con
         if (h[i]) atomicAdd(&L.hist[(int64_t)k * 2048 + i], h[i]);
 }
 
-__global__ void k_lvl_pick(LevelBufs L, int pass)
+// the digit that holds the rank still to select, eight bins a thread (one
+// thread over the 2048 bins took 75 us, three times a level); the bins are
+// cleared for the next pass
+__global__ void __launch_bounds__(256) k_lvl_pick(LevelBufs L, int pass)
 {
     const int k = blockIdx.x;
-    if (threadIdx.x != 0) return;
-    unsigned *h = L.hist + (int64_t)k * 2048;
-    int krem = L.sel_krem[k];
-    const int nbins = pass == 2 ? 1024 : 2048;
+    uint4 *h = reinterpret_cast<uint4 *>(L.hist + (int64_t)k * 2048) + 2 * threadIdx.x;
+    const uint4 a = h[0], b = h[1];
+    h[0] = h[1] = make_uint4(0u, 0u, 0u, 0u);
+    const unsigned c[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    const unsigned sum = a.x + a.y + a.z + a.w + b.x + b.y + b.z + b.w;
+    unsigned all;
+    unsigned acc = rs_block_scan<256>(sum, all);
+    const unsigned krem = (unsigned)L.sel_krem[k];
     const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
-    int acc = 0, d = 0;
-    for (d = 0; d < nbins; d++) {
-        if (acc + (int)h[d] >= krem) break;
-        acc += (int)h[d];
+    __syncthreads();
+    if (krem > all) {  // (fewer values than the rank: the last bin)
+        if (threadIdx.x == 0) {
+            L.sel_prefix[k] |= (pass == 2 ? 1023u : 2047u) << shift;
+            L.sel_krem[k] = (int)(krem - all);
+        }
+        return;
     }
-    if (d >= nbins) d = nbins - 1;
-    L.sel_prefix[k] |= (unsigned)d << shift;
-    L.sel_krem[k] = krem - acc;
-    for (int i = 0; i < 2048; i++) h[i] = 0;
+    if (!(acc < krem && krem <= acc + sum)) return;
+    int d = 0;
+    while (acc + c[d] < krem) acc += c[d++];
+    L.sel_prefix[k] |= (unsigned)(8 * threadIdx.x + d) << shift;
+    L.sel_krem[k] = (int)(krem - acc);
 }
 
 __global__ void __launch_bounds__(TQ) k_lvl_band(LevelBufs L, NodeArrays nd, const float *dnn)
@@ -3312,7 +3323,7 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
                 for (int pass = 0; pass < 3; pass++) {
                     RS_LAUNCH(ctx, "rf_sub_hist", k_sub_hist, T, TQ, 0, L, nd, (const int *)widx,
                               (unsigned long long)sub_seed, (int)sub_n, stage, pass);
-                    RS_LAUNCH(ctx, "rf_lvl_pick", k_lvl_pick, K, 32, 0, L, pass);
+                    RS_LAUNCH(ctx, "rf_lvl_pick", k_lvl_pick, K, 256, 0, L, pass);
                 }
                 RS_LAUNCH(ctx, "rf_sub_stage", k_sub_stage, ceil_div(K, 128), 128, 0, L, stage);
             }
@@ -3372,7 +3383,7 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
         RS_LAUNCH(ctx, "rf_lvl_initk", k_lvl_initk, ceil_div(K, 128), 128, 0, L, nd, f, (int)sub_n);
         for (int pass = 0; pass < 3; pass++) {
             RS_LAUNCH(ctx, "rf_lvl_hist", k_lvl_hist, T, TQ, 0, L, nd, (const float *)dnn, pass);
-            RS_LAUNCH(ctx, "rf_lvl_pick", k_lvl_pick, K, 32, 0, L, pass);
+            RS_LAUNCH(ctx, "rf_lvl_pick", k_lvl_pick, K, 256, 0, L, pass);
         }
         RS_LAUNCH(ctx, "rf_bracket_check", k_bracket_check, ceil_div(K, 128), 128, 0, L, R2,
                   (const float *)STOP, fallback, rs_fault("bracket") ? 1 : 0);
@@ -3385,7 +3396,7 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
             RS_LAUNCH(ctx, "rf_lvl_initk", k_lvl_initk, ceil_div(K, 128), 128, 0, L, nd, f, (int)sub_n);
             for (int pass = 0; pass < 3; pass++) {
                 RS_LAUNCH(ctx, "rf_lvl_hist", k_lvl_hist, T, TQ, 0, L, nd, (const float *)dnn, pass);
-                RS_LAUNCH(ctx, "rf_lvl_pick", k_lvl_pick, K, 32, 0, L, pass);
+                RS_LAUNCH(ctx, "rf_lvl_pick", k_lvl_pick, K, 256, 0, L, pass);
             }
             n_fallback_levels++;
         }
