@@ -1091,15 +1091,144 @@ struct LevelBufs {
     int *sub_cnt;            // per rank: members drawn into the subset
 };
 
-__global__ void k_lvl_prep(const int *list, int K, NodeArrays nd, int64_t *tiles, int64_t *segc,
-                           unsigned long long *max_count)
+// ---- sizes the level's setup needs of the hierarchies and splits below ----
+constexpr int BVH_LEAF = 32;
+constexpr int BVH_LOG = 5;  // log2 of the leaf size and of the fan-out
+constexpr int BVH_MAXH = 8;
+
+__device__ __forceinline__ int bvh_levels(int nl)
 {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
-    int c = nd.count[list[k]];
-    tiles[k] = ceil_div(c, TQ);
-    segc[k] = c;
-    atomicMax(max_count, (unsigned long long)c);
+    int h = 1;
+    while (nl > 1) {
+        nl = (nl + 31) >> BVH_LOG;
+        h++;
+    }
+    return h;
+}
+
+__device__ __forceinline__ int64_t bvh_total(int nl)
+{
+    int64_t t = nl;
+    while (nl > 1) {
+        nl = (nl + 31) >> BVH_LOG;
+        t += nl;
+    }
+    return t;
+}
+
+__host__ __device__ __forceinline__ int kd_split(int m)
+{
+    int h = ((m / 2 + 31) / 32) * 32;
+    h = h < 32 ? 32 : h;
+    return h > m - 1 ? m - 1 : h;
+}
+
+// splits until a range of m members is at most `limit`
+__host__ __device__ __forceinline__ int kd_rounds(int64_t m, int limit)
+{
+    int r = 0;
+    while (m > limit) {
+        m = kd_split((int)m);
+        r++;
+    }
+    return r;
+}
+
+constexpr int KD_CTA = 1024;  // ranges of at most this many members finish in one CTA
+
+constexpr int SMP_MAX = 1024;  // sample size of a node's search bracket
+
+// Per-rank offsets of one level (K + 1 entries each, the last the total)
+struct LevelOff {
+    int64_t *tile;   // tiles of TQ members
+    int64_t *seg;    // members
+    int64_t *box;    // hierarchy boxes
+    int64_t *block;  // blocks of KD_CTA members
+    int *smp;        // ranks of the nodes searched with a sampled bracket
+    int *smp_at;     // per rank: its place there, or -1
+};
+
+constexpr int KD_MAXR = 16;   // kd_rounds(2^26, KD_CTA) and more
+// words of the level's totals, read by the host in one go
+enum { LT_K = 0, LT_T, LT_LM, LT_NBX, LT_SMP, LT_SUB, LT_ROUNDS, LT_ROUND0 = 8, LT_WORDS = LT_ROUND0 + 3 * KD_MAXR };
+
+// One block sets a level up: the nodes in descending order of their k-d
+// rounds (so the nodes that a round still splits are a prefix of the level's
+// tiles, members and blocks), every per-rank offset and the totals, per round
+// the prefix's tiles, members and blocks.  One launch and one host read
+// instead of a count, a scan and a read for each array and each round.
+__global__ void __launch_bounds__(1024) k_lvl_setup(const int *raw, const int *len, int *list, NodeArrays nd,
+                                                    LevelOff O, int sub_n, int bracket_min, int64_t *tot)
+{
+    __shared__ int cls[KD_MAXR + 1], at[KD_MAXR + 1], start[KD_MAXR + 2], nsub;
+    const int K = *len, tid = threadIdx.x;
+    if (tid <= KD_MAXR) cls[tid] = 0;
+    if (tid == 0) nsub = 0;
+    __syncthreads();
+    for (int i = tid; i < K; i += 1024) atomicAdd(&cls[min(kd_rounds(nd.count[raw[i]], KD_CTA), KD_MAXR)], 1);
+    __syncthreads();
+    if (tid == 0) {
+        int s = 0;
+        for (int c = KD_MAXR; c >= 0; c--) {
+            start[c] = at[c] = s;  // start[c]: nodes of more than c rounds
+            s += cls[c];
+        }
+    }
+    __syncthreads();
+    for (int i = tid; i < K; i += 1024) {
+        const int node = raw[i];
+        list[atomicAdd(&at[min(kd_rounds(nd.count[node], KD_CTA), KD_MAXR)], 1)] = node;
+    }
+    __syncthreads();
+    long long c0 = 0, c1 = 0, c2 = 0, c3 = 0, c4 = 0;
+    for (int i0 = 0; i0 < K; i0 += 1024) {
+        const int i = i0 + tid;
+        const bool ok = i < K;
+        const int n = ok ? nd.count[list[i]] : 0;
+        if (ok && sub_n > 0 && n > sub_n) atomicAdd(&nsub, 1);
+        const bool smp = ok && n > bracket_min && !(sub_n > 0 && n > sub_n);
+        long long s0, s1, s2, s3, s4;
+        const long long v0 = rs_block_scan<1024, long long>(ceil_div(n, TQ), s0);
+        const long long v1 = rs_block_scan<1024, long long>(n, s1);
+        const long long v2 = rs_block_scan<1024, long long>(ok ? bvh_total((int)ceil_div(n, BVH_LEAF)) : 0, s2);
+        const long long v3 = rs_block_scan<1024, long long>(ceil_div(n, KD_CTA), s3);
+        const long long v4 = rs_block_scan<1024, long long>(smp ? 1 : 0, s4);
+        if (ok) {
+            O.tile[i] = c0 + v0;
+            O.seg[i] = c1 + v1;
+            O.box[i] = c2 + v2;
+            O.block[i] = c3 + v3;
+            O.smp_at[i] = smp ? (int)(c4 + v4) : -1;
+            if (smp) O.smp[c4 + v4] = i;
+        }
+        c0 += s0;
+        c1 += s1;
+        c2 += s2;
+        c3 += s3;
+        c4 += s4;
+    }
+    if (tid == 0) {
+        O.tile[K] = c0;
+        O.seg[K] = c1;
+        O.box[K] = c2;
+        O.block[K] = c3;
+        tot[LT_K] = K;
+        tot[LT_T] = c0;
+        tot[LT_LM] = c1;
+        tot[LT_NBX] = c2;
+        tot[LT_SMP] = c4;
+        tot[LT_SUB] = nsub;
+        int r = 0;
+        while (r < KD_MAXR && start[r] > 0) r++;
+        tot[LT_ROUNDS] = r;
+    }
+    __syncthreads();
+    if (tid < KD_MAXR) {
+        const int k = start[tid];
+        tot[LT_ROUND0 + 3 * tid] = O.tile[k];
+        tot[LT_ROUND0 + 3 * tid + 1] = O.seg[k];
+        tot[LT_ROUND0 + 3 * tid + 2] = O.block[k];
+    }
 }
 
 __global__ void k_lvl_tiles(int K, const int64_t *tile_off, int *tile_rank, int *tile_q0)
@@ -1236,40 +1365,8 @@ __device__ __forceinline__ MemberStore mem_shift(const MemberStore &M, int64_t b
 // warp width: a search gives each lane one child box of the box it opens, or
 // one member of the leaf it scans.  Boxes of a node are stored level by
 // level from its base offset.
-constexpr int BVH_LEAF = 32;
-constexpr int BVH_LOG = 5;  // log2 of the leaf size and of the fan-out
-constexpr int BVH_MAXH = 8;
-
-__device__ __forceinline__ int bvh_levels(int nl)
-{
-    int h = 1;
-    while (nl > 1) {
-        nl = (nl + 31) >> BVH_LOG;
-        h++;
-    }
-    return h;
-}
-
-__device__ __forceinline__ int64_t bvh_total(int nl)
-{
-    int64_t t = nl;
-    while (nl > 1) {
-        nl = (nl + 31) >> BVH_LOG;
-        t += nl;
-    }
-    return t;
-}
-
 // first member of box (h, i) and the end of its member range
 __device__ __forceinline__ int64_t bvh_m0(int h, int i) { return (int64_t)i << (BVH_LOG * (h + 1)); }
-
-__global__ void k_bvh_prep(const int *list, int K, NodeArrays nd, int64_t *nbox)
-{
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
-    const int n = nd.count[list[k]];
-    nbox[k] = bvh_total((int)ceil_div(n, BVH_LEAF));
-}
 
 __device__ __forceinline__ Box6 box_empty()
 {
@@ -1529,13 +1626,6 @@ __device__ __forceinline__ float4 shfl4(float4 a, int src)
     return make_float4(__shfl_sync(FULLW, a.x, src), __shfl_sync(FULLW, a.y, src), __shfl_sync(FULLW, a.z, src), 0.f);
 }
 
-struct WarpJobs {
-    const int *rank;  // per warp job: node rank
-    const int *q0;    // first member of the job's 32 queries (a multiple of 32)
-    const int *out;   // where the first query's result goes (query j writes out + j)
-    int64_t count;
-};
-
 // Nearest-neighbour distance of member q (coordinates pq, vq) among the
 // node's members P, Q (n of them), starting from the radius `best` (the own
 // leaf `own` already scanned).  Returns as soon as the radius drops below
@@ -1631,18 +1721,20 @@ __device__ __forceinline__ float w32_nn(const BvhView &V, const MemberStore &M, 
 constexpr int NN_WARPS = 4;
 template <int MINB>
 __global__ void __launch_bounds__(NN_WARPS * 32, MINB * W_WARPS / NN_WARPS)
-    k_bvh_nn(LevelBufs L, WarpJobs J, NodeArrays nd, const int64_t *box_base, BoxStore B, MemberStore MS,
-             const float *R2, const float *STOP, int redo_failed, float *out, rs_dev_status *st)
+    k_bvh_nn(LevelBufs L, NodeArrays nd, const int64_t *box_base, BoxStore B, MemberStore MS, const float *R2,
+             const float *STOP, int redo_failed, int sub_n, float *out, rs_dev_status *st)
 {
     __shared__ int si_s[NN_WARPS][W_STACK];
     __shared__ float sd_s[NN_WARPS][W_STACK];
     __shared__ int lv_s[NN_WARPS][2 * BVH_MAXH];
     const int w = warp_id(), lane = lane_id();
-    const int64_t gw = (int64_t)blockIdx.x * NN_WARPS + w;
-    if (gw >= J.count) return;
-    const int k = J.rank[gw], q0 = J.q0[gw];
+    // the grid holds exactly the tiles' warps
+    constexpr int bpt = (TQ / 32) / NN_WARPS;
+    const int tile = blockIdx.x / bpt;
+    const int k = L.tile_rank[tile], q0 = L.tile_q0[tile] + 32 * ((blockIdx.x % bpt) * NN_WARPS + w);
     const int node = L.list[k], first = nd.first[node], n = nd.count[node];
-    if (q0 >= n) return;
+    // (a node above the subset size searches its subset members one by one)
+    if (q0 >= n || (sub_n > 0 && n > sub_n)) return;
     const Metric6 met = L.met[k];
     BvhView V;
     bvh_view(V, B, box_base[k], n, lv_s[w]);
@@ -1674,24 +1766,22 @@ __global__ void __launch_bounds__(NN_WARPS * 32, MINB * W_WARPS / NN_WARPS)
         best = w32_nn(V, M, n, q0 + j, pq, vq, met, best, stop, own, si_s[w], sd_s[w], st, node);
         if (lane == j) res = best;
     }
-    if (have) out[J.out[gw] + lane] = res >= start ? INFINITY : res;
+    if (have) out[first + mo] = res >= start ? INFINITY : res;
 }
 
 // nearest-neighbour distance of single sampled members, one warp each
 __global__ void __launch_bounds__(W_WARPS * 32) k_bvh_nn_sample(LevelBufs L, NodeArrays nd, const int64_t *box_base,
-                                                                BoxStore B, MemberStore MS, const int64_t *soff,
+                                                                BoxStore B, MemberStore MS, const int *smp,
                                                                 float *out, rs_dev_status *st)
 {
     __shared__ int si_s[W_WARPS][W_STACK];
     __shared__ float sd_s[W_WARPS][W_STACK];
     __shared__ int lv_s[W_WARPS][2 * BVH_MAXH];
     const int w = warp_id(), lane = lane_id();
-    const int k = blockIdx.y;
+    const int64_t at = (int64_t)blockIdx.x * W_WARPS + w;  // the grid holds exactly the samples
+    const int k = smp[at / SMP_MAX], s = (int)(at % SMP_MAX);
     const int node = L.list[k], first = nd.first[node], n = nd.count[node];
-    const int S = (int)(soff[k + 1] - soff[k]);
-    const int s = blockIdx.x * W_WARPS + w;
-    if (s >= S) return;
-    const int q = (int)(((int64_t)s * n) / S);
+    const int q = (int)(((int64_t)s * n) / SMP_MAX);
     const Metric6 met = L.met[k];
     BvhView V;
     bvh_view(V, B, box_base[k], n, lv_s[w]);
@@ -1702,7 +1792,7 @@ __global__ void __launch_bounds__(W_WARPS * 32) k_bvh_nn_sample(LevelBufs L, Nod
     if (m < n) mem_get(M, m, pm, vm);
     const float d = (m < n && m != q) ? d2_32(pq, vq, pm, vm, met) : INFINITY;
     const float best = w32_nn(V, M, n, q, pq, vq, met, wmin(d), 0.f, own, si_s[w], sd_s[w], st, node);
-    if (lane == 0) out[soff[k] + s] = best;
+    if (lane == 0) out[at] = best;
 }
 
 // nearest-neighbour distance of listed members (rank, member), one warp
@@ -2126,58 +2216,29 @@ __global__ void __launch_bounds__(LK_WARPS * 32, WARPS / LK_WARPS)
 // stop early with "none within t_hi".  Only values up to the k-th are needed
 // for the linking length; if the k-th value is not within t_hi the level
 // falls back to the unbounded search, so the result is always exact.
-constexpr int SMP_MAX = 1024;       // sample size per node
-// (nodes of at most rs_tuning::bracket_min members, 4096 by default, are
-// searched without a bracket)
-
-// (nodes that draw a member subset for the linking length search only the
-// subset, without a bracket)
-__global__ void k_smp_prep(const int *list, int K, NodeArrays nd, int64_t *ns, int sub_n, int min_node)
-{
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
-    const int n = nd.count[list[k]];
-    ns[k] = (n > min_node && !(sub_n > 0 && n > sub_n)) ? SMP_MAX : 0;
-}
-
-// full-search warp jobs: every 32 consecutive members of every node
-__global__ void k_full_jobs(const int *list, int K, NodeArrays nd, const int64_t *woff, int *jrank, int *jq0,
-                            int *jout)
-{
-    const int k = blockIdx.x;
-    if (k >= K) return;
-    const int node = list[k], first = nd.first[node];
-    const int64_t a = woff[k], c = woff[k + 1] - woff[k];
-    for (int64_t j = threadIdx.x; j < c; j += blockDim.x) {
-        jrank[a + j] = k;
-        jq0[a + j] = (int)(32 * j);
-        jout[a + j] = first + (int)(32 * j);
-    }
-}
-
-// warp jobs of 32 members per node; none for a node above the subset size
-// (sub_n > 0), whose subset members are searched one by one instead
-__global__ void k_full_prep(const int *list, int K, NodeArrays nd, int64_t *nw, int sub_n)
-{
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
-    const int n = nd.count[list[k]];
-    nw[k] = (sub_n > 0 && n > sub_n) ? 0 : ceil_div(n, 32);
-}
+// (nodes of at most rs_tuning::bracket_min members, 4096 by default, and nodes
+// that draw a member subset for the linking length are searched without one)
 
 // bracket of the search from the sample: the radius R2 is the sample's
 // quantile at f + 5 sigma widened by 16 band widths; the stop value is the
 // quantile at f - 5 sigma narrowed by 16 band widths (a member with a
 // neighbour closer than it is certainly below the linking length)
-__global__ void k_smp_thresh(LevelBufs L, NodeArrays nd, const int64_t *soff, const float *sdnn, double f,
-                             float *R2, float *STOP)
+__global__ void k_smp_thresh(LevelBufs L, NodeArrays nd, const int *smp_at, const float *sdnn, double f, float *R2,
+                             float *STOP)
 {
     __shared__ float v[SMP_MAX];
     const int k = blockIdx.x;
     if (k >= L.K) return;
-    const int64_t a = soff[k];
-    const int S = (int)(soff[k + 1] - a);
-    for (int i = threadIdx.x; i < SMP_MAX; i += blockDim.x) v[i] = i < S ? sdnn[a + i] : INFINITY;
+    const int64_t a = (int64_t)smp_at[k] * SMP_MAX;
+    const int S = SMP_MAX;
+    if (a < 0) {  // not sampled: unbounded search, no early stop
+        if (threadIdx.x == 0) {
+            R2[k] = INFINITY;
+            STOP[k] = 0.f;
+        }
+        return;
+    }
+    for (int i = threadIdx.x; i < SMP_MAX; i += blockDim.x) v[i] = sdnn[a + i];
     __syncthreads();
     for (int kk = 2; kk <= SMP_MAX; kk <<= 1)
         for (int j = kk >> 1; j > 0; j >>= 1) {
@@ -2193,18 +2254,13 @@ __global__ void k_smp_thresh(LevelBufs L, NodeArrays nd, const int64_t *soff, co
             __syncthreads();
         }
     if (threadIdx.x == 0) {
-        if (S == 0) {  // not sampled: unbounded search, no early stop
-            R2[k] = INFINITY;
-            STOP[k] = 0.f;
-        } else {
-            const double sd = 5.0 * sqrt(f * (1.0 - f) / (double)S);
-            long long hi = (long long)ceil(fmin(1.0, f + sd) * (double)S) - 1;
-            long long lo = (long long)ceil(fmax(0.0, f - sd) * (double)S) - 2;
-            hi = hi < 0 ? 0 : (hi >= S ? S - 1 : hi);
-            const float th = v[hi];
-            R2[k] = isinf(th) ? INFINITY : (float)((double)th * (1.0 + 16.0 * RS_BAND));
-            STOP[k] = lo < 0 ? 0.f : (float)((double)v[lo] * (1.0 - 16.0 * RS_BAND));
-        }
+        const double sd = 5.0 * sqrt(f * (1.0 - f) / (double)S);
+        long long hi = (long long)ceil(fmin(1.0, f + sd) * (double)S) - 1;
+        long long lo = (long long)ceil(fmax(0.0, f - sd) * (double)S) - 2;
+        hi = hi < 0 ? 0 : (hi >= S ? S - 1 : hi);
+        const float th = v[hi];
+        R2[k] = isinf(th) ? INFINITY : (float)((double)th * (1.0 + 16.0 * RS_BAND));
+        STOP[k] = lo < 0 ? 0.f : (float)((double)v[lo] * (1.0 - 16.0 * RS_BAND));
     }
 }
 
@@ -2239,26 +2295,6 @@ __global__ void k_bracket_check(LevelBufs L, float *R2, const float *STOP, int *
 // positions depend only on the node's size, so each round is one stable sort
 // of all members by (segment, 16-bit coordinate), the coordinate relative to
 // the node's reference member in units of its dispersion.
-__host__ __device__ __forceinline__ int kd_split(int m)
-{
-    int h = ((m / 2 + 31) / 32) * 32;
-    h = h < 32 ? 32 : h;
-    return h > m - 1 ? m - 1 : h;
-}
-
-// splits until a range of m members is at most `limit`
-__host__ __device__ __forceinline__ int kd_rounds(int64_t m, int limit)
-{
-    int r = 0;
-    while (m > limit) {
-        m = kd_split((int)m);
-        r++;
-    }
-    return r;
-}
-
-constexpr int KD_CTA = 1024;  // ranges of at most this many members finish in one CTA
-
 // 16-bit coordinate of a member on an axis (x, vx, y, vy, z, vz), relative to
 // the node's reference member in units of its dispersion
 __device__ __forceinline__ unsigned kd_coord(const float4 *wpos, const float4 *wvel, unsigned slot, int axis,
@@ -2281,21 +2317,19 @@ __device__ __forceinline__ unsigned kd_coord(const float4 *wpos, const float4 *w
     return (unsigned)fminf(fmaxf(u, 0.f), 65535.f);
 }
 
-// One global round over the nodes still being split (act_off: their members'
-// offsets in the round's compact arrays; equal neighbours mark a node that is
-// done): ranges of more than KD_CTA members at this depth are sorted by the
+// One global round over the nodes still being split (a prefix of the level's
+// tiles and members): ranges of more than KD_CTA members at this depth are sorted by the
 // round's axis; smaller ranges keep their order (value 0).  vcur holds every
 // member's slot in the current order.
-__global__ void k_kd_keys(LevelBufs L, NodeArrays nd, const int64_t *seg_base, const int64_t *act_off,
-                          const float4 *wpos, const float4 *wvel, const unsigned *vcur, unsigned long long *kout,
+__global__ void k_kd_keys(LevelBufs L, NodeArrays nd, const int64_t *seg_base, const float4 *wpos, const float4 *wvel, const unsigned *vcur, unsigned long long *kout,
                           unsigned *vout, int round, int key32)
 {
     const int k = L.tile_rank[blockIdx.x], q0 = L.tile_q0[blockIdx.x];
     const int node = L.list[k], n = nd.count[node];
     const int p = q0 + threadIdx.x;
-    if (p >= n || act_off[k + 1] == act_off[k]) return;
-    const int64_t A = act_off[k] + p;
-    const unsigned slot = vcur[L.seg_off[k] + p];
+    if (p >= n) return;
+    const int64_t A = L.seg_off[k] + p;
+    const unsigned slot = vcur[A];
     int start = 0, size = n;
     for (int i = 0; i < round && size > KD_CTA; i++) {
         const int h = kd_split(size);
@@ -2327,16 +2361,6 @@ __global__ void k_kd_keys(LevelBufs L, NodeArrays nd, const int64_t *seg_base, c
     vout[A] = slot;
 }
 
-// the round's sorted slots back to their nodes' places in the current order
-__global__ void k_kd_back(LevelBufs L, NodeArrays nd, const int64_t *act_off, const unsigned *vs, unsigned *vcur)
-{
-    const int k = L.tile_rank[blockIdx.x], q0 = L.tile_q0[blockIdx.x];
-    const int n = nd.count[L.list[k]];
-    const int p = q0 + threadIdx.x;
-    if (p >= n || act_off[k + 1] == act_off[k]) return;
-    vcur[L.seg_off[k] + p] = vs[act_off[k] + p];
-}
-
 // the current order before the rounds: every member in its own place
 __global__ void k_kd_init(LevelBufs L, NodeArrays nd, unsigned *vcur)
 {
@@ -2346,55 +2370,29 @@ __global__ void k_kd_init(LevelBufs L, NodeArrays nd, unsigned *vcur)
     if (p < n) vcur[L.seg_off[k] + p] = (unsigned)(nd.first[node] + p);
 }
 
-// Nodes still being split in round r (their largest range at depth r, the
-// first, has more than KD_CTA members): blocks of KD_CTA members (the range
-// keys) and members; 0 for the others, which sit the round out.
-__global__ void k_kd_active(const int *list, int K, NodeArrays nd, int round, int64_t *nb, int64_t *na)
+// Ranges of 33 to KD_CTA members left by the global rounds, one entry per
+// range: (rank, start in the node, size, depth).  A thread per 32 members
+// descends the splits to its range and lists it if it holds the first ones
+// (a thread a node, over all its ranges, took up to 1.5 ms a path of 17M).
+__global__ void k_kd_ranges(LevelBufs L, NodeArrays nd, int64_t tiles, int4 *ranges, int *count)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
-    const int n = nd.count[list[k]];
-    const bool act = kd_rounds(n, KD_CTA) > round;
-    nb[k] = act ? ceil_div(n, KD_CTA) : 0;
-    na[k] = act ? n : 0;
-}
-
-// Ranges of at most KD_CTA members left by the global rounds, one entry per
-// range: (rank, start in the node, size, depth).  One thread per node.
-__global__ void k_kd_ranges(LevelBufs L, NodeArrays nd, int4 *ranges, int *count, int cap, rs_dev_status *st)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= L.K) return;
+    const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t tile = u / (TQ / 32);
+    if (tile >= tiles) return;
+    const int k = L.tile_rank[tile], p = L.tile_q0[tile] + 32 * (int)(u % (TQ / 32));
     const int n = nd.count[L.list[k]];
-    int stk_s[32], stk_m[32], stk_d[32];
-    int sp = 0;
-    stk_s[0] = 0;
-    stk_m[0] = n;
-    stk_d[0] = 0;
-    sp = 1;
-    for (int it = 0; sp > 0 && it < (1 << 26); it++) {
-        sp--;
-        const int s0 = stk_s[sp], m = stk_m[sp], d = stk_d[sp];
-        if (m <= KD_CTA) {
-            if (m > 32) {
-                const int slot = atomicAdd(count, 1);
-                if (slot < cap) ranges[slot] = make_int4(k, s0, m, d);
-                else dev_fail(st, DEV_OVERFLOW, 58, slot);
-            }
-            continue;
+    if (p >= n) return;
+    int start = 0, size = n, d = 0;
+    for (; size > KD_CTA; d++) {
+        const int h = kd_split(size);
+        if (p - start < h) {
+            size = h;
+        } else {
+            start += h;
+            size -= h;
         }
-        if (sp + 2 > 32) {
-            dev_fail(st, DEV_OVERFLOW, 59, k);
-            return;
-        }
-        const int h = kd_split(m);
-        stk_s[sp] = s0 + h;
-        stk_m[sp] = m - h;
-        stk_d[sp++] = d + 1;
-        stk_s[sp] = s0;
-        stk_m[sp] = h;
-        stk_d[sp++] = d + 1;
     }
+    if (p == start && size > 32) ranges[atomicAdd(count, 1)] = make_int4(k, start, size, d);
 }
 
 // Finish one range in shared memory: the remaining splits.  Round r orders
@@ -2772,15 +2770,14 @@ __global__ void __launch_bounds__(TQ) k_lvl_band(LevelBufs L, NodeArrays nd, con
     const int k = L.tile_rank[blockIdx.x], q0 = L.tile_q0[blockIdx.x];
     const int node = L.list[k], first = nd.first[node], n = nd.count[node];
     const int q = q0 + threadIdx.x;
-    if (q >= n) return;
     const float t32 = __uint_as_float(L.sel_prefix[k]);
-    const float blo = (float)((double)t32 * (1.0 - 2.0 * RS_BAND));
-    const float bhi = (float)((double)t32 * (1.0 + 2.0 * RS_BAND));
-    const float d = dnn[first + q];
-    if (__float_as_uint(d) >> 31) return;  // outside the subset
-    if (d < blo) {
-        atomicAdd(&L.below[k], 1);
-    } else if (d <= bhi) {
+    // t32 (1 -+ 2 RS_BAND), rounded once: 2 RS_BAND = 2^-19
+    const float blo = fmaf(t32, (float)(-2.0 * RS_BAND), t32), bhi = fmaf(t32, (float)(2.0 * RS_BAND), t32);
+    const float d = q < n ? dnn[first + q] : -1.f;  // (negative: outside the subset)
+    const bool in = !(__float_as_uint(d) >> 31);
+    const unsigned below = __ballot_sync(FULLW, in && d < blo);
+    if (below && lane_id() == 0) atomicAdd(&L.below[k], __popc(below));
+    if (in && d >= blo && d <= bhi) {
         int b = atomicAdd(L.band_len, 1);
         L.band_rank[b] = k;
         L.band_slot[b] = first + q;
@@ -3046,22 +3043,22 @@ size_t tree_bytes(int64_t M, int64_t cap)
 
 // the big-node nearest-neighbour search, compiled for 40, 48 or 56 resident
 // warps per SM (rs_tuning::nn_blocks_per_sm = 5, 6 or 7, in units of eight)
-static rs_status launch_nn(rs_ctx *ctx, const char *name, int64_t W, const LevelBufs &L, const WarpJobs &JF,
-                           const NodeArrays &nd, const int64_t *bo, const BoxStore &boxes, const MemberStore &ms,
-                           const float *R2, const float *STOP, int redo_failed, float *dnn)
+static rs_status launch_nn(rs_ctx *ctx, const char *name, int64_t T, const LevelBufs &L, const NodeArrays &nd,
+                           const int64_t *bo, const BoxStore &boxes, const MemberStore &ms, const float *R2,
+                           const float *STOP, int redo_failed, int sub_n, float *dnn)
 {
-    const int64_t g = ceil_div(W, NN_WARPS);
+    const int64_t g = T * (TQ / 32) / NN_WARPS;
     switch (ctx->tune.nn_blocks_per_sm) {
     case 5:
-        RS_LAUNCH(ctx, name, k_bvh_nn<5>, g, NN_WARPS * 32, 0, L, JF, nd, bo, boxes, ms, R2, STOP, redo_failed, dnn,
+        RS_LAUNCH(ctx, name, k_bvh_nn<5>, g, NN_WARPS * 32, 0, L, nd, bo, boxes, ms, R2, STOP, redo_failed, sub_n, dnn,
                   ctx->d_status);
         break;
     case 7:
-        RS_LAUNCH(ctx, name, k_bvh_nn<7>, g, NN_WARPS * 32, 0, L, JF, nd, bo, boxes, ms, R2, STOP, redo_failed, dnn,
+        RS_LAUNCH(ctx, name, k_bvh_nn<7>, g, NN_WARPS * 32, 0, L, nd, bo, boxes, ms, R2, STOP, redo_failed, sub_n, dnn,
                   ctx->d_status);
         break;
     default:
-        RS_LAUNCH(ctx, name, k_bvh_nn<6>, g, NN_WARPS * 32, 0, L, JF, nd, bo, boxes, ms, R2, STOP, redo_failed, dnn,
+        RS_LAUNCH(ctx, name, k_bvh_nn<6>, g, NN_WARPS * 32, 0, L, nd, bo, boxes, ms, R2, STOP, redo_failed, sub_n, dnn,
                   ctx->d_status);
     }
     return RS_OK;
@@ -3134,9 +3131,9 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
     int *shift_bits = gmisc, *gmin = gmisc + G, *slot_group = gmisc + 2 * G, *gred = gmisc + 2 * G + M;
     // node queues: big lists (ping-pong) and the small queue; counters
     // counters first (16 ints = 64 bytes, so everything after stays 8-byte aligned)
-    RS_WS(ctx, int, q, WS_RF_NODEQ, 6 * cap + 16);
+    RS_WS(ctx, int, q, WS_RF_NODEQ, 7 * cap + 16);
     int *ctr = q, *big_a = q + 16, *big_b = q + 16 + cap, *small_q = q + 16 + 2 * cap, *tiny_q = q + 16 + 3 * cap,
-        *mid_q = q + 16 + 4 * cap, *warp_q = q + 16 + 5 * cap;
+        *mid_q = q + 16 + 4 * cap, *warp_q = q + 16 + 5 * cap, *big_s = q + 16 + 6 * cap;
     // ctr: [0] big_a len, [1] big_b len, [2] small len, [3] small head, [4] band len,
     // [6..7] bracket fallback flag, [8] tiny len, [9] tiny head, [10] k-d ranges,
     // [11] middle len, [12] middle head, [13] subset query list length,
@@ -3161,32 +3158,35 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
     int *cur_len = ctr + 0, *nxt_len = ctr + 1;
     int64_t sum_level = 0;
     int n_fallback_levels = 0;
+    // per-rank offsets: a big node has more than SMALL_N members
+    const int64_t kcap = M / SMALL_N + 2;
+    RS_WS(ctx, int64_t, lv64, WS_RF_MISC1, 5 * kcap + LT_WORDS + 8);
+    LevelOff O;
+    O.tile = lv64;
+    O.seg = lv64 + kcap;
+    O.box = lv64 + 2 * kcap;
+    O.block = lv64 + 3 * kcap;
+    O.smp = (int *)(lv64 + 4 * kcap);
+    O.smp_at = O.smp + kcap;
+    int64_t *dtot = lv64 + 5 * kcap;
     for (int level = 0; level < 4096; level++) {
-        int64_t K;
-        RS_TRY(rs_read_i64(ctx, cur_len, 1, &K, "rs_refine6d"));
-        K &= 0xffffffffll;
+        RS_LAUNCH(ctx, "rf_lvl_setup", k_lvl_setup, 1, 1024, 0, (const int *)cur, (const int *)cur_len, big_s, nd, O,
+                  (int)sub_n, (int)ctx->tune.bracket_min, dtot);
+        int64_t tot[LT_WORDS];
+        static_assert(LT_WORDS <= 64, "the context's host scratch");
+        RS_TRY(rs_read_i64(ctx, dtot, LT_WORDS, tot, "rs_refine6d"));
+        const int64_t K = tot[LT_K], T = tot[LT_T], LM = tot[LT_LM], NBX = tot[LT_NBX];
         if (K == 0) break;
-        RS_WS(ctx, int64_t, lv64, WS_RF_MISC1, 4 * (K + 1) + 8);
-        int64_t *tiles = lv64, *segc = lv64 + (K + 1), *tot = lv64 + 2 * (K + 1);
-        RS_CUDA(ctx, cudaMemsetAsync(tot + 3, 0, sizeof(int64_t), ctx->stream));
-        RS_LAUNCH(ctx, "rf_lvl_prep", k_lvl_prep, ceil_div(K, 256), 256, 0, (const int *)cur, (int)K, nd, tiles,
-                  segc, (unsigned long long *)(tot + 3));
-        RS_CUDA(ctx, cudaMemsetAsync(tiles + K, 0, sizeof(int64_t), ctx->stream));
-        RS_CUDA(ctx, cudaMemsetAsync(segc + K, 0, sizeof(int64_t), ctx->stream));
-        RS_TRY(rs_scan_i64(ctx, tiles, K + 1, tot));
-        RS_TRY(rs_scan_i64(ctx, segc, K + 1, tot + 1));
-        int64_t TT[2];
-        RS_TRY(rs_read_i64(ctx, tot, 2, TT, "rs_refine6d"));
-        const int64_t T = TT[0], LM = TT[1];
         sum_level += LM;
         RS_WS(ctx, int, tl, WS_RF_MISC2, 2 * T + 8);
         LevelBufs L;
-        L.list = cur;
+        L.list = big_s;
         L.K = (int)K;
         L.tile_rank = tl;
         L.tile_q0 = tl + T;
-        L.seg_off = segc;
-        RS_LAUNCH(ctx, "rf_lvl_tiles", k_lvl_tiles, K, 256, 0, (int)K, (const int64_t *)tiles, tl, tl + T);
+        L.seg_off = O.seg;
+        const int64_t *bo = O.box;
+        RS_LAUNCH(ctx, "rf_lvl_tiles", k_lvl_tiles, K, 256, 0, (int)K, (const int64_t *)O.tile, tl, tl + T);
         // per-rank state
         size_t per = sizeof(MomAcc) + sizeof(Metric6) + 2 * sizeof(float4) + 2048 * sizeof(unsigned) +
                      7 * sizeof(int) + sizeof(double) + 64;
@@ -3225,32 +3225,19 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
             // medians (levels 0-2 by default, where most of the search work
             // is); deeper levels keep this order through the stable child
             // partition below
-            int64_t maxn = 0;
-            RS_TRY(rs_read_i64(ctx, tot + 3, 1, &maxn, "rs_refine6d"));
-            RS_WS(ctx, int64_t, kw, WS_RF_MISC5, 2 * (K + 1) + 8);
-            int64_t *kseg = kw, *aoff = kw + (K + 1), *ktot = kw + 2 * (K + 1);
             RS_WS(ctx, unsigned, vcur, WS_RF_KDV, LM);
             RS_LAUNCH(ctx, "rf_kd_init", k_kd_init, T, TQ, 0, L, nd, vcur);
             // each round sorts only the members of the nodes still being
             // split, so a node costs the rounds its own size needs, not the
             // largest node's; the range keys shrink with the active blocks
-            const int R = kd_rounds(maxn, KD_CTA);
-            for (int r = 0; r < R; r++) {
-                RS_LAUNCH(ctx, "rf_kd_active", k_kd_active, ceil_div(K, 256), 256, 0, (const int *)cur, (int)K, nd,
-                          r, kseg, aoff);
-                RS_CUDA(ctx, cudaMemsetAsync(kseg + K, 0, sizeof(int64_t), ctx->stream));
-                RS_CUDA(ctx, cudaMemsetAsync(aoff + K, 0, sizeof(int64_t), ctx->stream));
-                RS_TRY(rs_scan_i64(ctx, kseg, K + 1, ktot));
-                RS_TRY(rs_scan_i64(ctx, aoff, K + 1, ktot + 1));
-                int64_t tots[2];
-                RS_TRY(rs_read_i64(ctx, ktot, 2, tots, "rs_refine6d"));
-                const int64_t NS = tots[0], NA = tots[1];
-                if (NA <= 0) break;
+            for (int r = 0; r < (int)tot[LT_ROUNDS]; r++) {
+                const int64_t TA = tot[LT_ROUND0 + 3 * r], NA = tot[LT_ROUND0 + 3 * r + 1],
+                              NS = tot[LT_ROUND0 + 3 * r + 2];
                 int sbits = 0;
                 while (sbits < 40 && (NS >> sbits) != 0) sbits++;
                 // 32-bit keys (half the bytes, fewer passes) while the blocks fit in 16 bits
                 const int key32 = 16 + sbits <= 32 ? 1 : 0;
-                RS_LAUNCH(ctx, "rf_kd_keys", k_kd_keys, T, TQ, 0, L, nd, (const int64_t *)kseg, (const int64_t *)aoff,
+                RS_LAUNCH(ctx, "rf_kd_keys", k_kd_keys, TA, TQ, 0, L, nd, (const int64_t *)O.block,
                           (const float4 *)wpos, (const float4 *)wvel, (const unsigned *)vcur,
                           (unsigned long long *)k0, v0, r, key32);
                 bool kalt = false;
@@ -3259,16 +3246,16 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
                                              "sort_kd"));
                 else
                     RS_TRY(rs_radix_sort_u64(ctx, k0, k1, v0, v1, NA, 16 + sbits, &kalt, "sort_kd"));
-                RS_LAUNCH(ctx, "rf_kd_back", k_kd_back, T, TQ, 0, L, nd, (const int64_t *)aoff,
-                          (const unsigned *)(kalt ? v1 : v0), vcur);
+                RS_CUDA(ctx, cudaMemcpyAsync(vcur, kalt ? v1 : v0, sizeof(unsigned) * NA, cudaMemcpyDeviceToDevice,
+                                             ctx->stream));
             }
             // ranges of at most KD_CTA members finish in one CTA each
             const int64_t rcap = ceil_div(LM, 32) + K;
             RS_WS(ctx, int4, kranges, WS_RF_JOBS, rcap + 1);
             int *kcount = ctr + 10;
             RS_CUDA(ctx, cudaMemsetAsync(kcount, 0, sizeof(int), ctx->stream));
-            RS_LAUNCH(ctx, "rf_kd_ranges", k_kd_ranges, ceil_div(K, 128), 128, 0, L, nd, kranges, kcount, (int)rcap,
-                      ctx->d_status);
+            RS_LAUNCH(ctx, "rf_kd_ranges", k_kd_ranges, ceil_div(T * (TQ / 32), 256), 256, 0, L, nd, T, kranges,
+                      kcount);
             RS_LAUNCH(ctx, "rf_kd_finish", k_kd_finish, (int64_t)ctx->num_sms * 8, 256, 0, L, nd,
                       (const int4 *)kranges, (const int *)kcount, (const float4 *)wpos, (const float4 *)wvel, vcur);
             const unsigned *vsorted = vcur;
@@ -3282,12 +3269,6 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
             }
         }
         // bounding-volume hierarchy of every big node
-        RS_WS(ctx, int64_t, bo, WS_RF_MISC3, (K + 1) + 8);
-        RS_LAUNCH(ctx, "rf_bvh_prep", k_bvh_prep, ceil_div(K, 256), 256, 0, (const int *)cur, (int)K, nd, bo);
-        RS_CUDA(ctx, cudaMemsetAsync(bo + K, 0, sizeof(int64_t), ctx->stream));
-        RS_TRY(rs_scan_i64(ctx, bo, K + 1, tot + 2));
-        int64_t NBX;
-        RS_TRY(rs_read_i64(ctx, tot + 2, 1, &NBX, "rs_refine6d"));
         RS_WS(ctx, char, boxmem, WS_RF_HIST, NBX * 49 + 1024);
         BoxStore boxes;
         {
@@ -3304,17 +3285,17 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
             ms.a = carve<float4>(sp2, M);
             ms.b = carve<float2>(sp2, M);
         }
-        RS_LAUNCH(ctx, "rf_bvh_leaves", k_bvh_leaves<false>, T, TQ, 0, L, nd, (const int64_t *)bo, boxes, ms,
+        RS_LAUNCH(ctx, "rf_bvh_leaves", k_bvh_leaves<false>, T, TQ, 0, L, nd, bo, boxes, ms,
                   (const float4 *)wpos, (const float4 *)wvel, (const float *)nullptr, (int *)nullptr, (int *)nullptr,
                   (int *)nullptr, ctx->d_status);
-        RS_LAUNCH(ctx, "rf_bvh_build", k_bvh_build<false>, K, 256, 0, L, nd, (const int64_t *)bo, boxes,
+        RS_LAUNCH(ctx, "rf_bvh_build", k_bvh_build<false>, K, 256, 0, L, nd, bo, boxes,
                   (int *)nullptr, ctx->d_status);
         // ---- random member subsets of the nodes above sub_n (Sec. 3.2) ----
         int2 *sub_q = nullptr;
         int *sub_len = ctr + 13;
         int64_t QN = 0, qcap = 0;
         if (sub_n > 0) {
-            qcap = std::min<int64_t>(LM, K * sub_n);
+            QN = qcap = tot[LT_SUB] * sub_n;  // every node above sub_n draws exactly sub_n members
             RS_WS(ctx, int2, sq, WS_RF_SUBQ, qcap + 1);
             sub_q = sq;
             RS_CUDA(ctx, cudaMemsetAsync(sub_len, 0, sizeof(int), ctx->stream));
@@ -3330,55 +3311,23 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
             RS_LAUNCH(ctx, "rf_sub_mark", k_sub_mark, T, TQ, 0, L, nd, (const int *)widx,
                       (unsigned long long)sub_seed, (int)sub_n, dnn, sub_q, sub_len, (int)qcap, ctx->d_status);
             RS_LAUNCH(ctx, "rf_sub_check", k_sub_check, ceil_div(K, 128), 128, 0, L, nd, (int)sub_n, ctx->d_status);
-            RS_TRY(rs_read_i64(ctx, sub_len, 1, &QN, "rs_refine6d"));
-            QN = std::min<int64_t>(QN & 0xffffffffll, qcap);
         }
         // ---- linking length: sampled bracket, bounded nearest neighbours, exact select ----
-        RS_WS(ctx, int64_t, ch, WS_RF_MISC4, 2 * (K + 1) + 8);
-        int64_t *nsm = ch, *stot = ch + (K + 1);
-        RS_LAUNCH(ctx, "rf_smp_prep", k_smp_prep, ceil_div(K, 256), 256, 0, (const int *)cur, (int)K, nd, nsm,
-                  (int)sub_n, (int)ctx->tune.bracket_min);
-        RS_CUDA(ctx, cudaMemsetAsync(nsm + K, 0, sizeof(int64_t), ctx->stream));
-        RS_TRY(rs_scan_i64(ctx, nsm, K + 1, stot));
-        int64_t SS;
-        RS_TRY(rs_read_i64(ctx, stot, 1, &SS, "rs_refine6d"));
+        const int64_t SS = tot[LT_SMP] * SMP_MAX;
         RS_WS(ctx, float, sdnn, WS_RF_SDNN, SS + 32);
         RS_WS(ctx, float, R2, WS_RF_R2, 2 * K + 8);
         float *STOP = R2 + K;
-        if (SS > 0) {
-            dim3 grid((unsigned)ceil_div(SMP_MAX, W_WARPS), (unsigned)K);
-            int pr = rs_prof_begin(ctx, "rf_smp_nn");
-            k_bvh_nn_sample<<<grid, W_WARPS * 32, 0, ctx->stream>>>(L, nd, (const int64_t *)bo, boxes, ms,
-                                                                    (const int64_t *)nsm, sdnn, ctx->d_status);
-            ctx->launches++;
-            rs_prof_end(ctx, pr);
-            RS_CUDA(ctx, cudaGetLastError());
-        }
-        RS_LAUNCH(ctx, "rf_smp_thresh", k_smp_thresh, K, 256, 0, L, nd, (const int64_t *)nsm, (const float *)sdnn, f,
+        RS_LAUNCH(ctx, "rf_smp_nn", k_bvh_nn_sample, SS / W_WARPS, W_WARPS * 32, 0, L, nd, bo, boxes, ms,
+                  (const int *)O.smp, sdnn, ctx->d_status);
+        RS_LAUNCH(ctx, "rf_smp_thresh", k_smp_thresh, K, 256, 0, L, nd, (const int *)O.smp_at, (const float *)sdnn, f,
                   R2, STOP);
         int *fallback = ctr + 7;
         RS_CUDA(ctx, cudaMemsetAsync(ctr + 7, 0, sizeof(int), ctx->stream));
         // every member's nearest-neighbour distance, searched from the radius
-        RS_WS(ctx, int64_t, fw, WS_RF_MISC5, 2 * (K + 1) + 8);
-        int64_t *nw = fw, *wtot = fw + (K + 1);
-        RS_LAUNCH(ctx, "rf_full_prep", k_full_prep, ceil_div(K, 256), 256, 0, (const int *)cur, (int)K, nd, nw,
-                  (int)sub_n);
-        RS_CUDA(ctx, cudaMemsetAsync(nw + K, 0, sizeof(int64_t), ctx->stream));
-        RS_TRY(rs_scan_i64(ctx, nw, K + 1, wtot));
-        int64_t W;
-        RS_TRY(rs_read_i64(ctx, wtot, 1, &W, "rs_refine6d"));
-        RS_WS(ctx, int, jf, WS_RF_JOBS2, 3 * W + 8);
-        WarpJobs JF;
-        JF.rank = jf;
-        JF.q0 = jf + W;
-        JF.out = jf + 2 * W;
-        JF.count = W;
-        RS_LAUNCH(ctx, "rf_full_jobs", k_full_jobs, K, 128, 0, (const int *)cur, (int)K, nd, (const int64_t *)nw, jf,
-                  jf + W, jf + 2 * W);
-        RS_TRY(launch_nn(ctx, "rf_lvl_nn", W, L, JF, nd, bo, boxes, ms, R2, STOP, 0, dnn));
+        RS_TRY(launch_nn(ctx, "rf_lvl_nn", T, L, nd, bo, boxes, ms, R2, STOP, 0, (int)sub_n, dnn));
         if (QN > 0)
             RS_LAUNCH(ctx, "rf_sub_nn", k_bvh_nn_list, ceil_div(QN, W_WARPS), W_WARPS * 32, 0, L, nd,
-                      (const int64_t *)bo, boxes, ms, (const int2 *)sub_q, (const int *)sub_len, (int)qcap, dnn,
+                      bo, boxes, ms, (const int2 *)sub_q, (const int *)sub_len, (int)qcap, dnn,
                       ctx->d_status);
         RS_LAUNCH(ctx, "rf_lvl_initk", k_lvl_initk, ceil_div(K, 128), 128, 0, L, nd, f, (int)sub_n);
         for (int pass = 0; pass < 3; pass++) {
@@ -3387,29 +3336,32 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
         }
         RS_LAUNCH(ctx, "rf_bracket_check", k_bracket_check, ceil_div(K, 128), 128, 0, L, R2,
                   (const float *)STOP, fallback, rs_fault("bracket") ? 1 : 0);
-        int64_t fo;
-        RS_TRY(rs_read_i64(ctx, ctr + 6, 1, &fo, "rs_refine6d"));
-        if ((fo >> 32) != 0) {
-            // the bracket did not hold for some node: unbounded search of
-            // those nodes (the others keep their values and selection)
-            RS_TRY(launch_nn(ctx, "rf_lvl_nn_full", W, L, JF, nd, bo, boxes, ms, R2, nullptr, 1, dnn));
+        RS_LAUNCH(ctx, "rf_lvl_band", k_lvl_band, T, TQ, 0, L, nd, (const float *)dnn);
+        // ctr[4]: band members; ctr[7]: some node's bracket did not hold
+        int64_t flags[2];
+        RS_TRY(rs_read_i64(ctx, ctr + 4, 2, flags, "rs_refine6d"));
+        if ((flags[1] >> 32) != 0) {
+            // unbounded search of those nodes (the others keep their values
+            // and selection), and the band once more
+            RS_TRY(launch_nn(ctx, "rf_lvl_nn_full", T, L, nd, bo, boxes, ms, R2, nullptr, 1, (int)sub_n, dnn));
             RS_LAUNCH(ctx, "rf_lvl_initk", k_lvl_initk, ceil_div(K, 128), 128, 0, L, nd, f, (int)sub_n);
             for (int pass = 0; pass < 3; pass++) {
                 RS_LAUNCH(ctx, "rf_lvl_hist", k_lvl_hist, T, TQ, 0, L, nd, (const float *)dnn, pass);
                 RS_LAUNCH(ctx, "rf_lvl_pick", k_lvl_pick, K, 256, 0, L, pass);
             }
+            RS_CUDA(ctx, cudaMemsetAsync(ctr + 4, 0, sizeof(int), ctx->stream));
+            RS_CUDA(ctx, cudaMemsetAsync(L.below, 0, sizeof(int) * (size_t)K, ctx->stream));
+            RS_LAUNCH(ctx, "rf_lvl_band", k_lvl_band, T, TQ, 0, L, nd, (const float *)dnn);
+            RS_TRY(rs_read_i64(ctx, ctr + 4, 1, flags, "rs_refine6d"));
             n_fallback_levels++;
         }
-        RS_LAUNCH(ctx, "rf_lvl_band", k_lvl_band, T, TQ, 0, L, nd, (const float *)dnn);
-        int64_t NB;
-        RS_TRY(rs_read_i64(ctx, ctr + 4, 1, &NB, "rs_refine6d"));
-        const int nbv = (int)(NB & 0xffffffffll);
+        const int nbv = (int)(flags[0] & 0xffffffffll);
         RS_LAUNCH(ctx, "rf_lvl_band_exact", k_lvl_band_exact, ceil_div(nbv, W_WARPS), W_WARPS * 32, 0, L, nd,
-                  (const int64_t *)bo, boxes, ms, (const float *)dnn, ctx->d_status);
+                  bo, boxes, ms, (const float *)dnn, ctx->d_status);
         RS_LAUNCH(ctx, "rf_lvl_l2", k_lvl_l2, K, 128, 0, L, nd, f, (int)sub_n, ctx->d_status);
-        RS_LAUNCH(ctx, "rf_link_leaves", k_bvh_leaves<true>, T, TQ, 0, L, nd, (const int64_t *)bo, boxes, ms,
+        RS_LAUNCH(ctx, "rf_link_leaves", k_bvh_leaves<true>, T, TQ, 0, L, nd, bo, boxes, ms,
                   (const float4 *)wpos, (const float4 *)wvel, (const float *)dnn, uf, csize, cmin, ctx->d_status);
-        RS_LAUNCH(ctx, "rf_link_build", k_bvh_build<true>, K, 256, 0, L, nd, (const int64_t *)bo, boxes, uf,
+        RS_LAUNCH(ctx, "rf_link_build", k_bvh_build<true>, K, 256, 0, L, nd, bo, boxes, uf,
                   ctx->d_status);
         {
             // one warp per leaf job, LK_WARPS to a block; compiled for 24, 32
@@ -3418,15 +3370,15 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
             const int64_t njobs = T * (TQ / 32), lg = ceil_div(njobs, LK_WARPS);
             switch (ctx->tune.link_blocks_per_sm) {
             case 4:
-                RS_LAUNCH(ctx, "rf_lvl_link", k_bvh_link<24>, lg, LK_WARPS * 32, 0, L, nd, (const int64_t *)bo, boxes,
+                RS_LAUNCH(ctx, "rf_lvl_link", k_bvh_link<24>, lg, LK_WARPS * 32, 0, L, nd, bo, boxes,
                           ms, uf, ctx->d_status);
                 break;
             case 6:
-                RS_LAUNCH(ctx, "rf_lvl_link", k_bvh_link<40>, lg, LK_WARPS * 32, 0, L, nd, (const int64_t *)bo, boxes,
+                RS_LAUNCH(ctx, "rf_lvl_link", k_bvh_link<40>, lg, LK_WARPS * 32, 0, L, nd, bo, boxes,
                           ms, uf, ctx->d_status);
                 break;
             default:
-                RS_LAUNCH(ctx, "rf_lvl_link", k_bvh_link<32>, lg, LK_WARPS * 32, 0, L, nd, (const int64_t *)bo, boxes,
+                RS_LAUNCH(ctx, "rf_lvl_link", k_bvh_link<32>, lg, LK_WARPS * 32, 0, L, nd, bo, boxes,
                           ms, uf, ctx->d_status);
             }
         }
