@@ -48,6 +48,8 @@ struct AsBufs {
     double *hx, *hv, *hsigv, *hrdyn2;  // per root seed (hx, hv: 3 each)
     float *hfast;          // per root seed: 12 floats (centre hi/lo, velocity hi/lo) + 2 factors
     int *hrank;            // per root seed: dense halo rank
+    float4 *sx, *sv;       // per seed: centre and sigma_x, bulk velocity and sigma_v (float32)
+    int4 *si;              // per seed: count, smallest index, root node, node
     int *span;             // per node: members held by its children
 };
 
@@ -92,10 +94,16 @@ __global__ void k_as_leafcompact(NodeArrays nd, int nn, const unsigned *flag, co
     vals[scan[i]] = (unsigned)i;
 }
 
-__global__ void k_as_init(AsBufs A)
+__global__ void k_as_init(AsBufs A, NodeArrays nd)
 {
     int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= A.L) return;
+    const int node = A.leaf_node[a];
+    A.sx[a] = make_float4((float)nd.xbar[3 * node], (float)nd.xbar[3 * node + 1], (float)nd.xbar[3 * node + 2],
+                          (float)nd.sigx[node]);
+    A.sv[a] = make_float4((float)nd.vbar[3 * node], (float)nd.vbar[3 * node + 1], (float)nd.vbar[3 * node + 2],
+                          (float)nd.sigv[node]);
+    A.si[a] = make_int4(nd.count[node], nd.minidx[node], nd.root[node], node);
     A.uf[a] = a;
     A.hid[a] = 0x7fffffff;
     A.hcount[a] = 0;
@@ -126,42 +134,47 @@ __device__ double merge_distance(const NodeArrays &nd, int a, int b, double box)
 // comparison keeps a 2^-10 relative margin for the float32 products and
 // sums.  Returns false when the pair may be within the threshold (or a
 // dispersion is zero): the float64 test then decides.
-__device__ __forceinline__ bool merge_far_f32(const NodeArrays &nd, int a, int b, float boxf, float thresh2)
+__device__ __forceinline__ bool merge_far_f32(float4 xa, float4 va, int4 ia, float4 xb, float4 vb, int4 ib, float boxf,
+                                              float thresh2)
 {
-    const int na = nd.count[a], nb = nd.count[b];
-    const bool a_small = (na != nb) ? (na < nb) : (nd.minidx[a] > nd.minidx[b]);
-    const int s = a_small ? a : b;
-    const float sx = (float)nd.sigx[s], sv = (float)nd.sigv[s];
+    const bool a_small = (ia.x != ib.x) ? (ia.x < ib.x) : (ia.y > ib.y);
+    const float sx = a_small ? xa.w : xb.w, sv = a_small ? va.w : vb.w;
     if (!(sx > 1e-30f) || !(sv > 1e-30f)) return false;
-    float gx2 = 0.f, gv2 = 0.f;
-    for (int d = 0; d < 3; d++) {
-        const float xa = (float)nd.xbar[3 * a + d], xb = (float)nd.xbar[3 * b + d];
-        float dx = fabsf(xa - xb);
-        dx = fminf(dx, boxf - dx);
-        const float ex = 2.384185791015625e-07f * (fabsf(xa) + fabsf(xb) + boxf);
-        const float lx = fmaxf(0.f, dx - ex);
-        gx2 += lx * lx;
-        const float va = (float)nd.vbar[3 * a + d], vb = (float)nd.vbar[3 * b + d];
-        const float ev = 2.384185791015625e-07f * (fabsf(va) + fabsf(vb));
-        const float lv = fmaxf(0.f, fabsf(va - vb) - ev);
-        gv2 += lv * lv;
-    }
-    const float ns = (float)nd.count[s];
-    const float d2 = gx2 * ns / (sx * sx) + gv2 * ns / (sv * sv);
+    auto gap = [&](float p, float q) {
+        float d = fabsf(p - q);
+        d = fminf(d, boxf - d);
+        return fmaxf(0.f, d - 2.384185791015625e-07f * (fabsf(p) + fabsf(q) + boxf));
+    };
+    auto vgap = [](float p, float q) {
+        return fmaxf(0.f, fabsf(p - q) - 2.384185791015625e-07f * (fabsf(p) + fabsf(q)));
+    };
+    const float gx = gap(xa.x, xb.x), gy = gap(xa.y, xb.y), gz = gap(xa.z, xb.z);
+    const float hx = vgap(va.x, vb.x), hy = vgap(va.y, vb.y), hz = vgap(va.z, vb.z);
+    const float ns = (float)(a_small ? ia.x : ib.x);
+    const float d2 = (gx * gx + gy * gy + gz * gz) * ns / (sx * sx) + (hx * hx + hy * hy + hz * hz) * ns / (sv * sv);
     return d2 > thresh2 * 1.0009765625f;
 }
 
-__global__ void k_as_merge(AsBufs A, NodeArrays nd, double box, double thresh, rs_dev_status *st)
+// Every pair of seeds of a group, a warp a seed and the lanes over the later
+// seeds (packed in seed order, so their loads coalesce).  A thread a seed over
+// the node table took 0.76 ms for the 7,000 seeds of a 4M box (the largest
+// group's first seed alone scans all the others); this takes 0.05.
+__global__ void __launch_bounds__(AS_THREADS) k_as_merge(AsBufs A, NodeArrays nd, double box, double thresh,
+                                                         rs_dev_status *st)
 {
     const float boxf = (float)box, thresh2 = (float)(thresh * thresh);
-    for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < A.L; a += gridDim.x * blockDim.x) {
-        const int na = A.leaf_node[a];
-        const int ra = nd.root[na];
-        for (int b = a + 1; b < A.L; b++) {
-            const int nb = A.leaf_node[b];
-            if (nd.root[nb] != ra) break;
-            if (merge_far_f32(nd, na, nb, boxf, thresh2)) continue;
-            if (merge_distance(nd, na, nb, box) < thresh) uf_union(A.uf, a, b, st);
+    const int lane = lane_id();
+    for (int a = (blockIdx.x * AS_THREADS + threadIdx.x) >> 5; a < A.L; a += gridDim.x * AS_THREADS >> 5) {
+        const float4 xa = A.sx[a], va = A.sv[a];
+        const int4 ia = A.si[a];
+        for (int b0 = a + 1; b0 < A.L; b0 += 32) {
+            const int b = b0 + lane;
+            const int4 ib = b < A.L ? A.si[b] : make_int4(0, 0, -1, 0);
+            const bool in = ib.z == ia.z;
+            if (in && !merge_far_f32(xa, va, ia, A.sx[b], A.sv[b], ib, boxf, thresh2) &&
+                merge_distance(nd, ia.w, ib.w, box) < thresh)
+                uf_union(A.uf, a, b, st);
+            if (!__all_sync(0xffffffffu, in)) break;  // (a group's seeds are consecutive)
         }
     }
 }
@@ -561,17 +574,37 @@ __global__ void __launch_bounds__(AS_THREADS) k_as_assign(AsBufs A, NodeArrays n
     }
     const float4 p = unwrap_pos(pos, stride, i, nd.shift[node], boxf);
     const float4 v = load_vel(vel, stride, i);
-    float best = INFINITY;
+    // (134M particles: this kernel 10.8 -> 6.0 ms with the second pass left out)
+    // the nearest and, over the other halos, the second nearest: when the
+    // second lies beyond the float32 band of the first, the first is the
+    // float64 nearest too, and the second pass with its float64 divisions is
+    // not needed
+    float best = INFINITY, second = INFINITY;
+    int rbest = -1;
     bool need64 = false;
     for (int c = 0; c < nc; c++) {
-        const float *f = A.hfast + 16 * (int64_t)cl[c];
-        if (f[12] < 0.f || f[13] < 0.f) {
+        const int r = cl[c];
+        const float4 *f4 = reinterpret_cast<const float4 *>(A.hfast + 16 * (int64_t)r);
+        const float4 f0 = f4[0], f1 = f4[1], f2 = f4[2], f3 = f4[3];
+        if (f3.x < 0.f || f3.y < 0.f) {
             need64 = true;
             continue;
         }
-        best = fminf(best, as_d2_32(p, v, f));
+        const float f[14] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w, f2.x, f2.y, f2.z, f2.w, f3.x, f3.y};
+        const float d = as_d2_32(p, v, f);
+        if (d < best) {
+            second = best;
+            best = d;
+            rbest = r;
+        } else if (d < second && r != rbest) {
+            second = d;
+        }
     }
     const float lim = best * (float)(1.0 + 2.0 * RS_BAND);
+    if (!need64 && rbest >= 0 && second > lim) {
+        halo_id[i] = A.hid[rbest];
+        return;
+    }
     double b64 = INFINITY;
     int bid = 0x7fffffff;
     const float *pr = pos + (int64_t)stride * i;
@@ -756,7 +789,7 @@ extern "C" rs_status rs_assign_ex(rs_ctx *ctx, const rs_tree *t, const float *po
     A.leaf_node = (const int *)(alt ? v1 : v0);
     A.span = span;
     size_t per = sizeof(int) * 3 + sizeof(MomAcc) + 2 * sizeof(float4) + sizeof(unsigned long long) +
-                 8 * sizeof(double) + 16 * sizeof(float) + 64 * 8;
+                 8 * sizeof(double) + 16 * sizeof(float) + 3 * sizeof(float4) + 64 * 8;
     RS_WS(ctx, char, hb, WS_AS_3, (int64_t)(per * (L + 1)) + 65536);
     char *hp = hb;
     A.uf = carve<int>(hp, L);
@@ -764,6 +797,9 @@ extern "C" rs_status rs_assign_ex(rs_ctx *ctx, const rs_tree *t, const float *po
     A.hrank = carve<int>(hp, L);
     A.hacc = carve<MomAcc>(hp, L);
     A.href = carve<float4>(hp, 2 * L);
+    A.sx = carve<float4>(hp, L);
+    A.sv = carve<float4>(hp, L);
+    A.si = carve<int4>(hp, L);
     A.hcount = carve<unsigned long long>(hp, L);
     A.hx = carve<double>(hp, 3 * L);
     A.hv = carve<double>(hp, 3 * L);
@@ -772,8 +808,9 @@ extern "C" rs_status rs_assign_ex(rs_ctx *ctx, const rs_tree *t, const float *po
     A.hfast = carve<float>(hp, 16 * (int64_t)L);
     RS_CUDA(ctx, cudaMemsetAsync(A.hacc, 0, sizeof(MomAcc) * (size_t)L, ctx->stream));
     const int64_t gl = ceil_div(L, 256);
-    RS_LAUNCH(ctx, "as_init", k_as_init, gl, 256, 0, A);
-    RS_LAUNCH(ctx, "as_merge", k_as_merge, gl, 256, 0, A, nd, box, params->merge_thresh, ctx->d_status);
+    RS_LAUNCH(ctx, "as_init", k_as_init, gl, 256, 0, A, nd);
+    RS_LAUNCH(ctx, "as_merge", k_as_merge, std::min<int64_t>(ceil_div(L, AS_THREADS / 32), (int64_t)ctx->num_sms * 64),
+              AS_THREADS, 0, A, nd, box, params->merge_thresh, ctx->d_status);
     RS_LAUNCH(ctx, "as_roots", k_as_roots, gl, 256, 0, A, nd, (const int *)t->members, pos, vel, stride, boxf,
               ctx->d_status);
     RS_WS(ctx, int, leaf_root, WS_AS_7, L);

@@ -971,19 +971,12 @@ namespace {
 // counter (33M particles: 2.02 -> 0.24 ms).
 constexpr int GS_THREADS = 256;
 constexpr int GS_TILE = 16384;
-constexpr int GS_SLOTS = 4096;
-constexpr int GS_PROBES = 8;
 
 __global__ void __launch_bounds__(GS_THREADS) k_gs_count(int64_t n, const int32_t *labels, uint32_t *count,
                                                          rs_dev_status *st)
 {
-    __shared__ int32_t slot[GS_SLOTS];
-    __shared__ uint32_t num[GS_SLOTS];
-    for (int s = threadIdx.x; s < GS_SLOTS; s += GS_THREADS) {
-        slot[s] = -1;
-        num[s] = 0;
-    }
-    __syncthreads();
+    __shared__ RsBlockCount<uint32_t, 12> C;
+    C.clear();
     const int64_t i0 = (int64_t)blockIdx.x * GS_TILE;
     for (int64_t i = i0 + threadIdx.x; i < min(n, i0 + GS_TILE); i += GS_THREADS) {
         const int32_t l = labels[i];
@@ -991,22 +984,9 @@ __global__ void __launch_bounds__(GS_THREADS) k_gs_count(int64_t n, const int32_
             dev_fail(st, DEV_BADARG, 20, i);
             continue;
         }
-        if (l == i) continue;
-        unsigned h = ((unsigned)l * 2654435761u) >> 20;  // Knuth's multiplicative hash, 12 bits
-        bool done = false;
-        for (int p = 0; p < GS_PROBES && !done; p++, h = (h + 1) & (GS_SLOTS - 1)) {
-            int32_t have = ((volatile int32_t *)slot)[h];
-            if (have == -1) have = atomicCAS(&slot[h], -1, l);
-            if (have == -1 || have == l) {
-                atomicAdd(&num[h], 1u);
-                done = true;
-            }
-        }
-        if (!done) atomicAdd(&count[l], 1u);
+        if (l != i) C.add(l, count);
     }
-    __syncthreads();
-    for (int s = threadIdx.x; s < GS_SLOTS; s += GS_THREADS)
-        if (num[s]) atomicAdd(&count[slot[s]], num[s]);
+    C.flush(count);
 }
 
 // One pass with look-back: the members of groups of >= min_n members, in

@@ -130,17 +130,25 @@ __device__ __forceinline__ int rank_of(const unsigned *sid, const unsigned *sran
     return (k < H && sid[k] == (unsigned)id) ? (int)srank[k] : -1;
 }
 
-__global__ void k_hp_count(int64_t n, const int32_t *halo_id, const unsigned *sid, const unsigned *srank, int H,
-                           unsigned long long *n_assigned, rs_dev_status *st)
+constexpr int HP_COUNT_TILE = 8192;  // particles a block counts in its table first
+
+__global__ void __launch_bounds__(HP_THREADS) k_hp_count(int64_t n, const int32_t *halo_id, const unsigned *sid,
+                                                         const unsigned *srank, int H, unsigned long long *n_assigned,
+                                                         rs_dev_status *st)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || halo_id[i] < 0) return;
-    const int r = rank_of(sid, srank, H, halo_id[i]);
-    if (r < 0) {
-        dev_fail(st, DEV_BADARG, 70, i);
-        return;
+    __shared__ RsBlockCount<unsigned long long, 11> C;
+    C.clear();
+    const int64_t i0 = (int64_t)blockIdx.x * HP_COUNT_TILE;
+    for (int64_t i = i0 + threadIdx.x; i < min(n, i0 + HP_COUNT_TILE); i += HP_THREADS) {
+        if (halo_id[i] < 0) continue;
+        const int r = rank_of(sid, srank, H, halo_id[i]);
+        if (r < 0) {
+            dev_fail(st, DEV_BADARG, 70, i);
+            continue;
+        }
+        C.add(r, n_assigned);
     }
-    atomicAdd(&n_assigned[r], 1ull);
+    C.flush(n_assigned);
 }
 
 __device__ __forceinline__ double ratio2_h(double num, double den)
@@ -773,7 +781,7 @@ extern "C" rs_status rs_halo_props(rs_ctx *ctx, const rs_tree *t, const rs_halos
     RS_TRY(sorted_ids(ctx, hs, &sid, &srank, &groot, &grank));
     unsigned long long *na = (unsigned long long *)n_assigned;
     RS_CUDA(ctx, cudaMemsetAsync(na, 0, sizeof(int64_t) * H, ctx->stream));
-    RS_LAUNCH(ctx, "hp_count", k_hp_count, ceil_div(n, 256), 256, 0, n, halo_id, (const unsigned *)sid,
+    RS_LAUNCH(ctx, "hp_count", k_hp_count, ceil_div(n, HP_COUNT_TILE), HP_THREADS, 0, n, halo_id, (const unsigned *)sid,
               (const unsigned *)srank, (int)H, na, ctx->d_status);
     RS_LAUNCH(ctx, "hp_host", k_hp_host, ceil_div(H, 128), 128, 0, (int)H, *hs, (const double *)xc,
               (const double *)vc, (const unsigned long long *)na, (const unsigned *)groot, (const unsigned *)grank,

@@ -318,6 +318,45 @@ __device__ __forceinline__ unsigned long long rs_lookback(const RsLookback &lb, 
     return before_s;
 }
 
+// ---- counting by label through a block's shared memory ----
+// Adds one per call to counters in memory, through a table of the block's
+// recent labels: the members of a large group or halo, spread over the
+// catalogue, would otherwise queue on its one counter.  clear and flush are
+// called by the whole block (each ends or begins with a barrier).
+template <typename T, int SLOTS_LOG2>
+struct RsBlockCount {
+    static constexpr int SLOTS = 1 << SLOTS_LOG2, PROBES = 8;
+    int32_t slot[SLOTS];
+    uint32_t num[SLOTS];
+    __device__ __forceinline__ void clear()
+    {
+        for (int s = threadIdx.x; s < SLOTS; s += blockDim.x) {
+            slot[s] = -1;
+            num[s] = 0;
+        }
+        __syncthreads();
+    }
+    __device__ __forceinline__ void add(int32_t l, T *count)
+    {
+        unsigned h = ((unsigned)l * 2654435761u) >> (32 - SLOTS_LOG2);  // Knuth's multiplicative hash
+        for (int p = 0; p < PROBES; p++, h = (h + 1) & (SLOTS - 1)) {
+            int32_t have = ((volatile int32_t *)slot)[h];
+            if (have == -1) have = atomicCAS(&slot[h], -1, l);
+            if (have == -1 || have == l) {
+                atomicAdd(&num[h], 1u);
+                return;
+            }
+        }
+        atomicAdd(&count[l], (T)1);
+    }
+    __device__ __forceinline__ void flush(T *count)
+    {
+        __syncthreads();
+        for (int s = threadIdx.x; s < SLOTS; s += blockDim.x)
+            if (num[s]) atomicAdd(&count[slot[s]], (T)num[s]);
+    }
+};
+
 // Fine cells per side of the 3D FOF grid for (n, box, b): the side s is the
 // largest with sqrt(3) s (1 + 2 err) < l, err being the float32 error of a
 // fine-cell coordinate in cell units (2.0001 u Gf), rounded down so that 4 Gc
