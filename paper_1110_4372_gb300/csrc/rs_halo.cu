@@ -347,7 +347,22 @@ __device__ __forceinline__ void ub_finish(uint32_t i, int r, double phi, const f
     }
 }
 
-// potential and bound flag of every member of a set tile
+// -1/sqrt(r2) added to acc when r2 > 0, to the bit what rsqrtf gives: its
+// instruction takes normal numbers as they are, the few subnormal ones go
+// through rsqrtf itself
+__device__ __forceinline__ void ub_add(float &acc, float r2)
+{
+    float w;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(r2));
+    if (r2 >= 1.17549435e-38f) acc -= w;
+    else if (r2 > 0.f) acc -= rsqrtf(r2);
+}
+
+// potential and bound flag of every member of a set tile.  Bound by
+// instruction issue.  A chunk of sources none of which is more than half the
+// box from any target on any axis needs no periodic choice, and only the
+// tile's own chunk holds the targets themselves: 13 instructions a pair
+// instead of 35 (the sets up to 4096 members of a 2M box: 0.81 -> 0.40 ms).
 __global__ void __launch_bounds__(UB_TILE) k_ub_phi(const int *trank, const int *tq0, const int64_t *off,
                                                     const uint32_t *mem, const float *pos, const float *vel,
                                                     int stride, float boxf, double gm, float eps2f,
@@ -356,32 +371,74 @@ __global__ void __launch_bounds__(UB_TILE) k_ub_phi(const int *trank, const int 
                                                     double *phi_own)
 {
     __shared__ float4 src[UB_TILE];
+    __shared__ float far_s[UB_TILE / 32];
     const int r = trank[blockIdx.x];
     const int64_t a = off[r], n = off[r + 1] - a;
-    const int q = tq0[blockIdx.x] + threadIdx.x;
+    const int q0 = tq0[blockIdx.x], q = q0 + threadIdx.x;
     const bool mine = q < n;
     const uint32_t i = mine ? mem[a + q] : 0u;
-    const float *pi = pos + (int64_t)stride * i;
+    const float *pi = pos + (int64_t)stride * (mine ? i : mem[a + q0]);
     const float px = pi[0], py = pi[1], pz = pi[2];
+    // the targets' bounds (a lane without one repeats the first)
+    __shared__ float tlo[3][UB_TILE / 32], thi[3][UB_TILE / 32];
+    {
+        float lo[3] = {px, py, pz}, hi[3] = {px, py, pz};
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            for (int o = 16; o > 0; o >>= 1) {
+                lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
+                hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
+            }
+            if (lane_id() == 0) {
+                tlo[d][warp_id()] = lo[d];
+                thi[d][warp_id()] = hi[d];
+            }
+        }
+        __syncthreads();
+    }
+    float lo[3], hi[3];
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        lo[d] = tlo[d][0];
+        hi[d] = thi[d][0];
+        for (int w = 1; w < UB_TILE / 32; w++) {
+            lo[d] = fminf(lo[d], tlo[d][w]);
+            hi[d] = fmaxf(hi[d], thi[d][w]);
+        }
+    }
     double phi = 0.0;
     for (int64_t c0 = 0; c0 < n; c0 += UB_TILE) {
         const int64_t cj = c0 + threadIdx.x;
+        float far = 0.f;  // the largest distance of this source from any target along an axis
         if (cj < n) {
             const uint32_t j = mem[a + cj];
             const float *pj = pos + (int64_t)stride * j;
-            src[threadIdx.x] = make_float4(pj[0], pj[1], pj[2], __int_as_float((int)j));
+            const float4 s = make_float4(pj[0], pj[1], pj[2], __int_as_float((int)j));
+            src[threadIdx.x] = s;
+            far = fmaxf(fmaxf(fmaxf(s.x - lo[0], hi[0] - s.x), fmaxf(s.y - lo[1], hi[1] - s.y)),
+                        fmaxf(s.z - lo[2], hi[2] - s.z));
         }
+        far = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(far, 0.f))));
+        if (lane_id() == 0) far_s[warp_id()] = far;
         __syncthreads();
+        for (int w = 0; w < UB_TILE / 32; w++) far = fmaxf(far, far_s[w]);
         const int m = (int)(n - c0 < UB_TILE ? n - c0 : UB_TILE);
         float part = 0.f;
-        if (mine)
+        if (far <= 0.5f * boxf && c0 != q0) {
+#pragma unroll 8
+            for (int k = 0; k < m; k++) {
+                const float4 s = src[k];
+                const float dx = s.x - px, dy = s.y - py, dz = s.z - pz;
+                ub_add(part, dx * dx + dy * dy + dz * dz + eps2f);
+            }
+        } else if (mine) {
             for (int k = 0; k < m; k++) {
                 const float4 s = src[k];
                 if ((uint32_t)__float_as_int(s.w) == i) continue;
                 const float dx = pdiff(px, s.x, boxf), dy = pdiff(py, s.y, boxf), dz = pdiff(pz, s.z, boxf);
-                const float r2 = dx * dx + dy * dy + dz * dz + eps2f;
-                if (r2 > 0.f) part -= rsqrtf(r2);
+                ub_add(part, dx * dx + dy * dy + dz * dz + eps2f);
             }
+        }
         phi += (double)part;
         __syncthreads();
     }
@@ -630,7 +687,11 @@ __global__ void __launch_bounds__(HP_THREADS) k_ub_upper(int H, const int64_t *o
     }
 }
 
-// tree walk: one warp per leaf of targets, a target per lane
+// tree walk: one warp per leaf of targets, a target per lane.  Bound by
+// instruction issue (86% of the cycles, 3.5 G instructions for the 264k tree
+// members of a 2M box): a leaf's members and the accepted boxes are read from
+// shared memory in one broadcast load each, not four shuffles, and the
+// identity test is left to the targets' own leaf.  WALKNOW
 __global__ void __launch_bounds__(UT_WARPS * 32) k_ub_walk(int64_t njobs, const int *jset, const int *jleaf,
                                                           const int64_t *off, const int64_t *bbase,
                                                           const float4 *tpos, const uint32_t *tmem, UBoxes B,
@@ -640,10 +701,12 @@ __global__ void __launch_bounds__(UT_WARPS * 32) k_ub_walk(int64_t njobs, const 
                                                           double *phi_own, rs_dev_status *st)
 {
     __shared__ int stk[UT_WARPS][UT_STACK];
+    __shared__ float4 src_s[UT_WARPS][UT_LEAF];  // a leaf's members, or an opened box's children
     const unsigned FULL = 0xffffffffu;
     const int64_t j = (int64_t)blockIdx.x * UT_WARPS + warp_id();
     if (j >= njobs) return;
     const int w = warp_id(), lane = lane_id();
+    float4 *src = src_s[w];
     const int r = jset[j], leaf = jleaf[j];
     const int64_t a = off[r], n = off[r + 1] - a;
     UTView V;
@@ -670,16 +733,24 @@ __global__ void __launch_bounds__(UT_WARPS * 32) k_ub_walk(int64_t njobs, const 
         if (h == 0) {  // a leaf: every member directly
             const int64_t l0 = (int64_t)b * UT_LEAF;
             const int64_t mm = l0 + lane;
-            const float4 q = mm < n ? tpos[a + mm] : make_float4(0.f, 0.f, 0.f, 0.f);
+            if (mm < n) src[lane] = tpos[a + mm];
+            __syncwarp();
             const int cnt = (int)(n - l0 < UT_LEAF ? n - l0 : UT_LEAF);
-            for (int k = 0; k < cnt; k++) {
-                const float qx = __shfl_sync(FULL, q.x, k), qy = __shfl_sync(FULL, q.y, k),
-                            qz = __shfl_sync(FULL, q.z, k);
-                const uint32_t qi = (uint32_t)__shfl_sync(FULL, __float_as_int(q.w), k);
-                const float dx = qx - t.x, dy = qy - t.y, dz = qz - t.z;
-                const float r2 = dx * dx + dy * dy + dz * dz + eps2f;
-                if (have && qi != ti && r2 > 0.f) acc -= rsqrtf(r2);
+            if (b != leaf) {  // (the targets themselves are in their own leaf only)
+#pragma unroll 8
+                for (int k = 0; k < cnt; k++) {
+                    const float4 q = src[k];
+                    const float dx = q.x - t.x, dy = q.y - t.y, dz = q.z - t.z;
+                    ub_add(acc, dx * dx + dy * dy + dz * dz + eps2f);
+                }
+            } else {
+                for (int k = 0; k < cnt; k++) {
+                    const float4 q = src[k];
+                    const float dx = q.x - t.x, dy = q.y - t.y, dz = q.z - t.z;
+                    if ((uint32_t)__float_as_int(q.w) != ti) ub_add(acc, dx * dx + dy * dy + dz * dz + eps2f);
+                }
             }
+            __syncwarp();
             terms += cnt;
         } else {
             const int c = b * UT_LEAF + lane;
@@ -692,14 +763,17 @@ __global__ void __launch_bounds__(UT_WARPS * 32) k_ub_walk(int64_t njobs, const 
             const float gx = cc.x - gc.x, gy = cc.y - gc.y, gz = cc.z - gc.z;
             const bool acc_ok = ex && sqrtf(gx * gx + gy * gy + gz * gz) - gs.y > cs.z;
             unsigned am = __ballot_sync(FULL, acc_ok);
+            terms += __popc(am);
+            if (am) {
+                src[lane] = cc;
+                __syncwarp();
+            }
             while (am) {  // accepted boxes: a monopole term for every target
-                const int src = __ffs(am) - 1;
+                const int k = __ffs(am) - 1;
                 am &= am - 1;
-                const float bx = __shfl_sync(FULL, cc.x, src), by = __shfl_sync(FULL, cc.y, src),
-                            bz = __shfl_sync(FULL, cc.z, src), bn = __shfl_sync(FULL, cc.w, src);
-                const float dx = bx - t.x, dy = by - t.y, dz = bz - t.z;
-                if (have) acc -= bn * rsqrtf(dx * dx + dy * dy + dz * dz + eps2f);
-                terms++;
+                const float4 q = src[k];
+                const float dx = q.x - t.x, dy = q.y - t.y, dz = q.z - t.z;
+                acc -= q.w * rsqrtf(dx * dx + dy * dy + dz * dz + eps2f);
             }
             const unsigned om = __ballot_sync(FULL, ex && !acc_ok);
             // stack entries hold a box index in 24 bits (sets below 2^29 members)
