@@ -762,19 +762,13 @@ extern "C" rs_status rs_assign_ex(rs_ctx *ctx, const rs_tree *t, const float *po
     }
     // seeds
     RS_WS(ctx, unsigned, fl, WS_AS_0, 2 * (int64_t)nn + 8);
-    unsigned *flag = fl, *scan = fl + nn, *tot = fl + 2 * nn;
+    unsigned *flag = fl, *scan = fl + nn;
     RS_WS(ctx, int, span, WS_AS_1, nn);
     RS_LAUNCH(ctx, "as_leafflag", k_as_leafflag, ceil_div(nn, 256), 256, 0, nd, nn, flag, span);
     RS_LAUNCH(ctx, "as_span", k_as_span, ceil_div(nn, 256), 256, 0, nd, nn, span);
     RS_CUDA(ctx, cudaMemcpyAsync(scan, flag, sizeof(unsigned) * nn, cudaMemcpyDeviceToDevice, ctx->stream));
-    RS_TRY(rs_scan_u32(ctx, scan, nn, tot));
-    int64_t Lh;
-    {
-        RS_CUDA(ctx, cudaMemcpyAsync(ctx->h_scratch, tot, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream));
-        RS_TRY(rs_sync_check(ctx, "rs_assign"));
-        Lh = (int64_t)(*(unsigned *)ctx->h_scratch);
-    }
-    const int L = (int)Lh;
+    RS_TRY(rs_scan_u32(ctx, scan, nn, nullptr));
+    const int L = (int)t->n_seeds;
     RS_WS(ctx, unsigned, lk, WS_AS_2, 4 * (int64_t)L + 8);
     unsigned *k0 = lk, *k1 = lk + L, *v0 = lk + 2 * L, *v1 = lk + 3 * L;
     RS_LAUNCH(ctx, "as_leafcompact", k_as_leafcompact, ceil_div(nn, 256), 256, 0, nd, nn, (const unsigned *)flag,
@@ -834,10 +828,9 @@ extern "C" rs_status rs_assign_ex(rs_ctx *ctx, const rs_tree *t, const float *po
     RS_CUDA(ctx, cudaMemsetAsync(ho, 0, sizeof(unsigned long long) * (2 * (H + 1)), ctx->stream));
     RS_LAUNCH(ctx, "as_hrank", k_as_hrank, gl, 256, 0, A, (const unsigned *)rootflag, (const unsigned *)rscan, hoff);
     RS_TRY(rs_scan_i64(ctx, (int64_t *)hoff, H + 1, nullptr));
-    int64_t hm_total;
-    RS_TRY(rs_read_i64(ctx, hoff + H, 1, &hm_total, "rs_assign"));
-    RS_WS(ctx, int, hm, WS_AS_6, hm_total + H + 8);
-    int *hmem = hm, *root_of_rank = hm + hm_total;
+    // the seeds' members, at most all
+    RS_WS(ctx, int, hm, WS_AS_6, t->n_members + H + 8);
+    int *hmem = hm, *root_of_rank = hm + t->n_members;
     RS_LAUNCH(ctx, "as_root_of_rank", k_as_root_of_rank, gl, 256, 0, A, root_of_rank);
     RS_LAUNCH(ctx, "as_hmembers", k_as_hmembers, gblk, AS_THREADS, 0, A, nd, (const unsigned long long *)hoff, hfill,
               hmem, ctx->d_status);
@@ -852,11 +845,6 @@ extern "C" rs_status rs_assign_ex(rs_ctx *ctx, const rs_tree *t, const float *po
     RS_LAUNCH(ctx, "as_tiles_prep", k_as_tiles_prep, ceil_div(nn, 256), 256, 0, nd, nn, (const int *)span, tl);
     RS_CUDA(ctx, cudaMemsetAsync(tl + nn, 0, sizeof(int64_t), ctx->stream));
     RS_TRY(rs_scan_i64(ctx, tl, nn + 1, tl + nn + 2));
-    int64_t T;
-    RS_TRY(rs_read_i64(ctx, tl + nn, 1, &T, "rs_assign"));
-    RS_WS(ctx, int, tt, WS_RF_MISC2, 2 * T + 8);
-    RS_LAUNCH(ctx, "as_tiles_fill", k_as_tiles_fill, std::min<int64_t>(nn, 65535), 128, 0, nn, (const int64_t *)tl, tt,
-              tt + T);
     // distinct candidate halos of every node, once per node
     RS_WS(ctx, int64_t, cw, WS_AS_8, 2 * (int64_t)nn + 8);
     int64_t *coff = cw;
@@ -864,8 +852,13 @@ extern "C" rs_status rs_assign_ex(rs_ctx *ctx, const rs_tree *t, const float *po
     RS_LAUNCH(ctx, "as_nl", k_as_nl, ceil_div(nn, 256), 256, 0, A, nd, (int)nn, node_la, coff);
     RS_CUDA(ctx, cudaMemsetAsync(coff + nn, 0, sizeof(int64_t), ctx->stream));
     RS_TRY(rs_scan_i64(ctx, coff, nn + 1, coff + nn + 2));
-    int64_t CT;
-    RS_TRY(rs_read_i64(ctx, coff + nn, 1, &CT, "rs_assign"));
+    RS_CUDA(ctx, cudaMemcpyAsync(ctx->h_scratch + 1, coff + nn, sizeof(int64_t), cudaMemcpyDeviceToHost, ctx->stream));
+    int64_t T;
+    RS_TRY(rs_read_i64(ctx, tl + nn, 1, &T, "rs_assign"));
+    const int64_t CT = ctx->h_scratch[1];
+    RS_WS(ctx, int, tt, WS_RF_MISC2, 2 * T + 8);
+    RS_LAUNCH(ctx, "as_tiles_fill", k_as_tiles_fill, std::min<int64_t>(nn, 65535), 128, 0, nn, (const int64_t *)tl, tt,
+              tt + T);
     RS_WS(ctx, int, cand_g, WS_AS_9, CT + 8);
     RS_LAUNCH(ctx, "as_cand", k_as_cand, T, AS_THREADS, 0, A, nd, (const int *)leaf_root, (const int *)tt,
               (const int *)(tt + T), (const int *)node_la, (const int64_t *)coff, cand_g, ncand);
@@ -878,7 +871,7 @@ extern "C" rs_status rs_assign_ex(rs_ctx *ctx, const rs_tree *t, const float *po
         hs->n_halos = H;
         hs->n_nodes = nn;
         const size_t bytes = (size_t)(H + 1) * (4 + 48 + 8 + 8 + 4) + (size_t)(nn + 1) * 4 + 8 * 256;
-        if (cudaMalloc(&hs->block, bytes) != cudaSuccess) {
+        if (rs_block_alloc(ctx, &hs->block, bytes) != cudaSuccess) {
             cudaGetLastError();
             delete hs;
             return rs_fail(ctx, RS_ERR_OOM, "rs_assign: halo table allocation failed");
@@ -915,7 +908,7 @@ extern "C" rs_status rs_assign(rs_ctx *ctx, const rs_tree *t, const float *pos, 
 extern "C" void rs_halos_free(rs_halos *h)
 {
     if (!h) return;
-    if (h->block) cudaFree(h->block);
+    rs_block_free(h->block);
     delete h;
 }
 

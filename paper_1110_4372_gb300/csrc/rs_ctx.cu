@@ -146,6 +146,7 @@ extern "C" void rs_destroy(rs_ctx *c)
     cudaStreamSynchronize(c->stream);
     for (int i = 0; i < WS_NUM_SLOTS; i++)
         if (c->ws_ptr[i]) cudaFree(c->ws_ptr[i]);
+    if (c->pool) cudaMemPoolDestroy(c->pool);
     if (c->d_status) cudaFree(c->d_status);
     if (c->h_status) cudaFreeHost(c->h_status);
     if (c->h_scratch) cudaFreeHost(c->h_scratch);
@@ -192,18 +193,25 @@ bool rs_fault(const char *site)
 }
 
 // Frees the 3D FOF and group-sort slots whose call is not running (their
-// contents are scratch of that call); true if anything was freed.
+// contents are scratch of that call) and the pool's free memory; true if
+// anything was freed.
 static bool release_idle_slots(rs_ctx *c, int keep)
 {
     bool freed = false;
+    if (c->pool) {  // and what the pool keeps free
+        uint64_t before = 0, after = 0;
+        cudaStreamSynchronize(c->stream);
+        cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrReservedMemCurrent, &before);
+        cudaMemPoolTrimTo(c->pool, 0);
+        cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrReservedMemCurrent, &after);
+        freed = after < before;
+    }
     for (int s = 0; s < WS_NUM_SLOTS; s++) {
         const bool fof = s >= WS_FOF_CELLKEY && s <= WS_FOF_ACC;
         const bool gs = s == WS_GS_COUNT || s == WS_GS_FLAG;
         if (s == keep || !c->ws_ptr[s] || !((fof && !c->in_fof) || (gs && !c->in_gs))) continue;
-        if (!freed) {
-            cudaStreamSynchronize(c->stream);
-            if (c->aux) cudaStreamSynchronize(c->aux);
-        }
+        cudaStreamSynchronize(c->stream);
+        if (c->aux) cudaStreamSynchronize(c->aux);
         cudaFree(c->ws_ptr[s]);
         c->ws_ptr[s] = nullptr;
         c->ws_size[s] = 0;
@@ -217,6 +225,37 @@ size_t rs_ws_total(const rs_ctx *c)
     size_t t = 0;
     for (int s = 0; s < WS_NUM_SLOTS; s++) t += c->ws_size[s];
     return t;
+}
+
+cudaError_t rs_block_alloc(rs_ctx *c, void **p, size_t bytes)
+{
+    *p = nullptr;
+    if (!c->pool) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = c->device;
+        const cudaError_t e = cudaMemPoolCreate(&c->pool, &props);
+        if (e != cudaSuccess) {
+            c->pool = nullptr;
+            return e;
+        }
+        uint64_t keep = RS_POOL_KEEP;
+        cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    }
+    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, c->pool, c->stream);
+    if (e == cudaErrorMemoryAllocation && release_idle_slots(c, -1)) {
+        cudaGetLastError();
+        e = cudaMallocFromPoolAsync(p, bytes, c->pool, c->stream);
+    }
+    return e;
+}
+
+void rs_block_free(void *p)
+{
+    if (!p) return;
+    cudaDeviceSynchronize();  // cudaFree does not wait for a pool's block
+    cudaFree(p);
 }
 
 void *rs_ws(rs_ctx *c, int slot, size_t bytes)

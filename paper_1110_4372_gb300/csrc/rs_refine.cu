@@ -2988,9 +2988,11 @@ __global__ void k_lvl_store_tie(LevelBufs L, NodeArrays nd)
     nd.tie[L.list[k]] = L.tie[k];
 }
 
-__global__ void k_tree_stats(NodeArrays nd, int n_nodes, unsigned long long *out)
+__global__ void k_tree_stats(NodeArrays nd, unsigned long long *out)
 {
-    // out: [0] seeds, [1] tie sum, [2] max level, [3] sum of counts
+    // out: [0] nodes, [1] seeds, [2] tie sum, [3] max level, [4] sum of counts
+    const int n_nodes = min(*nd.counter, nd.cap);
+    if (blockIdx.x == 0 && threadIdx.x == 0) out[0] = (unsigned long long)*nd.counter;
     unsigned long long seeds = 0, tie = 0, sum = 0;
     int maxl = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_nodes; i += gridDim.x * blockDim.x) {
@@ -3008,10 +3010,10 @@ __global__ void k_tree_stats(NodeArrays nd, int n_nodes, unsigned long long *out
     sum = warp_sum(sum);
     maxl = warp_max(maxl);
     if (lane_id() == 0) {
-        atomicAdd(&out[0], seeds);
-        atomicAdd(&out[1], tie);
-        atomicMax(&out[2], (unsigned long long)maxl);
-        atomicAdd(&out[3], sum);
+        atomicAdd(&out[1], seeds);
+        atomicAdd(&out[2], tie);
+        atomicMax(&out[3], (unsigned long long)maxl);
+        atomicAdd(&out[4], sum);
     }
 }
 
@@ -3068,25 +3070,16 @@ static rs_status launch_nn(rs_ctx *ctx, const char *name, int64_t T, const Level
 // host driver
 // ---------------------------------------------------------------------------
 static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, int32_t stride, int64_t n, double box,
-                             const int32_t *perm, const int64_t *goff, int64_t G, double f, int32_t min_n,
+                             const int32_t *perm, const int64_t *goff, int64_t G, int64_t M, double f, int32_t min_n,
                              int64_t sub_n, uint64_t sub_seed, int64_t node_cap, rs_tree **out)
 {
-    int64_t h[2];
-    RS_TRY(rs_read_i64(ctx, goff, 1, h, "rs_refine6d"));
-    RS_CUDA(ctx, cudaMemcpyAsync(ctx->h_scratch + 1, goff + G, sizeof(int64_t), cudaMemcpyDeviceToHost, ctx->stream));
-    RS_TRY(rs_sync_check(ctx, "rs_refine6d"));
-    const int64_t M = ctx->h_scratch[1] - h[0];
-    if (M < 0 || M > n || h[0] < 0) return rs_fail(ctx, RS_ERR_INVALID_ARG, "rs_refine6d: inconsistent group offsets");
-    RS_LAUNCH(ctx, "rf_check_offsets", k_check_offsets, ceil_div(G, 256), 256, 0, G, goff, ctx->d_status);
-    RS_TRY(rs_sync_check(ctx, "rs_refine6d: group offsets must be non-decreasing"));
-
     rs_tree *t = new (std::nothrow) rs_tree();
     if (!t) return RS_ERR_OOM;
     t->n_total = n;
     t->n_members = M;
     t->box = box;
     const int64_t cap = node_cap;
-    cudaError_t e = cudaMalloc(&t->block, tree_bytes(M, cap));
+    cudaError_t e = rs_block_alloc(ctx, &t->block, tree_bytes(M, cap));
     if (e != cudaSuccess) {
         delete t;
         cudaGetLastError();
@@ -3438,16 +3431,14 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
     }
 
     // ---- summary ----
-    RS_WS(ctx, unsigned long long, so, WS_RF_MISC3, 4);
-    RS_CUDA(ctx, cudaMemsetAsync(so, 0, 4 * sizeof(unsigned long long), ctx->stream));
-    int64_t nn;
-    RS_TRY(rs_read_i64(ctx, nd.counter, 1, &nn, "rs_refine6d"));
-    nn &= 0xffffffffll;
+    RS_WS(ctx, unsigned long long, so, WS_RF_MISC3, 5);
+    RS_CUDA(ctx, cudaMemsetAsync(so, 0, 5 * sizeof(unsigned long long), ctx->stream));
+    RS_LAUNCH(ctx, "rf_tree_stats", k_tree_stats, std::min<int64_t>(ceil_div(cap, 256), ctx->num_sms * 4), 256, 0, nd,
+              so);
+    int64_t s5[5];
+    RS_TRY(rs_read_i64(ctx, so, 5, s5, "rs_refine6d"));
+    const int64_t *s4 = s5 + 1, nn = s5[0];
     if (nn > cap) return rs_fail(ctx, RS_ERR_INTERNAL, "rs_refine6d: node capacity exceeded");
-    RS_LAUNCH(ctx, "rf_tree_stats", k_tree_stats, std::min<int64_t>(ceil_div(nn, 256), ctx->num_sms * 4), 256, 0, nd,
-              (int)nn, so);
-    int64_t s4[4];
-    RS_TRY(rs_read_i64(ctx, so, 4, s4, "rs_refine6d"));
     t->n_nodes = nn;
     t->n_seeds = s4[0];
     t->n_tieband = s4[1];
@@ -3507,7 +3498,7 @@ __global__ void k_fill_i32(int32_t *p, int64_t n, int32_t v)
 extern "C" void rs_tree_free(rs_tree *t)
 {
     if (!t) return;
-    if (t->block) cudaFree(t->block);
+    rs_block_free(t->block);
     delete t;
 }
 
@@ -3527,20 +3518,21 @@ extern "C" rs_status rs_refine6d_sampled(rs_ctx *ctx, const float *pos, const fl
     if (n >= ((int64_t)1 << 31)) return rs_fail(ctx, RS_ERR_TOO_LARGE, "rs_refine6d: n >= 2^31");
     if ((double)(float)box != box) return rs_fail(ctx, RS_ERR_INVALID_ARG, "rs_refine6d: box must be a float32 value");
     RsRange range("rs_refine6d");
-    int64_t cap = 0;
-    {
-        int64_t h[2];
-        RS_TRY(rs_read_i64(ctx, group_offsets, 1, h, "rs_refine6d"));
-        RS_CUDA(ctx, cudaMemcpyAsync(ctx->h_scratch + 1, group_offsets + n_groups, sizeof(int64_t),
-                                     cudaMemcpyDeviceToHost, ctx->stream));
-        RS_TRY(rs_sync_check(ctx, "rs_refine6d"));
-        int64_t M = ctx->h_scratch[1] - h[0];
-        cap = M / 4 + 4096;
-    }
+    // the first and last offset, and the offsets' order, in one host read
+    RS_LAUNCH(ctx, "rf_check_offsets", k_check_offsets, ceil_div(n_groups, 256), 256, 0, n_groups, group_offsets,
+              ctx->d_status);
+    RS_CUDA(ctx, cudaMemcpyAsync(ctx->h_scratch, group_offsets, sizeof(int64_t), cudaMemcpyDeviceToHost, ctx->stream));
+    RS_CUDA(ctx, cudaMemcpyAsync(ctx->h_scratch + 1, group_offsets + n_groups, sizeof(int64_t),
+                                 cudaMemcpyDeviceToHost, ctx->stream));
+    RS_TRY(rs_sync_check(ctx, "rs_refine6d: group offsets must be non-decreasing"));
+    const int64_t first = ctx->h_scratch[0], M = ctx->h_scratch[1] - first;
+    if (M < 0 || M > n || first < 0)
+        return rs_fail(ctx, RS_ERR_INVALID_ARG, "rs_refine6d: inconsistent group offsets");
+    int64_t cap = M / 4 + 4096;
     for (int attempt = 0; attempt < 4; attempt++) {
         rs_tree *t = nullptr;
-        rs_status s = refine_impl(ctx, pos, vel, stride, n, box, perm, group_offsets, n_groups, f, min_n, subset_n,
-                                  subset_seed, cap, &t);
+        rs_status s = refine_impl(ctx, pos, vel, stride, n, box, perm, group_offsets, n_groups, M, f, min_n,
+                                  subset_n, subset_seed, cap, &t);
         if (s == RS_OK) {
             *out = t;
             return RS_OK;
