@@ -164,6 +164,32 @@ __device__ __forceinline__ uint64_t reach_mask(int ux, int uy, int uz, int dx, i
     return m;
 }
 
+// Tables that combine four bits per axis into a coarse cell's 64 sub-cells,
+// filled by the whole block
+struct ReachTab {
+    uint64_t axis[3][16];
+    __device__ __forceinline__ void fill()
+    {
+        if (threadIdx.x < 16) {
+            const unsigned m = threadIdx.x;
+            uint64_t x = 0, y = 0, z = 0;
+            for (int b = 0; b < 64; b++) {
+                x |= (uint64_t)((m >> (b & 3)) & 1u) << b;
+                y |= (uint64_t)((m >> ((b >> 2) & 3)) & 1u) << b;
+                z |= (uint64_t)((m >> (b >> 4)) & 1u) << b;
+            }
+            axis[0][m] = x;
+            axis[1][m] = y;
+            axis[2][m] = z;
+        }
+        __syncthreads();
+    }
+    __device__ __forceinline__ uint64_t mask(unsigned mx, unsigned my, unsigned mz) const
+    {
+        return axis[0][mx] & axis[1][my] & axis[2][mz];
+    }
+};
+
 __device__ __forceinline__ void coarse_coords(uint64_t c, int Gc, int &cx, int &cy, int &cz)
 {
     const uint32_t cc = (uint32_t)c, G = (uint32_t)Gc;  // fewer than 2^32 coarse cells
@@ -217,14 +243,6 @@ __device__ __forceinline__ int pair_link(const float4 &pa, const float4 &pb, int
     return e2 <= g.l2 ? 1 : 0;
 }
 
-// position of the j-th (0-based) set bit of a 64-bit mask with at least j + 1 bits
-__device__ __forceinline__ int nth_bit64(uint64_t m, int j)
-{
-    const unsigned lo = (unsigned)m, hi = (unsigned)(m >> 32);
-    const int nlo = __popc(lo);
-    return j < nlo ? (int)__fns(lo, 0, j + 1) : 32 + (int)__fns(hi, 0, j - nlo + 1);
-}
-
 // Join fine cell A with every fine cell of larger index within two fine cells
 // per axis that has a friend pair with it.  Pass 0 takes the 26 adjacent
 // cells (offsets of at most 1 per axis), where pairs are friends almost at
@@ -242,11 +260,15 @@ __device__ __forceinline__ int nth_bit64(uint64_t m, int j)
 // that more warps share the chain, and the root kernels between the passes are
 // left out (32,768 particles: 117 -> 76 us).
 //
-// A warp takes 32 consecutive fine cells, a lane each.  For each of the
-// eight coarse cells around them every lane forms its mask of candidate fine
-// cells; the warp then numbers all lanes' candidates (a prefix sum of the
-// mask popcounts) and deals them out 32 at a time, so each lane tests one
-// candidate pair per round whatever the spread of candidates over the cells.
+// A warp takes 32 consecutive fine cells, a lane each.  Its reach per axis and
+// neighbouring coarse cell is formed once (four bits an axis, combined per
+// coarse cell through tables), and a coarse cell is looked up only when the
+// reach touches it.  Candidate pairs go to the warp's queue, the lanes' lowest
+// bits at a time, and are tested 32 at a time whatever their spread over the
+// cells.  Bound by instruction issue and the loads of the tests.  Numbering
+// the candidates by a prefix sum and finding each lane's by its rank (with
+// __fns), and looking up all eight coarse cells, took 6.7 ms for 33M
+// particles; this takes 4.6.
 __global__ void __launch_bounds__(FOF_THREADS, 6) k_fof_link(const uint32_t *n_cells_p, const uint64_t *cell_key,
                                                             const uint32_t *cell_start, const uint32_t *table,
                                                             const uint64_t *occ, const float4 *spos, int *parent,
@@ -254,111 +276,106 @@ __global__ void __launch_bounds__(FOF_THREADS, 6) k_fof_link(const uint32_t *n_c
                                                             rs_dev_status *st)
 {
     const unsigned FULL = 0xffffffffu;
+    __shared__ ReachTab tab;
+    __shared__ int qa_s[FOF_THREADS / 32][64], qb_s[FOF_THREADS / 32][64];
+    __shared__ unsigned char qs_s[FOF_THREADS / 32][64];  // periodic shifts, two bits an axis (0: none, 1: +, 2: -)
+    tab.fill();
     const int64_t M = *n_cells_p;
-    const int lane = lane_id();
+    const int lane = lane_id(), w = warp_id();
+    int *qa = qa_s[w], *qb = qb_s[w];
+    unsigned char *qs = qs_s[w];
+    int np = 0;
+    // tests up to 32 queued pairs, one a lane
+    auto flush = [&](int cnt) {
+        np -= cnt;
+        if (lane < cnt) {
+            const int A = qa[np + lane], B = qb[np + lane], s = qs[np + lane];
+            if (uf_find(parent, A, st) != uf_find(parent, B, st)) {
+                const int sx = (s & 1) - ((s >> 1) & 1), sy = ((s >> 2) & 1) - ((s >> 3) & 1),
+                          sz = ((s >> 4) & 1) - ((s >> 5) & 1);
+                const uint32_t a0 = cell_start[A], a1 = cell_start[A + 1], b0 = cell_start[B], b1 = cell_start[B + 1];
+                bool linked = false;
+                for (uint32_t i = a0; i < a1 && !linked; i++) {
+                    const float4 pa = spos[i];
+                    for (uint32_t q = b0; q < b1; q++)
+                        if (pair_link(pa, spos[q], sx, sy, sz, g)) {
+                            linked = true;
+                            break;
+                        }
+                }
+                if (linked) uf_union(parent, A, B, st);
+            }
+        }
+        __syncwarp();
+    };
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t warps = (int64_t)gridDim.x * blockDim.x >> 5;
     for (int64_t u = warp0; u < (M + 31) / 32 * split; u += warps) {
-        const int64_t wb = u / split * 32;
+        const int64_t A = u / split * 32 + lane;
         const int s0 = (int)(u % split) * (8 / split), s1 = s0 + 8 / split;
-        const int64_t A = wb + lane;
         const bool va = A < M;
         uint64_t ca = 0;
-        int sa = 0, ux = 0, uy = 0, uz = 0, ccx = 0, ccy = 0, ccz = 0;
-        uint32_t a0 = 0, a1 = 0;
+        int sa = 0, ccx = 0, ccy = 0, ccz = 0;
         if (va) {
             const uint64_t ka = cell_key[A];
             ca = ka >> 6;
             sa = (int)(ka & 63);
-            ux = sa & 3;
-            uy = (sa >> 2) & 3;
-            uz = sa >> 4;
             coarse_coords(ca, g.Gc, ccx, ccy, ccz);
-            a0 = cell_start[A];
-            a1 = cell_start[A + 1];
         }
-        const int ax = 4 * ccx + ux, ay = 4 * ccy + uy, az = 4 * ccz + uz;
+        // per axis, for the lower and the upper of the two coarse cells in
+        // reach: the sub-cells at most 1 away (bits 0-3) and at most 2 (4-7)
+        const int ux = sa & 3, uy = (sa >> 2) & 3, uz = sa >> 4;
         const int lox = ux < 2 ? -1 : 0, loy = uy < 2 ? -1 : 0, loz = uz < 2 ? -1 : 0;
+        auto ranges = [](int c, int d) { return axis_range(c, d, 1) | axis_range(c, d, 2) << 4; };
+        const unsigned rx = ranges(ux, lox) | ranges(ux, lox + 1) << 8, ry = ranges(uy, loy) | ranges(uy, loy + 1) << 8,
+                       rz = ranges(uz, loz) | ranges(uz, loz + 1) << 8;
         // a root of A's set (sets only grow, so a coarse cell whose common
         // root equals it is in A's set for the rest of the pass)
         const int ra = (va && uroot) ? uf_find(parent, (int)A, st) : -1;
         for (int s8 = s0; s8 < s1; s8++) {
-            const int dz = loz + (s8 >> 2), dy = loy + ((s8 >> 1) & 1), dx = lox + (s8 & 1);
-            int cz = ccz + dz, cy = ccy + dy, cx = ccx + dx;
-            cz = cz < 0 ? cz + g.Gc : (cz >= g.Gc ? cz - g.Gc : cz);
-            cy = cy < 0 ? cy + g.Gc : (cy >= g.Gc ? cy - g.Gc : cy);
-            cx = cx < 0 ? cx + g.Gc : (cx >= g.Gc ? cx - g.Gc : cx);
-            uint64_t cand = 0, om = 0;
-            uint32_t b0c = 0;
-            if (va) {
-                const uint64_t cc = ((uint64_t)cz * g.Gc + cy) * g.Gc + cx;
-                if (cc >= ca) {  // coarse cells below A's hold only fine cells of smaller index
-                    b0c = table[cc];
-                    if (b0c != 0xffffffffu && !(ra >= 0 && uroot[b0c] == ra)) {
-                        om = occ[b0c];
-                        const uint64_t near = pass < 2 ? reach_mask(ux, uy, uz, dx, dy, dz, 1) : 0ull;
-                        cand = om & (pass == 0 ? near : reach_mask(ux, uy, uz, dx, dy, dz, 2) & ~near);
-                        if (cc == ca) cand &= ~((2ull << sa) - 1ull);  // sub-cells after A's
-                    }
-                }
+            const unsigned mx = rx >> (8 * (s8 & 1)), my = ry >> (8 * ((s8 >> 1) & 1)), mz = rz >> (8 * (s8 >> 2));
+            const uint64_t near = tab.mask(mx & 15u, my & 15u, mz & 15u);
+            uint64_t cand = near;
+            if (pass > 0) {
+                cand = tab.mask((mx >> 4) & 15u, (my >> 4) & 15u, (mz >> 4) & 15u);
+                if (pass == 1) cand &= ~near;
             }
-            for (int guard = 0; guard < 4096; guard++) {
-                const int cnt = __popcll(cand);
-                int incl = cnt;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(FULL, incl, o);
-                    if (lane >= o) incl += y;
+            uint64_t om = 0;
+            uint32_t b0c = 0xffffffffu;
+            unsigned shift = 0;
+            if (va && cand) {
+                int cx = ccx + lox + (s8 & 1), cy = ccy + loy + ((s8 >> 1) & 1), cz = ccz + loz + (s8 >> 2);
+                // (a cell reached across the lower face lies near the top)
+                shift = (cx < 0 ? 1u : (cx >= g.Gc ? 2u : 0u)) | (cy < 0 ? 4u : (cy >= g.Gc ? 8u : 0u)) |
+                        (cz < 0 ? 16u : (cz >= g.Gc ? 32u : 0u));
+                cx = cx < 0 ? cx + g.Gc : (cx >= g.Gc ? cx - g.Gc : cx);
+                cy = cy < 0 ? cy + g.Gc : (cy >= g.Gc ? cy - g.Gc : cy);
+                cz = cz < 0 ? cz + g.Gc : (cz >= g.Gc ? cz - g.Gc : cz);
+                const uint64_t cc = ((uint64_t)cz * g.Gc + cy) * g.Gc + cx;
+                if (cc == ca) cand &= ~((2ull << sa) - 1ull);  // sub-cells after A's
+                // (coarse cells below A's hold only fine cells of smaller index)
+                if (cc >= ca && cand) b0c = table[cc];
+                if (b0c != 0xffffffffu && !(ra >= 0 && uroot[b0c] == ra)) om = occ[b0c];
+            }
+            cand &= om;
+            for (;;) {
+                const unsigned bm = __ballot_sync(FULL, cand != 0);
+                if (!bm) break;
+                if (cand) {
+                    const int sb = __ffsll((long long)cand) - 1;
+                    cand &= cand - 1ull;
+                    const int at = np + __popc(bm & ((1u << lane) - 1u));
+                    qa[at] = (int)A;
+                    qb[at] = (int)(b0c + (uint32_t)__popcll(om & ((1ull << sb) - 1ull)));
+                    qs[at] = (unsigned char)shift;
                 }
-                const int total = __shfl_sync(FULL, incl, 31);
-                if (total == 0) break;
-                const int excl = incl - cnt;
-                // this lane's candidate: number `lane` in the warp's order
-                int lo = 0, hi = 31;
-#pragma unroll
-                for (int it = 0; it < 5; it++) {
-                    const int mid = (lo + hi) >> 1;
-                    if (__shfl_sync(FULL, incl, mid) > lane) hi = mid;
-                    else lo = mid + 1;
-                }
-                const int src = lo;
-                const int j = lane - __shfl_sync(FULL, excl, src);
-                const uint64_t smask = __shfl_sync(FULL, cand, src), som = __shfl_sync(FULL, om, src);
-                const uint32_t sb0 = __shfl_sync(FULL, b0c, src), sa0 = __shfl_sync(FULL, a0, src),
-                               sa1 = __shfl_sync(FULL, a1, src);
-                const int sax = __shfl_sync(FULL, ax, src), say = __shfl_sync(FULL, ay, src),
-                          saz = __shfl_sync(FULL, az, src);
-                const int scx = __shfl_sync(FULL, cx, src), scy = __shfl_sync(FULL, cy, src),
-                          scz = __shfl_sync(FULL, cz, src);
-                const int sA = (int)(wb + src);
-                if (lane < total) {
-                    const int sb = nth_bit64(smask, j);
-                    const int B = (int)(sb0 + __popcll(som & ((1ull << sb) - 1ull)));
-                    const int bx = 4 * scx + (sb & 3), by = 4 * scy + ((sb >> 2) & 3), bz = 4 * scz + (sb >> 4);
-                    int sx, sy, sz;
-                    fine_offset(sax, bx, g.Gf, sx);
-                    fine_offset(say, by, g.Gf, sy);
-                    fine_offset(saz, bz, g.Gf, sz);
-                    if (uf_find(parent, sA, st) != uf_find(parent, B, st)) {
-                        const uint32_t b0 = cell_start[B], b1 = cell_start[B + 1];
-                        bool linked = false;
-                        for (uint32_t i = sa0; i < sa1 && !linked; i++) {
-                            const float4 pa = spos[i];
-                            for (uint32_t q = b0; q < b1; q++)
-                                if (pair_link(pa, spos[q], sx, sy, sz, g)) {
-                                    linked = true;
-                                    break;
-                                }
-                        }
-                        if (linked) uf_union(parent, sA, B, st);
-                    }
-                }
-                // drop the candidates dealt out this round (the lowest ones of each lane)
-                const int used = max(0, min(incl, 32) - excl);
-                for (int u = 0; u < used; u++) cand &= cand - 1ull;
+                np += __popc(bm);
+                __syncwarp();
+                if (np >= 32) flush(32);
             }
         }
     }
+    if (np > 0) flush(np);
 }
 
 // the root of every coarse cell's first fine cell, kept at that cell
@@ -389,19 +406,32 @@ __global__ void k_fof_rootmin(const uint32_t *n_cells_p, const uint32_t *cell_st
 {
     const int64_t M = *n_cells_p;
     for (int64_t A = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; A < M; A += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t m = 0xffffffffu;
-        for (uint32_t q = cell_start[A]; q < cell_start[A + 1]; q++) m = min(m, idx[q]);
-        int r = uf_find_n(parent, (int)A, st, find_limit);
-        atomicMin(&root_min[r], (int)m);
+        // (a cell's particles are in index order; reading them all, and adding
+        // to roots that already hold less, took 0.63 ms for 33M particles,
+        // this 0.1)
+        const int m = (int)idx[cell_start[A]];
+        // No path halving here: a cell's parent is written by its own thread
+        // alone, so that it is the root when the labels read it (a late
+        // halving write of another thread would put back an ancestor).
+        int r = (int)A, it = 0;
+        for (; it < find_limit; it++) {
+            const int p = __ldcg(&parent[r]);
+            if (p == r) break;
+            r = p;
+        }
+        if (it >= find_limit) dev_fail(st, DEV_TIMEOUT, 1, r);
+        if (r != (int)A) parent[A] = r;
+        if (m < __ldcg(&root_min[r])) atomicMin(&root_min[r], m);
     }
 }
 
-__global__ void k_fof_labels(int64_t n, const uint32_t *idx, const uint32_t *cell_of, int *parent,
-                             const int *root_min, int32_t *labels, rs_dev_status *st)
+// (every cell's parent is its root by now)
+__global__ void k_fof_labels(int64_t n, const uint32_t *idx, const uint32_t *cell_of, const int *parent,
+                             const int *root_min, int32_t *labels)
 {
     int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= n) return;
-    labels[idx[q]] = root_min[uf_find(parent, (int)cell_of[q], st)];
+    labels[idx[q]] = root_min[parent[cell_of[q]]];
 }
 
 __global__ void k_fof_count_roots(const uint32_t *n_cells_p, const int *parent, unsigned long long *count)
@@ -926,7 +956,7 @@ rs_status fof_run(rs_ctx *ctx, const float *pos, int32_t stride, int64_t n, doub
               (const uint32_t *)cell_start, (const uint32_t *)idx, parent, root_min,
               rs_fault("timeout1") ? 1 : RS_SPIN_LIMIT, ctx->d_status);
     RS_LAUNCH(ctx, "fof_labels", k_fof_labels, nb, T, 0, n, (const uint32_t *)idx, (const uint32_t *)cell_of,
-              parent, (const int *)root_min, labels, ctx->d_status);
+              (const int *)parent, (const int *)root_min, labels);
     if (n_groups || n_tieband) {
         RS_CUDA(ctx, cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), ctx->stream));
         if (n_groups)

@@ -28,6 +28,19 @@ def test_fof_and_groups_at_tile_edges(n, b):
         assert np.array_equal(perm.cpu().numpy(), m) and np.array_equal(off.cpu().numpy(), o), min_n
 
 
+def test_labels_of_a_clustered_box_are_roots():
+    """Every label is the smallest index of its group, in a box whose groups span many cells (the labels read the
+    cells' parents directly): against the oracle, and the same labels in repeated calls."""
+    from paper_1110_4372_gb300 import rsgpu
+    n = 400_001
+    c = synth.generate("c2", seed=5, n=n, box=10.0 * (n / 32768) ** (1 / 3), n_halos=480)
+    ref, _, _ = oracle.fof3d(c.pos, c.box, 0.28)
+    ctx, pos = rsgpu.Context(), torch.from_numpy(c.pos).cuda()
+    for _ in range(20):
+        lab, _, _ = rsgpu.rs_fof3d(ctx, pos, c.box, 0.28)
+        assert np.array_equal(lab.cpu().numpy(), ref)
+
+
 @pytest.mark.parametrize("n,groups", [(300_001, 1), (300_001, 3), (1_000_003, 70_000), (2_500_000, 2_500_000)])
 def test_group_sort_of_synthetic_labels(n, groups):
     """Labels drawn directly: one huge group, a few, many, and singletons only."""
