@@ -1089,6 +1089,9 @@ struct LevelBufs {
     int *tie;                // per rank
     unsigned *sub_t;         // per rank: subset key threshold, high and low words (2 entries)
     int *sub_cnt;            // per rank: members drawn into the subset
+    float2 *lim;             // per rank: below it a friend in float32, beyond it none
+    int *need;               // per rank: the link search has to visit the node
+    int *ovf;                // per rank: its pair list did not fit
 };
 
 // ---- sizes the level's setup needs of the hierarchies and splits below ----
@@ -1453,17 +1456,21 @@ __device__ __forceinline__ float point_box_far2(float4 p, float4 v, const Box6 &
 }
 
 // ---- building the boxes ----
-// Two forms.  Before the searches (LINK false): boxes over all members, and
-// the packed member copy.  Once the linking length is known (LINK true): the
-// boxes are rebuilt over the members that can have a friend (nearest-
-// neighbour value within reach; the others are neither queries nor
-// candidates, and their packed x becomes infinite, which no box is within
+// Three forms.  BOX_ALL, before the searches: boxes over all members, and the
+// packed member copy.  BOX_PAIRS, for the nodes of the pair search (below):
+// their flags and union-find entries at the bracket's lower edge, the boxes as
+// they are.  BOX_LINK, for the nodes of the link search, once the linking
+// length is known: the boxes are rebuilt over the members that can have a
+// friend (nearest-neighbour value within reach; the others are neither queries
+// nor candidates, and their packed x becomes infinite, which no box is within
 // reach of), which drops the phase-space outliers that stretch them.  A box
 // whose members all can have a friend and whose diameter is within the clique
 // margin is flagged, and its members are joined: a leaf's when its members'
 // union-find entries are first written, an upper box's by joining the first
 // members of its children (a flagged box's children are flagged, their
 // diameters being no larger).
+enum { BOX_ALL, BOX_PAIRS, BOX_LINK };
+
 // the union of one box per lane, in every lane
 __device__ __forceinline__ Box6 warp_box(const Box6 &c)
 {
@@ -1475,67 +1482,96 @@ __device__ __forceinline__ Box6 warp_box(const Box6 &c)
     return b;
 }
 
+// whether the form visits node rank k, and the largest diameter of its cliques
+template <int MODE>
+__device__ __forceinline__ bool box_visits(const LevelBufs &L, int k, const float *R2, const float *STOP, float &clim)
+{
+    clim = 0.f;
+    if (MODE == BOX_PAIRS) {
+        clim = (float)((double)STOP[k] * RS_CLIQUE_MARGIN);
+        return isfinite(R2[k]);
+    }
+    if (MODE == BOX_LINK) {
+        clim = (float)(L.l2[k] * RS_CLIQUE_MARGIN);
+        return L.need[k] != 0;
+    }
+    return true;
+}
+
 // Leaf boxes (one warp a leaf) and the boxes of 32 leaves above them.  A
 // block takes the 1024 members of one such box: the tiles' grid, of which the
 // blocks of every fourth tile work.  Against one thread a leaf in one block a
 // node (the link form before: 3.5 ms of a 16.8M-particle path, its largest
 // node alone on one SM), the loads coalesce and a large node spreads over the
 // device.
-template <bool LINK>
-__global__ void __launch_bounds__(TQ) k_bvh_leaves(LevelBufs L, NodeArrays nd, const int64_t *box_base, BoxStore B,
-                                                   MemberStore MS, const float4 *wpos, const float4 *wvel,
-                                                   const float *dnn, int *parent, int *csize, int *cmin,
-                                                   rs_dev_status *st)
+template <int MODE>
+__global__ void __launch_bounds__(TQ) k_bvh_leaves(LevelBufs L, NodeArrays nd, int64_t tile0, const int64_t *box_base,
+                                                   BoxStore B, MemberStore MS, const float4 *wpos, const float4 *wvel,
+                                                   const float *R2, const float *STOP, float *dnn, int *parent,
+                                                   int *csize, int *cmin, rs_dev_status *st)
 {
     __shared__ float bs[32][12];
     __shared__ unsigned char cs[32];
-    const int qb = L.tile_q0[blockIdx.x];
+    const int64_t tile = tile0 + blockIdx.x;
+    const int qb = L.tile_q0[tile];
     if (qb & 1023) return;
-    const int k = L.tile_rank[blockIdx.x];
+    const int k = L.tile_rank[tile];
+    float clim;
+    if (!box_visits<MODE>(L, k, R2, STOP, clim)) return;
     const int node = L.list[k], first = nd.first[node], n = nd.count[node];
     const int lane = lane_id();
     const BoxStore bx = box_shift(B, box_base[k]);
     Metric6 met;
     met.ax = L.met[k].ax;
     met.av = L.met[k].av;
-    const float part = LINK ? link_part(L.l2[k]) : 0.f;
-    const float clim = LINK ? (float)(L.l2[k] * RS_CLIQUE_MARGIN) : 0.f;
+    const float part = MODE == BOX_LINK ? link_part(L.l2[k]) : 0.f;
     for (int j = warp_id(); j < 32; j += TQ / 32) {
         const int q0 = qb + 32 * j, m = q0 + lane;
         if (q0 >= n) break;
         const bool ok = m < n;
         bool act = ok;
-        float4 p = make_float4(0, 0, 0, 0), v = p;
-        if (ok) {
-            if (LINK) {
-                mem_get(mem_shift(MS, first), m, p, v);
-                act = dnn[first + m] <= part;
-                if (!act) MS.a[first + m].x = INFINITY;
-            } else {
-                p = wpos[first + m];
-                v = wvel[first + m];
-                MS.a[first + m] = make_float4(p.x, p.y, p.z, v.x);
-                MS.b[first + m] = make_float2(v.y, v.z);
+        Box6 b;
+        if (MODE == BOX_PAIRS) {
+            b = box_get(bx, q0 / BVH_LEAF);
+        } else {
+            float4 p = make_float4(0, 0, 0, 0), v = p;
+            if (ok) {
+                if (MODE == BOX_LINK) {
+                    mem_get(mem_shift(MS, first), m, p, v);
+                    act = dnn[first + m] <= part;
+                    if (!act) MS.a[first + m].x = INFINITY;
+                } else {
+                    p = wpos[first + m];
+                    v = wvel[first + m];
+                    MS.a[first + m] = make_float4(p.x, p.y, p.z, v.x);
+                    MS.b[first + m] = make_float2(v.y, v.z);
+                }
             }
+            b = box_empty();
+            if (act) {
+                b.plo = b.phi = p;
+                b.vlo = b.vhi = v;
+            }
+            b = warp_box(b);
         }
-        Box6 b = box_empty();
-        if (act) {
-            b.plo = b.phi = p;
-            b.vlo = b.vhi = v;
-        }
-        b = warp_box(b);
         bool clique = false;
-        if (LINK) {
-            clique = __ballot_sync(0xffffffffu, act) == __ballot_sync(0xffffffffu, ok) && box_diam2(b, met) <= clim;
+        if (MODE != BOX_ALL) {
+            const float diam = box_diam2(b, met);
+            clique = __ballot_sync(0xffffffffu, act) == __ballot_sync(0xffffffffu, ok) && diam <= clim;
+            // (a lone member has no neighbour in its leaf)
+            if (MODE == BOX_PAIRS) clique = clique && q0 + 1 < n;
             if (ok) {
                 parent[first + m] = clique ? first + q0 : first + m;
                 csize[first + m] = 0;
                 cmin[first + m] = 0x7fffffff;
+                // a clique's members have a neighbour below the bracket, which
+                // is all that matters of its distance
+                if (MODE == BOX_PAIRS) dnn[first + m] = clique ? diam : INFINITY;
             }
         }
         if (lane == 0) {
-            box_put(bx, q0 / BVH_LEAF, b);
-            if (LINK) bx.cl[q0 / BVH_LEAF] = cs[j] = clique ? 1 : 0;
+            if (MODE != BOX_PAIRS) box_put(bx, q0 / BVH_LEAF, b);
+            if (MODE != BOX_ALL) bx.cl[q0 / BVH_LEAF] = cs[j] = clique ? 1 : 0;
             float *o = bs[j];
             o[0] = b.plo.x; o[1] = b.plo.y; o[2] = b.plo.z; o[3] = b.vlo.x; o[4] = b.vlo.y; o[5] = b.vlo.z;
             o[6] = b.phi.x; o[7] = b.phi.y; o[8] = b.phi.z; o[9] = b.vhi.x; o[10] = b.vhi.y; o[11] = b.vhi.z;
@@ -1554,21 +1590,22 @@ __global__ void __launch_bounds__(TQ) k_bvh_leaves(LevelBufs L, NodeArrays nd, c
         b.vhi = make_float4(o[9], o[10], o[11], 0.f);
     }
     b = warp_box(b);
-    const bool clique = LINK && !__any_sync(0xffffffffu, have && !cs[lane]) && box_diam2(b, met) <= clim;
+    const bool clique = MODE != BOX_ALL && !__any_sync(0xffffffffu, have && !cs[lane]) && box_diam2(b, met) <= clim;
     if (lane == 0) {
-        box_put(bx, nl + (qb >> 10), b);
-        if (LINK) bx.cl[nl + (qb >> 10)] = clique ? 1 : 0;
+        if (MODE != BOX_PAIRS) box_put(bx, nl + (qb >> 10), b);
+        if (MODE != BOX_ALL) bx.cl[nl + (qb >> 10)] = clique ? 1 : 0;
     }
     if (clique && have && lane > 0) uf_union(parent, first + qb, first + qb + 32 * lane, st);
 }
 
 // the levels above, one block a node, one warp a box
-template <bool LINK>
+template <int MODE>
 __global__ void __launch_bounds__(256) k_bvh_build(LevelBufs L, NodeArrays nd, const int64_t *box_base, BoxStore B,
-                                                   int *parent, rs_dev_status *st)
+                                                   const float *R2, const float *STOP, int *parent, rs_dev_status *st)
 {
     const int k = blockIdx.x;
-    if (k >= L.K) return;
+    float clim;
+    if (k >= L.K || !box_visits<MODE>(L, k, R2, STOP, clim)) return;
     const int node = L.list[k], n = nd.count[node], first = nd.first[node];
     const int nl = (int)ceil_div(n, BVH_LEAF);
     const BoxStore bx = box_shift(B, box_base[k]);
@@ -1576,7 +1613,6 @@ __global__ void __launch_bounds__(256) k_bvh_build(LevelBufs L, NodeArrays nd, c
     Metric6 met;
     met.ax = L.met[k].ax;
     met.av = L.met[k].av;
-    const float clim = LINK ? (float)(L.l2[k] * RS_CLIQUE_MARGIN) : 0.f;
     int cprev = (nl + 31) >> BVH_LOG;
     int64_t off_prev = nl, off = nl + cprev;
     for (int h = 2; h < H; h++) {
@@ -1587,11 +1623,11 @@ __global__ void __launch_bounds__(256) k_bvh_build(LevelBufs L, NodeArrays nd, c
             Box6 b = box_empty();
             if (have) b = box_get(bx, off_prev + c);
             b = warp_box(b);
-            const bool clique = LINK && !__any_sync(0xffffffffu, have && !bx.cl[off_prev + c]) &&
+            const bool clique = MODE != BOX_ALL && !__any_sync(0xffffffffu, have && !bx.cl[off_prev + c]) &&
                                 box_diam2(b, met) <= clim;
             if (lane == 0) {
-                box_put(bx, off + i, b);
-                if (LINK) bx.cl[off + i] = clique ? 1 : 0;
+                if (MODE != BOX_PAIRS) box_put(bx, off + i, b);
+                if (MODE != BOX_ALL) bx.cl[off + i] = clique ? 1 : 0;
             }
             if (clique && have && lane > 0)
                 uf_union(parent, first + (int)bvh_m0(h, i), first + (int)bvh_m0(h - 1, c), st);
@@ -1722,7 +1758,7 @@ constexpr int NN_WARPS = 4;
 template <int MINB>
 __global__ void __launch_bounds__(NN_WARPS * 32, MINB * W_WARPS / NN_WARPS)
     k_bvh_nn(LevelBufs L, NodeArrays nd, const int64_t *box_base, BoxStore B, MemberStore MS, const float *R2,
-             const float *STOP, int redo_failed, int sub_n, float *out, rs_dev_status *st)
+             const float *STOP, int redo_failed, int sub_n, int pairs, float *out, rs_dev_status *st)
 {
     __shared__ int si_s[NN_WARPS][W_STACK];
     __shared__ float sd_s[NN_WARPS][W_STACK];
@@ -1735,6 +1771,7 @@ __global__ void __launch_bounds__(NN_WARPS * 32, MINB * W_WARPS / NN_WARPS)
     const int node = L.list[k], first = nd.first[node], n = nd.count[node];
     // (a node above the subset size searches its subset members one by one)
     if (q0 >= n || (sub_n > 0 && n > sub_n)) return;
+    if (pairs && isfinite(R2[k]) && R2[k] >= 0.f) return;  // the pair search took it
     const Metric6 met = L.met[k];
     BvhView V;
     bvh_view(V, B, box_base[k], n, lv_s[w]);
@@ -1915,7 +1952,49 @@ __device__ __forceinline__ float box_box_d2(const Box6 &a, const Box6 &b, const 
     return (gx * gx + gy * gy + gz * gz) * m.ax + (gu * gu + gv * gv + gw * gw) * m.av;
 }
 
-struct LinkWarp {
+// ---- nearest neighbours and friends in one search: the pair search ----
+// A node with a sampled bracket [stop, R2] around its linking length (squared)
+// needs one search only.  Walked at R2, leaf against leaf as above, it meets
+// every pair that matters: each evaluated pair lowers the nearest-neighbour
+// values of both its members; a pair below stop is a friend whatever the
+// linking length turns out to be, and is joined at once; the pairs between
+// stop and R2 (13 a member at f = 0.7) are listed, and once the linking length
+// is known the list is gone through (k_pair_link).  A node whose bracket
+// fails, or whose pairs do not fit the list, is searched for friends again
+// from scratch.
+//
+// Against a nearest-neighbour search a member and a link search a leaf: 118 +
+// 67 ms of a 134M-particle path became 83 (pairs) + 5 (list) + 21 (the nodes
+// without a bracket), 9.6M members in groups 19.5 + 13.7 became 15.9 + 1.1 +
+// 5.1.  The list moves 9 bytes a pair each way, a few percent of the search.
+//
+// The list is in chunks of PAIR_CHUNK pairs of one leaf, with a head (node
+// rank, first query, pairs), in PAIR_REGIONS regions with a counter each.
+constexpr int PAIR_CHUNK = 64;
+constexpr int PAIR_REGIONS = 64;
+constexpr int PAIR_PER_MEMBER = 20;                  // room for this many pairs a member
+constexpr int64_t PAIR_MAX_BYTES = (int64_t)16 << 30;  // no list beyond this
+
+struct PairList {
+    int4 *head;    // (rank, first query, pairs, 0) per chunk
+    int2 *pair;    // (query lane << 26 | member, float32 distance) per pair
+    int *len;      // chunks taken per region
+    int cap;       // chunks per region
+    const float *R2, *STOP;
+    float *dnn;
+};
+
+template <bool PAIRS>
+struct PairStage {
+    int2 out[96];  // pairs on their way to the list
+    int best[32];  // per query: nearest-neighbour value so far (bits)
+};
+template <>
+struct PairStage<false> {
+};
+
+template <bool PAIRS>
+struct LinkWarp : PairStage<PAIRS> {
     uint4 cand[32];         // 32 candidates (or, at first, the queries) as eight halves
     float4 qa[32];          // the queries: px, py, pz, vx
     float2 qb[32];          //              vy, vz
@@ -1936,27 +2015,29 @@ struct LinkWarp {
 // a small block frees its slot as soon as its own few warps end instead of
 // waiting for the slowest of eight.
 constexpr int LK_WARPS = 2;
-template <int WARPS>
+template <int WARPS, bool PAIRS>
 __global__ void __launch_bounds__(LK_WARPS * 32, WARPS / LK_WARPS)
-    k_bvh_link(LevelBufs L, NodeArrays nd, const int64_t *box_base, BoxStore B, MemberStore MS, int *parent,
-               rs_dev_status *st)
+    k_bvh_link(LevelBufs L, NodeArrays nd, int64_t tile0, const int64_t *box_base, BoxStore B, MemberStore MS,
+               int *parent, PairList P, rs_dev_status *st)
 {
     static_assert((TQ / 32) % LK_WARPS == 0, "a tile's warps fill whole blocks");
-    __shared__ LinkWarp sh[LK_WARPS];
+    __shared__ LinkWarp<PAIRS> sh[LK_WARPS];
     const int w = warp_id(), lane = lane_id();
-    LinkWarp &S = sh[w];
+    LinkWarp<PAIRS> &S = sh[w];
     // the grid holds exactly the tiles' warps: block b takes warps
     // (b % bpt) * LK_WARPS + w of tile b / bpt
     constexpr int bpt = (TQ / 32) / LK_WARPS;
-    const int tile = blockIdx.x / bpt, jw = (blockIdx.x % bpt) * LK_WARPS + w;
+    const int64_t tile = tile0 + blockIdx.x / bpt;
+    const int jw = (blockIdx.x % bpt) * LK_WARPS + w;
     const int k = L.tile_rank[tile], q0 = L.tile_q0[tile] + 32 * jw;
     const int node = L.list[k], first = nd.first[node], n = nd.count[node];
-    if (q0 >= n) return;
+    if (q0 >= n || (PAIRS ? !isfinite(P.R2[k]) : !L.need[k])) return;
     const MemberStore M = mem_shift(MS, first);
     const int mo = q0 + lane;
     float4 po = make_float4(INFINITY, 0, 0, 0), vo = make_float4(0, 0, 0, 0);
     if (mo < n) mem_get(M, mo, po, vo);
-    // (a member without a neighbour within reach has an infinite packed x)
+    // (in the link search a member without a neighbour within reach has an
+    // infinite packed x)
     const bool act = po.x < INFINITY;
     const unsigned actm = __ballot_sync(FULLW, act);
     if (!actm) return;
@@ -1965,13 +2046,22 @@ __global__ void __launch_bounds__(LK_WARPS * 32, WARPS / LK_WARPS)
     met.av = L.met[k].av;
     const Metric6 *met64 = L.met + k;
     const double *l2p = L.l2 + k;
-    const LinkLim lm = link_lim(L.l2[k]);
+    // search radius: every pair that matters is within it
+    LinkLim lm = link_lim(PAIRS ? 0.0 : L.l2[k]);
+    const float stop = PAIRS ? P.STOP[k] : 0.f;
+    if (PAIRS) {
+        lm.part = P.R2[k];
+        lm.lim = lm.part * RS_PRUNE_SLACK;
+        lm.cl_lim = (float)((double)stop * RS_CLIQUE_MARGIN);
+    }
     BvhView V;
     bvh_view(V, B, box_base[k], n, S.lv);
     const int own = q0 / BVH_LEAF;
     S.qa[lane] = make_float4(po.x, po.y, po.z, vo.x);
     S.qb[lane] = make_float2(vo.y, vo.z);
     S.rq[lane] = act ? __ldcg(&parent[first + mo]) : 0;
+    if constexpr (PAIRS) S.best[lane] = 0x7f800000;
+    const bool own_clique = PAIRS && V.S.cl[own] != 0;  // its own pairs are settled
 
     // ---- half-precision frame: centre, weights, the queries' fragments ----
     bool brute;
@@ -2016,14 +2106,60 @@ __global__ void __launch_bounds__(LK_WARPS * 32, WARPS / LK_WARPS)
         __syncwarp();
     }
 
-    int tie = 0, np = 0;               // queued pairs
+    int tie = 0, np = 0, no = 0;       // queued pairs, pairs on their way to the list
     int head = 0, nc = 0;              // ring of kept candidates
     const unsigned below = (1u << lane) - 1u;
+    // the last cnt staged pairs to a chunk of the list
+    auto put_chunk = [&](int cnt) {
+        if constexpr (PAIRS) {
+            const int region = blockIdx.x & (PAIR_REGIONS - 1);
+            no -= cnt;
+            int c = 0;
+            if (lane == 0) c = atomicAdd(&P.len[region], 1);
+            c = __shfl_sync(FULLW, c, 0);
+            if (c < P.cap) {
+                const int64_t at = (int64_t)region * P.cap + c;
+                for (int i = lane; i < cnt; i += 32) P.pair[at * PAIR_CHUNK + i] = S.out[no + i];
+                if (lane == 0) P.head[at] = make_int4(k, q0, cnt, 0);
+            } else if (lane == 0) {
+                L.ovf[k] = 1;
+            }
+            __syncwarp();
+        }
+    };
     // evaluates up to 32 queued pairs, one a lane
     auto flush = [&](int cnt) {
         np -= cnt;
         const int code = lane < cnt ? S.pairs[np + lane] : 0;
         const int r = code >> 26, m = code & 0x3ffffff;
+        if constexpr (PAIRS) {
+            bool keep = false;
+            float d2 = 0.f;
+            if (lane < cnt && m > q0 + r) {
+                float4 pm, vm;
+                mem_get(M, m, pm, vm);
+                const float4 x = S.qa[r];
+                const float2 y = S.qb[r];
+                d2 = d2_32(make_float4(x.x, x.y, x.z, 0.f), make_float4(x.w, y.x, y.y, 0.f), pm, vm, met);
+                if (d2 <= lm.part) {
+                    const int bits = __float_as_int(d2);
+                    int *dm = reinterpret_cast<int *>(P.dnn) + first + m;
+                    if (bits < ((volatile int *)S.best)[r]) atomicMin(&S.best[r], bits);
+                    if (bits < __ldcg(dm)) atomicMin(dm, bits);
+                    keep = !(d2 < stop);
+                    if (!keep) {
+                        const int root = join_friend(parent, first + q0 + r, first + m, ((volatile int *)S.rq)[r], st);
+                        if (root != 0x7fffffff) atomicMin(&S.rq[r], root);
+                    }
+                }
+            }
+            const unsigned km = __ballot_sync(FULLW, keep);
+            if (keep) S.out[no + __popc(km & below)] = make_int2(code, __float_as_int(d2));
+            no += __popc(km);
+            __syncwarp();
+            if (no >= PAIR_CHUNK) put_chunk(PAIR_CHUNK);
+            return;
+        }
         if (lane < cnt && m > q0 + r) {
             float4 pm, vm;
             mem_get(M, m, pm, vm);
@@ -2116,7 +2252,7 @@ __global__ void __launch_bounds__(LK_WARPS * 32, WARPS / LK_WARPS)
                 const int64_t bi = V.off[ch] + c;
                 cb = box_get(V.S, bi);
                 clique = V.S.cl[bi] != 0;
-                want = box_box_d2(own_box(), cb, met) <= lm.lim;
+                want = box_box_d2(own_box(), cb, met) <= lm.lim && !(own_clique && ch == 0 && c == own);
             }
         }
         unsigned cm = __ballot_sync(FULLW, want && clique && !(ch == 0 && c == own));
@@ -2137,6 +2273,9 @@ __global__ void __launch_bounds__(LK_WARPS * 32, WARPS / LK_WARPS)
             if (all) {
                 const int root = join_friend(parent, first + mo, first + m0, S.rq[lane], st);
                 if (root != 0x7fffffff) S.rq[lane] = min(S.rq[lane], root);
+                // (its members have a neighbour below the bracket already)
+                if constexpr (PAIRS)
+                    S.best[lane] = min(S.best[lane], __float_as_int(point_box_far2(po, vo, b, met)));
             }
             const bool open = __any_sync(FULLW, near && !all);
             if (lane == s) want = open;
@@ -2203,8 +2342,50 @@ __global__ void __launch_bounds__(LK_WARPS * 32, WARPS / LK_WARPS)
         while (nc >= 32 || (last && nc > 0)) test(min(nc, 32));
     }
     if (np > 0) flush(np);
+    if constexpr (PAIRS) {
+        if (no > 0) put_chunk(no);
+        if (act) atomicMin(reinterpret_cast<int *>(P.dnn) + first + mo, S.best[lane]);
+        return;
+    }
     tie = warp_sum(tie);
     if (lane == 0 && tie) atomicAdd(&L.tie[k], tie);
+}
+
+// the listed pairs at the linking length, a warp a chunk
+__global__ void __launch_bounds__(256) k_pair_link(LevelBufs L, NodeArrays nd, MemberStore MS, PairList P, int *parent,
+                                                   rs_dev_status *st)
+{
+    const int lane = lane_id(), gw = (int)((blockIdx.x * 256 + threadIdx.x) >> 5), warps = (int)(gridDim.x * 8);
+    const int region = gw & (PAIR_REGIONS - 1), len = min(P.len[region], P.cap);
+    for (int c = gw / PAIR_REGIONS; c < len; c += warps / PAIR_REGIONS) {
+        const int64_t at = (int64_t)region * P.cap + c;
+        const int4 h = P.head[at];
+        const int k = h.x;
+        if (L.need[k]) continue;
+        const float2 lim = L.lim[k];
+        const int first = nd.first[L.list[k]];
+        int tie = 0;
+        for (int i = lane; i < h.z; i += 32) {
+            const int2 e = P.pair[at * PAIR_CHUNK + i];
+            const float d2 = __int_as_float(e.y);
+            if (d2 > lim.y) continue;
+            const int q = first + h.y + (e.x >> 26), m = first + (e.x & 0x3ffffff);
+            bool link = d2 < lim.x;
+            if (!link) {
+                float4 pq, vq, pm, vm;
+                mem_get(MS, q, pq, vq);
+                mem_get(MS, m, pm, vm);
+                const double l2 = L.l2[k], l = sqrt(l2), e64 = d2_64(pq, vq, pm, vm, L.met[k]);
+                link = e64 <= l2;
+                tie += (l2 > 0 && e64 != l2 && fabs(sqrt(e64) - l) <= 1e-6 * l) ? 1 : 0;
+            }
+            if (link) join_friend(parent, q, m, __ldcg(&parent[q]), st);
+        }
+        if (__any_sync(FULLW, tie != 0)) {
+            tie = warp_sum(tie);
+            if (lane == 0) atomicAdd(&L.tie[k], tie);
+        }
+    }
 }
 
 // ---- sampled bracket for the nearest-neighbour search ----
@@ -2269,20 +2450,30 @@ __global__ void k_smp_thresh(LevelBufs L, NodeArrays nd, const int *smp_at, cons
 // A node whose bracket did not hold gets R2 = -1: the fallback search
 // redoes that node only (force_odd, from the injected fault
 // RS_FAULT=bracket, fails every node of odd rank that has a bracket).
-__global__ void k_bracket_check(LevelBufs L, float *R2, const float *STOP, int *fallback, int force_odd)
+// need marks the nodes left to the link search: all without a pair search,
+// and of those with one the failed ones and those whose list overflowed
+// (*again set).
+__global__ void k_bracket_check(LevelBufs L, float *R2, const float *STOP, int *fallback, int force_odd, int pairs,
+                                int *again)
 {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= L.K) return;
     // the whole float32 band around the k-th value must lie inside the radius,
-    // so no member that belongs in the band was cut off by it
+    // so no member that belongs in the band was cut off by it, and the linking
+    // and tie bands (within 5e-6 of t32) between the stop value and the radius,
+    // so the pair search joined friends only and listed every pair of the bands
     const float t32 = __uint_as_float(L.sel_prefix[k]);
-    bool fail = !((double)t32 * (1.0 + 4.0 * RS_BAND) <= (double)R2[k]) ||
-                !((double)t32 * (1.0 - 4.0 * RS_BAND) >= (double)STOP[k]);
+    const bool bracket = isfinite(R2[k]);
+    bool fail = !((double)t32 * (1.0 + 8.0 * RS_BAND) <= (double)R2[k]) ||
+                !((double)t32 * (1.0 - 8.0 * RS_BAND) >= (double)STOP[k]);
     if (force_odd && (k & 1) && !isinf(R2[k])) fail = true;
     if (fail) {
         R2[k] = -1.f;
         atomicExch(fallback, 1);
     }
+    const bool search = !pairs || !bracket || fail || L.ovf[k];
+    L.need[k] = search ? 1 : 0;
+    if (pairs && bracket && search) atomicExch(again, 1);
 }
 
 // ---- big-node member order: k-d splits at leaf-aligned medians ----
@@ -2883,7 +3074,9 @@ __global__ void k_lvl_l2(LevelBufs L, NodeArrays nd, double f, int sub_n, rs_dev
     found = __syncthreads_or(found);
     if (threadIdx.x == 0) {
         if (!found) dev_fail(st, DEV_INTERNAL, 50, node);
-        nd.lnk[node] = L.l2[k];  // k_tree_stats makes it a length
+        const double l2 = L.l2[k];
+        nd.lnk[node] = l2;  // k_tree_stats makes it a length
+        L.lim[k] = make_float2(fminf((float)(l2 * (1.0 - RS_BAND)), (float)(l2 * (1.0 - 3e-6))), link_part(l2));
     }
 }
 
@@ -3047,22 +3240,39 @@ size_t tree_bytes(int64_t M, int64_t cap)
 // warps per SM (rs_tuning::nn_blocks_per_sm = 5, 6 or 7, in units of eight)
 static rs_status launch_nn(rs_ctx *ctx, const char *name, int64_t T, const LevelBufs &L, const NodeArrays &nd,
                            const int64_t *bo, const BoxStore &boxes, const MemberStore &ms, const float *R2,
-                           const float *STOP, int redo_failed, int sub_n, float *dnn)
+                           const float *STOP, int redo_failed, int sub_n, int pairs, float *dnn)
 {
     const int64_t g = T * (TQ / 32) / NN_WARPS;
     switch (ctx->tune.nn_blocks_per_sm) {
     case 5:
-        RS_LAUNCH(ctx, name, k_bvh_nn<5>, g, NN_WARPS * 32, 0, L, nd, bo, boxes, ms, R2, STOP, redo_failed, sub_n, dnn,
-                  ctx->d_status);
+        RS_LAUNCH(ctx, name, k_bvh_nn<5>, g, NN_WARPS * 32, 0, L, nd, bo, boxes, ms, R2, STOP, redo_failed, sub_n,
+                  pairs, dnn, ctx->d_status);
         break;
     case 7:
-        RS_LAUNCH(ctx, name, k_bvh_nn<7>, g, NN_WARPS * 32, 0, L, nd, bo, boxes, ms, R2, STOP, redo_failed, sub_n, dnn,
-                  ctx->d_status);
+        RS_LAUNCH(ctx, name, k_bvh_nn<7>, g, NN_WARPS * 32, 0, L, nd, bo, boxes, ms, R2, STOP, redo_failed, sub_n,
+                  pairs, dnn, ctx->d_status);
         break;
     default:
-        RS_LAUNCH(ctx, name, k_bvh_nn<6>, g, NN_WARPS * 32, 0, L, nd, bo, boxes, ms, R2, STOP, redo_failed, sub_n, dnn,
-                  ctx->d_status);
+        RS_LAUNCH(ctx, name, k_bvh_nn<6>, g, NN_WARPS * 32, 0, L, nd, bo, boxes, ms, R2, STOP, redo_failed, sub_n,
+                  pairs, dnn, ctx->d_status);
     }
+    return RS_OK;
+}
+
+// the pair or the link search over tiles [t0, T): one warp per leaf, LK_WARPS
+// to a block, compiled for 24, 32 or 40 resident warps per SM
+// (rs_tuning::link_blocks_per_sm = 4, 5 or 6)
+template <bool PAIRS>
+static rs_status launch_link(rs_ctx *ctx, const char *name, int64_t t0, int64_t T, const LevelBufs &L,
+                             const NodeArrays &nd, const int64_t *bo, const BoxStore &boxes, const MemberStore &ms,
+                             int *uf, const PairList &pl)
+{
+    auto k24 = k_bvh_link<24, PAIRS>;
+    auto k32 = k_bvh_link<32, PAIRS>;
+    auto k40 = k_bvh_link<40, PAIRS>;
+    auto k = ctx->tune.link_blocks_per_sm == 4 ? k24 : (ctx->tune.link_blocks_per_sm == 6 ? k40 : k32);
+    RS_LAUNCH(ctx, name, k, (T - t0) * (TQ / 32) / LK_WARPS, LK_WARPS * 32, 0, L, nd, t0, bo, boxes, ms, uf, pl,
+              ctx->d_status);
     return RS_OK;
 }
 
@@ -3128,7 +3338,7 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
     int *ctr = q, *big_a = q + 16, *big_b = q + 16 + cap, *small_q = q + 16 + 2 * cap, *tiny_q = q + 16 + 3 * cap,
         *mid_q = q + 16 + 4 * cap, *warp_q = q + 16 + 5 * cap, *big_s = q + 16 + 6 * cap;
     // ctr: [0] big_a len, [1] big_b len, [2] small len, [3] small head, [4] band len,
-    // [6..7] bracket fallback flag, [8] tiny len, [9] tiny head, [10] k-d ranges,
+    // [6] pair-search nodes to link again, [7] bracket fallback flag, [8] tiny len, [9] tiny head, [10] k-d ranges,
     // [11] middle len, [12] middle head, [13] subset query list length,
     // [14] warp-tier len, [15] warp-tier head
     RS_CUDA(ctx, cudaMemsetAsync(ctr, 0, sizeof(int) * 16, ctx->stream));
@@ -3182,7 +3392,7 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
         RS_LAUNCH(ctx, "rf_lvl_tiles", k_lvl_tiles, K, 256, 0, (int)K, (const int64_t *)O.tile, tl, tl + T);
         // per-rank state
         size_t per = sizeof(MomAcc) + sizeof(Metric6) + 2 * sizeof(float4) + 2048 * sizeof(unsigned) +
-                     7 * sizeof(int) + sizeof(double) + 64;
+                     11 * sizeof(int) + sizeof(double) + 64;
         RS_WS(ctx, char, rk, WS_RF_ACC, (int64_t)(per * K + 4096));
         char *rp = rk;
         L.acc = carve<MomAcc>(rp, K);
@@ -3196,6 +3406,9 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
         L.tie = carve<int>(rp, K);
         L.sub_t = carve<unsigned>(rp, 2 * K);
         L.sub_cnt = carve<int>(rp, K);
+        L.lim = carve<float2>(rp, K);
+        L.need = carve<int>(rp, K);
+        L.ovf = carve<int>(rp, K);
         RS_CUDA(ctx, cudaMemsetAsync(rk, 0, (size_t)(rp - rk), ctx->stream));
         RS_WS(ctx, char, bandbuf, WS_RF_BAND, (int64_t)(LM * 16 + 64));
         char *bp = bandbuf;
@@ -3278,11 +3491,12 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
             ms.a = carve<float4>(sp2, M);
             ms.b = carve<float2>(sp2, M);
         }
-        RS_LAUNCH(ctx, "rf_bvh_leaves", k_bvh_leaves<false>, T, TQ, 0, L, nd, bo, boxes, ms,
-                  (const float4 *)wpos, (const float4 *)wvel, (const float *)nullptr, (int *)nullptr, (int *)nullptr,
-                  (int *)nullptr, ctx->d_status);
-        RS_LAUNCH(ctx, "rf_bvh_build", k_bvh_build<false>, K, 256, 0, L, nd, bo, boxes,
-                  (int *)nullptr, ctx->d_status);
+        const float *nof = nullptr;
+        int *noi = nullptr;
+        RS_LAUNCH(ctx, "rf_bvh_leaves", k_bvh_leaves<BOX_ALL>, T, TQ, 0, L, nd, (int64_t)0, bo, boxes, ms,
+                  (const float4 *)wpos, (const float4 *)wvel, nof, nof, (float *)nullptr, noi, noi, noi, ctx->d_status);
+        RS_LAUNCH(ctx, "rf_bvh_build", k_bvh_build<BOX_ALL>, K, 256, 0, L, nd, bo, boxes, nof, nof, noi,
+                  ctx->d_status);
         // ---- random member subsets of the nodes above sub_n (Sec. 3.2) ----
         int2 *sub_q = nullptr;
         int *sub_len = ctr + 13;
@@ -3315,9 +3529,37 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
         RS_LAUNCH(ctx, "rf_smp_thresh", k_smp_thresh, K, 256, 0, L, nd, (const int *)O.smp_at, (const float *)sdnn, f,
                   R2, STOP);
         int *fallback = ctr + 7;
-        RS_CUDA(ctx, cudaMemsetAsync(ctr + 7, 0, sizeof(int), ctx->stream));
+        RS_CUDA(ctx, cudaMemsetAsync(ctr + 6, 0, 2 * sizeof(int), ctx->stream));
         // every member's nearest-neighbour distance, searched from the radius
-        RS_TRY(launch_nn(ctx, "rf_lvl_nn", T, L, nd, bo, boxes, ms, R2, STOP, 0, (int)sub_n, dnn));
+        // the nodes with a bracket: nearest neighbours and friends in one
+        // search, while the list of pairs stays within bounds
+        PairList pl{};
+        const int64_t chunks = LM * PAIR_PER_MEMBER / PAIR_CHUNK / PAIR_REGIONS + 4;  // per region
+        const int64_t pl_bytes = PAIR_REGIONS * chunks * (int64_t)(sizeof(int4) + PAIR_CHUNK * sizeof(int2));
+        int pairs = 0;
+        if (SS > 0 && pl_bytes <= PAIR_MAX_BYTES) {
+            char *pp = (char *)rs_ws(ctx, WS_RF_PAIRS, (size_t)pl_bytes + 1024);
+            if (pp) {  // (without the room the nodes are searched twice)
+                pairs = 1;
+                pl.len = carve<int>(pp, PAIR_REGIONS);
+                pl.head = carve<int4>(pp, PAIR_REGIONS * chunks);
+                pl.pair = carve<int2>(pp, PAIR_REGIONS * chunks * PAIR_CHUNK);
+                pl.cap = (int)chunks;
+                pl.R2 = R2;
+                pl.STOP = STOP;
+                pl.dnn = dnn;
+            }
+        }
+        if (pairs) {
+            RS_CUDA(ctx, cudaMemsetAsync(pl.len, 0, sizeof(int) * PAIR_REGIONS, ctx->stream));
+            RS_LAUNCH(ctx, "rf_pair_leaves", k_bvh_leaves<BOX_PAIRS>, T, TQ, 0, L, nd, (int64_t)0, bo, boxes, ms,
+                      (const float4 *)wpos, (const float4 *)wvel, (const float *)R2, (const float *)STOP, dnn, uf, csize,
+                      cmin, ctx->d_status);
+            RS_LAUNCH(ctx, "rf_pair_build", k_bvh_build<BOX_PAIRS>, K, 256, 0, L, nd, bo, boxes, (const float *)R2,
+                      (const float *)STOP, uf, ctx->d_status);
+            RS_TRY(launch_link<true>(ctx, "rf_lvl_pairs", 0, T, L, nd, bo, boxes, ms, uf, pl));
+        }
+        RS_TRY(launch_nn(ctx, "rf_lvl_nn", T, L, nd, bo, boxes, ms, R2, STOP, 0, (int)sub_n, pairs, dnn));
         if (QN > 0)
             RS_LAUNCH(ctx, "rf_sub_nn", k_bvh_nn_list, ceil_div(QN, W_WARPS), W_WARPS * 32, 0, L, nd,
                       bo, boxes, ms, (const int2 *)sub_q, (const int *)sub_len, (int)qcap, dnn,
@@ -3328,15 +3570,16 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
             RS_LAUNCH(ctx, "rf_lvl_pick", k_lvl_pick, K, 256, 0, L, pass);
         }
         RS_LAUNCH(ctx, "rf_bracket_check", k_bracket_check, ceil_div(K, 128), 128, 0, L, R2,
-                  (const float *)STOP, fallback, rs_fault("bracket") ? 1 : 0);
+                  (const float *)STOP, fallback, rs_fault("bracket") ? 1 : 0, pairs, ctr + 6);
         RS_LAUNCH(ctx, "rf_lvl_band", k_lvl_band, T, TQ, 0, L, nd, (const float *)dnn);
-        // ctr[4]: band members; ctr[7]: some node's bracket did not hold
+        // ctr[4]: band members; ctr[6]: a node of the pair search needs the link
+        // search; ctr[7]: some node's bracket did not hold
         int64_t flags[2];
         RS_TRY(rs_read_i64(ctx, ctr + 4, 2, flags, "rs_refine6d"));
         if ((flags[1] >> 32) != 0) {
             // unbounded search of those nodes (the others keep their values
             // and selection), and the band once more
-            RS_TRY(launch_nn(ctx, "rf_lvl_nn_full", T, L, nd, bo, boxes, ms, R2, nullptr, 1, (int)sub_n, dnn));
+            RS_TRY(launch_nn(ctx, "rf_lvl_nn_full", T, L, nd, bo, boxes, ms, R2, nullptr, 1, (int)sub_n, 0, dnn));
             RS_LAUNCH(ctx, "rf_lvl_initk", k_lvl_initk, ceil_div(K, 128), 128, 0, L, nd, f, (int)sub_n);
             for (int pass = 0; pass < 3; pass++) {
                 RS_LAUNCH(ctx, "rf_lvl_hist", k_lvl_hist, T, TQ, 0, L, nd, (const float *)dnn, pass);
@@ -3352,29 +3595,19 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
         RS_LAUNCH(ctx, "rf_lvl_band_exact", k_lvl_band_exact, ceil_div(nbv, W_WARPS), W_WARPS * 32, 0, L, nd,
                   bo, boxes, ms, (const float *)dnn, ctx->d_status);
         RS_LAUNCH(ctx, "rf_lvl_l2", k_lvl_l2, K, 128, 0, L, nd, f, (int)sub_n, ctx->d_status);
-        RS_LAUNCH(ctx, "rf_link_leaves", k_bvh_leaves<true>, T, TQ, 0, L, nd, bo, boxes, ms,
-                  (const float4 *)wpos, (const float4 *)wvel, (const float *)dnn, uf, csize, cmin, ctx->d_status);
-        RS_LAUNCH(ctx, "rf_link_build", k_bvh_build<true>, K, 256, 0, L, nd, bo, boxes, uf,
+        if (pairs)
+            RS_LAUNCH(ctx, "rf_pair_link", k_pair_link, (int64_t)ctx->num_sms * 8, 256, 0, L, nd, ms, pl, uf,
+                      ctx->d_status);
+        // the other nodes: with every bracket kept and every list whole, the
+        // tiles of the nodes of more than two k-d rounds (all above 4096
+        // members, so all bracketed) need not be looked at
+        const bool again = (flags[1] & 0xffffffffll) != 0;
+        const int64_t t0 = pairs && !again && sub_n == 0 && ctx->tune.bracket_min <= 4096 ? tot[LT_ROUND0 + 3 * 2] : 0;
+        RS_LAUNCH(ctx, "rf_link_leaves", k_bvh_leaves<BOX_LINK>, T - t0, TQ, 0, L, nd, t0, bo, boxes, ms,
+                  (const float4 *)wpos, (const float4 *)wvel, nof, nof, dnn, uf, csize, cmin, ctx->d_status);
+        RS_LAUNCH(ctx, "rf_link_build", k_bvh_build<BOX_LINK>, K, 256, 0, L, nd, bo, boxes, nof, nof, uf,
                   ctx->d_status);
-        {
-            // one warp per leaf job, LK_WARPS to a block; compiled for 24, 32
-            // or 40 resident warps per SM (rs_tuning::link_blocks_per_sm = 4,
-            // 5 or 6)
-            const int64_t njobs = T * (TQ / 32), lg = ceil_div(njobs, LK_WARPS);
-            switch (ctx->tune.link_blocks_per_sm) {
-            case 4:
-                RS_LAUNCH(ctx, "rf_lvl_link", k_bvh_link<24>, lg, LK_WARPS * 32, 0, L, nd, bo, boxes,
-                          ms, uf, ctx->d_status);
-                break;
-            case 6:
-                RS_LAUNCH(ctx, "rf_lvl_link", k_bvh_link<40>, lg, LK_WARPS * 32, 0, L, nd, bo, boxes,
-                          ms, uf, ctx->d_status);
-                break;
-            default:
-                RS_LAUNCH(ctx, "rf_lvl_link", k_bvh_link<32>, lg, LK_WARPS * 32, 0, L, nd, bo, boxes,
-                          ms, uf, ctx->d_status);
-            }
-        }
+        RS_TRY(launch_link<false>(ctx, "rf_lvl_link", t0, T, L, nd, bo, boxes, ms, uf, PairList{}));
         RS_LAUNCH(ctx, "rf_lvl_comp", k_lvl_comp, T, TQ, 0, L, nd, (const int *)widx, uf, csize, cmin,
                   ctx->d_status);
         // reorder: children first, by smallest particle index, then the rest
