@@ -97,9 +97,9 @@ __global__ void k_refine_init(int64_t G, int *gred, int *gmin, int nmax, double 
 }
 
 // group of member slot m (off[g] <= base + m < off[g + 1])
-__device__ __forceinline__ int64_t group_of(const int64_t *off, int64_t G, int64_t at)
+__device__ __forceinline__ int64_t group_of(const int64_t *off, int64_t lo, int64_t hi, int64_t at)
 {
-    int64_t lo = 0, hi = G;  // off[lo] <= at < off[hi]
+    // off[lo] <= at < off[hi]
     while (hi - lo > 1) {
         const int64_t mid = (lo + hi) >> 1;
         if (off[mid] <= at) lo = mid;
@@ -112,23 +112,37 @@ __device__ __forceinline__ int64_t group_of(const int64_t *off, int64_t G, int64
 // and axis the minima of x and -x, unshifted and with the upper half of the
 // box shifted down by the box, and the smallest particle index.  Lanes of
 // one group (groups are contiguous runs of slots) combine before their
-// atomics, kept on order-preserving integer images of the floats.
+// atomics, kept on order-preserving integer images of the floats, and an
+// atomic that would change nothing is left out.  The positions go to the
+// member slots here, so k_gather gathers the velocities only; the group is
+// searched for a warp's first and last slot and, where they differ, between
+// (134M path: 6.6 -> 5.1 ms, k_gather 2.2 -> 1.3).
 __global__ void k_unwrap_tiles(int64_t G, const int64_t *off, const int32_t *perm, int64_t n, int64_t M,
                                const float *pos, int stride, float boxf, int *slot_group, int *gred, int *gmin,
-                               rs_dev_status *st)
+                               float4 *wpos, int *widx, rs_dev_status *st)
 {
     const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t mw = m & ~31ll;
+    if (mw >= M) return;
     const bool ok = m < M;
+    const int64_t at0 = off[0];
+    int64_t g0 = 0, g1 = 0;
+    if (lane_id() == 0) g0 = group_of(off, 0, G, at0 + mw);
+    g0 = __shfl_sync(0xffffffffu, g0, 0);
+    if (lane_id() == 0) g1 = off[g0 + 1] > at0 + min(mw + 31, M - 1) ? g0 : group_of(off, g0, G, at0 + min(mw + 31, M - 1));
+    g1 = __shfl_sync(0xffffffffu, g1, 0);
     int g = -1, i = 0x7fffffff;
     float r[12];
     for (int k = 0; k < 12; k++) r[k] = INFINITY;
     if (ok) {
-        g = (int)group_of(off, G, off[0] + m);
+        g = (int)(g0 == g1 ? g0 : group_of(off, g0, g1 + 1, at0 + m));
         slot_group[m] = g;
-        i = perm[off[0] + m];
+        i = perm[at0 + m];
         if (i < 0 || i >= n) {
             dev_fail(st, DEV_BADARG, 33, m);
             i = 0x7fffffff;
+            wpos[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+            widx[m] = 0;
         } else {
             float c[3];
             load3(pos, stride, i, c[0], c[1], c[2]);
@@ -139,6 +153,8 @@ __global__ void k_unwrap_tiles(int64_t G, const int64_t *off, const int32_t *per
                 r[6 + d] = sft;
                 r[9 + d] = -sft;
             }
+            wpos[m] = make_float4(c[0], c[1], c[2], 0.f);
+            widx[m] = i;
         }
     }
     const unsigned grp = __match_any_sync(0xffffffffu, g);
@@ -147,8 +163,9 @@ __global__ void k_unwrap_tiles(int64_t G, const int64_t *off, const int32_t *per
     for (int k = 0; k < 12; k++) v[k] = __reduce_min_sync(grp, ord_i(r[k]));
     const int mi = (int)__reduce_min_sync(grp, (unsigned)i);
     if (ok && lane_id() == lead) {
-        for (int k = 0; k < 12; k++) atomicMin(&gred[12 * (int64_t)g + k], v[k]);
-        atomicMin(&gmin[g], mi);
+        for (int k = 0; k < 12; k++)
+            if (v[k] < __ldcg(&gred[12 * (int64_t)g + k])) atomicMin(&gred[12 * (int64_t)g + k], v[k]);
+        if (mi < __ldcg(&gmin[g])) atomicMin(&gmin[g], mi);
     }
 }
 
@@ -173,24 +190,22 @@ __global__ void k_unwrap_bits(int64_t G, const int *gred, float boxf, int *shift
     shift_bits[g] = bits;
 }
 
-__global__ void k_gather(int64_t M, const int64_t *off, const int32_t *perm, int64_t n, const float *pos,
-                         const float *vel, int stride, float boxf, const int *slot_group, const int *shift_bits,
-                         float4 *wpos, float4 *wvel, int *widx)
+// the members' velocities to their slots, and their groups' unwrap
+__global__ void k_gather(int64_t M, const float *vel, int stride, float boxf, const int *slot_group,
+                         const int *shift_bits, float4 *wpos, float4 *wvel, const int *widx)
 {
     const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= M) return;
     const int bits = shift_bits[slot_group[m]];
-    int i = perm[off[0] + m];
-    if (i < 0 || i >= n) i = 0;  // recorded by k_unwrap_tiles
-    float x, y, z, u, v, w;
-    load3(pos, stride, i, x, y, z);
-    load3(vel, stride, i, u, v, w);
-    if ((bits & 1) && x >= 0.5f * boxf) x = x - boxf;
-    if ((bits & 2) && y >= 0.5f * boxf) y = y - boxf;
-    if ((bits & 4) && z >= 0.5f * boxf) z = z - boxf;
-    wpos[m] = make_float4(x, y, z, 0.f);
+    float u, v, w;
+    load3(vel, stride, widx[m], u, v, w);
     wvel[m] = make_float4(u, v, w, 0.f);
-    widx[m] = i;
+    if (!bits) return;
+    float4 p = wpos[m];
+    if ((bits & 1) && p.x >= 0.5f * boxf) p.x = p.x - boxf;
+    if ((bits & 2) && p.y >= 0.5f * boxf) p.y = p.y - boxf;
+    if ((bits & 4) && p.z >= 0.5f * boxf) p.z = p.z - boxf;
+    wpos[m] = p;
 }
 
 __global__ void k_check_offsets(int64_t G, const int64_t *off, rs_dev_status *st)
@@ -3347,11 +3362,11 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
     RS_LAUNCH(ctx, "rf_init", k_refine_init, ceil_div(std::max<int64_t>(12 * G, SMALL_N + 1), 256), 256, 0, G, gred,
               gmin, SMALL_N, f, size_tab);
     RS_LAUNCH(ctx, "rf_group_unwrap", k_unwrap_tiles, ceil_div(M, 256), 256, 0, G, goff, perm, n, M, pos, stride,
-              boxf, slot_group, gred, gmin, ctx->d_status);
+              boxf, slot_group, gred, gmin, wpos, widx, ctx->d_status);
     RS_LAUNCH(ctx, "rf_unwrap_bits", k_unwrap_bits, ceil_div(G, 256), 256, 0, G, (const int *)gred, boxf, shift_bits,
               ctx->d_status);
-    RS_LAUNCH(ctx, "rf_gather", k_gather, ceil_div(M, 256), 256, 0, M, goff, perm, n, pos, vel, stride, boxf,
-              (const int *)slot_group, (const int *)shift_bits, wpos, wvel, widx);
+    RS_LAUNCH(ctx, "rf_gather", k_gather, ceil_div(M, 256), 256, 0, M, vel, stride, boxf, (const int *)slot_group,
+              (const int *)shift_bits, wpos, wvel, (const int *)widx);
     RS_LAUNCH(ctx, "rf_roots", k_make_roots, ceil_div(G, 256), 256, 0, G, goff, (const int *)gmin,
               (const int *)shift_bits, (int)min_n, nd,
               big_a, ctr + 0, small_q, ctr + 2, ctx->d_status);
