@@ -116,7 +116,7 @@ __device__ __forceinline__ int64_t group_of(const int64_t *off, int64_t lo, int6
 // atomic that would change nothing is left out.  The positions go to the
 // member slots here, so k_gather gathers the velocities only; the group is
 // searched for a warp's first and last slot and, where they differ, between
-// (134M path: 6.6 -> 5.1 ms, k_gather 2.2 -> 1.3).
+// (134M path: 6.6 -> 5.0 ms, k_gather 2.2 -> 1.3).
 __global__ void k_unwrap_tiles(int64_t G, const int64_t *off, const int32_t *perm, int64_t n, int64_t M,
                                const float *pos, int stride, float boxf, int *slot_group, int *gred, int *gmin,
                                float4 *wpos, int *widx, rs_dev_status *st)
@@ -1260,26 +1260,36 @@ __global__ void k_lvl_tiles(int K, const int64_t *tile_off, int *tile_rank, int 
     }
 }
 
+// Four members a thread before the warp sums (the blocks of every fourth tile
+// work): the sums' instructions, not the members' bytes, are what this costs
+// (134M path, 7 levels: 5.4 -> 2.2 ms).
 __global__ void __launch_bounds__(TQ) k_lvl_moments(LevelBufs L, NodeArrays nd, const float4 *wpos,
                                                     const float4 *wvel)
 {
     const int k = L.tile_rank[blockIdx.x], q0 = L.tile_q0[blockIdx.x];
+    if (q0 & (4 * TQ - 1)) return;
     const int node = L.list[k], first = nd.first[node], n = nd.count[node];
     const float4 pref = wpos[first], vref = wvel[first];
     MomRef ref = mom_ref(pref, vref);
     MomAcc a;
     mom_zero(a);
-    int q = q0 + threadIdx.x;
-    if (q < n) mom_add(a, wpos[first + q], wvel[first + q], ref);
+#pragma unroll 1
+    for (int q = q0 + threadIdx.x; q < min(n, q0 + 4 * TQ); q += TQ) mom_add(a, wpos[first + q], wvel[first + q], ref);
     mom_warp_reduce(a);
     __shared__ MomAcc w[TQ / 32];
     if (lane_id() == 0) w[warp_id()] = a;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        MomAcc t = w[0];
-        for (int i = 1; i < TQ / 32; i++) mom_merge(t, w[i]);
-        mom_atomic_add(&L.acc[k], t);
-        if (q0 == 0) {
+    // a lane a sum
+    if (threadIdx.x < 8) {
+        const int j = threadIdx.x, lo_at = j < 6 ? j : 2 * j, hi_at = j < 6 ? j + 6 : 2 * j + 1;
+        unsigned long long lo = 0, hi = 0;
+        for (int i = 0; i < TQ / 32; i++) {
+            const unsigned long long *v = reinterpret_cast<const unsigned long long *>(&w[i]);
+            add128(lo, hi, v[lo_at], v[hi_at]);
+        }
+        unsigned long long *g = reinterpret_cast<unsigned long long *>(&L.acc[k]);
+        atomic_add128(g + lo_at, g + hi_at, lo, hi);
+        if (j == 0 && q0 == 0) {
             L.ref[2 * k] = pref;
             L.ref[2 * k + 1] = vref;
         }
