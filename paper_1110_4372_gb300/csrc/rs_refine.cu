@@ -3741,14 +3741,27 @@ __global__ void k_tree_export(NodeArrays nd, int nn, int32_t *parent, int32_t *l
     }
 }
 
-__global__ void k_level_labels(NodeArrays nd, int nn, int level, const int *members, int32_t *labels)
+// A warp looks at 32 nodes at once; LABEL_SPLIT rows of warps share the nodes,
+// and the members of the nodes above 1024 (9.6M members, 8 levels: 1.36
+// ms with a warp a node, 0.63 so).
+constexpr int LABEL_SPLIT = 16;
+
+__global__ void __launch_bounds__(256) k_level_labels(NodeArrays nd, int nn, int level, const int *members,
+                                                      int32_t *labels)
 {
+    const int lane = lane_id(), y = blockIdx.y;
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int i = w; i < nn; i += nw) {
-        if (nd.level[i] != level) continue;
-        const int a = nd.first[i], c = nd.count[i], id = nd.minidx[i];
-        for (int m = lane_id(); m < c; m += 32) labels[members[a + m]] = id;
+    const int i = 32 * w + lane;
+    const bool hit = i < nn && nd.level[i] == level;
+    const int a0 = hit ? nd.first[i] : 0, c0 = hit ? nd.count[i] : 0, id0 = hit ? nd.minidx[i] : 0;
+    unsigned m = __ballot_sync(0xffffffffu, hit && (c0 > 1024 || (lane & (LABEL_SPLIT - 1)) == y));
+    while (m) {
+        const int s = __ffs(m) - 1;
+        m &= m - 1;
+        const int a = __shfl_sync(0xffffffffu, a0, s), c = __shfl_sync(0xffffffffu, c0, s),
+                  id = __shfl_sync(0xffffffffu, id0, s);
+        const int rows = c > 1024 ? LABEL_SPLIT : 1;
+        for (int q = 32 * (rows > 1 ? y : 0) + lane; q < c; q += 32 * rows) labels[members[a + q]] = id;
     }
 }
 
@@ -3862,7 +3875,13 @@ extern "C" rs_status rs_tree_level_labels(rs_ctx *ctx, const rs_tree *t, int32_t
     if (n == 0) return RS_OK;
     RS_LAUNCH(ctx, "tree_fill", k_fill_i32, std::min<int64_t>(ceil_div(n, 256), 4096), 256, 0, labels, n, -1);
     const int nn = (int)t->n_nodes;
-    RS_LAUNCH(ctx, "tree_level_labels", k_level_labels, std::min<int64_t>(ceil_div((int64_t)nn * 32, 256), 8192),
-              256, 0, t->nd, nn, level, (const int *)t->members, labels);
+    if (nn > 0) {
+        const dim3 grid((unsigned)ceil_div(nn, 256), LABEL_SPLIT);
+        const int pr = rs_prof_begin(ctx, "tree_level_labels");
+        k_level_labels<<<grid, 256, 0, ctx->stream>>>(t->nd, nn, level, (const int *)t->members, labels);
+        ctx->launches++;
+        rs_prof_end(ctx, pr);
+        RS_CUDA(ctx, cudaGetLastError());
+    }
     return RS_OK;
 }
