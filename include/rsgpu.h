@@ -99,8 +99,9 @@ const char *rs_last_error(const rs_ctx *ctx);
  *                       of eight (5, 6 or 7: 40, 48 or 56 warps);
  *   kd_levels           big-node levels whose members are put in k-d order
  *                       (0-3; deeper levels keep their parent's order);
- *   bracket_min         big nodes above this many members search with the
- *                       sampled bracket of the linking length (>= 1024);
+ *   bracket_min         big nodes above this many members sample 1024 of
+ *                       them for the bracket of the linking length, the
+ *                       others 256 (>= 1024);
  *   mid_max             subtrees of at most this many members run in the
  *                       128-thread tier, and below 128 in the one-warp tier
  *                       (33-256); larger ones up to 1024 run in the

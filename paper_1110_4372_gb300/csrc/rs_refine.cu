@@ -1154,7 +1154,15 @@ __host__ __device__ __forceinline__ int kd_rounds(int64_t m, int limit)
 
 constexpr int KD_CTA = 1024;  // ranges of at most this many members finish in one CTA
 
-constexpr int SMP_MAX = 1024;  // sample size of a node's search bracket
+// Sample size of a node's search bracket: SMP_MAX above
+// rs_tuning::bracket_min members (4096 by default), a quarter of it below.  A
+// quarter costs up to a quarter of a small node's searches and gives twice as
+// wide a bracket, but without one the node takes a search a member and a
+// second one a leaf (2M path: the rest of the level's searches 1.3 -> 0.2 ms,
+// the whole path 7.2 -> 6.0; 9.6M grouped members 42.0 -> 39.0).
+constexpr int SMP_MAX = 1024;
+constexpr int SMP_UNIT = SMP_MAX / 4;
+__device__ __forceinline__ int smp_units(int n, int bracket_min) { return n > bracket_min ? SMP_MAX / SMP_UNIT : 1; }
 
 // Per-rank offsets of one level (K + 1 entries each, the last the total)
 struct LevelOff {
@@ -1162,8 +1170,8 @@ struct LevelOff {
     int64_t *seg;    // members
     int64_t *box;    // hierarchy boxes
     int64_t *block;  // blocks of KD_CTA members
-    int *smp;        // ranks of the nodes searched with a sampled bracket
-    int *smp_at;     // per rank: its place there, or -1
+    int *smp;        // per SMP_UNIT samples: the rank of their node
+    int *smp_at;     // per rank: its first unit of samples, or -1
 };
 
 constexpr int KD_MAXR = 16;   // kd_rounds(2^26, KD_CTA) and more
@@ -1204,20 +1212,21 @@ __global__ void __launch_bounds__(1024) k_lvl_setup(const int *raw, const int *l
         const bool ok = i < K;
         const int n = ok ? nd.count[list[i]] : 0;
         if (ok && sub_n > 0 && n > sub_n) atomicAdd(&nsub, 1);
-        const bool smp = ok && n > bracket_min && !(sub_n > 0 && n > sub_n);
+        const bool smp = ok && !(sub_n > 0 && n > sub_n);
+        const int units = smp ? smp_units(n, bracket_min) : 0;
         long long s0, s1, s2, s3, s4;
         const long long v0 = rs_block_scan<1024, long long>(ceil_div(n, TQ), s0);
         const long long v1 = rs_block_scan<1024, long long>(n, s1);
         const long long v2 = rs_block_scan<1024, long long>(ok ? bvh_total((int)ceil_div(n, BVH_LEAF)) : 0, s2);
         const long long v3 = rs_block_scan<1024, long long>(ceil_div(n, KD_CTA), s3);
-        const long long v4 = rs_block_scan<1024, long long>(smp ? 1 : 0, s4);
+        const long long v4 = rs_block_scan<1024, long long>(units, s4);
         if (ok) {
             O.tile[i] = c0 + v0;
             O.seg[i] = c1 + v1;
             O.box[i] = c2 + v2;
             O.block[i] = c3 + v3;
             O.smp_at[i] = smp ? (int)(c4 + v4) : -1;
-            if (smp) O.smp[c4 + v4] = i;
+            for (int u = 0; u < units; u++) O.smp[c4 + v4 + u] = i;
         }
         c0 += s0;
         c1 += s1;
@@ -1834,16 +1843,17 @@ __global__ void __launch_bounds__(NN_WARPS * 32, MINB * W_WARPS / NN_WARPS)
 // nearest-neighbour distance of single sampled members, one warp each
 __global__ void __launch_bounds__(W_WARPS * 32) k_bvh_nn_sample(LevelBufs L, NodeArrays nd, const int64_t *box_base,
                                                                 BoxStore B, MemberStore MS, const int *smp,
-                                                                float *out, rs_dev_status *st)
+                                                                const int *smp_at, int bracket_min, float *out,
+                                                                rs_dev_status *st)
 {
     __shared__ int si_s[W_WARPS][W_STACK];
     __shared__ float sd_s[W_WARPS][W_STACK];
     __shared__ int lv_s[W_WARPS][2 * BVH_MAXH];
     const int w = warp_id(), lane = lane_id();
     const int64_t at = (int64_t)blockIdx.x * W_WARPS + w;  // the grid holds exactly the samples
-    const int k = smp[at / SMP_MAX], s = (int)(at % SMP_MAX);
+    const int k = smp[at / SMP_UNIT], s = (int)(at - (int64_t)smp_at[k] * SMP_UNIT);
     const int node = L.list[k], first = nd.first[node], n = nd.count[node];
-    const int q = (int)(((int64_t)s * n) / SMP_MAX);
+    const int q = (int)(((int64_t)s * n) / (SMP_UNIT * smp_units(n, bracket_min)));
     const Metric6 met = L.met[k];
     BvhView V;
     bvh_view(V, B, box_base[k], n, lv_s[w]);
@@ -2422,21 +2432,20 @@ __global__ void __launch_bounds__(256) k_pair_link(LevelBufs L, NodeArrays nd, M
 // stop early with "none within t_hi".  Only values up to the k-th are needed
 // for the linking length; if the k-th value is not within t_hi the level
 // falls back to the unbounded search, so the result is always exact.
-// (nodes of at most rs_tuning::bracket_min members, 4096 by default, and nodes
-// that draw a member subset for the linking length are searched without one)
+// (nodes that draw a member subset for the linking length are searched without
+// one)
 
 // bracket of the search from the sample: the radius R2 is the sample's
 // quantile at f + 5 sigma widened by 16 band widths; the stop value is the
 // quantile at f - 5 sigma narrowed by 16 band widths (a member with a
 // neighbour closer than it is certainly below the linking length)
-__global__ void k_smp_thresh(LevelBufs L, NodeArrays nd, const int *smp_at, const float *sdnn, double f, float *R2,
-                             float *STOP)
+__global__ void k_smp_thresh(LevelBufs L, NodeArrays nd, const int *smp_at, int bracket_min, const float *sdnn, double f,
+                             float *R2, float *STOP)
 {
     __shared__ float v[SMP_MAX];
     const int k = blockIdx.x;
     if (k >= L.K) return;
-    const int64_t a = (int64_t)smp_at[k] * SMP_MAX;
-    const int S = SMP_MAX;
+    const int64_t a = (int64_t)smp_at[k] * SMP_UNIT;
     if (a < 0) {  // not sampled: unbounded search, no early stop
         if (threadIdx.x == 0) {
             R2[k] = INFINITY;
@@ -2444,11 +2453,12 @@ __global__ void k_smp_thresh(LevelBufs L, NodeArrays nd, const int *smp_at, cons
         }
         return;
     }
-    for (int i = threadIdx.x; i < SMP_MAX; i += blockDim.x) v[i] = sdnn[a + i];
+    const int S = SMP_UNIT * smp_units(nd.count[L.list[k]], bracket_min);
+    for (int i = threadIdx.x; i < S; i += blockDim.x) v[i] = sdnn[a + i];
     __syncthreads();
-    for (int kk = 2; kk <= SMP_MAX; kk <<= 1)
+    for (int kk = 2; kk <= S; kk <<= 1)
         for (int j = kk >> 1; j > 0; j >>= 1) {
-            for (int t = threadIdx.x; t < SMP_MAX / 2; t += blockDim.x) {
+            for (int t = threadIdx.x; t < S / 2; t += blockDim.x) {
                 int i = 2 * j * (t / j) + (t % j), l = i + j;
                 bool up = (i & kk) == 0;
                 float x = v[i], y = v[l];
@@ -2479,7 +2489,7 @@ __global__ void k_smp_thresh(LevelBufs L, NodeArrays nd, const int *smp_at, cons
 // and of those with one the failed ones and those whose list overflowed
 // (*again set).
 __global__ void k_bracket_check(LevelBufs L, float *R2, const float *STOP, int *fallback, int force_odd, int pairs,
-                                int *again)
+                                const int *smp_at, int *again)
 {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= L.K) return;
@@ -2498,7 +2508,7 @@ __global__ void k_bracket_check(LevelBufs L, float *R2, const float *STOP, int *
     }
     const bool search = !pairs || !bracket || fail || L.ovf[k];
     L.need[k] = search ? 1 : 0;
-    if (pairs && bracket && search) atomicExch(again, 1);
+    if (search && smp_at[k] >= 0) atomicExch(again, 1);
 }
 
 // ---- big-node member order: k-d splits at leaf-aligned medians ----
@@ -3392,15 +3402,15 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
     int n_fallback_levels = 0;
     // per-rank offsets: a big node has more than SMALL_N members
     const int64_t kcap = M / SMALL_N + 2;
-    RS_WS(ctx, int64_t, lv64, WS_RF_MISC1, 5 * kcap + LT_WORDS + 8);
+    RS_WS(ctx, int64_t, lv64, WS_RF_MISC1, 7 * kcap + LT_WORDS + 8);
     LevelOff O;
     O.tile = lv64;
     O.seg = lv64 + kcap;
     O.box = lv64 + 2 * kcap;
     O.block = lv64 + 3 * kcap;
     O.smp = (int *)(lv64 + 4 * kcap);
-    O.smp_at = O.smp + kcap;
-    int64_t *dtot = lv64 + 5 * kcap;
+    O.smp_at = O.smp + (SMP_MAX / SMP_UNIT) * kcap;
+    int64_t *dtot = lv64 + 7 * kcap;
     for (int level = 0; level < 4096; level++) {
         RS_LAUNCH(ctx, "rf_lvl_setup", k_lvl_setup, 1, 1024, 0, (const int *)cur, (const int *)cur_len, big_s, nd, O,
                   (int)sub_n, (int)ctx->tune.bracket_min, dtot);
@@ -3552,14 +3562,14 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
             RS_LAUNCH(ctx, "rf_sub_check", k_sub_check, ceil_div(K, 128), 128, 0, L, nd, (int)sub_n, ctx->d_status);
         }
         // ---- linking length: sampled bracket, bounded nearest neighbours, exact select ----
-        const int64_t SS = tot[LT_SMP] * SMP_MAX;
+        const int64_t SS = tot[LT_SMP] * SMP_UNIT;
         RS_WS(ctx, float, sdnn, WS_RF_SDNN, SS + 32);
         RS_WS(ctx, float, R2, WS_RF_R2, 2 * K + 8);
         float *STOP = R2 + K;
         RS_LAUNCH(ctx, "rf_smp_nn", k_bvh_nn_sample, SS / W_WARPS, W_WARPS * 32, 0, L, nd, bo, boxes, ms,
-                  (const int *)O.smp, sdnn, ctx->d_status);
-        RS_LAUNCH(ctx, "rf_smp_thresh", k_smp_thresh, K, 256, 0, L, nd, (const int *)O.smp_at, (const float *)sdnn, f,
-                  R2, STOP);
+                  (const int *)O.smp, (const int *)O.smp_at, (int)ctx->tune.bracket_min, sdnn, ctx->d_status);
+        RS_LAUNCH(ctx, "rf_smp_thresh", k_smp_thresh, K, 256, 0, L, nd, (const int *)O.smp_at,
+                  (int)ctx->tune.bracket_min, (const float *)sdnn, f, R2, STOP);
         int *fallback = ctr + 7;
         RS_CUDA(ctx, cudaMemsetAsync(ctr + 6, 0, 2 * sizeof(int), ctx->stream));
         // every member's nearest-neighbour distance, searched from the radius
@@ -3602,7 +3612,8 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
             RS_LAUNCH(ctx, "rf_lvl_pick", k_lvl_pick, K, 256, 0, L, pass);
         }
         RS_LAUNCH(ctx, "rf_bracket_check", k_bracket_check, ceil_div(K, 128), 128, 0, L, R2,
-                  (const float *)STOP, fallback, rs_fault("bracket") ? 1 : 0, pairs, ctr + 6);
+                  (const float *)STOP, fallback, rs_fault("bracket") ? 1 : 0, pairs,
+                  (const int *)O.smp_at, ctr + 6);
         RS_LAUNCH(ctx, "rf_lvl_band", k_lvl_band, T, TQ, 0, L, nd, (const float *)dnn);
         // ctr[4]: band members; ctr[6]: a node of the pair search needs the link
         // search; ctr[7]: some node's bracket did not hold
@@ -3630,14 +3641,13 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
         if (pairs)
             RS_LAUNCH(ctx, "rf_pair_link", k_pair_link, (int64_t)ctx->num_sms * 8, 256, 0, L, nd, ms, pl, uf,
                       ctx->d_status);
-        // the other nodes: with every bracket kept and every list whole, the
-        // tiles of the nodes of more than two k-d rounds (all above 4096
-        // members, so all bracketed) need not be looked at
+        // the other nodes; none when every node has a bracket, every bracket
+        // held and every list was whole
         const bool again = (flags[1] & 0xffffffffll) != 0;
-        const int64_t t0 = pairs && !again && sub_n == 0 && ctx->tune.bracket_min <= 4096 ? tot[LT_ROUND0 + 3 * 2] : 0;
+        const int64_t t0 = pairs && !again && sub_n == 0 ? T : 0;
         RS_LAUNCH(ctx, "rf_link_leaves", k_bvh_leaves<BOX_LINK>, T - t0, TQ, 0, L, nd, t0, bo, boxes, ms,
                   (const float4 *)wpos, (const float4 *)wvel, nof, nof, dnn, uf, csize, cmin, ctx->d_status);
-        RS_LAUNCH(ctx, "rf_link_build", k_bvh_build<BOX_LINK>, K, 256, 0, L, nd, bo, boxes, nof, nof, uf,
+        RS_LAUNCH(ctx, "rf_link_build", k_bvh_build<BOX_LINK>, t0 < T ? K : 0, 256, 0, L, nd, bo, boxes, nof, nof, uf,
                   ctx->d_status);
         RS_TRY(launch_link<false>(ctx, "rf_lvl_link", t0, T, L, nd, bo, boxes, ms, uf, PairList{}));
         RS_LAUNCH(ctx, "rf_lvl_comp", k_lvl_comp, T, TQ, 0, L, nd, (const int *)widx, uf, csize, cmin,

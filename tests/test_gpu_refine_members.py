@@ -41,6 +41,24 @@ def test_group_members_match_oracle(sizes, skip, stride):
     compare_trees(gpu_tree_dict(tree), oracle_tree_dict(o), box)
 
 
+@pytest.mark.parametrize("n,f,bracket_min", [(1025, 0.02, 4096), (1025, 0.99, 4096), (4096, 0.99, 4096),
+                                             (4097, 0.02, 4096), (9000, 0.7, 1 << 30), (1500, 0.98, 1024)])
+def test_sampled_brackets_match_oracle(n, f, bracket_min):
+    """Both sample sizes, where the bracket's quantiles are cut off at the
+    sample's ends (below the first or above the last value)."""
+    from paper_1110_4372_gb300 import rsgpu
+    rng = np.random.default_rng([n, bracket_min])
+    box = 20.0
+    pos = synth.wrap(rng.standard_normal((n, 3)) * 0.15, box)
+    vel = (rng.standard_normal((n, 3)) * 60.0).astype(np.float32)
+    perm, off = np.arange(n, dtype=np.int32), np.array([0, n], np.int64)
+    ctx = rsgpu.Context()
+    rsgpu.rs_set_tuning(ctx, bracket_min=bracket_min)
+    tree = rsgpu.rs_refine6d(ctx, *(torch.from_numpy(a).cuda() for a in (pos, vel)), box,
+                             torch.from_numpy(perm).cuda(), torch.from_numpy(off).cuda(), f)
+    compare_trees(gpu_tree_dict(tree), oracle_tree_dict(oracle.refine(pos, vel, box, perm, off, f)), box)
+
+
 @pytest.mark.parametrize("bad", [-1, 500])
 def test_index_out_of_range_is_an_error(bad):
     from paper_1110_4372_gb300 import rsgpu
