@@ -1318,6 +1318,11 @@ __global__ void k_lvl_finalize(LevelBufs L, NodeArrays nd, double box)
     nd.sigx[node] = o.sigx;
     nd.sigv[node] = o.sigv;
     L.met[k] = metric_of(o.sigx, o.sigv);
+    // the k-d order's scales, here and not in its kernels: two float64 divides
+    // a member and round were what k_kd_keys spent its time on (134M path:
+    // 12.4 -> 4.6 ms)
+    L.ref[2 * k].w = o.sigx > 0 ? (float)(1.0 / o.sigx) : 0.f;
+    L.ref[2 * k + 1].w = o.sigv > 0 ? (float)(1.0 / o.sigv) : 0.f;
 }
 
 // ---- raw-coordinate boxes ----
@@ -2522,9 +2527,9 @@ __global__ void k_bracket_check(LevelBufs L, float *R2, const float *STOP, int *
 // of all members by (segment, 16-bit coordinate), the coordinate relative to
 // the node's reference member in units of its dispersion.
 // 16-bit coordinate of a member on an axis (x, vx, y, vy, z, vz), relative to
-// the node's reference member in units of its dispersion
+// the node's reference member in units of its dispersion (.w: one over it)
 __device__ __forceinline__ unsigned kd_coord(const float4 *wpos, const float4 *wvel, unsigned slot, int axis,
-                                             float4 pref, float4 vref, float ix, float iv)
+                                             float4 pref, float4 vref)
 {
     const int d = axis >> 1;
     float c, r, inv;
@@ -2532,12 +2537,12 @@ __device__ __forceinline__ unsigned kd_coord(const float4 *wpos, const float4 *w
         const float4 a = wpos[slot];
         c = d == 0 ? a.x : (d == 1 ? a.y : a.z);
         r = d == 0 ? pref.x : (d == 1 ? pref.y : pref.z);
-        inv = ix;
+        inv = pref.w;
     } else {
         const float4 a = wvel[slot];
         c = d == 0 ? a.x : (d == 1 ? a.y : a.z);
         r = d == 0 ? vref.x : (d == 1 ? vref.y : vref.z);
-        inv = iv;
+        inv = vref.w;
     }
     const float u = ((c - r) * inv + 12.f) * (65536.f / 24.f);
     return (unsigned)fminf(fmaxf(u, 0.f), 65535.f);
@@ -2568,9 +2573,7 @@ __global__ void k_kd_keys(LevelBufs L, NodeArrays nd, const int64_t *seg_base, c
     }
     unsigned qv = 0;
     if (size > KD_CTA) {
-        const float ix = nd.sigx[node] > 0 ? (float)(1.0 / nd.sigx[node]) : 0.f;
-        const float iv = nd.sigv[node] > 0 ? (float)(1.0 / nd.sigv[node]) : 0.f;
-        qv = kd_coord(wpos, wvel, slot, round % 6, L.ref[2 * k], L.ref[2 * k + 1], ix, iv);
+        qv = kd_coord(wpos, wvel, slot, round % 6, L.ref[2 * k], L.ref[2 * k + 1]);
     }
     // Key: (block of KD_CTA members holding the range's start, coordinate).
     // A range still being split has more than KD_CTA members, so it is the
@@ -2713,10 +2716,7 @@ __global__ void __launch_bounds__(256) k_kd_finish(LevelBufs L, NodeArrays nd, c
     for (int ri = blockIdx.x; ri < nr; ri += gridDim.x) {
         const int4 rg = ranges[ri];
         const int k = rg.x, s0 = rg.y, m = rg.z, d0 = rg.w;
-        const int node = L.list[k];
         const int64_t P0 = L.seg_off[k] + s0;
-        const float ix = nd.sigx[node] > 0 ? (float)(1.0 / nd.sigx[node]) : 0.f;
-        const float iv = nd.sigv[node] > 0 ? (float)(1.0 / nd.sigv[node]) : 0.f;
         const float4 pref = L.ref[2 * k], vref = L.ref[2 * k + 1];
         const int R = kd_rounds(m, 32);
         for (int i = tid; i < m; i += blockDim.x) slot[i] = vals[P0 + i];
@@ -2724,7 +2724,7 @@ __global__ void __launch_bounds__(256) k_kd_finish(LevelBufs L, NodeArrays nd, c
         for (int r = 0; r < R; r++) {
             const int axis = (d0 + r) % 6;
             for (int i = tid; i < m; i += blockDim.x)
-                key[i] = (unsigned short)kd_coord(wpos, wvel, slot[i], axis, pref, vref, ix, iv);
+                key[i] = (unsigned short)kd_coord(wpos, wvel, slot[i], axis, pref, vref);
             __syncthreads();
             kdf_rank(m, key, rk[r], pm, wcnt, dstart, wsum);
         }
