@@ -203,6 +203,8 @@ rs_status rs_radix_sort_u64(rs_ctx *ctx, uint64_t *k0, uint64_t *k1, uint32_t *v
                             int nbits, bool *out_in_alt, const char *tag = "sort");
 rs_status rs_radix_sort_u32(rs_ctx *ctx, uint32_t *k0, uint32_t *k1, uint32_t *v0, uint32_t *v1, int64_t n,
                             int nbits, bool *out_in_alt, const char *tag = "sort");
+// whether a sort of n keys leaves its result in the second buffers
+bool rs_sort_alt(int64_t n, int nbits);
 
 // ---------------------------------------------------------------------------
 // Device helpers

@@ -2577,7 +2577,7 @@ __global__ void k_kd_keys(LevelBufs L, NodeArrays nd, const int64_t *seg_base, c
         ((unsigned *)kout)[A] = (unsigned)key;
     else
         kout[A] = key;
-    vout[A] = slot;
+    if (vout) vout[A] = slot;
 }
 
 // the current order before the rounds: every member in its own place
@@ -3475,17 +3475,19 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
                 while (sbits < 40 && (NS >> sbits) != 0) sbits++;
                 // 32-bit keys (half the bytes, fewer passes) while the blocks fit in 16 bits
                 const int key32 = 16 + sbits <= 32 ? 1 : 0;
+                // the order stays in place, or the sort's last pass writes it there
+                const bool odd = rs_sort_alt(NA, 16 + sbits);
+                unsigned *va = odd ? v0 : vcur, *vb = odd ? vcur : v1;
                 RS_LAUNCH(ctx, "rf_kd_keys", k_kd_keys, TA, TQ, 0, L, nd, (const int64_t *)O.block,
                           (const float4 *)wpos, (const float4 *)wvel, (const unsigned *)vcur,
-                          (unsigned long long *)k0, v0, r, key32);
+                          (unsigned long long *)k0, odd ? v0 : nullptr, r, key32);
                 bool kalt = false;
                 if (key32)
-                    RS_TRY(rs_radix_sort_u32(ctx, (uint32_t *)k0, (uint32_t *)k1, v0, v1, NA, 16 + sbits, &kalt,
+                    RS_TRY(rs_radix_sort_u32(ctx, (uint32_t *)k0, (uint32_t *)k1, va, vb, NA, 16 + sbits, &kalt,
                                              "sort_kd"));
                 else
-                    RS_TRY(rs_radix_sort_u64(ctx, k0, k1, v0, v1, NA, 16 + sbits, &kalt, "sort_kd"));
-                RS_CUDA(ctx, cudaMemcpyAsync(vcur, kalt ? v1 : v0, sizeof(unsigned) * NA, cudaMemcpyDeviceToDevice,
-                                             ctx->stream));
+                    RS_TRY(rs_radix_sort_u64(ctx, k0, k1, va, vb, NA, 16 + sbits, &kalt, "sort_kd"));
+                if (kalt != odd) return rs_fail(ctx, RS_ERR_INTERNAL, "rs_refine6d: k-d order");
             }
             // ranges of at most KD_CTA members finish in one CTA each
             const int64_t rcap = ceil_div(LM, 32) + K;

@@ -405,6 +405,12 @@ rs_status radix_sort(rs_ctx *ctx, K *k0, K *k1, uint32_t *v0, uint32_t *v1, int6
 
 }  // namespace
 
+bool rs_sort_alt(int64_t n, int nbits)
+{
+    if (n <= 1 || nbits <= 0) return false;
+    return n <= SORT_SMALL || ((nbits + RADIX_BITS - 1) / RADIX_BITS & 1);
+}
+
 rs_status rs_lookback_init(rs_ctx *ctx, int64_t tiles, RsLookback *lb)
 {
     unsigned long long *w = (unsigned long long *)rs_ws(ctx, WS_SCAN_TMP, sizeof(unsigned long long) * (tiles + 1));
