@@ -52,14 +52,9 @@ BYTES_LEVEL_PER_MEMBER = 28
 BYTES_ASSIGN_PER_MEMBER = 28
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per unit, from
-# one ncu capture of every launch of the kernel in one step of the 16.8M
-# workload (profiles/k_bvh_link_c3q_full.md, profiles/k_bvh_nn_c3q_full.md),
-# scaled to a step by the units processed.  An entry is dropped when its
-# kernel changes.
-NCU_TRAFFIC_PER_UNIT = {
-    "rf_lvl_link": 325757952 / 8612074,
-    "rf_lvl_nn": 241497088 / 8612074,
-}
+# an ncu capture of every launch of the kernel in one step, scaled to a step by
+# the units processed.  An entry is dropped when its kernel changes.
+NCU_TRAFFIC_PER_UNIT = {}
 
 # Which units each kernel processes per step (for its algorithmic bytes).
 KERNEL_UNITS = {
@@ -68,6 +63,7 @@ KERNEL_UNITS = {
     "rf_small_subtree": ("small_level_members", BYTES_LEVEL_PER_MEMBER),
     "rf_lvl_nn": ("big_level_members", BYTES_LEVEL_PER_MEMBER),
     "rf_lvl_link": ("big_level_members", BYTES_LEVEL_PER_MEMBER),
+    "rf_lvl_pairs": ("big_level_members", BYTES_LEVEL_PER_MEMBER),
     "as_assign": ("members", BYTES_ASSIGN_PER_MEMBER),
 }
 

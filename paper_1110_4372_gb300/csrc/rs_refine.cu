@@ -9,10 +9,11 @@
 // Size classes:
 //  * big nodes (> SMALL_N members): processed level by level by tiles of 256
 //    members spread over the whole GPU, with per-node accumulators and
-//    histograms in global memory.  At levels 0 and 1 their members are put in
-//    k-d order (splits at leaf-aligned medians); each node then has a 32-ary
-//    box hierarchy over 32-member leaves, searched one query per warp for
-//    nearest neighbours and friends.  Children above SMALL_N stay on the big
+//    histograms in global memory.  At the first levels (rs_tuning::kd_levels)
+//    their members are put in k-d order (splits at leaf-aligned medians); each
+//    node then has a 32-ary box hierarchy over 32-member leaves, searched a
+//    leaf a warp for nearest neighbours and friends together (a query a warp
+//    for the samples of its bracket).  Children above SMALL_N stay on the big
 //    path, smaller children join the small-node queue;
 //  * small nodes (<= SMALL_N members): one CTA loads the node into shared
 //    memory and builds its whole subtree there (moments, nearest neighbours,
@@ -1994,9 +1995,9 @@ __device__ __forceinline__ float box_box_d2(const Box6 &a, const Box6 &b, const 
 // from scratch.
 //
 // Against a nearest-neighbour search a member and a link search a leaf: 118 +
-// 67 ms of a 134M-particle path became 83 (pairs) + 5 (list) + 21 (the nodes
-// without a bracket), 9.6M members in groups 19.5 + 13.7 became 15.9 + 1.1 +
-// 5.1.  The list moves 9 bytes a pair each way, a few percent of the search.
+// 67 ms of a 134M-particle path became 89 (pairs) + 6 (list), 9.6M members in
+// groups 19.5 + 13.7 became 17.1 + 1.2.  The list moves 9 bytes a pair each
+// way, a few percent of the search.
 //
 // The list is in chunks of PAIR_CHUNK pairs of one leaf, with a head (node
 // rank, first query, pairs), in PAIR_REGIONS regions with a counter each.

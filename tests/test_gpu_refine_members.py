@@ -59,6 +59,23 @@ def test_sampled_brackets_match_oracle(n, f, bracket_min):
     compare_trees(gpu_tree_dict(tree), oracle_tree_dict(oracle.refine(pos, vel, box, perm, off, f)), box)
 
 
+@pytest.mark.parametrize("n", [2000, 6000])
+def test_more_pairs_than_listed_match_oracle(n):
+    """The bracket spans the gap between a core's neighbour distances and the
+    sparse rest's, so the core's pairs (n^2 / 5) lie inside it: far more than
+    the 20 a member that the pair search lists."""
+    from paper_1110_4372_gb300 import rsgpu
+    rng = np.random.default_rng(n)
+    box, f = 20.0, 0.7
+    scale = np.where(np.arange(n) < f * n, 0.05, 1.0)[:, None]
+    pos = synth.wrap(rng.standard_normal((n, 3)) * 0.15 * scale + 10.0, box)
+    vel = (rng.standard_normal((n, 3)) * 60.0 * scale).astype(np.float32)
+    perm, off = rng.permutation(n).astype(np.int32), np.array([0, n], np.int64)
+    tree = rsgpu.rs_refine6d(rsgpu.Context(), *(torch.from_numpy(a).cuda() for a in (pos, vel)), box,
+                             torch.from_numpy(perm).cuda(), torch.from_numpy(off).cuda(), f)
+    compare_trees(gpu_tree_dict(tree), oracle_tree_dict(oracle.refine(pos, vel, box, perm, off, f)), box)
+
+
 @pytest.mark.parametrize("bad", [-1, 500])
 def test_index_out_of_range_is_an_error(bad):
     from paper_1110_4372_gb300 import rsgpu
