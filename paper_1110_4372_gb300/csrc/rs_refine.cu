@@ -2515,7 +2515,7 @@ __global__ void k_bracket_check(LevelBufs L, float *R2, const float *STOP, int *
 // leaf of 32 consecutive members is one cell of the k-d tree: compact in
 // phase space, which is what the leaf boxes of the searches need.  The split
 // positions depend only on the node's size, so each round is one stable sort
-// of all members by (segment, 16-bit coordinate), the coordinate relative to
+// of all members by (segment, coordinate of 10 to 16 bits), relative to
 // the node's reference member in units of its dispersion.
 // 16-bit coordinate of a member on an axis (x, vx, y, vy, z, vz), relative to
 // the node's reference member in units of its dispersion (.w: one over it)
@@ -2544,7 +2544,7 @@ __device__ __forceinline__ unsigned kd_coord(const float4 *wpos, const float4 *w
 // round's axis; smaller ranges keep their order (value 0).  vcur holds every
 // member's slot in the current order.
 __global__ void k_kd_keys(LevelBufs L, NodeArrays nd, const int64_t *seg_base, const float4 *wpos, const float4 *wvel, const unsigned *vcur, unsigned long long *kout,
-                          unsigned *vout, int round, int key32)
+                          unsigned *vout, int round, int drop, int key32)
 {
     const int k = L.tile_rank[blockIdx.x], q0 = L.tile_q0[blockIdx.x];
     const int node = L.list[k], n = nd.count[node];
@@ -2573,7 +2573,7 @@ __global__ void k_kd_keys(LevelBufs L, NodeArrays nd, const int64_t *seg_base, c
     // block lie before it and keep their places under the stable sort.  So
     // the block number separates what must stay apart, with 5 fewer bits
     // than a leaf number.
-    const unsigned long long key = ((unsigned long long)(seg_base[k] + start / KD_CTA) << 16) | qv;
+    const unsigned long long key = ((unsigned long long)(seg_base[k] + start / KD_CTA) << (16 - drop)) | (qv >> drop);
     if (key32)
         ((unsigned *)kout)[A] = (unsigned)key;
     else
@@ -3474,20 +3474,26 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
                               NS = tot[LT_ROUND0 + 3 * r + 2];
                 int sbits = 0;
                 while (sbits < 40 && (NS >> sbits) != 0) sbits++;
-                // 32-bit keys (half the bytes, fewer passes) while the blocks fit in 16 bits
-                const int key32 = 16 + sbits <= 32 ? 1 : 0;
+                // the coordinate gives up to 6 of its 16 bits where that saves a
+                // pass: 9.6M grouped members' sorts 3.38 -> 2.53 ms, the 134M
+                // path's 17.1 -> 15.7, their searches unchanged; with 9 bits
+                // left the dense cores' members share a coordinate and the
+                // 134M path's searches lose more (89.1 -> 90.2 ms), with 8
+                // more yet (92.5)
+                const int kbits = std::min(16 + sbits, (10 + sbits + 7) / 8 * 8), drop = 16 + sbits - kbits;
+                const int key32 = kbits <= 32 ? 1 : 0;  // (half the bytes)
                 // the order stays in place, or the sort's last pass writes it there
-                const bool odd = rs_sort_alt(NA, 16 + sbits);
+                const bool odd = rs_sort_alt(NA, kbits);
                 unsigned *va = odd ? v0 : vcur, *vb = odd ? vcur : v1;
                 RS_LAUNCH(ctx, "rf_kd_keys", k_kd_keys, TA, TQ, 0, L, nd, (const int64_t *)O.block,
                           (const float4 *)wpos, (const float4 *)wvel, (const unsigned *)vcur,
-                          (unsigned long long *)k0, odd ? v0 : nullptr, r, key32);
+                          (unsigned long long *)k0, odd ? v0 : nullptr, r, drop, key32);
                 bool kalt = false;
                 if (key32)
-                    RS_TRY(rs_radix_sort_u32(ctx, (uint32_t *)k0, (uint32_t *)k1, va, vb, NA, 16 + sbits, &kalt,
+                    RS_TRY(rs_radix_sort_u32(ctx, (uint32_t *)k0, (uint32_t *)k1, va, vb, NA, kbits, &kalt,
                                              "sort_kd"));
                 else
-                    RS_TRY(rs_radix_sort_u64(ctx, k0, k1, va, vb, NA, 16 + sbits, &kalt, "sort_kd"));
+                    RS_TRY(rs_radix_sort_u64(ctx, k0, k1, va, vb, NA, kbits, &kalt, "sort_kd"));
                 if (kalt != odd) return rs_fail(ctx, RS_ERR_INTERNAL, "rs_refine6d: k-d order");
             }
             // ranges of at most KD_CTA members finish in one CTA each
