@@ -2515,8 +2515,8 @@ __global__ void k_bracket_check(LevelBufs L, float *R2, const float *STOP, int *
 // leaf of 32 consecutive members is one cell of the k-d tree: compact in
 // phase space, which is what the leaf boxes of the searches need.  The split
 // positions depend only on the node's size, so each round is one stable sort
-// of all members by (segment, coordinate of 10 to 16 bits), relative to
-// the node's reference member in units of its dispersion.
+// of all members by (segment, coordinate), the coordinate of 10 to 16 bits
+// relative to the node's reference member in units of its dispersion.
 // 16-bit coordinate of a member on an axis (x, vx, y, vy, z, vz), relative to
 // the node's reference member in units of its dispersion (.w: one over it)
 __device__ __forceinline__ unsigned kd_coord(const float4 *wpos, const float4 *wvel, unsigned slot, int axis,
