@@ -94,11 +94,12 @@ __global__ void k_as_leafcompact(NodeArrays nd, int nn, const unsigned *flag, co
     vals[scan[i]] = (unsigned)i;
 }
 
-__global__ void k_as_init(AsBufs A, NodeArrays nd)
+__global__ void k_as_init(AsBufs A, NodeArrays nd, const rs_dev_status *st)
 {
     int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= A.L) return;
     const int node = A.leaf_node[a];
+    if (dev_is_torn(st)) return;
     A.sx[a] = make_float4((float)nd.xbar[3 * node], (float)nd.xbar[3 * node + 1], (float)nd.xbar[3 * node + 2],
                           (float)nd.sigx[node]);
     A.sv[a] = make_float4((float)nd.vbar[3 * node], (float)nd.vbar[3 * node + 1], (float)nd.vbar[3 * node + 2],
@@ -162,6 +163,7 @@ __device__ __forceinline__ bool merge_far_f32(float4 xa, float4 va, int4 ia, flo
 __global__ void __launch_bounds__(AS_THREADS) k_as_merge(AsBufs A, NodeArrays nd, double box, double thresh,
                                                          rs_dev_status *st)
 {
+    if (dev_is_torn(st)) return;
     const float boxf = (float)box, thresh2 = (float)(thresh * thresh);
     const int lane = lane_id();
     for (int a = (blockIdx.x * AS_THREADS + threadIdx.x) >> 5; a < A.L; a += gridDim.x * AS_THREADS >> 5) {
@@ -183,7 +185,7 @@ __global__ void k_as_roots(AsBufs A, NodeArrays nd, const int *members, const fl
                            int stride, float boxf, rs_dev_status *st)
 {
     int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= A.L) return;
+    if (a >= A.L || dev_is_torn(st)) return;
     const int node = A.leaf_node[a];
     const int r = uf_find(A.uf, a, st);
     atomicMin(&A.hid[r], nd.minidx[node]);
@@ -201,6 +203,7 @@ __global__ void k_as_roots(AsBufs A, NodeArrays nd, const int *members, const fl
 __global__ void __launch_bounds__(AS_THREADS) k_as_hmom(AsBufs A, NodeArrays nd, const int *members, const float *pos,
                                                         const float *vel, int stride, float boxf, rs_dev_status *st)
 {
+    if (dev_is_torn(st)) return;
     __shared__ MomAcc w[AS_THREADS / 32];
     for (int a = blockIdx.x; a < A.L; a += gridDim.x) {
         const int node = A.leaf_node[a];
@@ -264,6 +267,7 @@ __global__ void k_as_hrank(AsBufs A, const unsigned *rootflag, const unsigned *r
 __global__ void k_as_hmembers(AsBufs A, NodeArrays nd, const unsigned long long *hoff, unsigned long long *hfill,
                               int *hmem, rs_dev_status *st)
 {
+    if (dev_is_torn(st)) return;
     for (int a = blockIdx.x; a < A.L; a += gridDim.x) {
         __shared__ unsigned long long base;
         const int node = A.leaf_node[a];
@@ -282,8 +286,9 @@ __global__ void k_as_hmembers(AsBufs A, NodeArrays nd, const unsigned long long 
 __global__ void __launch_bounds__(AS_THREADS) k_as_rdyn(AsBufs A, int n_halos, const int *root_of_rank,
                                                         const unsigned long long *hoff, const int *hmem,
                                                         const int *members, const float *pos, int stride,
-                                                        double box, double rho_term)
+                                                        double box, double rho_term, const rs_dev_status *st)
 {
+    if (dev_is_torn(st)) return;
     __shared__ unsigned long long key[RDYN_SMEM_N];
     __shared__ double wbest[AS_THREADS / 32];
     for (int k = blockIdx.x; k < n_halos; k += gridDim.x) {
@@ -393,11 +398,13 @@ __global__ void k_as_large_keys(int nlarge, const long long *loff, const int *lh
 }
 
 __global__ void k_as_large_max(long long total, const long long *loff, const unsigned long long *keys,
-                               const unsigned *vals, const double *r64, unsigned long long *best_bits)
+                               const unsigned *vals, const double *r64, unsigned long long *best_bits,
+                               const rs_dev_status *st)
 {
     long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= total) return;
     const unsigned long long key = keys[t];
+    if (dev_is_torn(st)) return;
     const int li = (int)(key >> 32);
     const long long start = loff[li];
     const double r = r64[vals[t]];
@@ -461,7 +468,7 @@ constexpr int AS_CAND = 4096;  // seeds deduplicated in shared memory per node
 __global__ void k_as_leafroot(AsBufs A, int *leaf_root, rs_dev_status *st)
 {
     int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= A.L) return;
+    if (a >= A.L || dev_is_torn(st)) return;
     leaf_root[a] = uf_find(A.uf, a, st);
 }
 
@@ -696,7 +703,7 @@ rs_status large_rdyn(rs_ctx *ctx, AsBufs A, int H, const int *root_of_rank, cons
     unsigned *lflag = lfl, *lscan = lfl + H, *ltot = lfl + 2 * H;
     RS_LAUNCH(ctx, "as_large_flag", k_as_large_flag, ceil_div(H, 256), 256, 0, H, hoff, lflag);
     RS_CUDA(ctx, cudaMemcpyAsync(lscan, lflag, sizeof(unsigned) * H, cudaMemcpyDeviceToDevice, ctx->stream));
-    RS_TRY(rs_scan_u32(ctx, lscan, H, ltot));
+    RS_TRY(rs_scan_u32(ctx, lscan, H, ltot, "scan_large"));
     RS_CUDA(ctx, cudaMemcpyAsync(ctx->h_scratch, ltot, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream));
     RS_TRY(rs_sync_check(ctx, "rs_assign"));
     const int NL = (int)(*(unsigned *)ctx->h_scratch);
@@ -723,10 +730,10 @@ rs_status large_rdyn(rs_ctx *ctx, AsBufs A, int H, const int *root_of_rank, cons
     int bits = 32;
     while (bits < 64 && ((uint64_t)(NL - 1) >> (bits - 32)) != 0) bits++;
     bool alt = false;
-    RS_TRY(rs_radix_sort_u64(ctx, k0, k1, v0, v1, total, bits, &alt, "sort_as"));
+    RS_TRY(rs_radix_sort_u64(ctx, k0, k1, v0, v1, total, bits, &alt, "sort_rdyn"));
     RS_LAUNCH(ctx, "as_large_max", k_as_large_max, ceil_div(total, 256), 256, 0, (long long)total,
               (const long long *)lsize, (const unsigned long long *)(alt ? k1 : k0), (const unsigned *)(alt ? v1 : v0),
-              (const double *)r64, bb);
+              (const double *)r64, bb, (const rs_dev_status *)ctx->d_status);
     RS_LAUNCH(ctx, "as_large_fin", k_as_large_fin, ceil_div(NL, 256), 256, 0, NL, (const int *)lhalo, root_of_rank,
               (const unsigned long long *)bb, A, rho_term);
     return RS_OK;
@@ -768,7 +775,7 @@ extern "C" rs_status rs_assign_ex(rs_ctx *ctx, const rs_tree *t, const float *po
     RS_LAUNCH(ctx, "as_leafflag", k_as_leafflag, ceil_div(nn, 256), 256, 0, nd, nn, flag, span);
     RS_LAUNCH(ctx, "as_span", k_as_span, ceil_div(nn, 256), 256, 0, nd, nn, span);
     RS_CUDA(ctx, cudaMemcpyAsync(scan, flag, sizeof(unsigned) * nn, cudaMemcpyDeviceToDevice, ctx->stream));
-    RS_TRY(rs_scan_u32(ctx, scan, nn, nullptr));
+    RS_TRY(rs_scan_u32(ctx, scan, nn, nullptr, "scan_leaf"));
     const int L = (int)t->n_seeds;
     RS_WS(ctx, unsigned, lk, WS_AS_2, 4 * (int64_t)L + 8);
     unsigned *k0 = lk, *k1 = lk + L, *v0 = lk + 2 * L, *v1 = lk + 3 * L;
@@ -803,7 +810,7 @@ extern "C" rs_status rs_assign_ex(rs_ctx *ctx, const rs_tree *t, const float *po
     A.hfast = carve<float>(hp, 16 * (int64_t)L);
     RS_CUDA(ctx, cudaMemsetAsync(A.hacc, 0, sizeof(MomAcc) * (size_t)L, ctx->stream));
     const int64_t gl = ceil_div(L, 256);
-    RS_LAUNCH(ctx, "as_init", k_as_init, gl, 256, 0, A, nd);
+    RS_LAUNCH(ctx, "as_init", k_as_init, gl, 256, 0, A, nd, (const rs_dev_status *)ctx->d_status);
     RS_LAUNCH(ctx, "as_merge", k_as_merge, std::min<int64_t>(ceil_div(L, AS_THREADS / 32), (int64_t)ctx->num_sms * 64),
               AS_THREADS, 0, A, nd, box, params->merge_thresh, ctx->d_status);
     RS_LAUNCH(ctx, "as_roots", k_as_roots, gl, 256, 0, A, nd, (const int *)t->members, pos, vel, stride, boxf,
@@ -817,7 +824,7 @@ extern "C" rs_status rs_assign_ex(rs_ctx *ctx, const rs_tree *t, const float *po
     unsigned *rootflag = rf, *rscan = rf + L, *rtot = rf + 2 * L;
     RS_LAUNCH(ctx, "as_hfin", k_as_hfin, gl, 256, 0, A, box, rootflag);
     RS_CUDA(ctx, cudaMemcpyAsync(rscan, rootflag, sizeof(unsigned) * L, cudaMemcpyDeviceToDevice, ctx->stream));
-    RS_TRY(rs_scan_u32(ctx, rscan, L, rtot));
+    RS_TRY(rs_scan_u32(ctx, rscan, L, rtot, "scan_root"));
     int64_t H;
     {
         RS_CUDA(ctx, cudaMemcpyAsync(ctx->h_scratch, rtot, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream));
@@ -828,7 +835,7 @@ extern "C" rs_status rs_assign_ex(rs_ctx *ctx, const rs_tree *t, const float *po
     unsigned long long *hoff = ho, *hfill = ho + (H + 1);
     RS_CUDA(ctx, cudaMemsetAsync(ho, 0, sizeof(unsigned long long) * (2 * (H + 1)), ctx->stream));
     RS_LAUNCH(ctx, "as_hrank", k_as_hrank, gl, 256, 0, A, (const unsigned *)rootflag, (const unsigned *)rscan, hoff);
-    RS_TRY(rs_scan_i64(ctx, (int64_t *)hoff, H + 1, nullptr));
+    RS_TRY(rs_scan_i64(ctx, (int64_t *)hoff, H + 1, nullptr, "scan_halo"));
     // the seeds' members, at most all
     RS_WS(ctx, int, hm, WS_AS_6, t->n_members + H + 8);
     int *hmem = hm, *root_of_rank = hm + t->n_members;
@@ -837,7 +844,7 @@ extern "C" rs_status rs_assign_ex(rs_ctx *ctx, const rs_tree *t, const float *po
               hmem, ctx->d_status);
     RS_LAUNCH(ctx, "as_rdyn", k_as_rdyn, std::min<int64_t>(H, (int64_t)ctx->num_sms * 8), AS_THREADS, 0, A, (int)H,
               (const int *)root_of_rank, (const unsigned long long *)hoff, (const int *)hmem,
-              (const int *)t->members, pos, stride, box, rho_term);
+              (const int *)t->members, pos, stride, box, rho_term, (const rs_dev_status *)ctx->d_status);
     // r_dyn of the halos too large for one block's shared memory
     RS_TRY(large_rdyn(ctx, A, (int)H, (const int *)root_of_rank, (const unsigned long long *)hoff, (const int *)hmem,
                       (const int *)t->members, pos, stride, box, rho_term));
@@ -845,14 +852,14 @@ extern "C" rs_status rs_assign_ex(rs_ctx *ctx, const rs_tree *t, const float *po
     RS_WS(ctx, int64_t, tl, WS_RF_MISC1, (int64_t)nn + 8);
     RS_LAUNCH(ctx, "as_tiles_prep", k_as_tiles_prep, ceil_div(nn, 256), 256, 0, nd, nn, (const int *)span, tl);
     RS_CUDA(ctx, cudaMemsetAsync(tl + nn, 0, sizeof(int64_t), ctx->stream));
-    RS_TRY(rs_scan_i64(ctx, tl, nn + 1, tl + nn + 2));
+    RS_TRY(rs_scan_i64(ctx, tl, nn + 1, tl + nn + 2, "scan_tile"));
     // distinct candidate halos of every node, once per node
     RS_WS(ctx, int64_t, cw, WS_AS_8, 2 * (int64_t)nn + 8);
     int64_t *coff = cw;
     int *node_la = (int *)(cw + nn + 4), *ncand = node_la + nn;
     RS_LAUNCH(ctx, "as_nl", k_as_nl, ceil_div(nn, 256), 256, 0, A, nd, (int)nn, node_la, coff);
     RS_CUDA(ctx, cudaMemsetAsync(coff + nn, 0, sizeof(int64_t), ctx->stream));
-    RS_TRY(rs_scan_i64(ctx, coff, nn + 1, coff + nn + 2));
+    RS_TRY(rs_scan_i64(ctx, coff, nn + 1, coff + nn + 2, "scan_cand"));
     RS_CUDA(ctx, cudaMemcpyAsync(ctx->h_scratch + 1, coff + nn, sizeof(int64_t), cudaMemcpyDeviceToHost, ctx->stream));
     int64_t T;
     RS_TRY(rs_read_i64(ctx, tl + nn, 1, &T, "rs_assign"));

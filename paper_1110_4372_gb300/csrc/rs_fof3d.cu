@@ -88,6 +88,8 @@ __global__ void __launch_bounds__(FOF_THREADS) k_fof_cells(const float *pos, int
                                                            uint32_t *n_cells, RsLookback lb, rs_dev_status *st)
 {
     const unsigned FULL = 0xffffffffu;
+    // (for the whole block: other blocks' look-backs may run out meanwhile)
+    if (__syncthreads_or(dev_is_torn(st))) return;
     const int64_t tile = rs_next_tile(lb);
     const int lane = lane_id();
     const int64_t base = tile * CELL_TILE + (int64_t)warp_id() * 32 * CELL_ROWS;
@@ -113,7 +115,7 @@ __global__ void __launch_bounds__(FOF_THREADS) k_fof_cells(const float *pos, int
         const int64_t q = base + 32 * j + lane;
         const uint32_t c = c0 + (uint32_t)__popc(starts[j] & upto) - 1u;
         c0 += (uint32_t)__popc(starts[j]);
-        if (q >= n || c >= n) continue;  // (a look-back that ran out of time leaves wrong numbers)
+        if (q >= n || c >= n) continue;  // (after a look-back that ran out of time: see dev_torn)
         float x, y, z;
         load_pos(pos, stride, idx[q], x, y, z);
         spos[q] = make_float4(x, y, z, 0.f);
@@ -133,9 +135,16 @@ __global__ void __launch_bounds__(FOF_THREADS) k_fof_cells(const float *pos, int
     }
 }
 
-// occupancy mask of each coarse cell, kept at its first fine cell
-__global__ void k_fof_occ(const uint32_t *n_cells_p, const uint64_t *cell_key, const uint32_t *table, uint64_t *occ)
+// occupancy mask of each coarse cell, kept at its first fine cell.  After a
+// torn sort or scan there are no cells: the kernels that go over them then do
+// nothing.
+__global__ void k_fof_occ(uint32_t *n_cells_p, const uint64_t *cell_key, const uint32_t *table, uint64_t *occ,
+                          const rs_dev_status *st)
 {
+    if (dev_is_torn(st)) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) *n_cells_p = 0u;
+        return;
+    }
     const int64_t M = *n_cells_p;
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < M; c += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t k = cell_key[c];
@@ -427,11 +436,13 @@ __global__ void k_fof_rootmin(const uint32_t *n_cells_p, const uint32_t *cell_st
 
 // (every cell's parent is its root by now)
 __global__ void k_fof_labels(int64_t n, const uint32_t *idx, const uint32_t *cell_of, const int *parent,
-                             const int *root_min, int32_t *labels)
+                             const int *root_min, int32_t *labels, const rs_dev_status *st)
 {
     int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= n) return;
-    labels[idx[q]] = root_min[parent[cell_of[q]]];
+    const uint32_t i = idx[q], c = cell_of[q];
+    if (dev_is_torn(st)) return;
+    labels[i] = root_min[parent[c]];
 }
 
 __global__ void k_fof_count_roots(const uint32_t *n_cells_p, const int *parent, unsigned long long *count)
@@ -590,10 +601,10 @@ __device__ __forceinline__ void acc_where(const uint64_t *cell_key, uint32_t A, 
 __global__ void __launch_bounds__(FOF_THREADS) k_acc_count(int64_t n, const uint32_t *cell_of, const uint64_t *cell_key,
                                                            const uint32_t *cell_start, const uint32_t *table,
                                                            const uint64_t *occ, const float4 *spos, FofGeom g,
-                                                           int dense_n, uint8_t *dense)
+                                                           int dense_n, uint8_t *dense, const rs_dev_status *st)
 {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
+    if (q >= n || dev_is_torn(st)) return;
     const uint32_t A = cell_of[q];
     int cnt = (int)(cell_start[A + 1] - cell_start[A]) - 1;
     if (cnt <= dense_n) {
@@ -877,13 +888,13 @@ rs_status fof_run(rs_ctx *ctx, const float *pos, int32_t stride, int64_t n, doub
     RS_WS(ctx, int, root_min, WS_FOF_ROOTMIN, n);
     const int64_t ctiles = ceil_div(n, CELL_TILE);
     RsLookback lb;
-    RS_TRY(rs_lookback_init(ctx, ctiles, &lb));
+    RS_TRY(rs_lookback_init(ctx, ctiles, &lb, "fof_cells"));
     RS_LAUNCH(ctx, "fof_cells", k_fof_cells, ctiles, T, 0, pos, stride, n, (const uint64_t *)keys,
               (const uint32_t *)idx, spos, cell_of, cell_start, cell_key, table, occ, parent, root_min, n_cells, lb,
               ctx->d_status);
     const int64_t grid = std::min<int64_t>(nb, (int64_t)ctx->num_sms * ctx->tune.fof_link_ctas_per_sm);
-    RS_LAUNCH(ctx, "fof_occ", k_fof_occ, grid, T, 0, (const uint32_t *)n_cells, (const uint64_t *)cell_key,
-              (const uint32_t *)table, occ);
+    RS_LAUNCH(ctx, "fof_occ", k_fof_occ, grid, T, 0, n_cells, (const uint64_t *)cell_key, (const uint32_t *)table, occ,
+              (const rs_dev_status *)ctx->d_status);
     const int64_t rows = ceil_div(n, 32), warps = (int64_t)ctx->num_sms * 48;
     const bool small = n <= FOF_ONE_PASS;
     int split = 1;
@@ -913,7 +924,7 @@ rs_status fof_run(rs_ctx *ctx, const float *pos, int32_t stride, int64_t n, doub
         unsigned long long *acnt = (unsigned long long *)len + 8;
         RS_LAUNCH(ctx, "fof_acc_count", k_acc_count, nb, T, 0, n, (const uint32_t *)cell_of,
                   (const uint64_t *)cell_key, (const uint32_t *)cell_start, (const uint32_t *)table,
-                  (const uint64_t *)occ, (const float4 *)spos, g, (int)dense_n, dense);
+                  (const uint64_t *)occ, (const float4 *)spos, g, (int)dense_n, dense, (const rs_dev_status *)ctx->d_status);
         RS_CUDA(ctx, cudaMemsetAsync(len, 0, 4, ctx->stream));
         RS_LAUNCH(ctx, "fof_acc_init", k_acc_init, grid, T, 0, (const uint32_t *)n_cells,
                   (const uint32_t *)cell_start, (const uint8_t *)dense, word, la, len);
@@ -956,7 +967,7 @@ rs_status fof_run(rs_ctx *ctx, const float *pos, int32_t stride, int64_t n, doub
               (const uint32_t *)cell_start, (const uint32_t *)idx, parent, root_min,
               rs_fault("timeout1") ? 1 : RS_SPIN_LIMIT, ctx->d_status);
     RS_LAUNCH(ctx, "fof_labels", k_fof_labels, nb, T, 0, n, (const uint32_t *)idx, (const uint32_t *)cell_of,
-              (const int *)parent, (const int *)root_min, labels);
+              (const int *)parent, (const int *)root_min, labels, (const rs_dev_status *)ctx->d_status);
     if (n_groups || n_tieband) {
         RS_CUDA(ctx, cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), ctx->stream));
         if (n_groups)
@@ -1103,7 +1114,7 @@ extern "C" rs_status rs_group_sort(rs_ctx *ctx, const int32_t *labels, int64_t n
     RS_LAUNCH(ctx, "gs_count", k_gs_count, ceil_div(n, GS_TILE), GS_THREADS, 0, n, labels, count, ctx->d_status);
     const int64_t tiles = ceil_div(n, GS_SCAN_TILE);
     RsLookback lb;
-    RS_TRY(rs_lookback_init(ctx, tiles, &lb));
+    RS_TRY(rs_lookback_init(ctx, tiles, &lb, "gs_select"));
     RS_LAUNCH(ctx, "gs_select", k_gs_select, tiles, GS_THREADS, 0, n, labels, (const uint32_t *)count, min_n,
               (uint32_t *)perm, group, offsets, offsets_cap, tot, lb, ctx->d_status);
     uint32_t h2[2];
@@ -1127,6 +1138,6 @@ extern "C" rs_status rs_group_sort(rs_ctx *ctx, const int32_t *labels, int64_t n
     if (alt)
         RS_CUDA(ctx, cudaMemcpyAsync(perm, vtmp, sizeof(uint32_t) * Mm, cudaMemcpyDeviceToDevice, ctx->stream));
     RS_CUDA(ctx, cudaMemsetAsync(offsets + G, 0, sizeof(int64_t), ctx->stream));
-    RS_TRY(rs_scan_i64(ctx, offsets, G + 1, nullptr));
+    RS_TRY(rs_scan_i64(ctx, offsets, G + 1, nullptr, "scan_gs"));
     return rs_sync_check(ctx, "rs_group_sort");
 }

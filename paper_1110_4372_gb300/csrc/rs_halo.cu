@@ -136,6 +136,7 @@ __global__ void __launch_bounds__(HP_THREADS) k_hp_count(int64_t n, const int32_
                                                          const unsigned *srank, int H, unsigned long long *n_assigned,
                                                          rs_dev_status *st)
 {
+    if (dev_is_torn(st)) return;
     __shared__ RsBlockCount<unsigned long long, 11> C;
     C.clear();
     const int64_t i0 = (int64_t)blockIdx.x * HP_COUNT_TILE;
@@ -167,10 +168,10 @@ __device__ __forceinline__ double min_image_h(double d, double box)
 // host of every halo: the Eq. 3 nearest larger halo of its group
 __global__ void k_hp_host(int H, rs_halos hs, const double *xc, const double *vc,
                           const unsigned long long *n_assigned, const unsigned *groot, const unsigned *grank,
-                          double box, int *host)
+                          double box, int *host, const rs_dev_status *st)
 {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= H) return;
+    if (s >= H || dev_is_torn(st)) return;
     const unsigned g = (unsigned)hs.root[s];
     const int a = lower_bound_u(groot, H, g);
     double best = INFINITY;
@@ -200,7 +201,7 @@ __global__ void k_ub_up(int H, const int32_t *host, const unsigned *sid, const u
                         rs_dev_status *st)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= H) return;
+    if (r >= H || dev_is_torn(st)) return;
     int u = -1;
     if (host[r] >= 0) {
         u = rank_of(sid, srank, H, host[r]);
@@ -217,6 +218,7 @@ __global__ void k_ub_up(int H, const int32_t *host, const unsigned *sid, const u
 __global__ void k_ub_count(int64_t n, const int32_t *halo_id, const unsigned *sid, const unsigned *srank, int H,
                            const int *up, unsigned long long *total, rs_dev_status *st)
 {
+    if (dev_is_torn(st)) return;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     unsigned long long c = 0;
     if (i < n && halo_id[i] >= 0) {
@@ -254,10 +256,10 @@ __global__ void k_ub_keys(int64_t n, const int32_t *halo_id, const unsigned *sid
 }
 
 // set boundaries from the sorted keys: off[r] = first position of set r
-__global__ void k_ub_bounds(int64_t total, const uint64_t *keys, int64_t *off, int H)
+__global__ void k_ub_bounds(int64_t total, const uint64_t *keys, int64_t *off, int H, const rs_dev_status *st)
 {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= total) return;
+    if (k >= total || dev_is_torn(st)) return;
     const int r = (int)(keys[k] >> 32);
     const int rp = k == 0 ? -1 : (int)(keys[k - 1] >> 32);
     for (int q = rp + 1; q <= r; q++) off[q] = k;
@@ -267,8 +269,10 @@ __global__ void k_ub_bounds(int64_t total, const uint64_t *keys, int64_t *off, i
 
 // bulk velocity of every set: one block per set, float64 reduction in a fixed order
 __global__ void __launch_bounds__(HP_THREADS) k_ub_bulk(int H, const int64_t *off, const uint32_t *mem,
-                                                        const float *vel, int stride, double *vbulk)
+                                                        const float *vel, int stride, double *vbulk,
+                                                        const rs_dev_status *st)
 {
+    if (dev_is_torn(st)) return;
     __shared__ double red[3][HP_THREADS];
     for (int r = blockIdx.x; r < H; r += gridDim.x) {
         const int64_t a = off[r], b = off[r + 1];
@@ -582,11 +586,12 @@ __global__ void k_ub_morton(int64_t total, const uint64_t *keys, const int64_t *
 }
 
 __global__ void k_ub_gather(int64_t total, const uint32_t *perm, const float4 *upos, const uint32_t *mem,
-                            float4 *tpos, uint32_t *tmem)
+                            float4 *tpos, uint32_t *tmem, const rs_dev_status *st)
 {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= total) return;
     const uint32_t s = perm[k];
+    if (dev_is_torn(st)) return;
     tpos[k] = upos[s];
     tmem[k] = mem[s];
 }
@@ -704,7 +709,7 @@ __global__ void __launch_bounds__(UT_WARPS * 32) k_ub_walk(int64_t njobs, const 
     __shared__ float4 src_s[UT_WARPS][UT_LEAF];  // a leaf's members, or an opened box's children
     const unsigned FULL = 0xffffffffu;
     const int64_t j = (int64_t)blockIdx.x * UT_WARPS + warp_id();
-    if (j >= njobs) return;
+    if (j >= njobs || dev_is_torn(st)) return;
     const int w = warp_id(), lane = lane_id();
     float4 *src = src_s[w];
     const int r = jset[j], leaf = jleaf[j];
@@ -816,11 +821,11 @@ rs_status sorted_ids(rs_ctx *ctx, const rs_halos *hs, unsigned **sid, unsigned *
     RS_LAUNCH(ctx, "hp_keys", k_hp_keys, ceil_div(H, 256), 256, 0, (int)H, (const int *)hs->id,
               (const int *)hs->root, k0, v0, g0, w0);
     bool alt = false;
-    RS_TRY(rs_radix_sort_u32(ctx, k0, k1, v0, v1, H, 31, &alt));
+    RS_TRY(rs_radix_sort_u32(ctx, k0, k1, v0, v1, H, 31, &alt, "sort_ids"));
     *sid = alt ? k1 : k0;
     *srank = alt ? v1 : v0;
     bool galt = false;
-    RS_TRY(rs_radix_sort_u32(ctx, g0, g1, w0, w1, H, 31, &galt));
+    RS_TRY(rs_radix_sort_u32(ctx, g0, g1, w0, w1, H, 31, &galt, "sort_hosts"));
     *groot = galt ? g1 : g0;
     *grank = galt ? w1 : w0;
     return RS_OK;
@@ -859,7 +864,7 @@ extern "C" rs_status rs_halo_props(rs_ctx *ctx, const rs_tree *t, const rs_halos
               (const unsigned *)srank, (int)H, na, ctx->d_status);
     RS_LAUNCH(ctx, "hp_host", k_hp_host, ceil_div(H, 128), 128, 0, (int)H, *hs, (const double *)xc,
               (const double *)vc, (const unsigned long long *)na, (const unsigned *)groot, (const unsigned *)grank,
-              t->box, host);
+              t->box, host, (const rs_dev_status *)ctx->d_status);
     return rs_sync_check(ctx, "rs_halo_props");
 }
 
@@ -903,20 +908,21 @@ extern "C" rs_status rs_unbind(rs_ctx *ctx, const rs_tree *t, const rs_halos *hs
     int rbits = 0;
     while (rbits < 32 && ((uint64_t)(H - 1) >> rbits) != 0) rbits++;
     bool alt = false;
-    if (total > 0) RS_TRY(rs_radix_sort_u64(ctx, k0, k1, v0, v1, total, 32 + rbits, &alt));
+    if (total > 0) RS_TRY(rs_radix_sort_u64(ctx, k0, k1, v0, v1, total, 32 + rbits, &alt, "sort_sets"));
     const uint64_t *sk = alt ? k1 : k0;
     const uint32_t *smem = alt ? v1 : v0;
     RS_WS(ctx, int64_t, ob, WS_HL_OFF, 2 * (H + 1) + 8);
     int64_t *off = ob, *toff = ob + (H + 1);
     if (total > 0)
-        RS_LAUNCH(ctx, "ub_bounds", k_ub_bounds, ceil_div(total, 256), 256, 0, total, sk, off, (int)H);
+        RS_LAUNCH(ctx, "ub_bounds", k_ub_bounds, ceil_div(total, 256), 256, 0, total, sk, off, (int)H,
+                  (const rs_dev_status *)ctx->d_status);
     else
         RS_CUDA(ctx, cudaMemsetAsync(off, 0, sizeof(int64_t) * (H + 1), ctx->stream));
     RS_LAUNCH(ctx, "ub_bulk", k_ub_bulk, std::min<int64_t>(H, (int64_t)ctx->num_sms * 8), HP_THREADS, 0, (int)H,
-              (const int64_t *)off, smem, vel, stride, vbulk);
+              (const int64_t *)off, smem, vel, stride, vbulk, (const rs_dev_status *)ctx->d_status);
     RS_LAUNCH(ctx, "ub_tiles", k_ub_tiles, ceil_div(H, 256), 256, 0, (int)H, (const int64_t *)off, tree_on, toff);
     RS_CUDA(ctx, cudaMemsetAsync(toff + H, 0, sizeof(int64_t), ctx->stream));
-    RS_TRY(rs_scan_i64(ctx, toff, H + 1, nullptr));
+    RS_TRY(rs_scan_i64(ctx, toff, H + 1, nullptr, "scan_tile"));
     int64_t T = 0;
     RS_TRY(rs_read_i64(ctx, toff + H, 1, &T, "rs_unbind"));
     RS_WS(ctx, int, tm, WS_HL_TILES, 2 * T + 8);
@@ -935,8 +941,8 @@ extern "C" rs_status rs_unbind(rs_ctx *ctx, const rs_tree *t, const rs_halos *hs
                   tree_on, nbox, nleaf);
         RS_CUDA(ctx, cudaMemsetAsync(nbox + H, 0, sizeof(int64_t), ctx->stream));
         RS_CUDA(ctx, cudaMemsetAsync(nleaf + H, 0, sizeof(int64_t), ctx->stream));
-        RS_TRY(rs_scan_i64(ctx, nbox, H + 1, nullptr));
-        RS_TRY(rs_scan_i64(ctx, nleaf, H + 1, nullptr));
+        RS_TRY(rs_scan_i64(ctx, nbox, H + 1, nullptr, "scan_box"));
+        RS_TRY(rs_scan_i64(ctx, nleaf, H + 1, nullptr, "scan_job"));
         int64_t NB = 0, NJ = 0;
         RS_TRY(rs_read_i64(ctx, nbox + H, 1, &NB, "rs_unbind"));
         RS_TRY(rs_read_i64(ctx, nleaf + H, 1, &NJ, "rs_unbind"));
@@ -960,9 +966,10 @@ extern "C" rs_status rs_unbind(rs_ctx *ctx, const rs_tree *t, const rs_halos *hs
             RS_LAUNCH(ctx, "ub_morton", k_ub_morton, ceil_div(total, 256), 256, 0, total, sk, (const int64_t *)off,
                       tree_on, (const float4 *)upos, (const float4 *)cube, mk0, mv0);
             bool malt = false;
-            RS_TRY(rs_radix_sort_u64(ctx, mk0, mk1, mv0, mv1, total, 30 + rbits, &malt));
+            RS_TRY(rs_radix_sort_u64(ctx, mk0, mk1, mv0, mv1, total, 30 + rbits, &malt, "sort_morton"));
             RS_LAUNCH(ctx, "ub_gather", k_ub_gather, ceil_div(total, 256), 256, 0, total,
-                      (const uint32_t *)(malt ? mv1 : mv0), (const float4 *)upos, smem, tpos, tmem);
+                      (const uint32_t *)(malt ? mv1 : mv0), (const float4 *)upos, smem, tpos, tmem,
+                      (const rs_dev_status *)ctx->d_status);
             RS_WS(ctx, float4, bx, WS_HL_BOX, 2 * NB + 2);
             UBoxes B;
             B.c = bx;

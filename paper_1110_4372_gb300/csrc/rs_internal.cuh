@@ -39,6 +39,8 @@ struct rs_dev_status {
     int32_t code;    // first error code recorded
     int32_t site;    // which check recorded it
     int64_t detail;  // site-specific value
+    int32_t torn;    // a sort or scan is incomplete (see dev_torn)
+    int32_t pad;
 };
 
 __device__ __forceinline__ void dev_fail(rs_dev_status *st, int32_t code, int32_t site, int64_t detail)
@@ -51,6 +53,23 @@ __device__ __forceinline__ void dev_fail(rs_dev_status *st, int32_t code, int32_
 
 // Upper bound on iterations of any retry or pointer-chasing loop.
 #define RS_SPIN_LIMIT (1 << 22)
+
+// A tile of a one-pass sort or scan whose wait for an earlier tile ran out
+// leaves places of the result unwritten: what lies there may be of an earlier
+// call.  It records that besides the time-out (whose code another error may
+// already hold the place of), and every kernel between the sort or scan and the
+// host's next look at the status that would use such a result as an index
+// returns at once when dev_is_torn says so.
+__device__ __forceinline__ void dev_torn(rs_dev_status *st, int32_t site, int64_t tile)
+{
+    *(volatile int32_t *)&st->torn = 1;
+    dev_fail(st, DEV_TIMEOUT, site, tile);
+}
+
+__device__ __forceinline__ bool dev_is_torn(const rs_dev_status *st)
+{
+    return *(const volatile int32_t *)&st->torn != 0;
+}
 
 // ---------------------------------------------------------------------------
 // Workspace slots (grow-only device buffers owned by the context)
@@ -148,6 +167,7 @@ rs_status rs_sync_check(rs_ctx *ctx, const char *where);
 rs_status rs_read_i64(rs_ctx *ctx, const void *dsrc, int count, int64_t *dst, const char *where);
 // Host-side fault injection for the failure-detection tests: true when the
 // environment variable RS_FAULT, a comma-separated list, names `site`.
+// ("wait_" and the tag of a one-pass sort or scan: its waits run out at once)
 // Sites: "alloc" (every workspace allocation fails), "timeout1" (the 3D FOF
 // label pass runs with a bound of one step per find), "offsets" (rs_find_halos
 // corrupts the group offsets it passes to the refinement), "bracket" (the
@@ -190,8 +210,8 @@ __host__ __device__ static inline int64_t ceil_div(int64_t a, int64_t b) { retur
 // Scan and sort (rs_scan_sort.cu)
 // ---------------------------------------------------------------------------
 // In-place exclusive prefix sum; *total (device, optional) receives the sum.
-rs_status rs_scan_u32(rs_ctx *ctx, uint32_t *data, int64_t n, uint32_t *total);
-rs_status rs_scan_i64(rs_ctx *ctx, int64_t *data, int64_t n, int64_t *total);
+rs_status rs_scan_u32(rs_ctx *ctx, uint32_t *data, int64_t n, uint32_t *total, const char *tag = "scan");
+rs_status rs_scan_i64(rs_ctx *ctx, int64_t *data, int64_t n, int64_t *total, const char *tag = "scan");
 // keys per radix-sort tile; the sort workspace holds, per pass of 8 key bits,
 // 320 words and 256 words per tile
 constexpr int64_t RS_SORT_TILE = 4096;
@@ -257,9 +277,10 @@ __device__ __forceinline__ double f64_sub(double a, double b) { return __dsub_rn
 struct RsLookback {
     unsigned *next;
     unsigned long long *state;
+    int limit;  // tries for a predecessor's word; -1: as if it never came
 };
 // cleared counter and states for a scan of this many tiles (rs_scan_sort.cu)
-rs_status rs_lookback_init(rs_ctx *ctx, int64_t tiles, RsLookback *lb);
+rs_status rs_lookback_init(rs_ctx *ctx, int64_t tiles, RsLookback *lb, const char *tag);
 
 // the block's tile
 __device__ __forceinline__ int64_t rs_next_tile(const RsLookback &lb)
@@ -309,14 +330,15 @@ __device__ __forceinline__ unsigned long long rs_lookback(const RsLookback &lb, 
         const int lane = lane_id();
         unsigned long long before = 0;
         if (lane == 0) s[tile] = tile == 0 ? PREFIX | sum : SUM | sum;
-        for (int64_t t = tile - 1; t >= 0; t -= 32) {
+        if (lb.limit < 0 && tile > 0 && lane == 0) dev_torn(st, 92, tile);
+        for (int64_t t = lb.limit < 0 ? -1 : tile - 1; t >= 0; t -= 32) {
             // the 32 tiles up to t, the nearest in lane 0
             unsigned long long x = t >= lane ? s[t - lane] : PREFIX;
-            for (int it = 0; it < RS_SPIN_LIMIT && __any_sync(0xffffffffu, x == 0); it++)
+            for (int it = 0; it < lb.limit && __any_sync(0xffffffffu, x == 0); it++)
                 if (x == 0) x = s[t - lane];
             const unsigned zero = __ballot_sync(0xffffffffu, x == 0);
             if (zero) {
-                if (lane == 0) dev_fail(st, DEV_TIMEOUT, 92, tile);
+                if (lane == 0) dev_torn(st, 92, tile);
                 break;
             }
             const unsigned pre = __ballot_sync(0xffffffffu, (x >> 63) != 0);

@@ -2543,13 +2543,14 @@ __device__ __forceinline__ unsigned kd_coord(const float4 *wpos, const float4 *w
 // tiles and members): ranges of more than KD_CTA members at this depth are sorted by the
 // round's axis; smaller ranges keep their order (value 0).  vcur holds every
 // member's slot in the current order.
-__global__ void k_kd_keys(LevelBufs L, NodeArrays nd, const int64_t *seg_base, const float4 *wpos, const float4 *wvel, const unsigned *vcur, unsigned long long *kout,
-                          unsigned *vout, int round, int drop, int key32)
+__global__ void k_kd_keys(LevelBufs L, NodeArrays nd, const int64_t *seg_base, const float4 *wpos, const float4 *wvel,
+                          const unsigned *vcur, unsigned long long *kout, unsigned *vout, int round, int drop,
+                          int key32, const rs_dev_status *st)
 {
     const int k = L.tile_rank[blockIdx.x], q0 = L.tile_q0[blockIdx.x];
     const int node = L.list[k], n = nd.count[node];
     const int p = q0 + threadIdx.x;
-    if (p >= n) return;
+    if (p >= n || dev_is_torn(st)) return;
     const int64_t A = L.seg_off[k] + p;
     const unsigned slot = vcur[A];
     int start = 0, size = n;
@@ -2691,8 +2692,10 @@ __device__ __forceinline__ void kdf_rank(int m, const unsigned short *key, unsig
 }
 
 __global__ void __launch_bounds__(256) k_kd_finish(LevelBufs L, NodeArrays nd, const int4 *ranges, const int *count,
-                                                     const float4 *wpos, const float4 *wvel, unsigned *vals)
+                                                     const float4 *wpos, const float4 *wvel, unsigned *vals,
+                                                     const rs_dev_status *st)
 {
+    if (dev_is_torn(st)) return;
     __shared__ unsigned slot[KD_CTA];
     __shared__ unsigned short rk[KDF_ROUNDS][KD_CTA];
     __shared__ unsigned short key[KD_CTA];
@@ -2777,7 +2780,8 @@ __global__ void __launch_bounds__(256) k_kd_finish(LevelBufs L, NodeArrays nd, c
 
 // members into the sorted order of their node's range
 __global__ void k_kd_place(LevelBufs L, NodeArrays nd, const unsigned *vals, const float4 *wpos, const float4 *wvel,
-                           const int *widx, float4 *wpos2, float4 *wvel2, int *widx2, unsigned *dest)
+                           const int *widx, float4 *wpos2, float4 *wvel2, int *widx2, unsigned *dest,
+                           const rs_dev_status *st)
 {
     const int k = L.tile_rank[blockIdx.x], q0 = L.tile_q0[blockIdx.x];
     const int node = L.list[k], first = nd.first[node], n = nd.count[node];
@@ -2785,6 +2789,7 @@ __global__ void k_kd_place(LevelBufs L, NodeArrays nd, const unsigned *vals, con
     if (p >= n) return;
     const int64_t P = L.seg_off[k] + p;
     const unsigned s = vals[P];
+    if (dev_is_torn(st)) return;
     const int dd = first + p;
     wpos2[dd] = wpos[s];
     wvel2[dd] = wvel[s];
@@ -3146,11 +3151,13 @@ __global__ void k_lvl_keys(LevelBufs L, NodeArrays nd, int *parent, const int *c
 
 __global__ void k_lvl_scatter(LevelBufs L, NodeArrays nd, int64_t LM, const unsigned long long *keys,
                               const unsigned *vals, const float4 *wpos, const float4 *wvel, const int *widx,
-                              float4 *wpos2, float4 *wvel2, int *widx2, unsigned *dest, int rank_shift)
+                              float4 *wpos2, float4 *wvel2, int *widx2, unsigned *dest, int rank_shift,
+                              const rs_dev_status *st)
 {
     int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= LM) return;
     const int k = (int)(keys[p] >> rank_shift);
+    if (dev_is_torn(st)) return;
     const int node = L.list[k];
     const int d = nd.first[node] + (int)(p - L.seg_off[k]);
     const unsigned s = vals[p];
@@ -3161,11 +3168,12 @@ __global__ void k_lvl_scatter(LevelBufs L, NodeArrays nd, int64_t LM, const unsi
 }
 
 __global__ void k_lvl_copyback(int64_t LM, const unsigned *dest, const float4 *wpos2, const float4 *wvel2,
-                               const int *widx2, float4 *wpos, float4 *wvel, int *widx)
+                               const int *widx2, float4 *wpos, float4 *wvel, int *widx, const rs_dev_status *st)
 {
     int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= LM) return;
     const unsigned d = dest[p];
+    if (dev_is_torn(st)) return;
     wpos[d] = wpos2[d];
     wvel[d] = wvel2[d];
     widx[d] = widx2[d];
@@ -3179,7 +3187,7 @@ __global__ void k_lvl_children(LevelBufs L, NodeArrays nd, int64_t LM, const uns
     if (p >= LM) return;
     const unsigned long long key = keys[p];
     const unsigned long long rest = (1ull << cbits) - 1ull, comp = key & rest;
-    if (comp == rest) return;
+    if (comp == rest || dev_is_torn(st)) return;
     if (p > 0 && keys[p - 1] == key) return;
     const int k = (int)(key >> cbits);
     const int node = L.list[k];
@@ -3487,7 +3495,8 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
                 unsigned *va = odd ? v0 : vcur, *vb = odd ? vcur : v1;
                 RS_LAUNCH(ctx, "rf_kd_keys", k_kd_keys, TA, TQ, 0, L, nd, (const int64_t *)O.block,
                           (const float4 *)wpos, (const float4 *)wvel, (const unsigned *)vcur,
-                          (unsigned long long *)k0, odd ? v0 : nullptr, r, drop, key32);
+                          (unsigned long long *)k0, odd ? v0 : nullptr, r, drop, key32,
+                          (const rs_dev_status *)ctx->d_status);
                 bool kalt = false;
                 if (key32)
                     RS_TRY(rs_radix_sort_u32(ctx, (uint32_t *)k0, (uint32_t *)k1, va, vb, NA, kbits, &kalt,
@@ -3504,15 +3513,17 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
             RS_LAUNCH(ctx, "rf_kd_ranges", k_kd_ranges, ceil_div(T * (TQ / 32), 256), 256, 0, L, nd, T, kranges,
                       kcount);
             RS_LAUNCH(ctx, "rf_kd_finish", k_kd_finish, (int64_t)ctx->num_sms * 8, 256, 0, L, nd,
-                      (const int4 *)kranges, (const int *)kcount, (const float4 *)wpos, (const float4 *)wvel, vcur);
+                      (const int4 *)kranges, (const int *)kcount, (const float4 *)wpos, (const float4 *)wvel, vcur,
+                      (const rs_dev_status *)ctx->d_status);
             const unsigned *vsorted = vcur;
             {
                 unsigned *kdest = v0;
                 RS_LAUNCH(ctx, "rf_kd_place", k_kd_place, T, TQ, 0, L, nd, vsorted, (const float4 *)wpos,
-                          (const float4 *)wvel, (const int *)widx, wpos2, wvel2, widx2, kdest);
+                          (const float4 *)wvel, (const int *)widx, wpos2, wvel2, widx2, kdest,
+                          (const rs_dev_status *)ctx->d_status);
                 RS_LAUNCH(ctx, "rf_lvl_copyback", k_lvl_copyback, ceil_div(LM, 256), 256, 0, LM,
                           (const unsigned *)kdest, (const float4 *)wpos2, (const float4 *)wvel2, (const int *)widx2,
-                          wpos, wvel, widx);
+                          wpos, wvel, widx, (const rs_dev_status *)ctx->d_status);
             }
         }
         // bounding-volume hierarchy of every big node
@@ -3662,9 +3673,11 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
         RS_LAUNCH(ctx, "rf_lvl_children", k_lvl_children, ceil_div(LM, 256), 256, 0, L, nd, LM, sk, sv, uf,
                   (const int *)csize, nxt, nxt_len, small_q, ctr + 2, cbits, ctx->d_status);
         RS_LAUNCH(ctx, "rf_lvl_scatter", k_lvl_scatter, ceil_div(LM, 256), 256, 0, L, nd, LM, sk, sv,
-                  (const float4 *)wpos, (const float4 *)wvel, (const int *)widx, wpos2, wvel2, widx2, dest, cbits);
+                  (const float4 *)wpos, (const float4 *)wvel, (const int *)widx, wpos2, wvel2, widx2, dest, cbits,
+                  (const rs_dev_status *)ctx->d_status);
         RS_LAUNCH(ctx, "rf_lvl_copyback", k_lvl_copyback, ceil_div(LM, 256), 256, 0, LM, (const unsigned *)dest,
-                  (const float4 *)wpos2, (const float4 *)wvel2, (const int *)widx2, wpos, wvel, widx);
+                  (const float4 *)wpos2, (const float4 *)wvel2, (const int *)widx2, wpos, wvel, widx,
+                  (const rs_dev_status *)ctx->d_status);
         RS_LAUNCH(ctx, "rf_lvl_tie", k_lvl_store_tie, ceil_div(K, 128), 128, 0, L, nd);
         // next level
         RS_CUDA(ctx, cudaMemsetAsync(cur_len, 0, sizeof(int), ctx->stream));

@@ -8,10 +8,19 @@
 // pass is one launch over tiles of 4096 keys that finds each digit's place by
 // looking back, so a pass reads and writes the data once.
 #include <algorithm>
+#include <cstdlib>
 
 #include "rs_internal.cuh"
 
 namespace {
+
+// tries for a predecessor's word in a look-back (-1 by the injected fault
+// wait_<tag>: as if no predecessor ever came)
+int wait_limit(const char *tag)
+{
+    if (!getenv("RS_FAULT")) return RS_SPIN_LIMIT;
+    return rs_fault((std::string("wait_") + tag).c_str()) ? -1 : RS_SPIN_LIMIT;
+}
 
 constexpr int SCAN_THREADS = 512;
 constexpr int SCAN_ITEMS = 8;
@@ -69,7 +78,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_lookback(T *data, int64_t
 }
 
 template <typename T>
-rs_status scan_top(rs_ctx *ctx, T *data, int64_t n, T *total)
+rs_status scan_top(rs_ctx *ctx, T *data, int64_t n, T *total, const char *tag)
 {
     if (n <= 0) {
         if (total) RS_CUDA(ctx, cudaMemsetAsync(total, 0, sizeof(T), ctx->stream));
@@ -81,7 +90,7 @@ rs_status scan_top(rs_ctx *ctx, T *data, int64_t n, T *total)
     }
     const int64_t tiles = ceil_div(n, SCAN_TILE);
     RsLookback lb;
-    RS_TRY(rs_lookback_init(ctx, tiles, &lb));
+    RS_TRY(rs_lookback_init(ctx, tiles, &lb, tag));
     RS_LAUNCH(ctx, "scan", k_scan_lookback<T>, tiles, SCAN_THREADS, 0, data, n, total, lb, ctx->d_status);
     return RS_OK;
 }
@@ -215,7 +224,7 @@ template <typename K, typename W>
 __global__ void __launch_bounds__(SORT_THREADS, 2) k_sort_pass(const K *kin, K *kout, const uint32_t *vin,
                                                               uint32_t *vout, int64_t n, int shift,
                                                               const uint32_t *hist, W *state, unsigned *next,
-                                                              rs_dev_status *st)
+                                                              int limit, rs_dev_status *st)
 {
     constexpr int WARPS = SORT_THREADS / 32, FB = 8 * (int)sizeof(W) - 2;
     constexpr W SUM = (W)1 << FB, PREFIX = (W)2 << FB, MASK = SUM - 1;
@@ -250,7 +259,8 @@ __global__ void __launch_bounds__(SORT_THREADS, 2) k_sort_pass(const K *kin, K *
             S.lstart[d] = at;
             // eight predecessors a step, their loads in flight together
             W before = 0;
-            bool open = true;
+            bool open = limit >= 0 || tile == 0;
+            if (!open) dev_torn(st, 91, tile);
             for (int64_t t = tile - 1; t >= 0 && open; t -= 8) {
                 W x[8];
 #pragma unroll
@@ -258,9 +268,9 @@ __global__ void __launch_bounds__(SORT_THREADS, 2) k_sort_pass(const K *kin, K *
 #pragma unroll
                 for (int u = 0; u < 8; u++) {
                     if (!open) continue;
-                    for (int it = 0; x[u] == 0 && it < RS_SPIN_LIMIT; it++)
+                    for (int it = 0; x[u] == 0 && it < limit; it++)
                         x[u] = *(const volatile W *)(state + (t - u) * RADIX + d);
-                    if (x[u] == 0) dev_fail(st, DEV_TIMEOUT, 91, tile);
+                    if (x[u] == 0) dev_torn(st, 91, tile);
                     before += x[u] & MASK;
                     open = x[u] != 0 && !(x[u] & PREFIX);
                 }
@@ -285,7 +295,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 2) k_sort_pass(const K *kin, K *
         const K k = S.key[i];
         const uint32_t d = (uint32_t)(k >> shift) & (RADIX - 1);
         const uint32_t pos = S.goff[d] + ((uint32_t)i - S.lstart[d]);
-        if (pos < n) {  // (a look-back that ran out of time leaves wrong places)
+        if (pos < n) {  // (after a look-back that ran out of time places are wrong: see dev_torn)
             kout[pos] = k;
             vout[pos] = S.val[i];
         }
@@ -370,10 +380,11 @@ rs_status sort_passes(rs_ctx *ctx, K *k0, K *k1, uint32_t *v0, uint32_t *v1, int
     RS_CUDA(ctx, cudaFuncSetAttribute(pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortShared<K>)));
     K *ki = k0, *ko = k1;
     uint32_t *vi = v0, *vo = v1;
+    const int limit = wait_limit(tag);
     for (int p = 0; p < passes; p++) {
-        RS_LAUNCH(ctx, pass_name.c_str(), pass, tiles, SORT_THREADS, (int)sizeof(SortShared<K>), (const K *)ki, ko, (const uint32_t *)vi, vo, n,
-                  p * RADIX_BITS, (const uint32_t *)hist + p * RADIX, state + p * tiles * RADIX, next + 64 * p,
-                  ctx->d_status);
+        RS_LAUNCH(ctx, pass_name.c_str(), pass, tiles, SORT_THREADS, (int)sizeof(SortShared<K>), (const K *)ki, ko,
+                  (const uint32_t *)vi, vo, n, p * RADIX_BITS, (const uint32_t *)hist + p * RADIX,
+                  state + p * tiles * RADIX, next + 64 * p, limit, ctx->d_status);
         std::swap(ki, ko);
         std::swap(vi, vo);
         *alt = !*alt;
@@ -411,24 +422,25 @@ bool rs_sort_alt(int64_t n, int nbits)
     return n <= SORT_SMALL || ((nbits + RADIX_BITS - 1) / RADIX_BITS & 1);
 }
 
-rs_status rs_lookback_init(rs_ctx *ctx, int64_t tiles, RsLookback *lb)
+rs_status rs_lookback_init(rs_ctx *ctx, int64_t tiles, RsLookback *lb, const char *tag)
 {
     unsigned long long *w = (unsigned long long *)rs_ws(ctx, WS_SCAN_TMP, sizeof(unsigned long long) * (tiles + 1));
     if (!w) return ctx->fixed_ws ? RS_ERR_INTERNAL : RS_ERR_OOM;
     RS_CUDA(ctx, cudaMemsetAsync(w, 0, sizeof(unsigned long long) * (tiles + 1), ctx->stream));
     lb->next = (unsigned *)w;
     lb->state = w + 1;
+    lb->limit = wait_limit(tag);
     return RS_OK;
 }
 
-rs_status rs_scan_u32(rs_ctx *ctx, uint32_t *data, int64_t n, uint32_t *total)
+rs_status rs_scan_u32(rs_ctx *ctx, uint32_t *data, int64_t n, uint32_t *total, const char *tag)
 {
-    return scan_top<uint32_t>(ctx, data, n, total);
+    return scan_top<uint32_t>(ctx, data, n, total, tag);
 }
 
-rs_status rs_scan_i64(rs_ctx *ctx, int64_t *data, int64_t n, int64_t *total)
+rs_status rs_scan_i64(rs_ctx *ctx, int64_t *data, int64_t n, int64_t *total, const char *tag)
 {
-    return scan_top<long long>(ctx, (long long *)data, n, (long long *)total);
+    return scan_top<long long>(ctx, (long long *)data, n, (long long *)total, tag);
 }
 
 rs_status rs_radix_sort_u64(rs_ctx *ctx, uint64_t *k0, uint64_t *k1, uint32_t *v0, uint32_t *v1, int64_t n,
