@@ -398,8 +398,9 @@ rs_status rs_profile_read(rs_ctx *ctx, int32_t i, const char **name, int64_t *la
 int64_t rs_launch_count(const rs_ctx *ctx);
 /* Bytes of device workspace the context holds now.  The workspace grows to
  * the largest call seen; when the device runs out of memory, the scratch of
- * the 3D FOF and of the group sort is released while neither runs, and the
- * allocation is retried (the 1.07B-particle path relies on this). */
+ * the 3D FOF and of the group sort and the refinement's list of pairs are
+ * released while not in use, and the allocation is retried (the
+ * 1.07B-particle path relies on this). */
 int64_t rs_workspace_bytes(const rs_ctx *ctx);
 
 #ifdef __cplusplus

@@ -193,8 +193,9 @@ bool rs_fault(const char *site)
 }
 
 // Frees the 3D FOF and group-sort slots whose call is not running (their
-// contents are scratch of that call) and the pool's free memory; true if
-// anything was freed.
+// contents are scratch of that call), the pair list while no level uses it
+// (up to 16 GB that a refinement can do without) and the pool's free memory;
+// true if anything was freed.
 static bool release_idle_slots(rs_ctx *c, int keep)
 {
     bool freed = false;
@@ -208,8 +209,9 @@ static bool release_idle_slots(rs_ctx *c, int keep)
     }
     for (int s = 0; s < WS_NUM_SLOTS; s++) {
         const bool fof = s >= WS_FOF_CELLKEY && s <= WS_FOF_ACC;
-        const bool gs = s == WS_GS_COUNT || s == WS_GS_FLAG;
-        if (s == keep || !c->ws_ptr[s] || !((fof && !c->in_fof) || (gs && !c->in_gs))) continue;
+        const bool gs = s == WS_GS_COUNT || s == WS_GS_FLAG, pairs = s == WS_RF_PAIRS;
+        if (s == keep || !c->ws_ptr[s] || !((fof && !c->in_fof) || (gs && !c->in_gs) || (pairs && !c->in_pairs)))
+            continue;
         cudaStreamSynchronize(c->stream);
         if (c->aux) cudaStreamSynchronize(c->aux);
         cudaFree(c->ws_ptr[s]);
@@ -227,6 +229,10 @@ size_t rs_ws_total(const rs_ctx *c)
     return t;
 }
 
+// (by the injected fault "full" the device is out of memory for as long as
+// the pair list is held)
+static bool device_full(const rs_ctx *c) { return c->ws_ptr[WS_RF_PAIRS] && rs_fault("full"); }
+
 cudaError_t rs_block_alloc(rs_ctx *c, void **p, size_t bytes)
 {
     *p = nullptr;
@@ -243,7 +249,7 @@ cudaError_t rs_block_alloc(rs_ctx *c, void **p, size_t bytes)
         uint64_t keep = RS_POOL_KEEP;
         cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep);
     }
-    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, c->pool, c->stream);
+    cudaError_t e = device_full(c) ? cudaErrorMemoryAllocation : cudaMallocFromPoolAsync(p, bytes, c->pool, c->stream);
     if (e == cudaErrorMemoryAllocation && release_idle_slots(c, -1)) {
         cudaGetLastError();
         e = cudaMallocFromPoolAsync(p, bytes, c->pool, c->stream);
@@ -279,7 +285,7 @@ void *rs_ws(rs_ctx *c, int slot, size_t bytes)
     // a little headroom against regrowth (at most 64 MB)
     size_t want = bytes + std::min<size_t>(bytes / 8, (size_t)64 << 20) + 256;
     void *p = nullptr;
-    cudaError_t e = cudaMalloc(&p, want);
+    cudaError_t e = device_full(c) ? cudaErrorMemoryAllocation : cudaMalloc(&p, want);
     if (e == cudaErrorMemoryAllocation && release_idle_slots(c, slot)) {
         cudaGetLastError();
         e = cudaMalloc(&p, want);

@@ -117,7 +117,8 @@ struct rs_ctx {
     int fixed_ws = 0;
     // set while a 3D FOF or group-sort call runs: its slots are in use and
     // must not be released to make room (see rs_ws)
-    int in_fof = 0, in_gs = 0;
+    // (in_pairs: while a level's pair list is in use)
+    int in_fof = 0, in_gs = 0, in_pairs = 0;
     // Pool of the trees and halo tables this context made: their blocks are
     // taken and given back on every call of a loop, and cudaMalloc with
     // cudaFree cost 100 us (1 MB) to 1.7 ms (2.2 GB) a pair, the pool 9 us.
@@ -140,8 +141,8 @@ rs_status rs_fail(rs_ctx *ctx, rs_status s, const std::string &msg);
 rs_status rs_cuda_fail(rs_ctx *ctx, cudaError_t e, const char *where);
 // Device buffer of at least `bytes` for a slot; contents are kept while the
 // slot does not grow.  When the device is out of memory, the slots of the 3D
-// FOF and of the group sort (scratch of those calls only) are released if
-// neither call is running, and the allocation is tried once more.  Returns
+// FOF and of the group sort (scratch of those calls only) and of the pair list
+// are released if not in use, and the allocation is tried once more.  Returns
 // nullptr (and records RS_ERR_OOM) on failure.
 void *rs_ws(rs_ctx *ctx, int slot, size_t bytes);
 // Device memory that outlives the call, from the context's pool, for use on
@@ -153,7 +154,7 @@ void rs_block_free(void *p);
 // Total bytes of the context's workspace slots.
 size_t rs_ws_total(const rs_ctx *ctx);
 
-// Marks a 3D FOF or group-sort call as running for its scope.
+// Marks a 3D FOF or group-sort call as running, or the pair list as used, for its scope.
 struct RsStageGuard {
     int *flag;
     explicit RsStageGuard(int *f) : flag(f) { *flag = 1; }

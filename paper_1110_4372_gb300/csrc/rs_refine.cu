@@ -3589,6 +3589,7 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
         const int64_t chunks = LM * PAIR_PER_MEMBER / PAIR_CHUNK / PAIR_REGIONS + 4;  // per region
         const int64_t pl_bytes = PAIR_REGIONS * chunks * (int64_t)(sizeof(int4) + PAIR_CHUNK * sizeof(int2));
         int pairs = 0;
+        RsStageGuard listed(&ctx->in_pairs);
         if (SS > 0 && pl_bytes <= PAIR_MAX_BYTES) {
             char *pp = (char *)rs_ws(ctx, WS_RF_PAIRS, (size_t)pl_bytes + 1024);
             if (pp) {  // (without the room the nodes are searched twice)
@@ -3651,6 +3652,7 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
         if (pairs)
             RS_LAUNCH(ctx, "rf_pair_link", k_pair_link, (int64_t)ctx->num_sms * 8, 256, 0, L, nd, ms, pl, uf,
                       ctx->d_status);
+        ctx->in_pairs = 0;  // (a release waits for the stream)
         // the other nodes; none when every node has a bracket, every bracket
         // held and every list was whole
         const bool again = (flags[1] & 0xffffffffll) != 0;
