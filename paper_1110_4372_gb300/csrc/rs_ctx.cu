@@ -300,6 +300,15 @@ void *rs_ws(rs_ctx *c, int slot, size_t bytes)
     return p;
 }
 
+void *rs_ws_optional(rs_ctx *c, int slot, size_t bytes, const char *site)
+{
+    if (rs_fault(site)) return nullptr;
+    const std::string before = c->last_error;
+    void *p = rs_ws(c, slot, bytes);
+    if (!p) c->last_error = before;
+    return p;
+}
+
 // ---------------------------------------------------------------------------
 // launch accounting
 // ---------------------------------------------------------------------------

@@ -145,6 +145,9 @@ rs_status rs_cuda_fail(rs_ctx *ctx, cudaError_t e, const char *where);
 // are released if not in use, and the allocation is tried once more.  Returns
 // nullptr (and records RS_ERR_OOM) on failure.
 void *rs_ws(rs_ctx *ctx, int slot, size_t bytes);
+// The same for a buffer that the call can do without: nullptr is no failure and
+// leaves rs_last_error as it was.  (nullptr too by the injected fault `site`)
+void *rs_ws_optional(rs_ctx *ctx, int slot, size_t bytes, const char *site);
 // Device memory that outlives the call, from the context's pool, for use on
 // the context's stream; given back by rs_block_free, from any thread, which
 // waits for the device first as cudaFree does.

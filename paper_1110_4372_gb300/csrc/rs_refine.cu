@@ -3591,7 +3591,7 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
         int pairs = 0;
         RsStageGuard listed(&ctx->in_pairs);
         if (SS > 0 && pl_bytes <= PAIR_MAX_BYTES) {
-            char *pp = (char *)rs_ws(ctx, WS_RF_PAIRS, (size_t)pl_bytes + 1024);
+            char *pp = (char *)rs_ws_optional(ctx, WS_RF_PAIRS, (size_t)pl_bytes + 1024, "pairs");
             if (pp) {  // (without the room the nodes are searched twice)
                 pairs = 1;
                 pl.len = carve<int>(pp, PAIR_REGIONS);
