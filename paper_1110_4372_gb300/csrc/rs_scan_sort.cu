@@ -409,8 +409,9 @@ rs_status radix_sort(rs_ctx *ctx, K *k0, K *k1, uint32_t *v0, uint32_t *v1, int6
         return RS_OK;
     }
     const int passes = (nbits + RADIX_BITS - 1) / RADIX_BITS;
-    // 32-bit states hold counts below 2^30
-    if (n < ((int64_t)1 << 30)) return sort_passes<K, uint32_t>(ctx, k0, k1, v0, v1, n, passes, alt, tag);
+    // 32-bit states hold counts below 2^30 (the injected fault sort64 takes the
+    // 64-bit ones at any size, for the tests)
+    if (n < ((int64_t)1 << 30) && !rs_fault("sort64")) return sort_passes<K, uint32_t>(ctx, k0, k1, v0, v1, n, passes, alt, tag);
     return sort_passes<K, unsigned long long>(ctx, k0, k1, v0, v1, n, passes, alt, tag);
 }
 
