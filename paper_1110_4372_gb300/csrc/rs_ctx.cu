@@ -257,13 +257,6 @@ cudaError_t rs_block_alloc(rs_ctx *c, void **p, size_t bytes)
     return e;
 }
 
-void rs_block_free(void *p)
-{
-    if (!p) return;
-    cudaDeviceSynchronize();  // cudaFree does not wait for a pool's block
-    cudaFree(p);
-}
-
 void *rs_ws(rs_ctx *c, int slot, size_t bytes)
 {
     if (c->ws_size[slot] >= bytes) return c->ws_ptr[slot];

@@ -149,11 +149,10 @@ void *rs_ws(rs_ctx *ctx, int slot, size_t bytes);
 // leaves rs_last_error as it was.  (nullptr too by the injected fault `site`)
 void *rs_ws_optional(rs_ctx *ctx, int slot, size_t bytes, const char *site);
 // Device memory that outlives the call, from the context's pool, for use on
-// the context's stream; given back by rs_block_free, from any thread, which
-// waits for the device first as cudaFree does.
+// the context's stream; given back by rs_block_give_back (rs_block.cuh), from any
+// thread, which waits for the block's device first.
 constexpr unsigned long long RS_POOL_KEEP = 4ull << 30;
 cudaError_t rs_block_alloc(rs_ctx *ctx, void **p, size_t bytes);
-void rs_block_free(void *p);
 // Total bytes of the context's workspace slots.
 size_t rs_ws_total(const rs_ctx *ctx);
 
