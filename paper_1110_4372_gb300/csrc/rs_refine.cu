@@ -2000,7 +2000,11 @@ __device__ __forceinline__ float box_box_d2(const Box6 &a, const Box6 &b, const 
 // way, a few percent of the search.
 //
 // The list is in chunks of PAIR_CHUNK pairs of one leaf, with a head (node
-// rank, first query, pairs), in PAIR_REGIONS regions with a counter each.
+// rank, first query, pairs), in PAIR_REGIONS regions with a counter each.  A
+// block takes its chunks of one region, and of the following ones once that is
+// full: a small level has fewer blocks than regions, and its first leaves list
+// twice the mean (a pair is listed with its first member), so without that a
+// node of 1100 members ran out of room with two thirds of the chunks unused.
 constexpr int PAIR_CHUNK = 64;
 constexpr int PAIR_REGIONS = 64;
 constexpr int PAIR_PER_MEMBER = 20;                  // room for this many pairs a member
@@ -2143,18 +2147,22 @@ __global__ void __launch_bounds__(LK_WARPS * 32, WARPS / LK_WARPS)
     // the last cnt staged pairs to a chunk of the list
     auto put_chunk = [&](int cnt) {
         if constexpr (PAIRS) {
-            const int region = blockIdx.x & (PAIR_REGIONS - 1);
             no -= cnt;
-            int c = 0;
-            if (lane == 0) c = atomicAdd(&P.len[region], 1);
-            c = __shfl_sync(FULLW, c, 0);
-            if (c < P.cap) {
-                const int64_t at = (int64_t)region * P.cap + c;
-                for (int i = lane; i < cnt; i += 32) P.pair[at * PAIR_CHUNK + i] = S.out[no + i];
-                if (lane == 0) P.head[at] = make_int4(k, q0, cnt, 0);
-            } else if (lane == 0) {
-                L.ovf[k] = 1;
+            int at = -1;
+            // (the pairs of a node that ran out are not needed)
+            if (lane == 0 && !__ldcg(&L.ovf[k])) {
+                for (int t = 0; t < PAIR_REGIONS && at < 0; t++) {
+                    const int region = (blockIdx.x + t) & (PAIR_REGIONS - 1);
+                    if (t > 0 && __ldcg(&P.len[region]) >= P.cap) continue;
+                    const int c = atomicAdd(&P.len[region], 1);
+                    if (c < P.cap) at = region * P.cap + c;
+                }
+                if (at >= 0) P.head[at] = make_int4(k, q0, cnt, 0);
+                else L.ovf[k] = 1;
             }
+            at = __shfl_sync(FULLW, at, 0);
+            if (at >= 0)
+                for (int i = lane; i < cnt; i += 32) P.pair[(int64_t)at * PAIR_CHUNK + i] = S.out[no + i];
             __syncwarp();
         }
     };
