@@ -878,9 +878,8 @@ extern "C" rs_status rs_assign_ex(rs_ctx *ctx, const rs_tree *t, const float *po
         if (!hs) return RS_ERR_OOM;
         hs->n_halos = H;
         hs->n_nodes = nn;
-        hs->device = ctx->device;
         const size_t bytes = (size_t)(H + 1) * (4 + 48 + 8 + 8 + 4) + (size_t)(nn + 1) * 4 + 8 * 256;
-        if (rs_block_alloc(ctx, &hs->block, bytes) != cudaSuccess) {
+        if (rs_block_alloc(ctx, &hs->block, &hs->pool, bytes) != cudaSuccess) {
             cudaGetLastError();
             delete hs;
             return rs_fail(ctx, RS_ERR_OOM, "rs_assign: halo table allocation failed");
@@ -917,7 +916,7 @@ extern "C" rs_status rs_assign(rs_ctx *ctx, const rs_tree *t, const float *pos, 
 extern "C" void rs_halos_free(rs_halos *h)
 {
     if (!h) return;
-    rs_block_give_back(h->block, h->device);
+    rs_block_give_back(h->block, h->pool);
     delete h;
 }
 

@@ -146,7 +146,7 @@ extern "C" void rs_destroy(rs_ctx *c)
     cudaStreamSynchronize(c->stream);
     for (int i = 0; i < WS_NUM_SLOTS; i++)
         if (c->ws_ptr[i]) cudaFree(c->ws_ptr[i]);
-    if (c->pool) cudaMemPoolDestroy(c->pool);
+    rs_pool_retire(c->pool);
     if (c->d_status) cudaFree(c->d_status);
     if (c->h_status) cudaFreeHost(c->h_status);
     if (c->h_scratch) cudaFreeHost(c->h_scratch);
@@ -202,9 +202,9 @@ static bool release_idle_slots(rs_ctx *c, int keep)
     if (c->pool) {  // and what the pool keeps free
         uint64_t before = 0, after = 0;
         cudaStreamSynchronize(c->stream);
-        cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrReservedMemCurrent, &before);
-        cudaMemPoolTrimTo(c->pool, 0);
-        cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrReservedMemCurrent, &after);
+        cudaMemPoolGetAttribute(c->pool->mem, cudaMemPoolAttrReservedMemCurrent, &before);
+        cudaMemPoolTrimTo(c->pool->mem, 0);
+        cudaMemPoolGetAttribute(c->pool->mem, cudaMemPoolAttrReservedMemCurrent, &after);
         freed = after < before;
     }
     for (int s = 0; s < WS_NUM_SLOTS; s++) {
@@ -233,26 +233,35 @@ size_t rs_ws_total(const rs_ctx *c)
 // the pair list is held)
 static bool device_full(const rs_ctx *c) { return c->ws_ptr[WS_RF_PAIRS] && rs_fault("full"); }
 
-cudaError_t rs_block_alloc(rs_ctx *c, void **p, size_t bytes)
+cudaError_t rs_block_alloc(rs_ctx *c, void **p, RsPool **pool, size_t bytes)
 {
     *p = nullptr;
+    *pool = nullptr;
     if (!c->pool) {
+        RsPool *made = new (std::nothrow) RsPool();
+        if (!made) return cudaErrorMemoryAllocation;
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = c->device;
-        const cudaError_t e = cudaMemPoolCreate(&c->pool, &props);
+        props.location.id = made->device = c->device;
+        const cudaError_t e = cudaMemPoolCreate(&made->mem, &props);
         if (e != cudaSuccess) {
-            c->pool = nullptr;
+            delete made;
             return e;
         }
         uint64_t keep = RS_POOL_KEEP;
-        cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        cudaMemPoolSetAttribute(made->mem, cudaMemPoolAttrReleaseThreshold, &keep);
+        c->pool = made;
     }
-    cudaError_t e = device_full(c) ? cudaErrorMemoryAllocation : cudaMallocFromPoolAsync(p, bytes, c->pool, c->stream);
+    const cudaMemPool_t mem = c->pool->mem;
+    cudaError_t e = device_full(c) ? cudaErrorMemoryAllocation : cudaMallocFromPoolAsync(p, bytes, mem, c->stream);
     if (e == cudaErrorMemoryAllocation && release_idle_slots(c, -1)) {
         cudaGetLastError();
-        e = cudaMallocFromPoolAsync(p, bytes, c->pool, c->stream);
+        e = cudaMallocFromPoolAsync(p, bytes, mem, c->stream);
+    }
+    if (e == cudaSuccess) {
+        c->pool->holders.fetch_add(1);
+        *pool = c->pool;
     }
     return e;
 }

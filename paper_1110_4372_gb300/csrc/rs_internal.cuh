@@ -12,6 +12,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "rs_block.cuh"
 #include "rsgpu.h"
 
 // NVTX range over a scope: each entry point and stage is named for a
@@ -122,10 +123,10 @@ struct rs_ctx {
     // Pool of the trees and halo tables this context made: their blocks are
     // taken and given back on every call of a loop, and cudaMalloc with
     // cudaFree cost 100 us (1 MB) to 1.7 ms (2.2 GB) a pair, the pool 9 us.
-    // It keeps at most RS_POOL_KEEP bytes
-    // free, gives them up when the device runs out (rs_ws) and with the
-    // context; blocks still in use then live on until they are freed.
-    cudaMemPool_t pool = nullptr;
+    // It keeps at most RS_POOL_KEEP bytes free, gives them up when the device
+    // runs out (rs_ws) and with the context; blocks still in use then, and the
+    // pool with them, live on until they are freed.
+    RsPool *pool = nullptr;
     rs_tuning tune;  // launch choices (rs_set_tuning)
     rs_ctx() { rs_tuning_default(&tune); }
     // second stream and events for copies that overlap the kernels of the
@@ -148,11 +149,11 @@ void *rs_ws(rs_ctx *ctx, int slot, size_t bytes);
 // The same for a buffer that the call can do without: nullptr is no failure and
 // leaves rs_last_error as it was.  (nullptr too by the injected fault `site`)
 void *rs_ws_optional(rs_ctx *ctx, int slot, size_t bytes, const char *site);
-// Device memory that outlives the call, from the context's pool, for use on
-// the context's stream; given back by rs_block_give_back (rs_block.cuh), from any
-// thread, which waits for the block's device first.
+// Device memory that outlives the call, from the context's pool (*pool, which
+// the block then holds), for use on the context's stream; given back by
+// rs_block_give_back, from any thread, which waits for the block's device first.
 constexpr unsigned long long RS_POOL_KEEP = 4ull << 30;
-cudaError_t rs_block_alloc(rs_ctx *ctx, void **p, size_t bytes);
+cudaError_t rs_block_alloc(rs_ctx *ctx, void **p, RsPool **pool, size_t bytes);
 // Total bytes of the context's workspace slots.
 size_t rs_ws_total(const rs_ctx *ctx);
 

@@ -3334,9 +3334,8 @@ static rs_status refine_impl(rs_ctx *ctx, const float *pos, const float *vel, in
     t->n_total = n;
     t->n_members = M;
     t->box = box;
-    t->device = ctx->device;
     const int64_t cap = node_cap;
-    cudaError_t e = rs_block_alloc(ctx, &t->block, tree_bytes(M, cap));
+    cudaError_t e = rs_block_alloc(ctx, &t->block, &t->pool, tree_bytes(M, cap));
     if (e != cudaSuccess) {
         delete t;
         cudaGetLastError();
@@ -3809,7 +3808,7 @@ __global__ void k_fill_i32(int32_t *p, int64_t n, int32_t v)
 extern "C" void rs_tree_free(rs_tree *t)
 {
     if (!t) return;
-    rs_block_give_back(t->block, t->device);
+    rs_block_give_back(t->block, t->pool);
     delete t;
 }
 

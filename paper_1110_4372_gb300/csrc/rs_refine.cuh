@@ -2,7 +2,6 @@
 // refinement kernels (rs_refine.cu) and the assignment (rs_assign.cu).
 #pragma once
 
-#include "rs_block.cuh"
 #include "rs_internal.cuh"
 
 // Node table (structure of arrays, device).  A node's members are the
@@ -26,7 +25,7 @@ struct rs_tree {
     NodeArrays nd{};
     int *members = nullptr;  // particle index per member slot
     void *block = nullptr;   // single device allocation holding everything
-    int device = 0;          // its device
+    RsPool *pool = nullptr;  // whose the allocation is
 };
 
 // Per-halo results of the assignment, kept for the halo-property steps
@@ -41,7 +40,7 @@ struct rs_halos {
     int *root = nullptr;       // root node of the halo's 3D group
     int *leaf_halo = nullptr;  // per tree node: the halo of a seed, -1 for inner nodes
     void *block = nullptr;
-    int device = 0;            // the block's device
+    RsPool *pool = nullptr;    // whose the block is
 };
 
 // Fixed-point scale of the exact moment sums: positions and velocities are

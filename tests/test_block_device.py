@@ -1,6 +1,7 @@
-"""Giving a pool's block back (rs_block.cuh) on a fake CUDA runtime of two
-devices: the wait and the free happen on the block's device, whatever device
-the calling thread has current, which it keeps."""
+"""A context's memory pool and its blocks (rs_block.cuh) on a fake CUDA runtime
+of two devices: the wait and the free of a block happen on the block's device,
+whatever device the calling thread has current, which it keeps; and the pool
+is destroyed by whoever lets go of it last, the context or a block."""
 import os
 import shutil
 import subprocess
@@ -10,6 +11,8 @@ import pytest
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_1110_4372_gb300", "csrc")
 
+# argv: the current device, the pool's device, and letters: a (a block is taken), f (one is given back), n (a null
+# one is), c (the context goes)
 PROGRAM = r"""
 #include <cstdio>
 #include <cstdlib>
@@ -18,14 +21,28 @@ static int current;
 extern "C" {
 cudaError_t cudaGetDevice(int *d) { *d = current; return cudaSuccess; }
 cudaError_t cudaSetDevice(int d) { current = d; return cudaSuccess; }
-cudaError_t cudaDeviceSynchronize() { printf("wait %d,", current); return cudaSuccess; }
-cudaError_t cudaFree(void *) { printf("free %d,", current); return cudaSuccess; }
+cudaError_t cudaDeviceSynchronize() { printf("wait%d ", current); return cudaSuccess; }
+cudaError_t cudaFree(void *) { printf("free%d ", current); return cudaSuccess; }
+cudaError_t cudaMemPoolDestroy(cudaMemPool_t) { printf("destroy "); return cudaSuccess; }
+cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t n) { printf("trim%d ", (int)n); return cudaSuccess; }
+cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void *v)
+{
+    printf("keep%d ", (int)*(unsigned long long *)v);
+    return cudaSuccess;
+}
 }
 int main(int, char **argv)
 {
     current = atoi(argv[1]);
-    rs_block_give_back(argv[3][0] == 'p' ? argv : nullptr, atoi(argv[2]));
-    printf("now %d", current);
+    RsPool *pool = new RsPool();
+    pool->device = atoi(argv[2]);
+    for (const char *s = argv[3]; *s; s++) {
+        if (*s == 'a') pool->holders.fetch_add(1);
+        if (*s == 'f') rs_block_give_back(argv, pool);
+        if (*s == 'n') rs_block_give_back(nullptr, nullptr);
+        if (*s == 'c') rs_pool_retire(pool);
+    }
+    printf("on%d", current);
 }
 """
 
@@ -39,15 +56,22 @@ def program(tmp_path_factory):
     src, exe = d / "block.cpp", d / "block"
     src.write_text(PROGRAM)
     subprocess.run(["g++", "-std=c++17", f"-I{CSRC}", f"-I{cuda}/include", str(src), "-o", str(exe)], check=True)
-    return str(exe)
+    return lambda *a: subprocess.run([str(exe), *map(str, a)], check=True, capture_output=True, text=True).stdout
 
 
 @pytest.mark.parametrize("current,device", [(0, 0), (0, 1), (1, 0), (1, 1)])
 def test_waits_and_frees_on_the_blocks_device(program, current, device):
-    out = subprocess.run([program, str(current), str(device), "p"], check=True, capture_output=True, text=True).stdout
-    assert out == f"wait {device},free {device},now {current}"
+    assert program(current, device, "af") == f"wait{device} free{device} on{current}"
 
 
 def test_nothing_to_free(program):
-    out = subprocess.run([program, "0", "1", "0"], check=True, capture_output=True, text=True).stdout
-    assert out == "now 0"
+    assert program(0, 1, "n") == "on0"
+
+
+@pytest.mark.parametrize("steps,out", [
+    ("c", "keep0 trim0 destroy on0"),
+    ("afc", "wait0 free0 keep0 trim0 destroy on0"),
+    ("aacff", "keep0 trim0 wait0 free0 wait0 free0 destroy on0"),
+    ("aafcf", "wait0 free0 keep0 trim0 wait0 free0 destroy on0")])
+def test_the_last_holder_destroys_the_pool(program, steps, out):
+    assert program(0, 0, steps) == out
