@@ -30,8 +30,11 @@
  *              device status word and reported by the next synchronising call.
  * Sizes.       n < 2^31 (RS_ERR_TOO_LARGE otherwise).  n = 0 is valid.
  * Memory.      The context owns a grow-only device workspace allocated with
- *              cudaMalloc and freed by rs_destroy.  rs_tree objects are owned
- *              by the library and freed by rs_tree_free.
+ *              cudaMalloc and freed by rs_destroy.  rs_tree and rs_halos
+ *              objects are owned by the library and freed by rs_tree_free and
+ *              rs_halos_free, before or after their context; their memory
+ *              comes from a pool of the context, which keeps up to 4 GiB of
+ *              what was freed for the next ones until rs_destroy.
  * Threads.     A context may be used by one host thread at a time.
  */
 #ifndef RSGPU_H
@@ -396,7 +399,8 @@ rs_status rs_profile_read(rs_ctx *ctx, int32_t i, const char **name, int64_t *la
 /* Number of kernel launches issued on the context since the last reset
  * (counted whether or not profiling is enabled). */
 int64_t rs_launch_count(const rs_ctx *ctx);
-/* Bytes of device workspace the context holds now.  The workspace grows to
+/* Bytes of device memory the context holds now: its workspace, and what its
+ * pool keeps free (trees and halo tables not counted).  The workspace grows to
  * the largest call seen; when the device runs out of memory, the scratch of
  * the 3D FOF and of the group sort and the refinement's list of pairs are
  * released while not in use, and the allocation is retried (the

@@ -32,10 +32,11 @@ inline void rs_pool_retire(RsPool *pool)
     rs_pool_release(pool);
 }
 
-// Frees a block of the pool, from any thread.  cudaFree does not wait for such a
-// block and cudaDeviceSynchronize waits for the current device, which in the
-// calling thread may be another one: the block's own is made current for both,
-// and the thread's restored.
+// Frees a block of the pool, from any thread.  Nothing that frees such a block
+// waits for the device and cudaDeviceSynchronize waits for the current one, which
+// in the calling thread may be another: the block's own is made current, and the
+// thread's restored.  (cudaFree gives the block back too, but the pool goes on
+// counting it as used.)
 inline void rs_block_give_back(void *p, RsPool *pool)
 {
     if (!p) return;
@@ -43,7 +44,8 @@ inline void rs_block_give_back(void *p, RsPool *pool)
     cudaGetDevice(&current);
     if (current != pool->device) cudaSetDevice(pool->device);
     cudaDeviceSynchronize();
-    cudaFree(p);
+    cudaFreeAsync(p, 0);
+    cudaStreamSynchronize(0);
     if (current != pool->device) cudaSetDevice(current);
     rs_pool_release(pool);
 }

@@ -396,7 +396,18 @@ extern "C" rs_status rs_profile_read(rs_ctx *c, int32_t i, const char **name, in
 
 extern "C" int64_t rs_launch_count(const rs_ctx *c) { return c ? c->launches : 0; }
 
-extern "C" int64_t rs_workspace_bytes(const rs_ctx *c) { return c ? (int64_t)rs_ws_total(c) : 0; }
+extern "C" int64_t rs_workspace_bytes(const rs_ctx *c)
+{
+    if (!c) return 0;
+    int64_t t = (int64_t)rs_ws_total(c);
+    if (c->pool) {  // and what the pool keeps free
+        uint64_t held = 0, used = 0;
+        cudaMemPoolGetAttribute(c->pool->mem, cudaMemPoolAttrReservedMemCurrent, &held);
+        cudaMemPoolGetAttribute(c->pool->mem, cudaMemPoolAttrUsedMemCurrent, &used);
+        if (held > used) t += (int64_t)(held - used);
+    }
+    return t;
+}
 
 rs_status rs_sync_check(rs_ctx *c, const char *where)
 {

@@ -22,7 +22,8 @@ extern "C" {
 cudaError_t cudaGetDevice(int *d) { *d = current; return cudaSuccess; }
 cudaError_t cudaSetDevice(int d) { current = d; return cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() { printf("wait%d ", current); return cudaSuccess; }
-cudaError_t cudaFree(void *) { printf("free%d ", current); return cudaSuccess; }
+cudaError_t cudaFreeAsync(void *, cudaStream_t) { printf("free%d ", current); return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { printf("done%d ", current); return cudaSuccess; }
 cudaError_t cudaMemPoolDestroy(cudaMemPool_t) { printf("destroy "); return cudaSuccess; }
 cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t n) { printf("trim%d ", (int)n); return cudaSuccess; }
 cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void *v)
@@ -61,7 +62,7 @@ def program(tmp_path_factory):
 
 @pytest.mark.parametrize("current,device", [(0, 0), (0, 1), (1, 0), (1, 1)])
 def test_waits_and_frees_on_the_blocks_device(program, current, device):
-    assert program(current, device, "af") == f"wait{device} free{device} on{current}"
+    assert program(current, device, "af") == f"wait{device} free{device} done{device} on{current}"
 
 
 def test_nothing_to_free(program):
@@ -70,8 +71,8 @@ def test_nothing_to_free(program):
 
 @pytest.mark.parametrize("steps,out", [
     ("c", "keep0 trim0 destroy on0"),
-    ("afc", "wait0 free0 keep0 trim0 destroy on0"),
-    ("aacff", "keep0 trim0 wait0 free0 wait0 free0 destroy on0"),
-    ("aafcf", "wait0 free0 keep0 trim0 wait0 free0 destroy on0")])
+    ("afc", "wait0 free0 done0 keep0 trim0 destroy on0"),
+    ("aacff", "keep0 trim0 wait0 free0 done0 wait0 free0 done0 destroy on0"),
+    ("aafcf", "wait0 free0 done0 keep0 trim0 wait0 free0 done0 destroy on0")])
 def test_the_last_holder_destroys_the_pool(program, steps, out):
     assert program(0, 0, steps) == out
