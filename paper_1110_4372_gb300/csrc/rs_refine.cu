@@ -1957,8 +1957,8 @@ __device__ __forceinline__ int join_friend(int *parent, int a, int b, int rq, rs
 // the few pairs it lets through (about 20 of 1024) are nearly all friends;
 // they are queued and evaluated 32 at a time in full, as float32 differences
 // of the members' own coordinates with the float64 recheck in the band.  A
-// leaf whose box is too large for half precision (or whose l is 0) queues
-// every kept pair instead.
+// leaf whose box is too large for half precision (or whose l is 0, or so small
+// that float32 cannot hold one over it) queues every kept pair instead.
 //
 // Bound by instruction issue and the latency of the dependent walk.  Walking
 // once a leaf instead of once a query cut the link of the 134M-particle path
@@ -2110,7 +2110,8 @@ __global__ void __launch_bounds__(LK_WARPS * 32, WARPS / LK_WARPS)
                                   0.5f * bx.vlo.z + 0.5f * bx.vhi.z, 0.f);
     const float wx = sqrtf(met.ax / lm.part), wv = sqrtf(met.av / lm.part);
     const float rb = sqrtf(point_box_far2(pc, vc, bx, met) / lm.part);
-    brute = !(rb <= LK_RMAX && lm.part < 1e30f);
+    // (weights beyond float32's range would make every product a NaN)
+    brute = !(rb <= LK_RMAX && lm.part < 1e30f && lm.part > 1e-30f);
     if (lane == 0) {
         S.box[0] = bx.plo;
         S.box[1] = bx.phi;
