@@ -475,13 +475,23 @@ def rs_set_tuning(ctx: Context, **fields) -> dict:
 TUNING_FILE = os.path.join(_HERE, "tuning_gb300.json")
 
 
+# What the fields of a tuner record mean: 1 (records without the key) counted
+# the link search's warps per SM as 32, 40 and 48 for 4, 5 and 6, and bracketed
+# the nodes above bracket_min only.
+TUNING_MEANING = 2
+TUNING_CHANGED = {1: ("link_blocks_per_sm", "bracket_min")}
+
+
 def apply_tuning(ctx: Context, path: str = TUNING_FILE) -> dict:
     """Applies the "tuned" table of a tuner record (tune.py --out; by default
     the record of the GB300 run shipped with the package, whose table the
-    library's defaults already equal) to the context."""
+    library's defaults already equal) to the context.  Fields that meant
+    something else when an older record was made keep the context's values."""
     import json
     with open(path) as fh:
-        return rs_set_tuning(ctx, **json.load(fh)["tuned"])
+        rec = json.load(fh)
+    changed = TUNING_CHANGED.get(rec.get("meaning", 1), ())
+    return rs_set_tuning(ctx, **{k: v for k, v in rec["tuned"].items() if k not in changed})
 
 
 def rs_workspace_bytes(ctx: Context) -> int:

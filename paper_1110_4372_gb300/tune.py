@@ -120,9 +120,9 @@ def main(argv=None):
     vel = torch.from_numpy(cat.vel).cuda()
     best, best_ms, base_ms, trials = tune(rsgpu, ctx, pos, vel, cat.box, args.reps, args.sweeps,
                                           log=lambda m: print(m, file=sys.stderr, flush=True))
-    rec = {"device": torch.cuda.get_device_name(0), "workload": args.config, "particles": cat.n,
-           "default": rsgpu.rs_tuning_default(), "default_ms": base_ms, "tuned": best, "tuned_ms": best_ms,
-           "reps": args.reps, "trials": trials}
+    rec = {"meaning": rsgpu.TUNING_MEANING, "device": torch.cuda.get_device_name(0), "workload": args.config,
+           "particles": cat.n, "default": rsgpu.rs_tuning_default(), "default_ms": base_ms, "tuned": best,
+           "tuned_ms": best_ms, "reps": args.reps, "trials": trials}
     text = json.dumps(rec, indent=1)
     if args.out:
         with open(args.out, "w") as fh:
