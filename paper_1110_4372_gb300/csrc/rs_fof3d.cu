@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(FOF_THREADS) k_fof_cells(const float *pos, int
 {
     const unsigned FULL = 0xffffffffu;
     // (for the whole block: other blocks' look-backs may run out meanwhile)
-    if (__syncthreads_or(dev_is_torn(st))) return;
+    if (__syncthreads_or(*(volatile int32_t *)&st->torn)) return;
     const int64_t tile = rs_next_tile(lb);
     const int lane = lane_id();
     const int64_t base = tile * CELL_TILE + (int64_t)warp_id() * 32 * CELL_ROWS;

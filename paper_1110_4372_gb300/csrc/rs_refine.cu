@@ -2559,9 +2559,10 @@ __global__ void k_kd_keys(LevelBufs L, NodeArrays nd, const int64_t *seg_base, c
     const int k = L.tile_rank[blockIdx.x], q0 = L.tile_q0[blockIdx.x];
     const int node = L.list[k], n = nd.count[node];
     const int p = q0 + threadIdx.x;
-    if (p >= n || dev_is_torn(st)) return;
+    if (p >= n) return;
     const int64_t A = L.seg_off[k] + p;
     const unsigned slot = vcur[A];
+    if (dev_is_torn(st)) return;
     int start = 0, size = n;
     for (int i = 0; i < round && size > KD_CTA; i++) {
         const int h = kd_split(size);
@@ -3196,8 +3197,8 @@ __global__ void k_lvl_children(LevelBufs L, NodeArrays nd, int64_t LM, const uns
     if (p >= LM) return;
     const unsigned long long key = keys[p];
     const unsigned long long rest = (1ull << cbits) - 1ull, comp = key & rest;
-    if (comp == rest || dev_is_torn(st)) return;
-    if (p > 0 && keys[p - 1] == key) return;
+    if (comp == rest) return;
+    if ((p > 0 && keys[p - 1] == key) || dev_is_torn(st)) return;
     const int k = (int)(key >> cbits);
     const int node = L.list[k];
     const int r = uf_find(parent, (int)vals[p], st);

@@ -209,7 +209,8 @@ __global__ void __launch_bounds__(HIST_THREADS) k_sort_hist(const K *keys, int64
 // consecutive global slots (coalesced stores).  A digit's place is the count
 // of smaller digits in all keys plus that of its own digit in earlier tiles,
 // which thread d looks back for (W: one word per tile and digit, two flag
-// bits over the count).
+// bits over the count; LIMIT: tries for a word, -1 as if none ever came -- a
+// constant, which as an argument took 7% of a pass).
 template <typename K>
 struct SortShared {
     K key[SORT_TILE];
@@ -220,11 +221,11 @@ struct SortShared {
     unsigned tile;
 };
 
-template <typename K, typename W>
+template <typename K, typename W, int LIMIT>
 __global__ void __launch_bounds__(SORT_THREADS, 2) k_sort_pass(const K *kin, K *kout, const uint32_t *vin,
                                                               uint32_t *vout, int64_t n, int shift,
                                                               const uint32_t *hist, W *state, unsigned *next,
-                                                              int limit, rs_dev_status *st)
+                                                              rs_dev_status *st)
 {
     constexpr int WARPS = SORT_THREADS / 32, FB = 8 * (int)sizeof(W) - 2;
     constexpr W SUM = (W)1 << FB, PREFIX = (W)2 << FB, MASK = SUM - 1;
@@ -259,7 +260,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 2) k_sort_pass(const K *kin, K *
             S.lstart[d] = at;
             // eight predecessors a step, their loads in flight together
             W before = 0;
-            bool open = limit >= 0 || tile == 0;
+            bool open = LIMIT >= 0 || tile == 0;
             if (!open) dev_torn(st, 91, tile);
             for (int64_t t = tile - 1; t >= 0 && open; t -= 8) {
                 W x[8];
@@ -268,7 +269,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 2) k_sort_pass(const K *kin, K *
 #pragma unroll
                 for (int u = 0; u < 8; u++) {
                     if (!open) continue;
-                    for (int it = 0; x[u] == 0 && it < limit; it++)
+                    for (int it = 0; x[u] == 0 && it < LIMIT; it++)
                         x[u] = *(const volatile W *)(state + (t - u) * RADIX + d);
                     if (x[u] == 0) dev_torn(st, 91, tile);
                     before += x[u] & MASK;
@@ -376,15 +377,14 @@ rs_status sort_passes(rs_ctx *ctx, K *k0, K *k1, uint32_t *v0, uint32_t *v1, int
     const int64_t per = rows * std::max<int64_t>(1, n / (rows * ctx->num_sms * 8));
     RS_LAUNCH(ctx, hist_name.c_str(), k_sort_hist<K>, ceil_div(n, per), HIST_THREADS, 4 * passes * RADIX,
               (const K *)k0, n, passes, hist, per);
-    auto pass = k_sort_pass<K, W>;
+    auto pass = wait_limit(tag) < 0 ? k_sort_pass<K, W, -1> : k_sort_pass<K, W, RS_SPIN_LIMIT>;
     RS_CUDA(ctx, cudaFuncSetAttribute(pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortShared<K>)));
     K *ki = k0, *ko = k1;
     uint32_t *vi = v0, *vo = v1;
-    const int limit = wait_limit(tag);
     for (int p = 0; p < passes; p++) {
         RS_LAUNCH(ctx, pass_name.c_str(), pass, tiles, SORT_THREADS, (int)sizeof(SortShared<K>), (const K *)ki, ko,
                   (const uint32_t *)vi, vo, n, p * RADIX_BITS, (const uint32_t *)hist + p * RADIX,
-                  state + p * tiles * RADIX, next + 64 * p, limit, ctx->d_status);
+                  state + p * tiles * RADIX, next + 64 * p, ctx->d_status);
         std::swap(ki, ko);
         std::swap(vi, vo);
         *alt = !*alt;
