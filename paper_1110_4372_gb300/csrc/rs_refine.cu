@@ -2019,6 +2019,19 @@ struct PairList {
     float *dnn;
 };
 
+// a region after a full one with a chunk left, and the chunk (cap when there is
+// none), for a whole warp; the pairs of a node that ran out are not needed
+static __device__ __noinline__ int2 next_chunk(int *len, int cap, const int *ovf, int full)
+{
+    int c = cap, r = full;
+    if (lane_id() == 0 && !__ldcg(ovf))
+        for (int t = 1; t < PAIR_REGIONS && c >= cap; t++) {
+            r = (full + t) & (PAIR_REGIONS - 1);
+            if (__ldcg(&len[r]) < cap) c = atomicAdd(&len[r], 1);
+        }
+    return make_int2(__shfl_sync(0xffffffffu, r, 0), __shfl_sync(0xffffffffu, c, 0));
+}
+
 template <bool PAIRS>
 struct PairStage {
     int2 out[96];  // pairs on their way to the list
@@ -2148,22 +2161,23 @@ __global__ void __launch_bounds__(LK_WARPS * 32, WARPS / LK_WARPS)
     // the last cnt staged pairs to a chunk of the list
     auto put_chunk = [&](int cnt) {
         if constexpr (PAIRS) {
+            int region = blockIdx.x & (PAIR_REGIONS - 1);
             no -= cnt;
-            int at = -1;
-            // (the pairs of a node that ran out are not needed)
-            if (lane == 0 && !__ldcg(&L.ovf[k])) {
-                for (int t = 0; t < PAIR_REGIONS && at < 0; t++) {
-                    const int region = (blockIdx.x + t) & (PAIR_REGIONS - 1);
-                    if (t > 0 && __ldcg(&P.len[region]) >= P.cap) continue;
-                    const int c = atomicAdd(&P.len[region], 1);
-                    if (c < P.cap) at = region * P.cap + c;
-                }
-                if (at >= 0) P.head[at] = make_int4(k, q0, cnt, 0);
-                else L.ovf[k] = 1;
+            int c = 0;
+            if (lane == 0) c = atomicAdd(&P.len[region], 1);
+            c = __shfl_sync(FULLW, c, 0);
+            if (c >= P.cap) {
+                const int2 next = next_chunk(P.len, P.cap, L.ovf + k, region);
+                region = next.x;
+                c = next.y;
             }
-            at = __shfl_sync(FULLW, at, 0);
-            if (at >= 0)
-                for (int i = lane; i < cnt; i += 32) P.pair[(int64_t)at * PAIR_CHUNK + i] = S.out[no + i];
+            if (c < P.cap) {
+                const int64_t at = (int64_t)region * P.cap + c;
+                for (int i = lane; i < cnt; i += 32) P.pair[at * PAIR_CHUNK + i] = S.out[no + i];
+                if (lane == 0) P.head[at] = make_int4(k, q0, cnt, 0);
+            } else if (lane == 0) {
+                L.ovf[k] = 1;
+            }
             __syncwarp();
         }
     };
