@@ -106,9 +106,9 @@ const char *rs_last_error(const rs_ctx *ctx);
  *                       them for the bracket of the linking length, the
  *                       others 256 (>= 1024);
  *   mid_max             subtrees of at most this many members run in the
- *                       128-thread tier, and below 128 in the one-warp tier
- *                       (33-256); larger ones up to 1024 run in the
- *                       256-thread tier;
+ *                       128-thread tier, and of at most 128 of them in the
+ *                       one-warp tier (33-256); larger ones up to 1024 run
+ *                       in the 256-thread tier;
  *   tiny_max            subtrees of at most this many members run in a
  *                       warp's registers (10-32);
  *   small_ctas_per_sm, mid_ctas_per_sm, tiny_ctas_per_sm

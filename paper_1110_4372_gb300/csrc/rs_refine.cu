@@ -407,8 +407,9 @@ __device__ __forceinline__ float4 sv4(const SS &S, int i)
 // pair loops for both rounds and little unrolling: 2.05 -> 1.52 ms), and
 // earlier by the float64 unit, which executes about 2 lanes a clock: what can
 // be is taken from tables, done in float32 with the same rounding, or left to
-// k_tree_stats.  5.0M members in 29,000 groups of 20-600: nodes above 256
-// members 6.9 -> 2.0 ms, 33-256 3.9 -> 2.5 ms (as one 128-thread tier 4.1), up
+// k_tree_stats.  The one-warp tier spills 108 bytes at its 80 registers, the
+// others about 50.  5.0M members in 29,000 groups of 20-600: nodes above 256
+// members 6.9 -> 2.0 ms, 129-256 and 33-128 3.9 -> 2.5 ms (as one 128-thread tier 4.1), up
 // to 32 1.08 -> 0.67 ms.
 template <int NMAX, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
@@ -1964,7 +1965,8 @@ __device__ __forceinline__ int join_friend(int *parent, int a, int b, int rq, rs
 // once a leaf instead of once a query cut the link of the 134M-particle path
 // (7 levels) from 240 to 68 ms, of 9.6M members in independent groups from 46
 // to 13.8 ms, of a 2M path from 4.3 to 0.85 ms.  32 resident warps (64
-// registers) against 40 (48, spilling: 74 ms) and 48 (81 ms).
+// registers, the pair search spilling 40 bytes) against 40 (48 registers and
+// 112 bytes: 74 ms) and 48 (81 ms).
 constexpr int LK_STACK = 256;   // link stack entries per warp
 constexpr int LK_LEAVES = 128;  // pending leaves per warp
 constexpr int LK_RING = 128;    // kept candidates per warp (a ring; 32 are consumed at a time)

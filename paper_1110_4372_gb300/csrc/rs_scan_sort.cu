@@ -2,7 +2,9 @@
 //
 // Scan: one launch.  Up to SCAN_SMALL elements one block loops over them;
 // above, tiles of SCAN_TILE elements in one pass: each tile publishes its sum,
-// looks back over its predecessors' (rs_lookback) and publishes its prefix.
+// looks back over its predecessors' (rs_lookback) and publishes its prefix
+// (decoupled look-back: Merrill & Garland 2016; per digit in a radix sort:
+// Adinets & Merrill 2022).
 // Sort: 8-bit digits.  Up to SORT_SMALL keys one block does all passes in
 // shared memory.  Above, one launch counts the digits of every pass, and each
 // pass is one launch over tiles of 4096 keys that finds each digit's place by
